@@ -231,6 +231,22 @@ static Inst make_inst(const Params& P) {
     // shifted by up to 21 bits, or a 33-bit noise integer times one shifted
     // by up to 40
     I.ou_int = (I.stn_s <= I.ctm1_s) ? (I.ctm1_s - I.stn_s <= 40) : (I.stn_s - I.ctm1_s <= 21);
+    // the shifts that bring the products' scale to 2^-64 (the operand keeps
+    // two spare bits)
+    auto pre = [](int s, int& t, long long& lim) {
+        t = 64 - s;
+        lim = (t >= 0 && t <= 40) ? 1ll << (61 - t) : 0;
+        if (lim == 0) t = 0;
+    };
+    pre(I.hm8_s, I.hm8_t, I.hm8_lim);
+    pre(I.hdt_s, I.hdt_t, I.hdt_lim);
+    I.ou_vt = 64 - I.ctm1_s;
+    I.ou_nt = 64 - I.stn_s;
+    // (the noise integer has 33 bits)
+    const bool ou64 = I.ou_int && I.ou_vt >= 0 && I.ou_vt <= 40 && I.ou_nt >= 0 && I.ou_nt <= 28;
+    I.ou_lim = ou64 ? 1ll << (61 - I.ou_vt) : 0;
+    if (!ou64) I.ou_vt = I.ou_nt = 0;
+    I.rot = rot_constants(0.5 * h, I.h_i_d, I.cr_m1_d, I.srn_d);
     I.h_m = (float)I.h_m_d; I.h_i = (float)I.h_i_d; I.hdt = (float)I.hdt_d;
     I.ct_m1 = (float)I.ct_m1_d; I.cr_m1 = (float)I.cr_m1_d; I.st = (float)I.st_d; I.sr = (float)I.sr_d;
     I.mass = P.mass; I.inertia = P.inertia;
@@ -317,6 +333,7 @@ void Ensemble::alloc_core(const std::vector<int>& p0, const std::vector<int>& k0
     d_grank = alloc<unsigned char>(N);
     d_dmax = alloc<unsigned>(B);
     d_fbcount = alloc<int>(1);
+    d_rot_n = alloc<int>(1);
     d_adjpad = alloc<int>((size_t)Ktot * 64);
     d_seglist = alloc<int>((size_t)2 * Ktot);
     d_seglist_n = alloc<int>(2);

@@ -313,6 +313,7 @@ public:
     float4* d_cnorm = nullptr;               // [Ktot] cell normals (pair-kernel frames)
     unsigned char* d_grank = nullptr;        // [N] pair-kernel group ranks
     unsigned* d_dmax = nullptr;              // [B] largest centroid move of the last M-step (float bits)
+    int* d_rot_n = nullptr;                  // lipids whose rotation the fixed-point update left to FP64
     int* d_fbcount = nullptr;                // particles the certified E-step left to the grid search
     int* d_adjpad = nullptr;                 // [Ktot][64] neighbouring-cell rows before compaction
     int* d_seglist = nullptr;                // [2][Ktot] cells for the block sort / the rank sort

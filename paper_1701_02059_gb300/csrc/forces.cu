@@ -1285,7 +1285,8 @@ template <int Z, bool S0, bool D>
 __global__ void __launch_bounds__(128, 4)
     k_pair_eval_step(View v, View o, const int* __restrict__ nlist, const int* __restrict__ ncnt, int cap,
                      const int4* __restrict__ rowoff, unsigned char* __restrict__ sflag,
-                     const long long* __restrict__ steps, long long* __restrict__ msum, int* __restrict__ mcnt) {
+                     const long long* __restrict__ steps, long long* __restrict__ msum, int* __restrict__ mcnt,
+                     int* __restrict__ rot_list, int* __restrict__ rot_n) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned live = __ballot_sync(0xffffffffu, q < v.N);
     if (q >= v.N) return;
@@ -1323,7 +1324,7 @@ __global__ void __launch_bounds__(128, 4)
     }
     for (int a = 0; a < 3; a++) { v.F[a * N + pi] = F[a]; v.T[a * N + pi] = Tq[a]; }
     __syncwarp(live);
-    if (D) baoa_d_body<true>(v, o, pi, F, Tq, steps, msum, mcnt, live, true);
+    if (D) baoa_d_body<true>(v, o, pi, F, Tq, steps, msum, mcnt, live, true, rot_list, rot_n);
     else baoa_body<float, true>(v, o, pi, F, Tq, steps, msum, mcnt, live, true);
 }
 
@@ -1600,7 +1601,8 @@ void Ensemble::launch_pairs_step(bool msums) {
     const int ng = (int)((N + 127) / 128);
     const bool d = !step_f32();
 #define ORBC_EVAL_STEP(Z, S, D) \
-    k_pair_eval_step<Z, S, D><<<ng, 128, 0, stream>>>(v, o, d_nlist, d_ncnt, list_cap, d_rowoff, d_sflag, d_step, ms, mc)
+    k_pair_eval_step<Z, S, D><<<ng, 128, 0, stream>>>(v, o, d_nlist, d_ncnt, list_cap, d_rowoff, d_sflag, d_step, ms, mc, \
+                                                     d_cell_tmp, d_rot_n)
     if (z4 && s0z) { if (d) ORBC_EVAL_STEP(4, false, true); else ORBC_EVAL_STEP(4, false, false); }
     else if (z4) { if (d) ORBC_EVAL_STEP(4, true, true); else ORBC_EVAL_STEP(4, true, false); }
     else { if (d) ORBC_EVAL_STEP(0, true, true); else ORBC_EVAL_STEP(0, true, false); }
@@ -1608,8 +1610,12 @@ void Ensemble::launch_pairs_step(bool msums) {
     launches++;
     CK(cudaGetLastError());
     toc();
+    if (d) {
+        k_rot_rest<<<152, 128, 0, stream>>>(v, o, d_step, 1, d_cell_tmp, d_rot_n);
+        launches++;
+    }
     swap_state();
-    k_step_advance<<<1, 64, 0, stream>>>(d_step, B);
+    k_step_advance<<<1, 64, 0, stream>>>(d_step, B, 1, d_rot_n);
     launches++;
     CK(cudaGetLastError());
     forces_valid = false;   // F and T belong to the positions before the update

@@ -29,39 +29,72 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 4) k_baoa(View v, co
     baoa_body<T, FUSED>(v, v, p, F, Tq, steps, msum, mcnt, __activemask(), false);
 }
 
+// FP64-accurate increments on the integer pipes.  With the rotation in FP64
+// the kernel was bound by the FP64 pipe (85% busy): 0.81 ms on the 4M cell,
+// against 0.14 ms for its 240 B per particle at the copy bandwidth; with the
+// fixed-point rotation it is bound by integer issue: 0.47 ms with
+// k_rot_rest.  Four CTAs per SM (64 registers, some spilled) against 0.48 ms
+// at three.
 template <bool FUSED>
-__global__ void __launch_bounds__(256, 3) k_baoa_d(View v, const long long* __restrict__ steps,
-                                                   long long* __restrict__ msum, int* __restrict__ mcnt) {
+__global__ void __launch_bounds__(256, 4) k_baoa_d(View v, const long long* __restrict__ steps,
+                                                   long long* __restrict__ msum, int* __restrict__ mcnt,
+                                                   int* __restrict__ rot_list, int* __restrict__ rot_n) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= v.N) return;
     const size_t N = v.N;
     long long F[3], Tq[3];
     for (int a = 0; a < 3; a++) { F[a] = v.F[a * N + p]; Tq[a] = v.T[a * N + p]; }
-    baoa_d_body<FUSED>(v, v, p, F, Tq, steps, msum, mcnt, __activemask(), false);
+    baoa_d_body<FUSED>(v, v, p, F, Tq, steps, msum, mcnt, __activemask(), false, rot_list, rot_n);
 }
 
-__global__ void k_kick_d(View v, long long* __restrict__ steps) {
+// The rotational update in FP64 of the lipids that k_baoa_d (or the
+// evaluation with the update in its epilogue) listed: from the state of v
+// into the state arrays of o.  About 1e-3 of the lipids; taken inside
+// k_baoa_d, 4% of its warps would wait for one lane's FP64 code (0.49-0.50
+// against 0.47 ms for both launches on the 4M cell).
+__global__ void __launch_bounds__(128) k_rot_rest(View v, View o, const long long* __restrict__ steps, int fused,
+                                                  const int* __restrict__ rot_list, const int* __restrict__ rot_n) {
+    const int n = *rot_n;
+    const size_t N = v.N;
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+        const int p = rot_list[q];
+        const int b = find_inst(v.inst_p0, v.B, p);
+        const Inst& I = v.inst[b];
+        const unsigned id = (unsigned)I.id_base + v.id[p];
+        const unsigned long long step = (unsigned long long)steps[b] + (fused ? 1ull : 0ull);
+        const uint2 key = make_uint2((unsigned)I.seed, (unsigned)(I.seed >> 32) ^ I.instance);
+        const uint4 w1 = philox4x32_10(make_uint4(id, (unsigned)step, (unsigned)(step >> 32), 1u), key);
+        rot_fp64(v.nq + p, v.wq + p, o.nq + p, o.wq + p, N, I, fused ? 2 : 1, v.T[p], v.T[N + p], v.T[2 * N + p], w1);
+    }
+}
+
+__global__ void __launch_bounds__(256) k_kick_d(View v, long long* __restrict__ steps) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= v.N) return;
     const int b = find_inst(v.inst_p0, v.B, p);
     const Inst& I = v.inst[b];
     const size_t N = v.N;
-    const bool lipid = bilayer(v.type[p]);
-    long long vq[3], wq[3] = {0, 0, 0};
-    double Nd[3] = {0.0, 0.0, 0.0};
-    for (int a = 0; a < 3; a++) vq[a] = v.vq[a * N + p];
-    if (lipid) for (int a = 0; a < 3; a++) { Nd[a] = gd(v.nq[a * N + p]); wq[a] = v.wq[a * N + p]; }
-    long long F[3], Tq[3];
-    for (int a = 0; a < 3; a++) { F[a] = v.F[a * N + p]; Tq[a] = v.T[a * N + p]; }
-    kick_grid(vq, wq, Nd, lipid, I, 1, F, Tq);
-    for (int a = 0; a < 3; a++) v.vq[a * N + p] = vq[a];
-    if (lipid) for (int a = 0; a < 3; a++) v.wq[a * N + p] = wq[a];
+    for (int a = 0; a < 3; a++)
+        v.vq[a * N + p] += mul_round_pre(v.F[a * N + p], I.hm8_m, I.hm8_s, I.hm8_t, I.hm8_lim);
+    if (bilayer(v.type[p])) {
+        long long nq[3], wq[3], Tq[3];
+        for (int a = 0; a < 3; a++) { nq[a] = v.nq[a * N + p]; wq[a] = v.wq[a * N + p]; Tq[a] = v.T[a * N + p]; }
+        if (!(I.rot.ok && dir_ok(nq) && rot_kick(wq, dir_of(nq), Tq, I.rot, 1))) {
+            const double Nd[3] = {gd(nq[0]), gd(nq[1]), gd(nq[2])};
+            for (int a = 0; a < 3; a++) wq[a] = v.wq[a * N + p];
+            kick_rot_grid(wq, Nd, I, 1, Tq);
+        }
+        for (int a = 0; a < 3; a++) v.wq[a * N + p] = wq[a];
+    }
     if (p == I.p0) steps[b] += 1;
 }
 
-// Counts the previous step after a fused launch read the counters.
-__global__ void k_step_advance(long long* __restrict__ steps, int B) {
-    for (int b = threadIdx.x; b < B; b += blockDim.x) steps[b] += 1;
+// After a B-A-O-A: counts the previous step once a fused launch has read the
+// counters, and empties the list of left-over rotations.
+__global__ void k_step_advance(long long* __restrict__ steps, int B, int fused, int* __restrict__ rot_n) {
+    for (int b = threadIdx.x; b < B; b += blockDim.x)
+        if (fused) steps[b] += 1;
+    if (threadIdx.x == 0) *rot_n = 0;
 }
 
 // Final B of the step; advances the step counter of every instance.
@@ -195,12 +228,15 @@ void Ensemble::launch_integrate_first(bool fused, bool msums) {
         if (fused) k_baoa<float, true><<<nblk(N, 256), 256, 0, stream>>>(view(), d_step, ms, mc);
         else k_baoa<float, false><<<nblk(N, 256), 256, 0, stream>>>(view(), d_step, ms, mc);
     } else {
-        if (fused) k_baoa_d<true><<<nblk(N, 256), 256, 0, stream>>>(view(), d_step, ms, mc);
-        else k_baoa_d<false><<<nblk(N, 256), 256, 0, stream>>>(view(), d_step, ms, mc);
+        // (the left-over list shares the E-step's, which the rebuild uses later)
+        if (fused) k_baoa_d<true><<<nblk(N, 256), 256, 0, stream>>>(view(), d_step, ms, mc, d_cell_tmp, d_rot_n);
+        else k_baoa_d<false><<<nblk(N, 256), 256, 0, stream>>>(view(), d_step, ms, mc, d_cell_tmp, d_rot_n);
+        k_rot_rest<<<152, 128, 0, stream>>>(view(), view(), d_step, fused, d_cell_tmp, d_rot_n);
+        launches++;
     }
     launches++;
-    if (fused) {
-        k_step_advance<<<1, 64, 0, stream>>>(d_step, B);
+    if (fused || !step_f32()) {
+        k_step_advance<<<1, 64, 0, stream>>>(d_step, B, fused, d_rot_n);
         launches++;
     }
     CK(cudaGetLastError());

@@ -240,18 +240,26 @@ __device__ inline long long mul_round(long long q, unsigned long long m, int s) 
     return q < 0 ? -(long long)r : (long long)r;
 }
 
-// Half kick(s): v += round(h_m 2^8 F), w += round(h_i 2^8 (T - (T.n) n)) in
-// grid units, with N the director in grid units.
-__device__ inline void kick_grid(long long vq[3], long long wq[3], const double N[3], bool lipid, const Inst& I,
-                                 int reps, const long long F[3], const long long Tq[3]) {
-    for (int a = 0; a < 3; a++) vq[a] += reps * mul_round(F[a], I.hm8_m, I.hm8_s);
-    if (lipid) {
-        const double T0 = gd(Tq[0]), T1 = gd(Tq[1]), T2 = gd(Tq[2]);
-        const double u = (T0 * N[0] + T1 * N[1] + T2 * N[2]) * 8.271806125530277e-25;   // (T.N) 2^-80
-        wq[0] += reps * rg(I.hi8_d * (T0 - u * N[0]));
-        wq[1] += reps * rg(I.hi8_d * (T1 - u * N[1]));
-        wq[2] += reps * rg(I.hi8_d * (T2 - u * N[2]));
-    }
+// round(q m 2^-s) as mul_round, with q << t (t = 64 - s, |q| <= lim) so that
+// the product's upper word is the floor and its lower word decides the
+// rounding: no variable 128-bit shift.  Anything else takes mul_round.
+static __device__ __noinline__ long long mul_round_any(long long q, unsigned long long m, int s) { return mul_round(q, m, s); }
+__device__ inline long long mul_round_pre(long long q, unsigned long long m, int s, int t, long long lim) {
+    if (lim == 0 || !below(q, lim)) return mul_round_any(q, m, s);
+    const long long a = q << t;
+    const long long hi = __mul64hi(a, (long long)m);      // m < 2^54
+    const unsigned long long lo = (unsigned long long)a * m, half = 1ull << 63;
+    return hi + ((lo > half || (lo == half && (hi & 1))) ? 1 : 0);
+}
+
+// Rotational half of the half kick(s) in FP64: w += round(h_i 2^8 (T - (T.n)
+// n)) in grid units, with N the director in grid units.
+__device__ inline void kick_rot_grid(long long wq[3], const double N[3], const Inst& I, int reps, const long long Tq[3]) {
+    const double T0 = gd(Tq[0]), T1 = gd(Tq[1]), T2 = gd(Tq[2]);
+    const double u = (T0 * N[0] + T1 * N[1] + T2 * N[2]) * 8.271806125530277e-25;   // (T.N) 2^-80
+    wq[0] += reps * rg(I.hi8_d * (T0 - u * N[0]));
+    wq[1] += reps * rg(I.hi8_d * (T1 - u * N[1]));
+    wq[2] += reps * rg(I.hi8_d * (T2 - u * N[2]));
 }
 
 // Cayley increment of the director in grid units: a = (dt/4 2^-40) W,
@@ -302,11 +310,62 @@ __device__ inline double noise_int(unsigned w) {
     return (double)(2 * (long long)(int)(w ^ 0x80000000u) + 1);
 }
 
-// The same with FP64 increments in grid units.
+// round((exp(-gamma dt) - 1) v + s z), the exact sum of the two products
+static __device__ __noinline__ long long ou_any(long long vq, long long z, const Inst& I) {
+    return I.ou_int ? mul2_round(vq, I.ctm1_m, I.ctm1_s, z, I.stn_m, I.stn_s)
+                    : rg(fma(I.ct_m1_d, gd(vq), I.stn_d * (double)z));
+}
+__device__ inline long long ou_increment(long long vq, long long z, const Inst& I) {
+    if (I.ou_lim == 0 || !below(vq, I.ou_lim)) return ou_any(vq, z, I);
+    // both scales at 2^-64 (see mul_round_pre)
+    const unsigned __int128 t = (unsigned __int128)((__int128)(vq << I.ou_vt) * I.ctm1_m) +
+                                (unsigned __int128)((__int128)(z << I.ou_nt) * I.stn_m);
+    const long long hi = (long long)(unsigned long long)(t >> 64);
+    const unsigned long long lo = (unsigned long long)t, half = 1ull << 63;
+    return hi + ((lo > half || (lo == half && (hi & 1))) ? 1 : 0);
+}
+
+// The rotational B-A-O-A of one lipid in FP64 (director and angular velocity
+// ni, wi to no, wo, axis stride N): for the values that the fixed-point code
+// leaves to it.
+static __device__ __noinline__ void rot_fp64(const long long* ni, const long long* wi, long long* no, long long* wo,
+                                             size_t N, const Inst& I, int reps, long long T0, long long T1,
+                                             long long T2, uint4 noise) {
+    const long long Tq[3] = {T0, T1, T2};
+    long long nq[3], wq[3], d[3];
+    double Nd[3], Wd[3];
+    for (int a = 0; a < 3; a++) { nq[a] = ni[a * N]; wq[a] = wi[a * N]; Nd[a] = gd(nq[a]); }
+    kick_rot_grid(wq, Nd, I, reps, Tq);
+    for (int a = 0; a < 3; a++) Wd[a] = gd(wq[a]);
+    cayley_grid(Nd, Wd, I, d);
+    for (int a = 0; a < 3; a++) { nq[a] += d[a]; Nd[a] = gd(nq[a]); }
+    // the noise scaled by sr first: its projection is linear
+    const double r0 = I.srn_d * noise_int(noise.x), r1 = I.srn_d * noise_int(noise.y), r2 = I.srn_d * noise_int(noise.z);
+    const double u = (r0 * Nd[0] + r1 * Nd[1] + r2 * Nd[2]) * 8.271806125530277e-25;   // (r.N) 2^-80
+    const double rp[3] = {r0 - u * Nd[0], r1 - u * Nd[1], r2 - u * Nd[2]};
+    for (int a = 0; a < 3; a++) {
+        wq[a] += rg(fma(I.cr_m1_d, Wd[a], rp[a]));
+        Wd[a] = gd(wq[a]);
+    }
+    cayley_grid(Nd, Wd, I, d);
+    for (int a = 0; a < 3; a++) { nq[a] += d[a]; Nd[a] = gd(nq[a]); }
+    // unit-norm correction n <- n (1 - delta/2), delta = |n|^2 - 1, with
+    // |N|^2 - 2^80 exact in 128-bit integer arithmetic and delta/2 = that
+    // 2^-81, one conversion and one product
+    const double hdelta = gd(norm2_excess(nq)) * 4.1359030627651384e-25;   // 2^-81
+    for (int a = 0; a < 3; a++) nq[a] -= rg(Nd[a] * hdelta);
+    for (int a = 0; a < 3; a++) { no[a * N] = nq[a]; wo[a * N] = wq[a]; }
+}
+
+// The same with FP64-accurate increments in grid units, all of them on the
+// integer pipes: the translational products exact (mul_round), the rotation
+// in fixed point (rotation.cuh); the lipids whose rotation it leaves to FP64
+// go to rot_list (n and w untouched) for k_rot_rest.
 template <bool FUSED>
 __device__ inline void baoa_d_body(const View& v, const View& o, int p, const long long F[3], const long long Tq[3],
                                    const long long* __restrict__ steps, long long* __restrict__ msum,
-                                   int* __restrict__ mcnt, unsigned mask, bool copy_static) {
+                                   int* __restrict__ mcnt, unsigned mask, bool copy_static,
+                                   int* __restrict__ rot_list, int* __restrict__ rot_n) {
     const int b = find_inst(v.inst_p0, v.B, p);
     const Inst& I = v.inst[b];
     const size_t N = v.N;
@@ -315,63 +374,52 @@ __device__ inline void baoa_d_body(const View& v, const View& o, int p, const lo
     long long xq[3], vq[3], nq[3] = {0, 0, 0}, wq[3] = {0, 0, 0};
     for (int a = 0; a < 3; a++) { xq[a] = v.xq[a * N + p]; vq[a] = v.vq[a * N + p]; }
     if (lipid) for (int a = 0; a < 3; a++) { nq[a] = v.nq[a * N + p]; wq[a] = v.wq[a * N + p]; }
-    double Nd[3] = {0.0, 0.0, 0.0};
-    if (lipid) for (int a = 0; a < 3; a++) Nd[a] = gd(nq[a]);
-    // (final B of the previous step), B
-    kick_grid(vq, wq, Nd, lipid, I, FUSED ? 2 : 1, F, Tq);
-    // A
-    double Wd[3] = {0.0, 0.0, 0.0};
-    for (int a = 0; a < 3; a++) xq[a] += mul_round(vq[a], I.hdt_m, I.hdt_s);
-    if (lipid) {
-        for (int a = 0; a < 3; a++) Wd[a] = gd(wq[a]);
-        long long d[3];
-        cayley_grid(Nd, Wd, I, d);
-        for (int a = 0; a < 3; a++) { nq[a] += d[a]; Nd[a] = gd(nq[a]); }
-    }
-    // O
     const unsigned id = (unsigned)I.id_base + v.id[p];   // the id in the membrane
     const unsigned long long step = (unsigned long long)steps[b] + (FUSED ? 1ull : 0ull);
     const uint2 key = make_uint2((unsigned)I.seed, (unsigned)(I.seed >> 32) ^ I.instance);
-    const uint4 w0 = philox4x32_10(make_uint4(id, (unsigned)step, (unsigned)(step >> 32), 0u), key);
-    const unsigned wv[3] = {w0.x, w0.y, w0.z};
-    for (int a = 0; a < 3; a++) {
-        const long long sn = 2 * (long long)(int)(wv[a] ^ 0x80000000u) + 1;   // the noise's exact integer
-        vq[a] += I.ou_int ? mul2_round(vq[a], I.ctm1_m, I.ctm1_s, sn, I.stn_m, I.stn_s)
-                          : rg(fma(I.ct_m1_d, gd(vq[a]), I.stn_d * (double)sn));
-    }
-    if (lipid) {
-        const uint4 w1 = philox4x32_10(make_uint4(id, (unsigned)step, (unsigned)(step >> 32), 1u), key);
-        // the noise scaled by sr first: its projection is linear
-        const double r0 = I.srn_d * noise_int(w1.x), r1 = I.srn_d * noise_int(w1.y), r2 = I.srn_d * noise_int(w1.z);
-        const double u = (r0 * Nd[0] + r1 * Nd[1] + r2 * Nd[2]) * 8.271806125530277e-25;   // (r.N) 2^-80
-        const double rp[3] = {r0 - u * Nd[0], r1 - u * Nd[1], r2 - u * Nd[2]};
+    const int reps = FUSED ? 2 : 1;      // (final B of the previous step), B
+    {
+        const uint4 w0 = philox4x32_10(make_uint4(id, (unsigned)step, (unsigned)(step >> 32), 0u), key);
+        const unsigned wv[3] = {w0.x, w0.y, w0.z};
         for (int a = 0; a < 3; a++) {
-            const long long d = rg(fma(I.cr_m1_d, Wd[a], rp[a]));
-            wq[a] += d;
-            Wd[a] = gd(wq[a]);
+            vq[a] += reps * mul_round_pre(F[a], I.hm8_m, I.hm8_s, I.hm8_t, I.hm8_lim);
+            xq[a] += mul_round_pre(vq[a], I.hdt_m, I.hdt_s, I.hdt_t, I.hdt_lim);
+            vq[a] += ou_increment(vq[a], 2 * (long long)(int)(wv[a] ^ 0x80000000u) + 1, I);
+            xq[a] += mul_round_pre(vq[a], I.hdt_m, I.hdt_s, I.hdt_t, I.hdt_lim);
         }
     }
-    // A
-    for (int a = 0; a < 3; a++) xq[a] += mul_round(vq[a], I.hdt_m, I.hdt_s);
-    if (lipid) {
-        long long d[3];
-        cayley_grid(Nd, Wd, I, d);
-        for (int a = 0; a < 3; a++) { nq[a] += d[a]; Nd[a] = gd(nq[a]); }
-        // unit-norm correction n <- n (1 - delta/2), delta = |n|^2 - 1, with
-        // |N|^2 - 2^80 exact in 128-bit integer arithmetic (integer pipes)
-        // and delta/2 = that 2^-81, one conversion and one product
-        const double hdelta = gd(norm2_excess(nq)) * 4.1359030627651384e-25;   // 2^-81
-        for (int a = 0; a < 3; a++) nq[a] -= rg(Nd[a] * hdelta);
-    }
     for (int a = 0; a < 3; a++) { o.xq[a * N + p] = xq[a]; o.vq[a * N + p] = vq[a]; }
-    // in place a protein's (zero) director and angular velocity need no
-    // store; into the other buffer, whose slot held another particle, they do
-    if (lipid || copy_static) for (int a = 0; a < 3; a++) { o.nq[a * N + p] = nq[a]; o.wq[a * N + p] = wq[a]; }
-    if (copy_static) { o.type[p] = type; o.id[p] = v.id[p]; }
     if (msum) mstep_sums(v, I, p, centroid_member(I, type), xq, msum, mcnt, mask);
+    if (lipid) {
+        const uint4 w1 = philox4x32_10(make_uint4(id, (unsigned)step, (unsigned)(step >> 32), 1u), key);
+        const unsigned zw[3] = {w1.x, w1.y, w1.z};
+        if (!I.rot.ok) {
+            rot_fp64(v.nq + p, v.wq + p, o.nq + p, o.wq + p, N, I, reps, Tq[0], Tq[1], Tq[2], w1);
+        } else {
+            bool ok = dir_ok(nq);
+            if (ok) {
+                Dir d = dir_of(nq);
+                ok = rot_kick(wq, d, Tq, I.rot, reps) && rot_turn(nq, d, wq, I.rot);
+                if (ok) {
+                    d = dir_of(nq);
+                    ok = rot_noise(wq, d, zw, I.rot) && rot_turn(nq, d, wq, I.rot) && rot_renorm(nq);
+                }
+            }
+            // the few left over run together in k_rot_rest: in here each
+            // would hold its warp for the length of the FP64 code
+            if (ok) for (int a = 0; a < 3; a++) { o.nq[a * N + p] = nq[a]; o.wq[a * N + p] = wq[a]; }
+            else rot_list[atomicAdd(rot_n, 1)] = p;
+        }
+    } else if (copy_static) {
+        // in place a protein's (zero) director and angular velocity need no
+        // store; into the other buffer, whose slot held another particle, they do
+        for (int a = 0; a < 3; a++) { o.nq[a * N + p] = 0; o.wq[a * N + p] = 0; }
+    }
+    if (copy_static) { o.type[p] = type; o.id[p] = v.id[p]; }
 }
 
-// Counts the previous step after a fused launch read the counters.
-__global__ void k_step_advance(long long* __restrict__ steps, int B);
+__global__ void k_step_advance(long long* __restrict__ steps, int B, int fused, int* __restrict__ rot_n);
+__global__ void k_rot_rest(View v, View o, const long long* __restrict__ steps, int fused,
+                           const int* __restrict__ rot_list, const int* __restrict__ rot_n);
 
 }  // namespace orbc

@@ -16,6 +16,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "rotation.cuh"
+
 namespace orbc {
 
 constexpr int kGridShift = 40;                       // state: 2^-40
@@ -93,6 +95,13 @@ struct Inst {
     // (ou_int), else in FP64
     long long ctm1_m, stn_m;
     int ctm1_s, stn_s, ou_int;
+    // the same products with the shift taken on the 64-bit operand, so that
+    // the result is the upper word of the product and only its rounding is
+    // left: q << hm8_t, q << hdt_t for |q| up to hm8_lim, hdt_lim (0: shift
+    // not possible, see mul_round), and v << ou_vt, noise << ou_nt (ou_lim)
+    int hm8_t, hdt_t, ou_vt, ou_nt;
+    long long hm8_lim, hdt_lim, ou_lim;
+    RotK rot;           // the rotational update's constants in fixed point
     // st and sr 2^40 times the noise's scale sqrt(12) 2^-33 (multiplying the
     // noise's exact integer part)
     double stn_d, srn_d;
