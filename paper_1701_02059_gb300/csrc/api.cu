@@ -53,9 +53,9 @@ void Ensemble::free_all() {
     for (void* p : allocs_) cudaFreeAsync(p, stream);
     allocs_.clear();
     bytes_ = 0;
-    for (int* p : scan_tmp_) if (p) cudaFreeAsync(p, stream);
-    scan_tmp_.clear();
-    scan_tmp_n_.clear();
+    if (d_scan_) cudaFreeAsync(d_scan_, stream);
+    d_scan_ = nullptr;
+    scan_words_ = 0;
     if (ev0_) { cudaEventDestroy(ev0_); ev0_ = nullptr; }
     if (ev1_) { cudaEventDestroy(ev1_); ev1_ = nullptr; }
     d_dump = nullptr;
@@ -87,9 +87,9 @@ View Ensemble::view() {
     v.cell = d_cell; v.slot_of_id = d_slot_of_id;
     v.F = d_F; v.T = d_T; v.Fbig = d_Fbig;
     v.mq = d_mq; v.mo = d_mo; v.mqr = d_mqr; v.mor = d_mor; v.cnorm = d_cnorm; v.grank = d_grank;
-    v.cq = d_cq; v.cell_start = d_cell_start; v.R = d_R; v.Rf = d_Rf; v.adj_ptr = d_adj_ptr; v.adj = d_adj; v.adj_cap = adj_cap; v.adjd = d_adjd;
+    v.cq = d_cq; v.cell_start = d_cell_start; v.R2 = d_R2; v.Rf = d_Rf; v.adj_ptr = d_adj_ptr; v.adj = d_adj; v.adj_cap = adj_cap; v.adjd = d_adjd;
     v.adjn = d_adjcount;
-    v.gstart = d_gstart; v.gcent = d_gcent; v.gcf = d_gcf;
+    v.gstart = d_gstart; v.gcf = d_gcf;
     v.bptr = d_bptr; v.bpartner = d_bpartner;
     v.nbond = nbond; v.bij = d_bij; v.binst = d_binst; v.bkf = d_bkf; v.bkd = d_bkd;
     v.status = d_status;
@@ -302,13 +302,12 @@ void Ensemble::alloc_core(const std::vector<int>& p0, const std::vector<int>& k0
     d_cq = alloc<long long>((size_t)3 * Ktot);
     d_cq_tmp = alloc<long long>((size_t)3 * Ktot);
     d_cell_start = alloc<int>(Ktot + 1);
-    d_R = alloc<double>(Ktot);
+    d_R2 = alloc<double>(Ktot);
     d_Rf = alloc<float>(Ktot);
     d_adj_ptr = alloc<int>(Ktot + 1);
     d_adjcount = alloc<int>(Ktot + 1);
     adj_cap = (long long)Ktot * 64;
     d_adj = alloc<int>(adj_cap);
-    d_gcent = alloc<int>(Ktot);
     d_gcf = alloc<float4>(Ktot);
     d_gidx = alloc<int>(Ktot);
     d_status = alloc<unsigned>(1);
@@ -334,9 +333,8 @@ void Ensemble::alloc_core(const std::vector<int>& p0, const std::vector<int>& k0
     d_dmax = alloc<unsigned>(B);
     d_fbcount = alloc<int>(1);
     d_rot_n = alloc<int>(1);
+    d_flag = alloc<int>(1);
     d_adjpad = alloc<int>((size_t)Ktot * 64);
-    d_seglist = alloc<int>((size_t)2 * Ktot);
-    d_seglist_n = alloc<int>(2);
     d_adjd = alloc<AdjDesc>(adj_cap);
     d_candrows = alloc<float4>(adj_cap);
     alloc_lists();
@@ -349,6 +347,7 @@ void Ensemble::alloc_core(const std::vector<int>& p0, const std::vector<int>& k0
     d_step = alloc<long long>(B);
     CK(cudaMemcpyAsync(d_step, step_h.data(), sizeof(long long) * B, cudaMemcpyHostToDevice, stream));
     d_xref = any_skin ? alloc<long long>((size_t)3 * N) : nullptr;
+    reset_scratch();
 }
 
 // Bond CSR by (p0 + id), both directions; r0 and kb per entry in FP32 and FP64.
@@ -653,6 +652,7 @@ void Ensemble::init_cells() {
         mstep_iter(d_cell, it, d_dmax);
         toc();
     }
+    CK(cudaMemsetAsync(d_dmax, 0, sizeof(unsigned) * B, stream));
     finish_cells();
     unsigned st = read_status(true);
     if (st) throw StateError("cell initialisation flagged status " + std::to_string(st));
@@ -779,7 +779,7 @@ void Ensemble::get_cells(int b, int* cell_of_id, unsigned* slot_ids, double* cen
     CK(cudaMemcpyAsync(cs.data(), d_cell_start + I.k0, sizeof(int) * (K + 1), cudaMemcpyDeviceToHost, stream));
     CK(cudaMemcpyAsync(ap.data(), d_adj_ptr + I.k0, sizeof(int) * (K + 1), cudaMemcpyDeviceToHost, stream));
     std::vector<double> R(K);
-    CK(cudaMemcpyAsync(R.data(), d_R + I.k0, sizeof(double) * K, cudaMemcpyDeviceToHost, stream));
+    CK(cudaMemcpyAsync(R.data(), d_R2 + I.k0, sizeof(double) * K, cudaMemcpyDeviceToHost, stream));
     std::vector<long long> c((size_t)3 * K);
     for (int a = 0; a < 3; a++)
         CK(cudaMemcpyAsync(c.data() + (size_t)a * K, d_cq + (size_t)a * Ktot + I.k0, sizeof(long long) * K,
@@ -793,7 +793,8 @@ void Ensemble::get_cells(int b, int* cell_of_id, unsigned* slot_ids, double* cen
         for (int k = 0; k < K; k++)
             for (int a = 0; a < 3; a++) centroids[(size_t)3 * k + a] = (double)c[(size_t)a * K + k] * kGridInv;
     if (cell_start) for (int k = 0; k <= K; k++) cell_start[k] = cs[k] - I.p0;
-    if (radius) std::copy(R.begin(), R.end(), radius);
+    // (the device keeps the squares; the host's square root is correctly rounded too)
+    if (radius) std::transform(R.begin(), R.end(), radius, [](double r2) { return std::sqrt(r2); });
     if (adj_ptr) for (int k = 0; k <= K; k++) adj_ptr[k] = ap[k] - ap[0];
     if (adj) {
         long long L = ap[K] - ap[0];
@@ -819,7 +820,7 @@ void Ensemble::get_cells_all(int* cell_of_id, unsigned* slot_ids, double* centro
     CK(cudaMemcpyAsync(cs.data(), d_cell_start, sizeof(int) * (Ktot + 1), cudaMemcpyDeviceToHost, stream));
     CK(cudaMemcpyAsync(ap.data(), d_adj_ptr, sizeof(int) * (Ktot + 1), cudaMemcpyDeviceToHost, stream));
     std::vector<double> R(Ktot);
-    CK(cudaMemcpyAsync(R.data(), d_R, sizeof(double) * Ktot, cudaMemcpyDeviceToHost, stream));
+    CK(cudaMemcpyAsync(R.data(), d_R2, sizeof(double) * Ktot, cudaMemcpyDeviceToHost, stream));
     std::vector<long long> c((size_t)3 * Ktot);
     CK(cudaMemcpyAsync(c.data(), d_cq, sizeof(long long) * 3 * Ktot, cudaMemcpyDeviceToHost, stream));
     CK(cudaStreamSynchronize(stream));
@@ -833,7 +834,8 @@ void Ensemble::get_cells_all(int* cell_of_id, unsigned* slot_ids, double* centro
         for (int k = 0; k < Ktot; k++)
             for (int a = 0; a < 3; a++) centroids[(size_t)3 * k + a] = (double)c[(size_t)a * Ktot + k] * kGridInv;
     if (cell_start) std::copy(cs.begin(), cs.end(), cell_start);
-    if (radius) std::copy(R.begin(), R.end(), radius);
+    // (the device keeps the squares; the host's square root is correctly rounded too)
+    if (radius) std::transform(R.begin(), R.end(), radius, [](double r2) { return std::sqrt(r2); });
     if (adj_ptr) for (int k = 0; k <= Ktot; k++) adj_ptr[k] = ap[k] - ap[0];
     if (adj) {
         const long long L = ap[Ktot] - ap[0];

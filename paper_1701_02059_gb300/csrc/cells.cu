@@ -8,7 +8,7 @@
 // integer arithmetic where the definition is integer (M-step, sort), FP32
 // prefilters with a proven rounding band and an FP64 re-decision inside the
 // band where the definition compares FP64 distances.
-#include "ensemble.cuh"
+#include "integrator.cuh"
 
 #include <algorithm>
 
@@ -162,9 +162,17 @@ __global__ void k_mstep_sorted(View v, long long* __restrict__ bb, unsigned* __r
 // k_mstep_sorted, so the same centroids): one thread per cell updates c_k,
 // clears the sums for the next step and folds the centroid into the
 // instance's bounding box and its largest move (warp-reduced before the
-// atomics).
+// atomics).  The blocks from rot_block on take the B-A-O-A's left-over
+// rotations instead (rot_rest; one launch fewer than on their own).
 __global__ void __launch_bounds__(256) k_mstep_apply(View v, long long* __restrict__ S, int* __restrict__ cnt,
-                                                     long long* __restrict__ bb, unsigned* __restrict__ dmax) {
+                                                     long long* __restrict__ bb, unsigned* __restrict__ dmax,
+                                                     int rot_block, const long long* __restrict__ steps, int fused,
+                                                     const int* __restrict__ rot_list, const int* __restrict__ rot_n) {
+    if ((int)blockIdx.x >= rot_block) {
+        rot_rest(v, v, steps, fused, rot_list, rot_n, (blockIdx.x - rot_block) * blockDim.x + threadIdx.x,
+                 (gridDim.x - rot_block) * blockDim.x);
+        return;
+    }
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= v.Ktot) return;
     const size_t K = v.Ktot;
@@ -247,16 +255,29 @@ __device__ inline unsigned long long spread3(unsigned long long x) {
 }
 
 // Key: 21 bits per axis, q = min(2^21 - 1, floor((c - lo) * 2^21 / (hi - lo)))
-// in FP64 exactly as the definition (c - lo is exact on the grid).
-__global__ void k_morton_keys(View v, const long long* __restrict__ bb, unsigned long long* __restrict__ key) {
+// in FP64 exactly as the definition (c - lo is exact on the grid).  Also
+// copies the centroids for the permutation that follows, and does what the
+// step's earlier launches left to a later one (K >= B): the step counters
+// (advance), the empty list of left-over rotations, the largest radii and
+// the overflow count of the pair search to come.
+__global__ void k_morton_keys(View v, const long long* __restrict__ bb, unsigned long long* __restrict__ key,
+                              long long* __restrict__ cq_copy, long long* __restrict__ steps, int advance,
+                              int* __restrict__ rot_n, unsigned long long* __restrict__ rmax, int* __restrict__ novf) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= v.Ktot) return;
+    if (k < v.B) {
+        if (advance) steps[k] += 1;
+        rmax[k] = 0ull;
+        if (k == 0) { *rot_n = 0; *novf = 0; }
+    }
     int b = find_inst(v.inst_k0, v.B, k);
     unsigned long long kk = 0;
     for (int a = 0; a < 3; a++) {
+        const long long c = v.cq[(size_t)a * v.Ktot + k];
+        cq_copy[(size_t)a * v.Ktot + k] = c;
         double lo = grid_to_double(bb[b * 6 + a]), hi = grid_to_double(bb[b * 6 + 3 + a]);
         double s = (hi > lo) ? __ddiv_rn(2097152.0, __dsub_rn(hi, lo)) : 0.0;
-        double t = __dmul_rn(__dsub_rn(grid_to_double(v.cq[(size_t)a * v.Ktot + k]), lo), s);
+        double t = __dmul_rn(__dsub_rn(grid_to_double(c), lo), s);
         double f = floor(t);
         unsigned long long q = (f >= 2097151.0) ? 2097151ull : (unsigned long long)f;
         kk |= spread3(q) << a;
@@ -297,7 +318,10 @@ __global__ void __launch_bounds__(kTile) k_tile_sort(View v, const unsigned long
     SortRec r;
     if (k < v.Ktot) { r.key = key[k]; r.idx = k; r.inst = find_inst(v.inst_k0, v.B, k); }
     else { r.key = ~0ull; r.idx = 0x7fffffff; r.inst = 0x7fffffff; }
-    for (int size = 2; size <= kTile; size <<= 1) {
+    // the padding records sort last, so the network stops at the tile's
+    // record count rounded up
+    const int m = min(kTile, v.Ktot - (int)blockIdx.x * kTile);
+    for (int size = 2; size < 2 * m; size <<= 1) {
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
             SortRec o;
             if (stride >= 32) {
@@ -317,13 +341,68 @@ __global__ void __launch_bounds__(kTile) k_tile_sort(View v, const unsigned long
     out[blockIdx.x * kTile + t] = r;
 }
 
-// rank -> new cell index; writes order[new] = old and the permuted centroids.
+// ============================================================== centroid grid
+// Fixed per-instance geometry (origin, edge, dims); edge cells extend to
+// infinity, so the face-distance bound of the shell search stays valid for
+// centroids and particles outside the box.
+__device__ inline int grid_coord(long long xq, const Inst& I, int a, float& rel) {
+    long long d = xq - I.gorg[a];
+    if (I.periodic[a]) d = floor_mod_ll(d, I.boxq[a]);
+    // >> 20: units of 2^-20 sigma, |.| < 2^31 for |d| < 2048 sigma
+    long long s = d >> 20;
+    if (s > 2147483647ll) s = 2147483647ll;
+    if (s < -2147483647ll) s = -2147483647ll;
+    rel = (float)(int)s * 9.5367431640625e-07f;
+    int g = (int)floorf(rel * I.ginv[a]);
+    if (g < 0) g = 0;
+    if (g >= I.gdim[a]) g = I.gdim[a] - 1;
+    return g;
+}
+
+// Centroid k's grid cell: counted (gcount), noted (gidx) and its FP32 position
+// relative to the grid origin (cf).
+__device__ inline void grid_count_one(const Inst& I, int k, long long x, long long y, long long z,
+                                      int* __restrict__ gcount, int* __restrict__ gidx, float4* __restrict__ cf) {
+    float r[3];
+    const int gx = grid_coord(x, I, 0, r[0]), gy = grid_coord(y, I, 1, r[1]), gz = grid_coord(z, I, 2, r[2]);
+    const long long g = I.g0 + ((long long)gz * I.gdim[1] + gy) * I.gdim[0] + gx;
+    gidx[k] = (int)g;
+    cf[k] = make_float4(r[0], r[1], r[2], 0.f);
+    atomicAdd(&gcount[g], 1);
+}
+
+__global__ void k_grid_count(View v, int* __restrict__ gcount, int* __restrict__ gidx, float4* __restrict__ cf) {
+    int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= v.Ktot) return;
+    const Inst& I = v.inst[find_inst(v.inst_k0, v.B, k)];
+    grid_count_one(I, k, v.cq[k], v.cq[(size_t)v.Ktot + k], v.cq[(size_t)2 * v.Ktot + k], gcount, gidx, cf);
+}
+
+// Centroid k to its place in grid order.  The counts are taken down to zero,
+// ready for the next count.
+__device__ inline void grid_fill_one(const View& v, int k, const int* __restrict__ gidx, int* __restrict__ gcount,
+                                     const float4* __restrict__ cf) {
+    const int g = gidx[k];
+    const int pos = v.gstart[g] + atomicSub(&gcount[g], 1) - 1;
+    float4 c = cf[k];
+    c.w = __int_as_float(k);
+    v.gcf[pos] = c;
+}
+
+__global__ void k_grid_fill(View v, const int* __restrict__ gidx, int* __restrict__ gcount, const float4* __restrict__ cf) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < v.Ktot) grid_fill_one(v, k, gidx, gcount, cf);
+}
+
+// rank -> new cell index; writes order[new] = old and the permuted centroids,
+// and counts each into its grid cell.
 // Tiles wholly below or above a record need no search (nearly sorted keys
 // between rebuilds make this the common case).
 constexpr int kBoundTiles = 1024;   // tiles whose bounds a block keeps in shared memory
 
 __global__ void k_rank_scatter(View v, const SortRec* __restrict__ tiles, int ntiles, const long long* __restrict__ cq_old,
-                               int* __restrict__ new_of_old) {
+                               int* __restrict__ new_of_old, int* __restrict__ gcount, int* __restrict__ gidx,
+                               float4* __restrict__ cf, long long* __restrict__ bb) {
     // first and last record of every tile (most tiles lie wholly below or
     // above a record, which these settle without a search)
     __shared__ SortRec tb[2][kBoundTiles];
@@ -335,6 +414,10 @@ __global__ void k_rank_scatter(View v, const SortRec* __restrict__ tiles, int nt
         }
     __syncthreads();
     int pos = blockIdx.x * blockDim.x + threadIdx.x;   // position in the tiled array
+    // the bounding boxes, read by the keys, empty for the next step
+    // (ntiles * kTile >= K >= B)
+    if (pos < v.B)
+        for (int a = 0; a < 6; a++) bb[pos * 6 + a] = a < 3 ? 0x7fffffffffffffffll : (-0x7fffffffffffffffll - 1);
     if (pos >= ntiles * kTile) return;
     SortRec me = tiles[pos];
     if (me.idx >= v.Ktot) return;
@@ -367,55 +450,12 @@ __global__ void k_rank_scatter(View v, const SortRec* __restrict__ tiles, int nt
     }
     int nk = I.k0 + rank;
     new_of_old[me.idx] = nk;
-    for (int a = 0; a < 3; a++) v.cq[(size_t)a * v.Ktot + nk] = cq_old[(size_t)a * v.Ktot + me.idx];
-}
-
-// ============================================================== centroid grid
-// Fixed per-instance geometry (origin, edge, dims); edge cells extend to
-// infinity, so the face-distance bound of the shell search stays valid for
-// centroids and particles outside the box.
-__device__ inline int grid_coord(long long xq, const Inst& I, int a, float& rel) {
-    long long d = xq - I.gorg[a];
-    if (I.periodic[a]) d = floor_mod_ll(d, I.boxq[a]);
-    // >> 20: units of 2^-20 sigma, |.| < 2^31 for |d| < 2048 sigma
-    long long s = d >> 20;
-    if (s > 2147483647ll) s = 2147483647ll;
-    if (s < -2147483647ll) s = -2147483647ll;
-    rel = (float)(int)s * 9.5367431640625e-07f;
-    int g = (int)floorf(rel * I.ginv[a]);
-    if (g < 0) g = 0;
-    if (g >= I.gdim[a]) g = I.gdim[a] - 1;
-    return g;
-}
-
-__global__ void k_grid_count(View v, int* __restrict__ gcount, int* __restrict__ gidx) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= v.Ktot) return;
-    int b = find_inst(v.inst_k0, v.B, k);
-    const Inst& I = v.inst[b];
-    float r[3];
-    int gx = grid_coord(v.cq[k], I, 0, r[0]);
-    int gy = grid_coord(v.cq[(size_t)v.Ktot + k], I, 1, r[1]);
-    int gz = grid_coord(v.cq[(size_t)2 * v.Ktot + k], I, 2, r[2]);
-    long long g = I.g0 + ((long long)gz * I.gdim[1] + gy) * I.gdim[0] + gx;
-    gidx[k] = (int)g;
-    atomicAdd(&gcount[g], 1);
-}
-
-__global__ void k_grid_fill(View v, const int* __restrict__ gidx, int* __restrict__ cursor, float4* __restrict__ cf) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= v.Ktot) return;
-    int b = find_inst(v.inst_k0, v.B, k);
-    const Inst& I = v.inst[b];
-    int g = gidx[k];
-    int pos = v.gstart[g] + atomicAdd(&cursor[g], 1);
-    float r[3];
-    grid_coord(v.cq[k], I, 0, r[0]);
-    grid_coord(v.cq[(size_t)v.Ktot + k], I, 1, r[1]);
-    grid_coord(v.cq[(size_t)2 * v.Ktot + k], I, 2, r[2]);
-    v.gcent[pos] = k;
-    v.gcf[pos] = make_float4(r[0], r[1], r[2], __int_as_float(k));
-    if (cf) cf[k] = make_float4(r[0], r[1], r[2], 0.f);
+    long long c[3];
+    for (int a = 0; a < 3; a++) {
+        c[a] = cq_old[(size_t)a * v.Ktot + me.idx];
+        v.cq[(size_t)a * v.Ktot + nk] = c[a];
+    }
+    grid_count_one(I, nk, c[0], c[1], c[2], gcount, gidx, cf);
 }
 
 // ============================================================== E-step
@@ -690,17 +730,99 @@ __global__ void k_estep_warp(View v, int* __restrict__ cell_out, float* __restri
     }
 }
 
-__global__ void k_estep(View v, int* __restrict__ cell_out) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < v.N) estep_one(v, i, cell_out);
+// One particle's nearest centroid by a whole warp: the lanes share the grid
+// cells of each shell (see estep_one for the bounds; the same answer: the
+// FP32 best alone in its band, else the FP64 best, ties to the lowest index).
+__device__ int estep_warp_one(const View& v, int i) {
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    const Inst& I = v.inst[find_inst(v.inst_p0, v.B, i)];
+    const long long xq[3] = { v.xq[i], v.xq[(size_t)v.N + i], v.xq[(size_t)2 * v.N + i] };
+    float p[3];
+    int g[3];
+    for (int a = 0; a < 3; a++) g[a] = grid_coord(xq[a], I, a, p[a]);
+    // visits the centroids of cube(r) (skipping cube(r - 1) when shell is set)
+    auto scan = [&](int r, bool shell, auto&& f) {
+        int lo[3], ext[3];
+        for (int a = 0; a < 3; a++) {
+            int l, h;
+            if (I.periodic[a]) {
+                if (2 * r + 1 >= I.gdim[a]) { l = 0; h = I.gdim[a] - 1; }
+                else { l = g[a] - r; h = g[a] + r; }
+            } else {
+                l = max(0, g[a] - r);
+                h = min(I.gdim[a] - 1, g[a] + r);
+            }
+            lo[a] = l;
+            ext[a] = h - l + 1;
+        }
+        const long long n = (long long)ext[0] * ext[1] * ext[2];
+        for (long long t = lane; t < n; t += 32) {
+            const int x = lo[0] + (int)(t % ext[0]), y = lo[1] + (int)(t / ext[0] % ext[1]),
+                      z = lo[2] + (int)(t / ((long long)ext[0] * ext[1]));
+            const int w[3] = { I.periodic[0] ? wrap_idx(x, I.gdim[0]) : x, I.periodic[1] ? wrap_idx(y, I.gdim[1]) : y,
+                               I.periodic[2] ? wrap_idx(z, I.gdim[2]) : z };
+            if (shell && r > 0 && in_cube(w, g, r - 1, I)) continue;
+            const long long gg = I.g0 + ((long long)w[2] * I.gdim[1] + w[1]) * I.gdim[0] + w[0];
+            const int q1 = v.gstart[gg + 1];
+            for (int q = v.gstart[gg]; q < q1; q++) {
+                const float4 c = v.gcf[q];
+                const float dx = axis_dist(p[0], c.x, I, 0), dy = axis_dist(p[1], c.y, I, 1), dz = axis_dist(p[2], c.z, I, 2);
+                f(fmaf(dx, dx, fmaf(dy, dy, dz * dz)), __float_as_int(c.w));
+            }
+        }
+    };
+    float best = 3.0e38f;
+    int r = 0;
+    const int rmax = max(I.gdim[0], max(I.gdim[1], I.gdim[2]));
+    for (;; r++) {
+        scan(r, true, [&](float d2, int) { best = fminf(best, d2); });
+        // non-negative floats order like their bits
+        best = __uint_as_float(__reduce_min_sync(full, __float_as_uint(best)));
+        bool ex;
+        const float lb = shell_bound(p, g, r, I, ex);
+        if (ex || r >= rmax || (best < 3.0e38f && lb > sqrtf(best) + kBandE)) break;
+    }
+    const float lim = sqrtf(best) + kBandE, lim2 = lim * lim;
+    int ncand = 0, bk = 0x7fffffff;
+    scan(r, false, [&](float d2, int k) { if (d2 <= lim2) { ncand++; bk = min(bk, k); } });
+    ncand = (int)__reduce_add_sync(full, (unsigned)ncand);
+    if (ncand == 0) {   // unreachable for finite input: the search covers every centroid
+        if (lane == 0) flag_inst(v, I, kStatusGridRange);
+        return I.k0;
+    }
+    if (ncand > 1) {
+        // (squared distances are non-negative: their bits order like them)
+        unsigned long long b64 = ~0ull;
+        bk = 0x7fffffff;
+        scan(r, false, [&](float d2, int k) {
+            if (d2 > lim2) return;
+            const unsigned long long d = (unsigned long long)__double_as_longlong(
+                dist2_grid_d(xq[0], xq[1], xq[2], v.cq[k], v.cq[(size_t)v.Ktot + k], v.cq[(size_t)2 * v.Ktot + k], I));
+            if (d < b64 || (d == b64 && k < bk)) { b64 = d; bk = k; }
+        });
+        unsigned long long m = b64;
+        for (int off = 16; off; off >>= 1) m = min(m, (unsigned long long)__shfl_xor_sync(full, m, off));
+        if (b64 != m) bk = 0x7fffffff;
+    }
+    return __reduce_min_sync(full, bk);
 }
 
-// Grid search for the particles the certified E-step could not decide.
-__global__ void k_estep_list(View v, const int* __restrict__ fb_list, const int* __restrict__ fb_count,
-                             int* __restrict__ cell_out, float* __restrict__ lbound = nullptr) {
+// Grid search for the particles the certified E-step could not decide, a
+// warp each (one thread each took 70 us for the few of the 4M cell: a chain
+// of dependent loads per shell); counts them into their cells.
+__global__ void __launch_bounds__(128) k_estep_list(View v, const int* __restrict__ fb_list,
+                                                    const int* __restrict__ fb_count, int* __restrict__ cell_out,
+                                                    int* __restrict__ cnt) {
     const int n = *fb_count;
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x)
-        estep_one(v, fb_list[q], cell_out, lbound);
+    for (int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < n; q += (gridDim.x * blockDim.x) >> 5) {
+        const int i = fb_list[q];
+        const int c = estep_warp_one(v, i);
+        if ((threadIdx.x & 31) == 0) {
+            cell_out[i] = c;
+            atomicAdd(&cnt[c], 1);
+        }
+    }
 }
 
 // Largest move of the centroids now in each grid cell (FP32 bits:
@@ -767,12 +889,14 @@ __global__ void __launch_bounds__(256) k_estep_bound(View v, const int* __restri
 
 // The previous rows with their cells renumbered and the renumbered cells'
 // FP32 centroids (w = new index), so the E-step reads one record per
-// candidate instead of three dependent loads.
-__global__ void k_cand_rows(const int* __restrict__ cnt_old, int Ktot, const int* __restrict__ pad_old,
+// candidate instead of three dependent loads; the first K threads also put
+// the centroids in grid order.
+__global__ void k_cand_rows(View v, const int* __restrict__ cnt_old, const int* __restrict__ pad_old,
                             const int* __restrict__ new_of_old, const float4* __restrict__ cf,
-                            float4* __restrict__ rows) {
+                            float4* __restrict__ rows, const int* __restrict__ gidx, int* __restrict__ gcount) {
     const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // one thread per row slot
-    if (q >= (long long)Ktot * kAdjRow || (int)(q % kAdjRow) >= cnt_old[q / kAdjRow]) return;
+    if (q < v.Ktot) grid_fill_one(v, (int)q, gidx, gcount, cf);
+    if (q >= (long long)v.Ktot * kAdjRow || (int)(q % kAdjRow) >= cnt_old[q / kAdjRow]) return;
     const int j = new_of_old[pad_old[q]];
     float4 c = cf[j];
     c.w = __int_as_float(j);
@@ -788,14 +912,17 @@ __global__ void k_cand_rows(const int* __restrict__ cnt_old, int Ktot, const int
 // non-neighbour), and every centroid has since moved at most dmax, so none
 // of them is within best + band of the particle when
 //   sqrt(best) + band < rho_k - 2 dmax - |x - c_k|   (FP32 with margins).
-// Particles that fail the test take the grid search.
+// Particles that fail the test take the grid search.  The others are counted
+// into their cells (a histogram pass of its own cost 13 us at 4M).
 __global__ void __launch_bounds__(128, 16) k_estep_rows(View v, const int* __restrict__ cell_old,
                                                     const int* __restrict__ cnt_old, const float4* __restrict__ rows,
                                                     const float* __restrict__ rho_old, const int* __restrict__ new_of_old,
                                                     const unsigned* __restrict__ dmax, int* __restrict__ cell_out,
-                                                    int* __restrict__ fb_list, int* __restrict__ fb_count) {
+                                                    int* __restrict__ fb_list, int* __restrict__ fb_count,
+                                                    int* __restrict__ cnt) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     bool fail = false;
+    int to = -1;
     if (i < v.N) {
         const int b = find_inst(v.inst_p0, v.B, i);
         const Inst& I = v.inst[b];
@@ -823,9 +950,8 @@ __global__ void __launch_bounds__(128, 16) k_estep_rows(View v, const int* __res
         const float cert = rho_old[ko] - 2.0f * __uint_as_float(dmax[b]) - sqrtf(dself2) - kCertMargin;
         fail = bk < 0 || dself2 >= 3.0e38f || !(lim < cert);
         if (!fail) {
-            if (second > lim * lim) {
-                cell_out[i] = bk;
-            } else {
+            to = bk;
+            if (second <= lim * lim) {
                 // tie band: FP64 among the row's candidates within it
                 double best64 = 1e300;
                 int bk64 = -1;
@@ -841,10 +967,14 @@ __global__ void __launch_bounds__(128, 16) k_estep_rows(View v, const int* __res
                         if (d64 < best64 || (d64 == best64 && j < bk64)) { best64 = d64; bk64 = j; }
                     }
                 }
-                cell_out[i] = bk64;
+                to = bk64;
             }
+            cell_out[i] = to;
         }
     }
+    // the counts of the sort that follows: one atomic per distinct cell of a warp
+    const unsigned peers = __match_any_sync(0xffffffffu, to);
+    if (to >= 0 && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&cnt[to], __popc(peers));
     // the rare failures to the grid search's list, one atomic per warp
     const unsigned m = __ballot_sync(0xffffffffu, fail);
     if (m) {
@@ -868,16 +998,20 @@ __global__ void k_hist(int N, const int* __restrict__ cell, int* __restrict__ cn
 }
 
 // Slot of each particle inside its cell's range (in any order across warps;
-// the per-cell sort that follows restores the storage order).
-__global__ void k_scatter(int N, const int* __restrict__ cell, const int* __restrict__ start, int* __restrict__ cursor,
-                          int* __restrict__ tmp) {
+// the per-cell sort that follows restores the storage order).  The counts
+// are taken down to zero, ready for the next histogram.  dmax, fb_count
+// (nullable): the E-step's inputs, cleared for the next rebuild (N >= B).
+__global__ void k_scatter(int N, const int* __restrict__ cell, const int* __restrict__ start, int* __restrict__ cnt,
+                          int* __restrict__ tmp, int B, unsigned* __restrict__ dmax, int* __restrict__ fb_count) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < B) dmax[i] = 0u;
+    if (i == 0 && fb_count) *fb_count = 0;
     const int c = (i < N) ? cell[i] : -1;
     const unsigned peers = __match_any_sync(0xffffffffu, c);
     const int lane = threadIdx.x & 31;
     const int leader = __ffs(peers) - 1;
     int base = 0;
-    if (c >= 0 && lane == leader) base = atomicAdd(&cursor[c], __popc(peers));
+    if (c >= 0 && lane == leader) base = atomicSub(&cnt[c], __popc(peers)) - __popc(peers);
     base = __shfl_sync(peers, base, leader);
     if (c >= 0) tmp[start[c] + base + __popc(peers & ((1u << lane) - 1u))] = i;
 }
@@ -913,12 +1047,8 @@ __global__ void k_segsort(int Ktot, const int* __restrict__ start, int* __restri
 
 // Cells of up to 128 particles: one warp, bitonic network over 4 values per
 // lane (element e = lane + 32 q), shuffles for strides < 32.
-__global__ void k_segsort_warp(int Ktot, const int* __restrict__ start, int* __restrict__ tmp) {
-    const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+__device__ inline void segsort_warp(int s, int n, int* __restrict__ tmp) {
     const int lane = threadIdx.x & 31;
-    if (k >= Ktot) return;
-    const int s = start[k], n = start[k + 1] - s;
-    if (n <= 1 || n > 128) return;
     int val[4];
 #pragma unroll
     for (int q = 0; q < 4; q++) val[q] = (lane + 32 * q < n) ? tmp[s + lane + 32 * q] : 0x7fffffff;
@@ -954,6 +1084,60 @@ __global__ void k_segsort_warp(int Ktot, const int* __restrict__ start, int* __r
         if (lane + 32 * q < n) tmp[s + lane + 32 * q] = val[q];
 }
 
+__global__ void k_segsort_warp(int Ktot, const int* __restrict__ start, int* __restrict__ tmp) {
+    const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (k >= Ktot) return;
+    const int s = start[k], n = start[k + 1] - s;
+    if (n > 1 && n <= 128) segsort_warp(s, n, tmp);
+}
+
+// The rebuild's form, one launch for every size: 256 threads, eight cells; a
+// warp sorts its cell when it holds up to 128 particles, then the block takes
+// the larger ones (rare) one after the other, bitonic in shared memory up to
+// kSegMax, beyond it each slot's rank among its cell's (distinct) slots, out
+// being scratch.
+__global__ void __launch_bounds__(256) k_segsort_cells(int Ktot, const int* __restrict__ start, int* __restrict__ tmp,
+                                                       int* __restrict__ out) {
+    __shared__ int sh[kSegMax];
+    const int k0 = blockIdx.x * 8, k = k0 + (threadIdx.x >> 5);
+    const int s = k < Ktot ? start[k] : 0, n = k < Ktot ? start[k + 1] - s : 0;
+    if (n > 1 && n <= 128) segsort_warp(s, n, tmp);
+    if (!__syncthreads_or(n > 128)) return;
+    for (int c = k0; c < min(k0 + 8, Ktot); c++) {
+        const int s0 = start[c], m0 = start[c + 1] - s0;
+        if (m0 <= 128) continue;
+        if (m0 <= kSegMax) {
+            int m = 1;
+            while (m < m0) m <<= 1;
+            for (int t = threadIdx.x; t < m; t += blockDim.x) sh[t] = (t < m0) ? tmp[s0 + t] : 0x7fffffff;
+            __syncthreads();
+            for (int size = 2; size <= m; size <<= 1)
+                for (int stride = size >> 1; stride > 0; stride >>= 1) {
+                    for (int t = threadIdx.x; t < m; t += blockDim.x) {
+                        const int p = t ^ stride;
+                        if (p > t) {
+                            const bool up = (t & size) == 0;
+                            const int a = sh[t], b = sh[p];
+                            if ((b < a) == up) { sh[t] = b; sh[p] = a; }
+                        }
+                    }
+                    __syncthreads();
+                }
+            for (int t = threadIdx.x; t < m0; t += blockDim.x) tmp[s0 + t] = sh[t];
+        } else {
+            for (int q = s0 + threadIdx.x; q < s0 + m0; q += blockDim.x) {
+                const int me = tmp[q];
+                int r = 0;
+                for (int t = s0; t < s0 + m0; t++) r += (tmp[t] < me);
+                out[s0 + r] = me;
+            }
+            __syncthreads();
+            for (int q = s0 + threadIdx.x; q < s0 + m0; q += blockDim.x) tmp[q] = out[q];
+        }
+        __syncthreads();
+    }
+}
+
 // Cells larger than kSegMax: each slot's rank among its cell's (distinct)
 // old indices, O(n^2) per such cell; writes the ordered list to out.
 __global__ void k_segrank(int N, const int* __restrict__ cell, const int* __restrict__ start, const int* __restrict__ tmp,
@@ -974,74 +1158,6 @@ __global__ void k_segcopy(int N, const int* __restrict__ cell, const int* __rest
     if (q >= N) return;
     int c = cell[tmp[q]];
     if (start[c + 1] - start[c] > kSegMax) tmp[q] = src[q];
-}
-
-// Cells that the warp sort cannot take: 128 < n <= kSegMax into list A
-// (block bitonic), n > kSegMax into list B (exact rank); counts in cnt[0..1].
-__global__ void k_seglist(int Ktot, const int* __restrict__ start, int* __restrict__ la, int* __restrict__ lb,
-                          int* __restrict__ cnt) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n = (k < Ktot) ? start[k + 1] - start[k] : 0;
-    const bool a = n > 128 && n <= kSegMax, bb = n > kSegMax;
-    const int lane = threadIdx.x & 31;
-    const unsigned ma = __ballot_sync(0xffffffffu, a), mb = __ballot_sync(0xffffffffu, bb);
-    int baseA = 0, baseB = 0;
-    if (ma && lane == __ffs(ma) - 1) baseA = atomicAdd(&cnt[0], __popc(ma));
-    if (mb && lane == __ffs(mb) - 1) baseB = atomicAdd(&cnt[1], __popc(mb));
-    baseA = __shfl_sync(0xffffffffu, baseA, ma ? __ffs(ma) - 1 : 0);
-    baseB = __shfl_sync(0xffffffffu, baseB, mb ? __ffs(mb) - 1 : 0);
-    const unsigned lt = (1u << lane) - 1u;
-    if (a) la[baseA + __popc(ma & lt)] = k;
-    if (bb) lb[baseB + __popc(mb & lt)] = k;
-}
-
-// List A: one block per cell, bitonic sort of its slot list in shared memory.
-__global__ void k_segsort_list(const int* __restrict__ start, const int* __restrict__ la, const int* __restrict__ cnt,
-                               int* __restrict__ tmp) {
-    __shared__ int sh[kSegMax];
-    const int nl = cnt[0];
-    for (int e = blockIdx.x; e < nl; e += gridDim.x) {
-        const int k = la[e];
-        const int s0 = start[k], n = start[k + 1] - s0;
-        int m = 1;
-        while (m < n) m <<= 1;
-        for (int t = threadIdx.x; t < m; t += blockDim.x) sh[t] = (t < n) ? tmp[s0 + t] : 0x7fffffff;
-        __syncthreads();
-        for (int size = 2; size <= m; size <<= 1)
-            for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                for (int t = threadIdx.x; t < m; t += blockDim.x) {
-                    const int p = t ^ stride;
-                    if (p > t) {
-                        const bool up = (t & size) == 0;
-                        const int a = sh[t], c = sh[p];
-                        if ((c < a) == up) { sh[t] = c; sh[p] = a; }
-                    }
-                }
-                __syncthreads();
-            }
-        for (int t = threadIdx.x; t < n; t += blockDim.x) tmp[s0 + t] = sh[t];
-        __syncthreads();
-    }
-}
-
-// List B: one block per cell; every slot's rank among the cell's slots (they
-// are distinct), written to out, then copied back.
-__global__ void k_segrank_list(const int* __restrict__ start, const int* __restrict__ lb, const int* __restrict__ cnt,
-                               int* __restrict__ tmp, int* __restrict__ out) {
-    const int nl = cnt[1];
-    for (int e = blockIdx.x; e < nl; e += gridDim.x) {
-        const int k = lb[e];
-        const int s0 = start[k], s1 = start[k + 1];
-        for (int q = s0 + threadIdx.x; q < s1; q += blockDim.x) {
-            const int me = tmp[q];
-            int r = 0;
-            for (int t = s0; t < s1; t++) r += (tmp[t] < me);
-            out[s0 + r] = me;
-        }
-        __syncthreads();
-        for (int q = s0 + threadIdx.x; q < s1; q += blockDim.x) tmp[q] = out[q];
-        __syncthreads();
-    }
 }
 
 // ============================================================== gather + mirrors
@@ -1152,7 +1268,7 @@ __device__ inline void warp_bitonic_u32(unsigned (&r)[4], int lane) {
 
 // Per-cell quantities read back from the gathered mirrors: one warp per cell
 // computes the squared cell radius R_k^2 = max |x - c_k|^2 (FP32 with the
-// FP64 definition inside a band; left in R for k_cell_radius), the pair
+// FP64 definition inside a band) and the radius in FP32, the pair
 // kernel's cell normal (mean bilayer director, unit; +z without one) and, in
 // each tile of 128 particles, every particle's rank along the tile's longer
 // tangent extent.  rmax_bits: each instance's largest R_k^2 (bit pattern).
@@ -1196,10 +1312,12 @@ __global__ void __launch_bounds__(256, 6) k_cell_props(View v, unsigned long lon
     unsigned long long bb = (unsigned long long)__double_as_longlong(best);
     for (int off = 16; off; off >>= 1) bb = max(bb, (unsigned long long)__shfl_xor_sync(0xffffffffu, bb, off));
     best = __longlong_as_double((long long)bb);
-    // the squared radius for now (k_cell_radius takes the square roots, one
-    // cell per thread), and each instance's largest square
+    // the squared radius (an FP64 square root per cell would cost a whole
+    // warp's turn on the FP64 pipe each: the neighbour rule takes the few it
+    // needs), the radius in FP32, and each instance's largest square
     if (lane == 0) {
-        v.R[k] = best;
+        v.R2[k] = best;
+        v.Rf[k] = sqrtf((float)best);
         atomicMax(&rmax_bits[b], bb);
     }
     // pair-kernel frame
@@ -1284,17 +1402,6 @@ __global__ void k_mirrors(View v) {
     v.mor[q] = no;
 }
 
-// Cell radii R_k = sqrt(R_k^2) from k_cell_props and their FP32 copies, one
-// thread per cell: an FP64 instruction occupies the FP64 pipe for a whole
-// warp, so 32 cells share each square root instead of one.
-__global__ void k_cell_radius(View v) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= v.Ktot) return;
-    const double R = __dsqrt_rn(v.R[k]);
-    v.R[k] = R;
-    v.Rf[k] = (float)R;
-}
-
 // ============================================================== neighbouring cells
 // nbr(k) = { j : |c_k - c_j| < ((R_k + R_j) + r_s + 2 skin)(1 + 1e-12) },
 // evaluated exactly as the FP64 definition for candidates within a band of
@@ -1303,16 +1410,16 @@ constexpr float kBandA = 2e-3f;
 
 // exact neighbouring-cell test of (k, j), FP32 with a margin outside the
 // band and the definition's FP64 operations inside it
-__device__ inline bool adj_test(const View& v, const Inst& I, int k, int j, double Rk, float Rkf, float df,
-                                long long cx, long long cy, long long cz, float tailf) {
-    // FP32 prefilter: radii rounded to FP32 differ from the definition's
-    // FP64 sum by far less than the band
+__device__ inline bool adj_test(const View& v, const Inst& I, int k, int j, float Rkf, float df, long long cx,
+                                long long cy, long long cz, float tailf) {
+    // FP32 prefilter: FP32 radii differ from the definition's FP64 sum by far
+    // less than the band
     const float tf = (Rkf + v.Rf[j]) + tailf;
     if (df < tf - kBandA) return true;
     if (df > tf + kBandA) return false;
     const double d = __dsqrt_rn(dist2_grid_d(cx, cy, cz, v.cq[j], v.cq[(size_t)v.Ktot + j], v.cq[(size_t)2 * v.Ktot + j], I));
     // same operation order as the definition: ((Rk + Rj) + rs) + (skin + skin)
-    double tt = __dadd_rn(__dadd_rn(__dadd_rn(Rk, v.R[j]), I.rs), __dadd_rn(I.skin, I.skin));
+    double tt = __dadd_rn(__dadd_rn(__dadd_rn(__dsqrt_rn(v.R2[k]), __dsqrt_rn(v.R2[j])), I.rs), __dadd_rn(I.skin, I.skin));
     tt = __dmul_rn(tt, 1.0 + 1e-12);
     return d < tt;
 }
@@ -1335,7 +1442,6 @@ __global__ void __launch_bounds__(256, 6) k_adj_warp(View v, const unsigned long
     if (k >= v.Ktot) return;
     const int b = find_inst(v.inst_k0, v.B, k);
     const Inst& I = v.inst[b];
-    const double Rk = v.R[k];
     const float Rkf = v.Rf[k];
     const long long cx = v.cq[k], cy = v.cq[(size_t)v.Ktot + k], cz = v.cq[(size_t)2 * v.Ktot + k];
     // the cell's scalars in FP32 (every lane of the warp computes them, and
@@ -1418,7 +1524,7 @@ __global__ void __launch_bounds__(256, 6) k_adj_warp(View v, const unsigned long
                     const float dx = axis_dist(p[0], c.x, G, 0), dy = axis_dist(p[1], c.y, G, 1),
                                 dz = axis_dist(p[2], c.z, G, 2);
                     const float df = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-                    if (adj_test(v, I, k, j, Rk, Rkf, df, cx, cy, cz, tailf)) {
+                    if (adj_test(v, I, k, j, Rkf, df, cx, cy, cz, tailf)) {
                         const int at = atomicAdd(&rown[wb], 1);
                         if (at < kAdjRow) row[wb][at] = j;
                     } else if (own) {
@@ -1481,14 +1587,21 @@ __global__ void k_adj_csr(View v, const int* __restrict__ pad) {
 // ============================================================== host side
 static inline int nblk(long long n, int t) { return (int)((n + t - 1) / t); }
 
+void Ensemble::reset_scratch() {
+    // every other scratch array starts at zero (alloc)
+    k_fill_bbox<<<1, 64, 0, stream>>>(d_bbox, B);
+    launches++;
+    CK(cudaGetLastError());
+    after_baoa_ = -1;
+    ovf_clean_ = true;
+}
+
 void Ensemble::build_grid() {
     View v = view();
-    CK(cudaMemsetAsync(d_gcount, 0, sizeof(int) * (Gtot + 1), stream));
-    k_grid_count<<<nblk(Ktot, 256), 256, 0, stream>>>(v, d_gcount, d_gidx);
+    k_grid_count<<<nblk(Ktot, 256), 256, 0, stream>>>(v, d_gcount, d_gidx, d_cf);
     launches++;
     CK(cudaGetLastError());
     scan_exclusive(d_gcount, d_gstart, Gtot + 1);
-    CK(cudaMemsetAsync(d_gcount, 0, sizeof(int) * (Gtot + 1), stream));
     k_grid_fill<<<nblk(Ktot, 256), 256, 0, stream>>>(v, d_gidx, d_gcount, d_cf);
     launches++;
     CK(cudaGetLastError());
@@ -1530,12 +1643,12 @@ __global__ void k_displacement(View v, const long long* __restrict__ xref, unsig
 }
 
 bool Ensemble::displacement_exceeds_skin() {
-    CK(cudaMemsetAsync(d_cnt + Ktot, 0, sizeof(int), stream));
-    k_displacement<<<nblk(N, 256), 256, 0, stream>>>(view(), d_xref, (unsigned*)(d_cnt + Ktot));
+    CK(cudaMemsetAsync(d_flag, 0, sizeof(int), stream));
+    k_displacement<<<nblk(N, 256), 256, 0, stream>>>(view(), d_xref, (unsigned*)d_flag);
     launches++;
     CK(cudaGetLastError());
     unsigned f = 0;
-    CK(cudaMemcpyAsync(&f, d_cnt + Ktot, sizeof(unsigned), cudaMemcpyDeviceToHost, stream));
+    CK(cudaMemcpyAsync(&f, d_flag, sizeof(unsigned), cudaMemcpyDeviceToHost, stream));
     CK(cudaStreamSynchronize(stream));
     return f != 0;
 }
@@ -1553,28 +1666,27 @@ void Ensemble::estep_bounded(int* cell) {
     k_estep_bound<<<nblk(N, 256), 256, 0, stream>>>(view(), cell, d_lbound, d_cf, d_dmax, d_gmove, d_cell_tmp,
                                                     d_fbcount);
     k_estep_warp<<<nblk(N, 128), 128, 0, stream>>>(view(), cell, d_lbound, d_cell_tmp, d_fbcount);
-    launches += 2;
+    launches += 3;
     CK(cudaGetLastError());
 }
 
 void Ensemble::morton_relabel() {
     View v = view();
     if (!bbox_ready_) {
-        // bbox init: min = +inf, max = -inf
-        k_fill_bbox<<<1, 64, 0, stream>>>(d_bbox, B);
-        launches++;
         k_bbox<<<nblk(Ktot, 256), 256, 0, stream>>>(v, d_bbox);
         launches++;
     }
     bbox_ready_ = false;
-    k_morton_keys<<<nblk(Ktot, 256), 256, 0, stream>>>(v, d_bbox, d_keys);
+    k_morton_keys<<<nblk(Ktot, 256), 256, 0, stream>>>(v, d_bbox, d_keys, d_cq_tmp, d_step, after_baoa_ == 1, d_rot_n,
+                                                       d_rmax, d_novf_n);
+    after_baoa_ = -1;
+    ovf_clean_ = true;
     launches++;
     int ntiles = nblk(Ktot, kTile);
     k_tile_sort<<<ntiles, kTile, 0, stream>>>(v, d_keys, (SortRec*)d_sortrec);
     launches++;
-    CK(cudaMemcpyAsync(d_cq_tmp, d_cq, sizeof(long long) * 3 * Ktot, cudaMemcpyDeviceToDevice, stream));
     k_rank_scatter<<<nblk((long long)ntiles * kTile, 256), 256, 0, stream>>>(v, (const SortRec*)d_sortrec, ntiles, d_cq_tmp,
-                                                                            d_new_of_old);
+                                                                            d_new_of_old, d_gcount, d_gidx, d_cf, d_bbox);
     launches++;
     CK(cudaGetLastError());
 }
@@ -1582,45 +1694,34 @@ void Ensemble::morton_relabel() {
 void Ensemble::finish_cells() {
     View v = view();
     morton_relabel();
-    build_grid();
+    scan_exclusive(d_gcount, d_gstart, Gtot + 1);
     if (prev_adj_valid_) {
-        CK(cudaMemsetAsync(d_fbcount, 0, sizeof(int), stream));
-        k_cand_rows<<<nblk((long long)Ktot * kAdjRow, 256), 256, 0, stream>>>(d_adjcount, Ktot, d_adjpad, d_new_of_old, d_cf,
-                                                                          d_candrows);
+        k_cand_rows<<<nblk((long long)Ktot * kAdjRow, 256), 256, 0, stream>>>(v, d_adjcount, d_adjpad, d_new_of_old, d_cf,
+                                                                          d_candrows, d_gidx, d_gcount);
         k_estep_rows<<<nblk(N, 128), 128, 0, stream>>>(v, d_cell, d_adjcount, d_candrows, d_rho, d_new_of_old, d_dmax,
-                                                      d_cell_new, d_cell_tmp, d_fbcount);
-        k_estep_list<<<152 * 4, 128, 0, stream>>>(v, d_cell_tmp, d_fbcount, d_cell_new);
+                                                      d_cell_new, d_cell_tmp, d_fbcount, d_cnt);
+        k_estep_list<<<152 * 4, 128, 0, stream>>>(v, d_cell_tmp, d_fbcount, d_cell_new, d_cnt);
         launches += 3;
         CK(cudaGetLastError());
     } else {
+        k_grid_fill<<<nblk(Ktot, 256), 256, 0, stream>>>(v, d_gidx, d_gcount, d_cf);
         estep(d_cell_new, nullptr);
+        k_hist<<<nblk(N, 256), 256, 0, stream>>>(N, d_cell_new, d_cnt);
+        launches += 2;
     }
     // stable counting sort
-    CK(cudaMemsetAsync(d_cnt, 0, sizeof(int) * (Ktot + 1), stream));
-    k_hist<<<nblk(N, 256), 256, 0, stream>>>(N, d_cell_new, d_cnt);
-    launches++;
     scan_exclusive(d_cnt, d_cell_start, Ktot + 1);
-    CK(cudaMemsetAsync(d_cnt, 0, sizeof(int) * (Ktot + 1), stream));
-    k_scatter<<<nblk(N, 256), 256, 0, stream>>>(N, d_cell_new, d_cell_start, d_cnt, d_perm);
-    launches++;
-    k_segsort_warp<<<nblk((long long)Ktot * 32, 256), 256, 0, stream>>>(Ktot, d_cell_start, d_perm);
-    // larger cells (rare) from lists, so that no launch scans every cell or particle
-    CK(cudaMemsetAsync(d_seglist_n, 0, sizeof(int) * 2, stream));
-    k_seglist<<<nblk(Ktot, 256), 256, 0, stream>>>(Ktot, d_cell_start, d_seglist, d_seglist + Ktot, d_seglist_n);
-    k_segsort_list<<<152, 256, 0, stream>>>(d_cell_start, d_seglist, d_seglist_n, d_perm);
-    k_segrank_list<<<152, 256, 0, stream>>>(d_cell_start, d_seglist + Ktot, d_seglist_n, d_perm, d_cell_tmp);
-    launches += 4;
+    k_scatter<<<nblk(N, 256), 256, 0, stream>>>(N, d_cell_new, d_cell_start, d_cnt, d_perm, B, d_dmax, d_fbcount);
+    k_segsort_cells<<<nblk(Ktot, 8), 256, 0, stream>>>(Ktot, d_cell_start, d_perm, d_cell_tmp);
+    launches += 2;
     CK(cudaGetLastError());
-    CK(cudaMemsetAsync(d_cnt, 0, sizeof(int) * (Ktot + 1), stream));
     // gather into the second buffer set, then swap
     swap_state();
     View nv = view();
     View ov = view_alt();
-    CK(cudaMemsetAsync(d_rmax, 0, sizeof(unsigned long long) * B, stream));
     k_gather_particles<<<nblk(N, 256), 256, 0, stream>>>(nv, ov, d_perm, d_cell_new, d_xref);
     k_cell_props<<<nblk((long long)Ktot * 32, 256), 256, 0, stream>>>(nv, d_rmax);
-    k_cell_radius<<<nblk(Ktot, 256), 256, 0, stream>>>(nv);
-    launches += 3;
+    launches += 2;
     CK(cudaGetLastError());
     // neighbouring cells
     k_adj_warp<<<nblk((long long)Ktot * 32, 256), 256, 0, stream>>>(nv, d_rmax, d_adjcount, d_rho, d_adjpad);
@@ -1645,12 +1746,15 @@ void Ensemble::adjacency_csr() {
 }
 
 void Ensemble::rebuild(bool sums_ready) {
-    // M-step on the cell-sorted particles, fused with the centroid bounding box
-    k_fill_bbox<<<1, 64, 0, stream>>>(d_bbox, B);
-    launches++;
-    CK(cudaMemsetAsync(d_dmax, 0, sizeof(unsigned) * B, stream));
-    if (sums_ready) k_mstep_apply<<<nblk(Ktot, 256), 256, 0, stream>>>(view(), d_msum, d_mcnt, d_bbox, d_dmax);
-    else k_mstep_sorted<<<nblk(Ktot, 8), 256, 0, stream>>>(view(), d_bbox, d_dmax);
+    // M-step on the cell-sorted particles, fused with the centroid bounding
+    // box (and the B-A-O-A's left-over rotations)
+    if (sums_ready) {
+        const int nb = nblk(Ktot, 256);
+        k_mstep_apply<<<nb + (after_baoa_ >= 0 ? 152 : 0), 256, 0, stream>>>(
+            view(), d_msum, d_mcnt, d_bbox, d_dmax, nb, d_step, after_baoa_, d_cell_tmp, d_rot_n);
+    } else {
+        k_mstep_sorted<<<nblk(Ktot, 8), 256, 0, stream>>>(view(), d_bbox, d_dmax);
+    }
     launches++;
     CK(cudaGetLastError());
     bbox_ready_ = true;

@@ -14,8 +14,8 @@ namespace orbc {
 
 // kernels defined in cells.cu
 __global__ void k_hist(int N, const int* __restrict__ cell, int* __restrict__ cnt);
-__global__ void k_scatter(int N, const int* __restrict__ cell, const int* __restrict__ start, int* __restrict__ cursor,
-                          int* __restrict__ tmp);
+__global__ void k_scatter(int N, const int* __restrict__ cell, const int* __restrict__ start, int* __restrict__ cnt,
+                          int* __restrict__ tmp, int B, unsigned* __restrict__ dmax, int* __restrict__ fb_count);
 __global__ void k_segsort_warp(int Ktot, const int* __restrict__ start, int* __restrict__ tmp);
 __global__ void k_segsort(int Ktot, const int* __restrict__ start, int* __restrict__ tmp, unsigned* status);
 __global__ void k_segrank(int N, const int* __restrict__ cell, const int* __restrict__ start, const int* __restrict__ tmp,
@@ -55,14 +55,13 @@ __global__ void k_check_cells(const int* __restrict__ cell, int n, int K, unsign
 
 static inline int nblk(long long n, int t) { return (int)((n + t - 1) / t); }
 
-// scratch: counts [K+1], cursor [K+1], tmp [n], flag [1]
-void cell_sort_run(const int* d_cell, int n, int K, int* d_perm, int* d_start, cudaStream_t st, int* counts,
-                   int* cursor, int* tmp, unsigned* flag) {
+// scratch: counts [K+1], tmp [n], flag [1]
+void cell_sort_run(const int* d_cell, int n, int K, int* d_perm, int* d_start, cudaStream_t st, int* counts, int* tmp,
+                   unsigned* flag) {
     CK(cudaMemsetAsync(counts, 0, sizeof(int) * (K + 1), st));
-    CK(cudaMemsetAsync(cursor, 0, sizeof(int) * (K + 1), st));
     k_hist<<<nblk(n, 256), 256, 0, st>>>(n, d_cell, counts);
     k_scan_single<<<1, 1024, 0, st>>>(counts, d_start, K + 1);
-    k_scatter<<<nblk(n, 256), 256, 0, st>>>(n, d_cell, d_start, cursor, d_perm);
+    k_scatter<<<nblk(n, 256), 256, 0, st>>>(n, d_cell, d_start, counts, d_perm, 0, nullptr, nullptr);
     k_segsort_warp<<<nblk((long long)K * 32, 256), 256, 0, st>>>(K, d_start, d_perm);
     k_segsort<<<std::min(K, 1024), 256, 0, st>>>(K, d_start, d_perm, flag);
     k_segrank<<<nblk(n, 256), 256, 0, st>>>(n, d_cell, d_start, d_perm, tmp);
@@ -87,18 +86,17 @@ extern "C" int orbc_cell_sort(const int* d_cell, int n, int K, int* d_perm, int*
     cudaStream_t st = (cudaStream_t)cuda_stream;
     void* buf = nullptr;
     try {
-        const size_t bytes = sizeof(int) * ((size_t)2 * (K + 1) + (size_t)n + 1);
+        const size_t bytes = sizeof(int) * ((size_t)(K + 1) + (size_t)n + 1);
         if (cudaMallocAsync(&buf, bytes, st) != cudaSuccess) {
             cudaGetLastError();
             return ORBC_E_NOMEM;
         }
         int* counts = (int*)buf;
-        int* cursor = counts + (K + 1);
-        int* tmp = cursor + (K + 1);
+        int* tmp = counts + (K + 1);
         unsigned* flag = (unsigned*)(tmp + n);
         int rc = ORBC_OK;
         if (n > 0 && !cell_sort_cells_valid(d_cell, n, K, st, flag)) rc = ORBC_E_ARG;
-        else if (n > 0) cell_sort_run(d_cell, n, K, d_perm, d_cell_start, st, counts, cursor, tmp, flag);
+        else if (n > 0) cell_sort_run(d_cell, n, K, d_perm, d_cell_start, st, counts, tmp, flag);
         else CK(cudaMemsetAsync(d_cell_start, 0, sizeof(int) * (K + 1), st));
         CK(cudaFreeAsync(buf, st));
         CK(cudaStreamSynchronize(st));
@@ -162,11 +160,10 @@ extern "C" int orbc_cell_sort_noalloc(const int* d_cell, int n, int K, int* d_pe
     if (!base) return ORBC_E_CUDA;
     try {
         int* counts = base;
-        int* cursor = counts + (K + 1);
-        int* tmp = cursor + (K + 1);
+        int* tmp = counts + (K + 1);
         unsigned* flag = (unsigned*)(tmp + n);
         if (n > 0 && !cell_sort_cells_valid(d_cell, n, K, st, flag)) return ORBC_E_ARG;
-        if (n > 0) cell_sort_run(d_cell, n, K, d_perm, d_cell_start, st, counts, cursor, tmp, flag);
+        if (n > 0) cell_sort_run(d_cell, n, K, d_perm, d_cell_start, st, counts, tmp, flag);
         else CK(cudaMemsetAsync(d_cell_start, 0, sizeof(int) * (K + 1), st));
         CK(cudaStreamSynchronize(st));
         return ORBC_OK;

@@ -213,6 +213,7 @@ public:
     void scan_exclusive(const int* in, int* out, long long n);
 
     // phases
+    void reset_scratch();       // the scratch that each step's launches leave ready for the next
     void build_grid();
     void mstep(const int* cell_of) { mstep_iter(cell_of, -1); }
     // iter < 0: every instance updates; dmax (nullable): largest centroid move per instance
@@ -233,6 +234,7 @@ public:
     bool fuse_steps = false;                 // run each step's B-A-O-A in the previous step's force launch
     void launch_volume(bool energies);       // after the pair and bond forces
     void alloc_lists();
+    void clear_overflow();
     void launch_integrate_first(bool fused, bool msums = false);
     void launch_kick(bool energies);
     void mirrors();
@@ -257,6 +259,10 @@ private:
     std::vector<void*> allocs_;
     int cur_ = 0;
     bool bbox_ready_ = false;   // set by the fused M-step of a rebuild
+    // what the launches of a rebuild that follows a B-A-O-A do on its behalf:
+    // -1 nothing, 0 the left-over rotations, 1 also the step counters
+    int after_baoa_ = -1;
+    bool ovf_clean_ = false;    // d_novf_n is zero
     bool csr_valid_ = false;        // d_adj_ptr / d_adj hold the current rows as CSR
     bool prev_adj_valid_ = false;   // the cell list of the previous rebuild can seed the E-step
     // timing state
@@ -279,11 +285,11 @@ public:
     float4* d_mor = nullptr;
     long long *d_cq = nullptr, *d_cq_tmp = nullptr;
     int* d_cell_start = nullptr;
-    double* d_R = nullptr;
+    double* d_R2 = nullptr;
     float* d_Rf = nullptr;
     int *d_adj_ptr = nullptr, *d_adj = nullptr, *d_adjcount = nullptr;
     long long adj_cap = 0;
-    int *d_gstart = nullptr, *d_gcount = nullptr, *d_gcent = nullptr, *d_gidx = nullptr;
+    int *d_gstart = nullptr, *d_gcount = nullptr, *d_gidx = nullptr;
     float4* d_gcf = nullptr;
     int *d_bptr = nullptr, *d_bpartner = nullptr;
     int nbond = 0;
@@ -298,7 +304,8 @@ public:
     long long* d_S = nullptr;
     long long* d_msum = nullptr;   // [3][Ktot] M-step sums from the B-A-O-A launch (zero between uses)
     int* d_mcnt = nullptr;         // [Ktot] lipids per cell, same
-    int* d_cnt = nullptr;
+    int* d_cnt = nullptr;          // [Ktot + 1] particles per cell (zero between uses)
+    int* d_flag = nullptr;         // skin trigger
     long long* d_bbox = nullptr;
     unsigned long long* d_keys = nullptr;
     void* d_sortrec = nullptr;
@@ -316,8 +323,6 @@ public:
     int* d_rot_n = nullptr;                  // lipids whose rotation the fixed-point update left to FP64
     int* d_fbcount = nullptr;                // particles the certified E-step left to the grid search
     int* d_adjpad = nullptr;                 // [Ktot][64] neighbouring-cell rows before compaction
-    int* d_seglist = nullptr;                // [2][Ktot] cells for the block sort / the rank sort
-    int* d_seglist_n = nullptr;              // [2] their counts
     AdjDesc* d_adjd = nullptr;               // [adj_cap] staging descriptors of the rows
     float4* d_candrows = nullptr;            // [adj_cap] previous rows renumbered, with centroids (E-step)
     // neighbour lists of the split pair path (valid until the next reorder)
@@ -338,8 +343,8 @@ public:
     unsigned long long* d_dump_count = nullptr;
     long long dump_cap = 0;
     std::vector<int> n_lloyd_;
-    std::vector<int*> scan_tmp_;
-    std::vector<long long> scan_tmp_n_;
+    unsigned long long* d_scan_ = nullptr;   // scan: counters, then one word per block (zero between launches)
+    long long scan_words_ = 0;
 };
 
 }  // namespace orbc

@@ -1334,11 +1334,12 @@ __global__ void __launch_bounds__(128, 4)
 // sflag (nullable): add to the side array instead, and flag the particle
 // (the evaluation with the update in its epilogue collects it).
 template <int Z, bool S0>
-__global__ void k_pair_overflow(View v, const int2* __restrict__ ovf, const int* __restrict__ novf, int ovf_cap,
-                                const int4* __restrict__ rowoff, unsigned char* __restrict__ sflag) {
+__device__ inline void pair_overflow(const View& v, const int2* __restrict__ ovf, const int* __restrict__ novf,
+                                     int ovf_cap, const int4* __restrict__ rowoff, unsigned char* __restrict__ sflag,
+                                     int at, int threads) {
     const int n = min(*novf, ovf_cap);
     const size_t N = v.N;
-    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < n; x += gridDim.x * blockDim.x) {
+    for (int x = at; x < n; x += threads) {
         const int2 pr = ovf[x];
         const int q = pr.x, e = pr.y;
         const int4 qi = v.mqr[q];
@@ -1370,6 +1371,13 @@ __global__ void k_pair_overflow(View v, const int2* __restrict__ ovf, const int*
     }
 }
 
+template <int Z, bool S0>
+__global__ void k_pair_overflow(View v, const int2* __restrict__ ovf, const int* __restrict__ novf, int ovf_cap,
+                                const int4* __restrict__ rowoff, unsigned char* __restrict__ sflag) {
+    pair_overflow<Z, S0>(v, ovf, novf, ovf_cap, rowoff, sflag, blockIdx.x * blockDim.x + threadIdx.x,
+                         gridDim.x * blockDim.x);
+}
+
 // Harmonic bonds ("Force Evaluation": a list of bonds between proteins is
 // maintained): one thread per bond, after the pair kernel wrote F.  The bond
 // force is rounded to the 2^-32 grid once and added to both ends with
@@ -1377,8 +1385,8 @@ __global__ void k_pair_overflow(View v, const int2* __restrict__ ovf, const int*
 // the order, and the result equals evaluating the bond from each end.
 // sflag (nullable): add to the side array instead, and flag both ends.
 template <typename T, bool ENERGY>
-__global__ void k_bonds(View v, long long* __restrict__ energy /* [B][8] */, unsigned char* __restrict__ sflag) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ inline void bond_one(const View& v, int q, long long* __restrict__ energy /* [B][8] */,
+                                unsigned char* __restrict__ sflag) {
     int b = -1;
     long long eb = 0, ew = 0;
     if (q < v.nbond) {
@@ -1444,6 +1452,24 @@ __global__ void k_bonds(View v, long long* __restrict__ energy /* [B][8] */, uns
     }
 }
 
+template <typename T, bool ENERGY>
+__global__ void k_bonds(View v, long long* __restrict__ energy, unsigned char* __restrict__ sflag) {
+    bond_one<T, ENERGY>(v, blockIdx.x * blockDim.x + threadIdx.x, energy, sflag);
+}
+
+// The bonds and the listed pairs beyond the lists' capacity (blocks from
+// ovf_block on) in one launch: both add to F by integer atomics after the
+// evaluation wrote it.
+template <int Z, bool S0>
+__global__ void k_bonds_overflow(View v, int ovf_block, const int2* __restrict__ ovf, const int* __restrict__ novf,
+                                 int ovf_cap, const int4* __restrict__ rowoff) {
+    if ((int)blockIdx.x < ovf_block)
+        bond_one<float, false>(v, blockIdx.x * blockDim.x + threadIdx.x, nullptr, nullptr);
+    else
+        pair_overflow<Z, S0>(v, ovf, novf, ovf_cap, rowoff, nullptr, (blockIdx.x - ovf_block) * blockDim.x + threadIdx.x,
+                             (gridDim.x - ovf_block) * blockDim.x);
+}
+
 // The pair kernel runs five CTAs per SM only with the whole unified L1 /
 // shared memory given to shared memory; ask for that once per process.
 template <typename Kern> static void prefer_shared(Kern k) {
@@ -1478,6 +1504,13 @@ void Ensemble::alloc_lists() {
     list_valid = false;
 }
 
+// The search's overflow count starts at zero: the rebuild before it left it
+// so, unless the lists are searched again without a rebuild.
+void Ensemble::clear_overflow() {
+    if (!ovf_clean_) CK(cudaMemsetAsync(d_novf_n, 0, sizeof(int), stream));
+    ovf_clean_ = false;
+}
+
 void Ensemble::launch_pairs(bool energies, bool dump) {
     View v = view();
     if (energies) CK(cudaMemsetAsync(d_energy, 0, sizeof(long long) * 8 * B, stream));
@@ -1490,7 +1523,7 @@ void Ensemble::launch_pairs(bool energies, bool dump) {
         // listed pairs beyond the lists' capacity
         if (!list_valid) {
             tic("pair_search");
-            CK(cudaMemsetAsync(d_novf_n, 0, sizeof(int), stream));
+            clear_overflow();
             if (any_mp())
                 k_pair_search<true><<<g, t, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_novf, d_novf_n, ovf_cap, d_rowoff);
             else
@@ -1521,21 +1554,30 @@ void Ensemble::launch_pairs(bool energies, bool dump) {
                 if (ctas == 5) k_pair_eval<0, true, 5, true><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff);
                 else k_pair_eval<0, true, 7, true><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff);
             }
-            k_pair_overflow<0, true><<<152, 128, 0, stream>>>(v, d_novf, d_novf_n, ovf_cap, d_rowoff, nullptr);
         } else if (z4 && s0z) {
             ORBC_EVAL(4, false);
-            k_pair_overflow<4, false><<<152, 128, 0, stream>>>(v, d_novf, d_novf_n, ovf_cap, d_rowoff, nullptr);
         } else if (z4) {
             ORBC_EVAL(4, true);
-            k_pair_overflow<4, true><<<152, 128, 0, stream>>>(v, d_novf, d_novf_n, ovf_cap, d_rowoff, nullptr);
         } else {
             ORBC_EVAL(0, true);
-            k_pair_overflow<0, true><<<152, 128, 0, stream>>>(v, d_novf, d_novf_n, ovf_cap, d_rowoff, nullptr);
         }
 #undef ORBC_EVAL
-        launches += 2;
+        launches++;
         CK(cudaGetLastError());
         toc();
+        tic("bonds");
+        const int nbb = (nbond + 255) / 256, nov = 76;
+#define ORBC_BONDS(Z, S) k_bonds_overflow<Z, S><<<nbb + nov, 256, 0, stream>>>(v, nbb, d_novf, d_novf_n, ovf_cap, d_rowoff)
+        if (any_mp()) ORBC_BONDS(0, true);
+        else if (z4 && s0z) ORBC_BONDS(4, false);
+        else if (z4) ORBC_BONDS(4, true);
+        else ORBC_BONDS(0, true);
+#undef ORBC_BONDS
+        launches++;
+        CK(cudaGetLastError());
+        toc();
+        launch_volume(false);
+        return;
     } else {
     tic("pairs");
     if (!force_f64()) {
@@ -1576,7 +1618,7 @@ void Ensemble::launch_pairs_step(bool msums) {
     prefer_shared_all();
     if (!list_valid) {
         tic("pair_search");
-        CK(cudaMemsetAsync(d_novf_n, 0, sizeof(int), stream));
+        clear_overflow();
         k_pair_search<false><<<Ktot, kPairThreads, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_novf, d_novf_n, ovf_cap,
                                                                 d_rowoff);
         launches++;

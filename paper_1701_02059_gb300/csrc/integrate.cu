@@ -47,25 +47,10 @@ __global__ void __launch_bounds__(256, 4) k_baoa_d(View v, const long long* __re
     baoa_d_body<FUSED>(v, v, p, F, Tq, steps, msum, mcnt, __activemask(), false, rot_list, rot_n);
 }
 
-// The rotational update in FP64 of the lipids that k_baoa_d (or the
-// evaluation with the update in its epilogue) listed: from the state of v
-// into the state arrays of o.  About 1e-3 of the lipids; taken inside
-// k_baoa_d, 4% of its warps would wait for one lane's FP64 code (0.49-0.50
-// against 0.47 ms for both launches on the 4M cell).
+// The left-over rotations in a launch of their own (when no rebuild follows).
 __global__ void __launch_bounds__(128) k_rot_rest(View v, View o, const long long* __restrict__ steps, int fused,
                                                   const int* __restrict__ rot_list, const int* __restrict__ rot_n) {
-    const int n = *rot_n;
-    const size_t N = v.N;
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
-        const int p = rot_list[q];
-        const int b = find_inst(v.inst_p0, v.B, p);
-        const Inst& I = v.inst[b];
-        const unsigned id = (unsigned)I.id_base + v.id[p];
-        const unsigned long long step = (unsigned long long)steps[b] + (fused ? 1ull : 0ull);
-        const uint2 key = make_uint2((unsigned)I.seed, (unsigned)(I.seed >> 32) ^ I.instance);
-        const uint4 w1 = philox4x32_10(make_uint4(id, (unsigned)step, (unsigned)(step >> 32), 1u), key);
-        rot_fp64(v.nq + p, v.wq + p, o.nq + p, o.wq + p, N, I, fused ? 2 : 1, v.T[p], v.T[N + p], v.T[2 * N + p], w1);
-    }
+    rot_rest(v, o, steps, fused, rot_list, rot_n, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 __global__ void __launch_bounds__(256) k_kick_d(View v, long long* __restrict__ steps) {
@@ -231,10 +216,18 @@ void Ensemble::launch_integrate_first(bool fused, bool msums) {
         // (the left-over list shares the E-step's, which the rebuild uses later)
         if (fused) k_baoa_d<true><<<nblk(N, 256), 256, 0, stream>>>(view(), d_step, ms, mc, d_cell_tmp, d_rot_n);
         else k_baoa_d<false><<<nblk(N, 256), 256, 0, stream>>>(view(), d_step, ms, mc, d_cell_tmp, d_rot_n);
+    }
+    launches++;
+    CK(cudaGetLastError());
+    if (msums) {
+        // the rebuild's first launches do the rest
+        after_baoa_ = fused ? 1 : 0;
+        return;
+    }
+    if (!step_f32()) {
         k_rot_rest<<<152, 128, 0, stream>>>(view(), view(), d_step, fused, d_cell_tmp, d_rot_n);
         launches++;
     }
-    launches++;
     if (fused || !step_f32()) {
         k_step_advance<<<1, 64, 0, stream>>>(d_step, B, fused, d_rot_n);
         launches++;

@@ -357,6 +357,27 @@ static __device__ __noinline__ void rot_fp64(const long long* ni, const long lon
     for (int a = 0; a < 3; a++) { no[a * N] = nq[a]; wo[a * N] = wq[a]; }
 }
 
+// The rotational update in FP64 of the lipids that k_baoa_d (or the
+// evaluation with the update in its epilogue) listed: from the state of v
+// into the state arrays of o, thread `at` of `threads`.  About 1e-3 of the
+// lipids; taken inside k_baoa_d, 4% of its warps would wait for one lane's
+// FP64 code (0.49-0.50 against 0.47 ms for both launches on the 4M cell).
+__device__ inline void rot_rest(const View& v, const View& o, const long long* __restrict__ steps, int fused,
+                                const int* __restrict__ rot_list, const int* __restrict__ rot_n, int at, int threads) {
+    const int n = *rot_n;
+    const size_t N = v.N;
+    for (int q = at; q < n; q += threads) {
+        const int p = rot_list[q];
+        const int b = find_inst(v.inst_p0, v.B, p);
+        const Inst& I = v.inst[b];
+        const unsigned id = (unsigned)I.id_base + v.id[p];
+        const unsigned long long step = (unsigned long long)steps[b] + (fused ? 1ull : 0ull);
+        const uint2 key = make_uint2((unsigned)I.seed, (unsigned)(I.seed >> 32) ^ I.instance);
+        const uint4 w1 = philox4x32_10(make_uint4(id, (unsigned)step, (unsigned)(step >> 32), 1u), key);
+        rot_fp64(v.nq + p, v.wq + p, o.nq + p, o.wq + p, N, I, fused ? 2 : 1, v.T[p], v.T[N + p], v.T[2 * N + p], w1);
+    }
+}
+
 // The same with FP64-accurate increments in grid units, all of them on the
 // integer pipes: the translational products exact (mul_round), the rotation
 // in fixed point (rotation.cuh); the lipids whose rotation it leaves to FP64

@@ -45,13 +45,47 @@
 
 namespace orbc {
 
-__global__ void k_scan_block(const int* __restrict__ in, int* __restrict__ out, long long n, int* __restrict__ sums);
-__global__ void k_scan_add(int* __restrict__ out, long long n, const int* __restrict__ offs);
 __global__ void k_scan_single(const int* __restrict__ in, int* __restrict__ out, int m);
 
 namespace {
 
-constexpr int kBlk = 1024;   // elements per k_scan_block
+constexpr int kBlk = 1024;   // elements per k_scan_block (256 threads x 4)
+
+__global__ void k_scan_block(const int* __restrict__ in, int* __restrict__ out, long long n, int* __restrict__ sums) {
+    __shared__ int warp_tot[8];
+    long long base = (long long)blockIdx.x * kBlk + threadIdx.x * 4;
+    int v[4];
+    for (int q = 0; q < 4; q++) v[q] = (base + q < n) ? in[base + q] : 0;
+    int t = v[0] + v[1] + v[2] + v[3];
+    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int x = t;
+    for (int off = 1; off < 32; off <<= 1) {
+        int y = __shfl_up_sync(0xffffffffu, x, off);
+        if (lane >= off) x += y;
+    }
+    if (lane == 31) warp_tot[w] = x;
+    __syncthreads();
+    if (w == 0) {
+        int s = (lane < 8) ? warp_tot[lane] : 0;
+        for (int off = 1; off < 8; off <<= 1) {
+            int y = __shfl_up_sync(0xffffffffu, s, off);
+            if (lane >= off) s += y;
+        }
+        if (lane < 8) warp_tot[lane] = s;
+    }
+    __syncthreads();
+    int excl = x - t + (w > 0 ? warp_tot[w - 1] : 0);
+    for (int q = 0; q < 4; q++) {
+        if (base + q < n) out[base + q] = excl;
+        excl += v[q];
+    }
+    if (threadIdx.x == blockDim.x - 1 && sums) sums[blockIdx.x] = warp_tot[7];
+}
+
+__global__ void k_scan_add(int* __restrict__ out, long long n, const int* __restrict__ offs) {
+    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] += offs[i / kBlk];
+}
 inline int nb(long long n, int t) { return (int)((n + t - 1) / t); }
 
 // Exclusive scan of n ints with a caller scratch of 2 * ceil(n / 1024) + 2.

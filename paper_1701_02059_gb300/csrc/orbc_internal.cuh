@@ -174,8 +174,8 @@ struct View {
     // cells
     long long* cq;                  // [3][Ktot] centroids on the 2^-40 grid
     int* cell_start;                // [Ktot+1]
-    double* R;                      // [Ktot] cell radius
-    float* Rf;                      // [Ktot] the same rounded to FP32 (the neighbour rule's prefilter)
+    double* R2;                     // [Ktot] squared cell radius
+    float* Rf;                      // [Ktot] cell radius in FP32 (the neighbour rule's prefilter)
     int* adj_ptr;                   // [Ktot+1]
     int* adj;                       // [adj_cap]
     struct AdjDesc* adjd;           // [Ktot][kAdjRow] staging descriptors, row k ascending by cell
@@ -183,7 +183,6 @@ struct View {
     long long adj_cap;
     // centroid search grid
     int* gstart;                    // [Gtot+1]
-    int* gcent;                     // [Ktot] centroid ids in grid order
     float4* gcf;                    // [Ktot] centroid xyz rel. to grid origin, w = id bits
     // bonds: CSR by (p0 + id)
     int* bptr;                      // [N+1]
