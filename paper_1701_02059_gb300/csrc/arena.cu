@@ -177,57 +177,6 @@ void Ensemble::setup_from(const std::vector<const Snapshot*>& list) {
     list_valid = false;
 }
 
-// ---------------------------------------------------------------- graphs
-void Ensemble::integrate_graph(int nsteps) {
-    if (!cells_valid) throw StateError("cells not initialised");
-    const bool eager = timing || d_xref != nullptr || prm_h[0].rebuild_every != 1;
-    if (eager) {
-        integrate(nsteps);
-        return;
-    }
-    if (!forces_valid) {
-        launch_pairs(false, false);
-        forces_valid = true;
-    }
-    if (nsteps <= 0) return;
-    // the first step runs eagerly (unfused; after a set-up it also seeds the
-    // E-step from the grid search); the fused steps are graph replays
-    step_body(false);
-    for (auto& x : step_h) x++;
-    for (int s = 1; s < nsteps; s++) {
-        const int p = cur_;
-        if (!graph_[p]) {
-            const long long l0 = launches, r0 = n_rebuilds;
-            cudaGraph_t g = nullptr;
-            CK(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
-            try {
-                step_body(true);
-            } catch (...) {
-                cudaStreamEndCapture(stream, &g);
-                if (g) cudaGraphDestroy(g);
-                cur_ = p;
-                throw;
-            }
-            CK(cudaStreamEndCapture(stream, &g));
-            cudaError_t e = cudaGraphInstantiate(&graph_[p], g, 0);
-            cudaGraphDestroy(g);
-            CK(e);
-            // capturing ran no kernel: restore the host-side state it advanced
-            graph_launches_ = launches - l0;
-            launches = l0;
-            n_rebuilds = r0;
-            cur_ = p;
-        }
-        CK(cudaGraphLaunch(graph_[p], stream));
-        cur_ = p ^ 1;   // the step's gather swapped the state buffers
-        launches += graph_launches_;
-        n_rebuilds++;
-        for (auto& x : step_h) x++;
-    }
-    launch_kick(false);
-    forces_valid = true;
-}
-
 // ---------------------------------------------------------------- arena
 struct ArenaSlot {
     // kFailed: the instance's own data raised a device flag (non-finite or
@@ -479,8 +428,7 @@ public:
         if (!batch_) return 0;
         long long s = max_steps;
         for (int slot : batch_slot_) s = std::min(s, slots_[slot].target - slots_[slot].done);
-        if (graphs) batch_->integrate_graph((int)s);
-        else batch_->integrate((int)s);
+        batch_->integrate((int)s, graphs);
         const unsigned st = batch_->read_status(true);
         if (st) {
             // flags that belong to single instances fail those instances

@@ -138,16 +138,17 @@ public:
     void setup_from(const std::vector<const Snapshot*>& list);
     void export_instance(int b, Snapshot& s);
     size_t bytes_allocated() const { return bytes_; }
-    // one step captured as a CUDA graph per state-buffer parity, replayed
-    void integrate_graph(int nsteps);
     void init_cells();                       // seeding + Lloyd + reorder
     // one EM update + reorder; sums_ready: the B-A-O-A launch before it
     // already summed each cell's lipid displacements (d_msum, d_mcnt)
     void rebuild(bool sums_ready = false);
     void compute_forces(bool energies);
-    void integrate(int nsteps);
+    // graphs: replay captured steps where the step's launches allow it
+    void integrate(int nsteps, bool graphs);
+    // the captured steps are stale (launch arguments or choices changed)
+    void drop_graphs();
     // velocity quench; returns the largest |F| at the end
-    double quench(int nsteps, double dt, double max_move, double max_turn);
+    double quench(int nsteps, double dt, double max_move, double max_turn, bool graphs);
     void energies(std::vector<double>& out); // [B][5] after compute_forces(true)
     // volume constraint of instance b (kv = 0: off); forces become stale
     void set_volume(int b, double kv, double v0, double area, const double xc[3]);
@@ -237,6 +238,8 @@ public:
     void clear_overflow();
     void launch_integrate_first(bool fused, bool msums = false);
     void launch_kick(bool energies);
+    void launch_quench(double dt, double max_move, double max_turn);
+    double quench_end();                     // zero velocities; the largest |F|
     void mirrors();
 
     // timing helpers
@@ -253,8 +256,17 @@ private:
     // force launch also runs the next step's B-A-O-A
     void step_body(bool fused, bool baoa_done = false, bool eval_step = false);
     size_t bytes_ = 0;
-    cudaGraphExec_t graph_[2] = {nullptr, nullptr};
-    long long graph_launches_ = 0;
+    // one step as a CUDA graph, by kind (first step of a call, a later one,
+    // quench step) and state-buffer parity
+    struct StepGraph {
+        cudaGraphExec_t exec = nullptr;
+        long long launches = 0;
+        int uses = 0;
+    };
+    StepGraph graph_[3][2];
+    bool graphs_off_ = false;      // the stream cannot be captured
+    double quench_key_[3] = {0, 0, 0};
+    template <typename F> void step_or_replay(int kind, bool graphs, F&& body);
     template <typename T> T* alloc(size_t count);
     std::vector<void*> allocs_;
     int cur_ = 0;

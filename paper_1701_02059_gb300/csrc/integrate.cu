@@ -243,17 +243,13 @@ void Ensemble::launch_kick(bool energies) {
     (void)energies;
 }
 
-double Ensemble::quench(int nsteps, double dt, double max_move, double max_turn) {
-    if (!cells_valid) throw StateError("cells not initialised");
-    if (!forces_valid) launch_pairs(false, false);
-    for (int s = 0; s < nsteps; s++) {
-        k_quench<<<nblk(N, 256), 256, 0, stream>>>(view(), dt, max_move, max_turn);
-        launches++;
-        CK(cudaGetLastError());
-        rebuild(false);
-        launch_pairs(false, false);
-    }
-    forces_valid = true;
+void Ensemble::launch_quench(double dt, double max_move, double max_turn) {
+    k_quench<<<nblk(N, 256), 256, 0, stream>>>(view(), dt, max_move, max_turn);
+    launches++;
+    CK(cudaGetLastError());
+}
+
+double Ensemble::quench_end() {
     // velocities and angular velocities zero at the end
     CK(cudaMemsetAsync(d_state[cur_][1], 0, sizeof(long long) * 3 * (size_t)N, stream));
     CK(cudaMemsetAsync(d_state[cur_][3], 0, sizeof(long long) * 3 * (size_t)N, stream));

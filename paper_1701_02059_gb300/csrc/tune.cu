@@ -83,12 +83,12 @@ static double time_tile(const HostInstance& h, int K, int ctas, int steps, cudaS
     Ensemble e(st);
     e.setup(c);
     e.init_cells();
-    e.integrate(2);
+    e.integrate(7, true);   // (captures the step)
     cudaEvent_t a, b;
     CK(cudaEventCreate(&a));
     CK(cudaEventCreate(&b));
     CK(cudaEventRecord(a, st));
-    e.integrate(steps);
+    e.integrate(steps, true);
     CK(cudaEventRecord(b, st));
     CK(cudaEventSynchronize(b));
     float ms = 0.f;

@@ -207,8 +207,7 @@ void Ensemble::set_volume(int b, double kv, double v0, double area, const double
     for (const Inst& J : inst_h) any = any || J.vol_on;
     if (any != vol_any) {
         // the captured step holds the volume launches or not
-        for (int q = 0; q < 2; q++)
-            if (graph_[q]) { cudaGraphExecDestroy(graph_[q]); graph_[q] = nullptr; }
+        drop_graphs();
     }
     vol_any = any;
     forces_valid = false;
