@@ -261,6 +261,8 @@ static Inst make_inst(const Params& P) {
         I.mm_eps_d[q] = e;
         I.mm_rc_d[q] = rc;
         I.mm_rc2[q] = rc * rc;
+        I.mm_w_d[q] = w;
+        I.mm_e2zw_d[q] = e * (2.0 * P.zeta) * w;
         I.mm_eps[q] = (float)e;
         I.mm_aw[q] = (float)w;
         I.mm_e2za[q] = (float)(e * 2.0 * P.zeta * w);

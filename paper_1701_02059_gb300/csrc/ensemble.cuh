@@ -235,6 +235,7 @@ public:
     bool fuse_steps = false;                 // run each step's B-A-O-A in the previous step's force launch
     void launch_volume(bool energies);       // after the pair and bond forces
     void alloc_lists();
+    void launch_search();
     void clear_overflow();
     void launch_integrate_first(bool fused, bool msums = false);
     void launch_kick(bool energies);

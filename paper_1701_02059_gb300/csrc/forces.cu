@@ -39,10 +39,6 @@ constexpr float kFilterBand = 1e-4f;
 // ---------------------------------------------------------------- pair terms
 // Lipid pair (see the header of orbc.h for the potential).  d = x_j - x_i.
 // Returns U; adds force on i and torque on i.
-template <typename T, typename IC>
-__device__ inline T lipid_terms(const IC& I, T dx, T dy, T dz, T r2, T nix, T niy, T niz, T njx, T njy, T njz,
-                                T& fx, T& fy, T& fz, T& tx, T& ty, T& tz, T* tj);
-
 __device__ inline float taylor_cos(float x) {
     // Maclaurin series of cos through x^14 on [0, pi/2]; truncation < 1e-9
     float x2 = x * x;
@@ -148,81 +144,23 @@ __device__ inline float lipid_terms_f(const IC& I, float dx, float dy, float dz,
     return U;
 }
 
-template <typename T, typename IC>
-__device__ inline T lipid_terms(const IC& I, T dx, T dy, T dz, T r2, T nix, T niy, T niz, T njx, T njy, T njz,
-                                T& fx, T& fy, T& fz, T& tx, T& ty, T& tz, T* tj) {
-    static_assert(sizeof(T) == 8, "the FP32 terms are lipid_terms_f");
-    double r = sqrt(r2);
-    double hx = -dx / r, hy = -dy / r, hz = -dz / r;
-    double s0 = I.s0_d;
-    double nin = nix * njx + niy * njy + niz * njz;
-    double nir = nix * hx + niy * hy + niz * hz;
-    double njr = njx * hx + njy * hy + njz * hz;
-    double a = nin - nir * njr + s0 * (njr - nir) - s0 * s0;
-    double phi = 1.0 + I.mu_d * (a - 1.0);
-    double f, fp, g, gp;
-    if (r < I.rmin_d) {
-        double q = I.rmin_d / r;
-        double q2 = q * q, q4 = q2 * q2;
-        f = I.eps_d * (q4 - 2.0 * q2) + I.eps_d;
-        fp = I.eps_d * (-4.0 * q4 / r + 4.0 * q2 / r);
-        g = -I.eps_d;
-        gp = 0.0;
-    } else {
-        double w = 1.5707963267948966 / (I.rc_d - I.rmin_d);
-        double th = w * (r - I.rmin_d);
-        double c, sn;
-        sincos(th, &sn, &c);
-        double cp = 1.0;
-        for (int k = 0; k < 2 * I.zeta - 1; k++) cp *= c;
-        f = 0.0;
-        fp = 0.0;
-        g = -I.eps_d * cp * c;
-        gp = I.eps_d * (double)(2 * I.zeta) * cp * sn * w;
-    }
-    double U = f + g * phi;
-    double wx = -njr * nix - nir * njx + s0 * (njx - nix);
-    double wy = -njr * niy - nir * njy + s0 * (njy - niy);
-    double wz = -njr * niz - nir * njz + s0 * (njz - niz);
-    double wr = wx * hx + wy * hy + wz * hz;
-    double radial = fp + gp * phi;
-    double gm = g * I.mu_d;
-    fx += -radial * hx - gm * (wx - wr * hx) / r;
-    fy += -radial * hy - gm * (wy - wr * hy) / r;
-    fz += -radial * hz - gm * (wz - wr * hz) / r;
-    double js = njr + s0;
-    double gx = njx - js * hx, gy = njy - js * hy, gz = njz - js * hz;
-    tx += -gm * (niy * gz - niz * gy);
-    ty += -gm * (niz * gx - nix * gz);
-    tz += -gm * (nix * gy - niy * gx);
-    if (tj) {
-        double is = nir - s0;
-        double ux = nix - is * hx, uy = niy - is * hy, uz = niz - is * hz;
-        tj[0] = -gm * (njy * uz - njz * uy);
-        tj[1] = -gm * (njz * ux - njx * uz);
-        tj[2] = -gm * (njx * uy - njy * ux);
-    }
-    return U;
-}
-
 // WCA; d = x_j - x_i; adds the force on i.  pp: protein-protein size.
-template <typename T>
-__device__ inline T wca_terms(const Inst& I, bool pp, T dx, T dy, T dz, T r2, T& fx, T& fy, T& fz) {
-    T sig = (sizeof(T) == 4) ? (T)(pp ? I.sig_pp : I.sig_wca) : (T)(pp ? I.sig_pp_d : I.sig_wca_d);
-    T e = (sizeof(T) == 4) ? (T)I.eps_wca : (T)I.eps_wca_d;
-    T s2 = sig * sig / r2;
-    T s6 = s2 * s2 * s2;
-    T s12 = s6 * s6;
-    T fr = (T)4 * e * ((T)12 * s12 - (T)6 * s6) / r2;
+__device__ inline float wca_terms(const Inst& I, bool pp, float dx, float dy, float dz, float r2, float& fx, float& fy,
+                                  float& fz) {
+    const float sig = pp ? I.sig_pp : I.sig_wca;
+    const float e = I.eps_wca;
+    const float s2 = sig * sig / r2;
+    const float s6 = s2 * s2 * s2;
+    const float s12 = s6 * s6;
+    const float fr = 4.0f * e * (12.0f * s12 - 6.0f * s6) / r2;
     fx -= fr * dx;
     fy -= fr * dy;
     fz -= fr * dz;
-    return (T)4 * e * (s12 - s6) + e;
+    return 4.0f * e * (s12 - s6) + e;
 }
 
 // ---------------------------------------------------------------- accumulators
-template <typename T> struct Acc;
-template <> struct Acc<float> {
+struct Acc {
     // fast path: split int32 sums (|component sum| < 1000); wider values go
     // to an int64 side array with atomics (exact, rare)
     SplitAcc f[3], t[3];
@@ -248,22 +186,6 @@ template <> struct Acc<float> {
     }
     __device__ void add_bond(const View& v, int p, float fx, float fy, float fz) { add3(v, p, f, nf, 0, fx, fy, fz); }
 };
-template <> struct Acc<double> {
-    long long f[3], t[3];
-    int np, nb;
-    __device__ void zero() { for (int a = 0; a < 3; a++) { f[a] = 0; t[a] = 0; } np = 0; nb = 0; }
-    __device__ static long long q(double v) { return __double2ll_rn(v * 4294967296.0); }
-    __device__ void add_pair(const View& v, int p, double fx, double fy, double fz, double tx, double ty, double tz) {
-        const double mag = fabs(fx) + fabs(fy) + fabs(fz) + fabs(tx) + fabs(ty) + fabs(tz);
-        if (!(mag < (double)kMaxTerm))
-            flag_inst(v, v.inst[find_inst(v.inst_p0, v.B, p)], (mag == mag) ? kStatusPairForceRange : kStatusNaN);
-        f[0] += q(fx); f[1] += q(fy); f[2] += q(fz); t[0] += q(tx); t[1] += q(ty); t[2] += q(tz); np++;
-    }
-    __device__ void add_bond(const View&, int, double fx, double fy, double fz) { f[0] += q(fx); f[1] += q(fy); f[2] += q(fz); nb++; }
-    __device__ long long F(int a) const { return f[a]; }
-    __device__ long long Tq(int a) const { return t[a]; }
-};
-
 // exact FP64 inclusion decision for a pair inside the cutoff band; m: the
 // bilayer species pair (cls 0)
 __device__ inline bool exact_inside(const View& v, const Inst& I, int pi, int pj, int cls, int m = 0) {
@@ -281,15 +203,13 @@ __device__ inline int pair_class(int ti, int tj, int& m) {
     return (bi && bj) ? 0 : ((bi || bj) ? 1 : 2);
 }
 
-// The lipid potential's constants of one bilayer species pair, in the field
-// names of Inst (FP32 and FP64), for the pair-term functions.
+// The lipid potential's FP32 constants of one bilayer species pair, in the
+// field names of Inst, for the pair-term functions.
 struct LipK {
     float eps, rmin, mu, s0, aw, eps2z_aw;
     int zeta;
-    double eps_d, rmin_d, rc_d, mu_d, s0_d;
     __device__ LipK(const Inst& I, int m)
-        : eps(I.mm_eps[m]), rmin(I.rmin), mu(I.mu), s0(I.s0), aw(I.mm_aw[m]), eps2z_aw(I.mm_e2za[m]), zeta(I.zeta),
-          eps_d(I.mm_eps_d[m]), rmin_d(I.rmin_d), rc_d(I.mm_rc_d[m]), mu_d(I.mu_d), s0_d(I.s0_d) {}
+        : eps(I.mm_eps[m]), rmin(I.rmin), mu(I.mu), s0(I.s0), aw(I.mm_aw[m]), eps2z_aw(I.mm_e2za[m]), zeta(I.zeta) {}
 };
 
 // 1-2 and 1-3 bonded pairs carry no excluded-volume term (bonded directly,
@@ -355,21 +275,17 @@ struct NbrInfo {
     int ox, oy, oz; // exact offset c_l - c_k at 2^-26 sigma (wrap-around int32)
 };
 
-template <typename T, bool S0, typename IC = Inst>
-__device__ inline T lipid_dispatch(const IC& I, T dx, T dy, T dz, T r2, T nix, T niy, T niz, T njx, T njy, T njz,
-                                   T& fx, T& fy, T& fz, T& tx, T& ty, T& tz, int zc, T* tj) {
-    if constexpr (sizeof(T) == 4) {
-        if (zc == 4)
-            return lipid_terms_f<4, S0, IC>(I, dx, dy, dz, r2, nix, niy, niz, njx, njy, njz, fx, fy, fz, tx, ty, tz, tj);
-        return lipid_terms_f<0, true, IC>(I, dx, dy, dz, r2, nix, niy, niz, njx, njy, njz, fx, fy, fz, tx, ty, tz, tj);
-    } else {
-        return lipid_terms<double, IC>(I, dx, dy, dz, r2, nix, niy, niz, njx, njy, njz, fx, fy, fz, tx, ty, tz, tj);
-    }
+template <bool S0, typename IC = Inst>
+__device__ inline float lipid_dispatch(const IC& I, float dx, float dy, float dz, float r2, float nix, float niy, float niz,
+                                       float njx, float njy, float njz, float& fx, float& fy, float& fz, float& tx,
+                                       float& ty, float& tz, int zc, float* tj) {
+    if (zc == 4)
+        return lipid_terms_f<4, S0, IC>(I, dx, dy, dz, r2, nix, niy, niz, njx, njy, njz, fx, fy, fz, tx, ty, tz, tj);
+    return lipid_terms_f<0, true, IC>(I, dx, dy, dz, r2, nix, niy, niz, njx, njy, njz, fx, fy, fz, tx, ty, tz, tj);
 }
 
-
 // S0: some instance has a spontaneous-curvature term (s0 != 0).
-template <typename T, bool ENERGY, bool DUMP, int Z, bool S0>
+template <bool ENERGY, bool DUMP, int Z, bool S0>
 __global__ void __launch_bounds__(kPairThreads, 5) k_pairs(View v, long long* __restrict__ energy /* [B][8] */,
                                                             unsigned* __restrict__ dump,
                                                             unsigned long long* __restrict__ dump_count,
@@ -528,7 +444,7 @@ __global__ void __launch_bounds__(kPairThreads, 5) k_pairs(View v, long long* __
                 blo[a] = fminf(blo[a], __shfl_xor_sync(0xffffffffu, blo[a], off));
                 bhi[a] = fmaxf(bhi[a], __shfl_xor_sync(0xffffffffu, bhi[a], off));
             }
-        Acc<T> acc;
+        Acc acc;
         acc.zero();
         double up = 0, vir = 0;     // per-particle energy and virial partials, FP64 in every mode
 
@@ -625,35 +541,16 @@ __global__ void __launch_bounds__(kPairThreads, 5) k_pairs(View v, long long* __
                         if (!in) in = exact_inside(v, I, pi, pj, cls, m);
                         if (in && cls != 0 && is_excluded(v, I, v.id[pi], v.id[pj], pj)) in = false;
                         if (!in) continue;
-                        T fx = 0, fy = 0, fz = 0, tx = 0, ty = 0, tz = 0, U;
-                        T dx, dy, dz, r2;
-                        if constexpr (sizeof(T) == 4) {
-                            dx = dxf; dy = dyf; dz = dzf; r2 = r2f;
-                        } else {
-                            dx = grid_to_double(minimg_q(v.xq[pj] - v.xq[pi], I.boxq[0], I.periodic[0]));
-                            dy = grid_to_double(minimg_q(v.xq[N + pj] - v.xq[N + pi], I.boxq[1], I.periodic[1]));
-                            dz = grid_to_double(minimg_q(v.xq[2 * N + pj] - v.xq[2 * N + pi], I.boxq[2], I.periodic[2]));
-                            r2 = dx * dx + dy * dy + dz * dz;
-                        }
-                        if (ll) {
-                            T nix, niy, niz, njx, njy, njz;
-                            if constexpr (sizeof(T) == 4) {
-                                nix = oi.x; niy = oi.y; niz = oi.z; njx = oj.x; njy = oj.y; njz = oj.z;
-                            } else {
-                                nix = grid_to_double(v.nq[pi]); niy = grid_to_double(v.nq[N + pi]);
-                                niz = grid_to_double(v.nq[2 * N + pi]);
-                                njx = grid_to_double(v.nq[pj]); njy = grid_to_double(v.nq[N + pj]);
-                                njz = grid_to_double(v.nq[2 * N + pj]);
-                            }
-                            if (I.has_mp)
-                                U = lipid_dispatch<T, S0, LipK>(LipK(I, m), dx, dy, dz, r2, nix, niy, niz, njx, njy, njz,
-                                                                fx, fy, fz, tx, ty, tz, zc, (T*)nullptr);
-                            else
-                                U = lipid_dispatch<T, S0>(I, dx, dy, dz, r2, nix, niy, niz, njx, njy, njz, fx, fy, fz, tx,
-                                                          ty, tz, zc, (T*)nullptr);
-                        } else {
-                            U = wca_terms<T>(I, cls == 2, dx, dy, dz, r2, fx, fy, fz);
-                        }
+                        float fx = 0, fy = 0, fz = 0, tx = 0, ty = 0, tz = 0, U;
+                        const float dx = dxf, dy = dyf, dz = dzf, r2 = r2f;
+                        if (ll && I.has_mp)
+                            U = lipid_dispatch<S0, LipK>(LipK(I, m), dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, fx,
+                                                         fy, fz, tx, ty, tz, zc, (float*)nullptr);
+                        else if (ll)
+                            U = lipid_dispatch<S0>(I, dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, fx, fy, fz, tx, ty,
+                                                   tz, zc, (float*)nullptr);
+                        else
+                            U = wca_terms(I, cls == 2, dx, dy, dz, r2, fx, fy, fz);
                         acc.add_pair(v, pi, fx, fy, fz, tx, ty, tz);
                         if (ENERGY) {
                             up += 0.5 * (double)U;
@@ -699,7 +596,7 @@ __global__ void __launch_bounds__(kPairThreads, 5) k_pairs(View v, long long* __
         // ((nsplit - 1) x nti <= 96 rows of 56 bytes) fit in sY, which no
         // warp reads any more.
         __syncthreads();
-        if constexpr (sizeof(T) == 4) {
+        {
             // the warps of a group hold partial sums of the same particles:
             // the later splits hand theirs over by plain stores, split 0 adds
             // them and writes the particle
@@ -718,11 +615,11 @@ __global__ void __launch_bounds__(kPairThreads, 5) k_pairs(View v, long long* __
                               acc.t[0].h, acc.t[0].l, acc.t[1].h, acc.t[1].l, acc.t[2].h, acc.t[2].l, acc.nf, acc.nt};
                 for (int q = 1; q < nsplit; q++) {
                     const int* d = red[(q - 1) * nti + r];
-#pragma unroll
+    #pragma unroll
                     for (int c = 0; c < 14; c++) sm[c] += d[c];
                 }
                 const int p = pi;
-#pragma unroll
+    #pragma unroll
                 for (int a = 0; a < 3; a++) {
                     SplitAcc f; f.h = sm[2 * a]; f.l = sm[2 * a + 1];
                     SplitAcc t; t.h = sm[6 + 2 * a]; t.l = sm[6 + 2 * a + 1];
@@ -735,20 +632,6 @@ __global__ void __launch_bounds__(kPairThreads, 5) k_pairs(View v, long long* __
                     v.F[a * N + p] = f.finish(sm[12]) + fb;
                     v.T[a * N + p] = t.finish(sm[13]) + tb;
                 }
-            }
-        } else {
-            long long (*red64)[6] = reinterpret_cast<long long (*)[6]>(&sY[0]);
-            for (int q = tid; q < kPairThreads * 6; q += kPairThreads) (&red64[0][0])[q] = 0;
-            __syncthreads();
-            if (ivalid)
-                for (int a = 0; a < 3; a++) {
-                    atomicAdd((unsigned long long*)&red64[r][a], (unsigned long long)acc.F(a));
-                    atomicAdd((unsigned long long*)&red64[r][3 + a], (unsigned long long)acc.Tq(a));
-                }
-            __syncthreads();
-            if (tid < nti) {
-                const int p = __float_as_int(v.mor[it0 + tid].w);   // slot of rank tid
-                for (int a = 0; a < 3; a++) { v.F[a * N + p] = red64[tid][a]; v.T[a * N + p] = red64[tid][3 + a]; }
             }
         }
         if (ENERGY) {
@@ -795,15 +678,231 @@ struct SNbr {
     int ox, oy, oz;
 };
 
+// The FP32 constants of the pair terms, held in registers by the evaluation.
+struct PairC {
+    float eps, rmin, mu, s0, aw, eps2z_aw, eps_wca, sig_wca, sig_pp;
+    int zeta;
+    float ll_lo, ll_hi, w_lo, w_hi, p_lo, p_hi;   // squared cutoffs -+ the FP64 decision band
+    __device__ explicit PairC(const Inst& I)
+        : eps(I.eps), rmin(I.rmin), mu(I.mu), s0(I.s0), aw(I.aw), eps2z_aw(I.eps2z_aw), eps_wca(I.eps_wca),
+          sig_wca(I.sig_wca), sig_pp(I.sig_pp), zeta(I.zeta) {
+        const float rcl = sqrtf(I.rc2f_ll), rcw = sqrtf(I.rc2f_wca), rcp = sqrtf(I.rc2f_pp);
+        ll_lo = (rcl - kCutBand) * (rcl - kCutBand); ll_hi = (rcl + kCutBand) * (rcl + kCutBand);
+        w_lo = (rcw - kCutBand) * (rcw - kCutBand); w_hi = (rcw + kCutBand) * (rcw + kCutBand);
+        p_lo = (rcp - kCutBand) * (rcp - kCutBand); p_hi = (rcp + kCutBand) * (rcp + kCutBand);
+    }
+};
+
+// ================================================================ FP64 pair forces
+// The quad loop with FP64 terms: the neighbour search below (its DIRECT form)
+// evaluates the pairs it finds instead of listing them.  GB300 issues one
+// FP64 instruction per 16 cycles and SM, so it is bound by their number:
+//   - each pair is evaluated once, by the particle of the lower id (so the
+//     result does not depend on the cell list), and both sides get their
+//     force and torque as 2^-32 integers by atomics: integer sums, any order;
+//   - a warp collects its interacting pairs in shared memory (integer and
+//     FP32 work) and evaluates 32 at a time, with all lanes full (no list, so
+//     no limit to the partners of a particle either);
+//   - the terms are arranged for few FP64 operations (about 120 a pair): one
+//     reciprocal square root by a third-order step from the FP32 one, no
+//     division, sine and cosine from their series about pi/4, positions and
+//     directors in grid units with the powers of two folded into constants.
+// The one-launch kernel that it replaces (both sides, six divisions, sqrt and
+// sincos per pair, lanes idle when their queues ran dry) took 6.30 ms for the
+// 250k vesicle, this one 0.54 ms, its FP64 pipe 81% busy; 55.0 and 9.4 ms for the 4M
+// cell.
+constexpr int kQueue64 = 64;      // a warp's queued pairs: fewer than 32 left over and up to 32 new ones
+constexpr double kTwo40 = 1099511627776.0, kTwo80 = kTwo40 * kTwo40;
+constexpr double kTwo32 = 4294967296.0;
+
+// 1/sqrt(x) for 0 < x < 2^127: y from the FP32 estimate (error below 2^-21)
+// with the third-order step y (1 + e/2 + 3 e^2/8), e = 1 - x y^2 (error e^3).
+__device__ inline double rsqrt_d(double x) {
+    const double y = (double)rsqrtf((float)x);
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+
+// sine and cosine of pi/4 + x, |x| <= pi/4: Maclaurin series through x^15 and
+// x^16 (truncation below 5e-17), combined by the addition theorem.
+__device__ inline void sincos_quarter(double x, double& s, double& c) {
+    const double x2 = x * x;
+    double p = -7.6471637318198164759e-13;          // -1/15!
+    p = fma(p, x2, 1.6059043836821614599e-10);      // 1/13!
+    p = fma(p, x2, -2.5052108385441718775e-08);     // -1/11!
+    p = fma(p, x2, 2.7557319223985890653e-06);      // 1/9!
+    p = fma(p, x2, -1.9841269841269841270e-04);     // -1/7!
+    p = fma(p, x2, 8.3333333333333333333e-03);      // 1/5!
+    p = fma(p, x2, -1.6666666666666666667e-01);     // -1/3!
+    const double sx = fma(p * x2, x, x);
+    double q = 4.7794773323873852974e-14;           // 1/16!
+    q = fma(q, x2, -1.1470745597729724714e-11);     // -1/14!
+    q = fma(q, x2, 2.0876756987868098979e-09);      // 1/12!
+    q = fma(q, x2, -2.7557319223985890653e-07);     // -1/10!
+    q = fma(q, x2, 2.4801587301587301587e-05);      // 1/8!
+    q = fma(q, x2, -1.3888888888888888889e-03);     // -1/6!
+    q = fma(q, x2, 4.1666666666666666667e-02);      // 1/4!
+    q = fma(q, x2, -0.5);
+    const double cx = fma(q, x2, 1.0);
+    const double h = 0.70710678118654752440;        // sqrt(1/2)
+    s = h * (cx + sx);
+    c = h * (cx - sx);
+}
+
+// One interacting pair from the side of pi: d = x_j - x_i and the directors in
+// grid units.  F on i (the reaction is its negative) and the torques on both,
+// as 2^-32 fixed point before rounding; the potential energy when EN.
+template <bool Z4, bool S0, bool EN>
+__device__ inline void pair_terms_d(const Inst& I, int cls, int m, const double D[3], const double A[3], const double B[3],
+                                    double f[3], double ti[3], double tj[3], double& U) {
+    const double R2 = fma(D[2], D[2], fma(D[1], D[1], D[0] * D[0]));
+    const double ri = rsqrt_d(R2 * (1.0 / kTwo80)) * (1.0 / kTwo40);      // 1/r, grid units
+    if (cls != 0) {
+        const double sig = cls == 2 ? I.sig_pp_d : I.sig_wca_d, e = I.eps_wca_d;
+        const double i2 = ri * ri, s2 = (sig * sig * kTwo80) * i2;
+        const double s6 = s2 * s2 * s2;
+        const double K = (-48.0 * e * kTwo32 * kTwo40) * (s6 * (s6 - 0.5)) * i2;
+        for (int a = 0; a < 3; a++) { f[a] = K * D[a]; ti[a] = 0.0; tj[a] = 0.0; }
+        U = EN ? fma(4.0 * e, s6 * (s6 - 1.0), e) : 0.0;
+        return;
+    }
+    const double r = R2 * ri;                                             // grid units
+    const double h[3] = {-D[0] * ri, -D[1] * ri, -D[2] * ri};
+    const double nn = fma(A[2], B[2], fma(A[1], B[1], A[0] * B[0]));      // n_i.n_j 2^80
+    const double ir = fma(A[2], h[2], fma(A[1], h[1], A[0] * h[0]));      // n_i.h 2^40
+    const double jr = fma(B[2], h[2], fma(B[1], h[1], B[0] * h[0]));
+    const double s0 = S0 ? I.s0_d * kTwo40 : 0.0;
+    double av = fma(-ir, jr, nn);                                         // a 2^80
+    if (S0) av += fma(s0, jr - ir, -s0 * s0);
+    const double mu = I.mu_d;
+    const double phi = fma(mu * (1.0 / kTwo80), av, 1.0 - mu);
+    const double eps = I.mm_eps_d[m];
+    double g, rad;                                                        // g, (f' + g' phi) 2^32
+    double fu = 0.0;
+    if (r < I.rmin_d * kTwo40) {
+        const double q = (I.rmin_d * kTwo40) * ri, q2 = q * q;
+        rad = (4.0 * eps * kTwo32 * kTwo40) * ri * fma(-q2, q2, q2);
+        if (EN) fu = fma(eps, fma(q2, q2, -2.0 * q2), eps);
+        g = -eps;
+    } else {
+        const double w = I.mm_w_d[m];
+        double c, s;
+        sincos_quarter(fma(w * (1.0 / kTwo40), r, fma(-w, I.rmin_d, -0.78539816339744830962)), s, c);
+        double cp;
+        if (Z4) {
+            const double c2 = c * c;
+            cp = (c * c2) * (c2 * c2);
+        } else {
+            cp = 1.0;
+            double bp = c;
+            for (int e = 2 * I.zeta - 1; e > 0; e >>= 1) {
+                if (e & 1) cp *= bp;
+                bp *= bp;
+            }
+        }
+        g = -eps * (cp * c);
+        rad = (I.mm_e2zw_d[m] * kTwo32) * (cp * s) * phi;
+    }
+    U = EN ? fma(g, phi, fu) : 0.0;
+    const double gm = g * (mu * kTwo32 / kTwo80);      // g mu 2^32, per product of two grid directors
+    const double gr = gm * (ri * kTwo40);              // ... / r
+    const double js = S0 ? jr + s0 : jr, is = S0 ? ir - s0 : ir;
+    // F = -(radial - g mu wr / r) h - (g mu / r) w with w = -js n_i - is n_j,
+    // wr = w.h = -(js ir + is jr)
+    const double ca = fma(gr, fma(js, ir, is * jr), rad);
+    const double cb = gr * js, cc = gr * is;
+    double gi[3], gj[3];
+    for (int a = 0; a < 3; a++) {
+        f[a] = fma(-ca, h[a], fma(cb, A[a], cc * B[a]));
+        gi[a] = fma(-js, h[a], B[a]);                  // da/dn_i
+        gj[a] = fma(-is, h[a], A[a]);                  // da/dn_j
+    }
+    for (int a = 0; a < 3; a++) {
+        const int u = a == 2 ? 0 : a + 1, w = a == 0 ? 2 : a - 1;
+        ti[a] = -gm * fma(A[u], gi[w], -(A[w] * gi[u]));
+        tj[a] = -gm * fma(B[u], gj[w], -(B[w] * gj[u]));
+    }
+}
+
+// Does the found particle interact with particle pi (mirror displacement d:
+// FP32 outside the cutoff band, exact inside it, exclusions), and is the pair
+// pi's to evaluate?  Returns the pair's class and species in code, its other
+// slot in pj.
+__device__ inline bool own_pair_d(const View& v, const Inst& I, const PairC& C, int4 qi, int pi, unsigned idi, int qj,
+                                  int ox, int oy, int oz, int& pj, int& code) {
+    const int4 mj = __ldg(v.mqr + qj);
+    int m;
+    const int cls = pair_class(qi.w & 0xff, mj.w & 0xff, m);
+    const float dx = (float)(int)((unsigned)mj.x + (unsigned)ox - (unsigned)qi.x) * kMirrorUnit,
+                dy = (float)(int)((unsigned)mj.y + (unsigned)oy - (unsigned)qi.y) * kMirrorUnit,
+                dz = (float)(int)((unsigned)mj.z + (unsigned)oz - (unsigned)qi.z) * kMirrorUnit;
+    const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+    const float lo = cls == 0 ? I.mm_lo[m] : (cls == 1 ? C.w_lo : C.p_lo);
+    const float hi = cls == 0 ? I.mm_hi[m] : (cls == 1 ? C.w_hi : C.p_hi);
+    if (r2 >= hi) return false;
+    pj = __float_as_int(__ldg(&v.mor[qj].w));
+    const Inst& J = (unsigned)(pj - I.p0) < (unsigned)I.n ? I : v.inst[I.partner];
+    if (idi > (unsigned)J.id_base + v.id[pj]) return false;
+    if (!(r2 < lo) && !exact_inside(v, I, pi, pj, cls, m)) return false;
+    if (cls != 0 && (qi.w & mj.w & kMirrorBonded) && is_excluded(v, I, v.id[pi], v.id[pj], pj)) return false;
+    code = cls | (m << 2);
+    return true;
+}
+
+// One pair's terms into F and T of both particles.
+template <bool Z4, bool S0, bool EN>
+__device__ inline void eval_pair_d(const View& v, const Inst& I, int pi, int pj, int code, long long& eu, long long& ew) {
+    const size_t N = v.N;
+    const int cls = code & 3, m = code >> 2;
+    double D[3], A[3], B[3], f[3], ti[3], tj[3], U;
+    for (int a = 0; a < 3; a++)
+        D[a] = __ll2double_rn(minimg_q(v.xq[a * N + pj] - v.xq[a * N + pi], I.boxq[a], I.periodic[a]));
+    if (cls == 0)
+        for (int a = 0; a < 3; a++) {
+            A[a] = __ll2double_rn(v.nq[a * N + pi]);
+            B[a] = __ll2double_rn(v.nq[a * N + pj]);
+        }
+    pair_terms_d<Z4, S0, EN>(I, cls, m, D, A, B, f, ti, tj, U);
+    // (a conversion saturates and turns a NaN into the most negative integer,
+    // so one integer test finds terms beyond the range and NaN)
+    const long long lim = (long long)((double)kMaxTerm * kTwo32);
+    long long q[9];
+    for (int a = 0; a < 3; a++) { q[a] = __double2ll_rn(f[a]); q[3 + a] = __double2ll_rn(ti[a]); q[6 + a] = __double2ll_rn(tj[a]); }
+    bool big = false;
+    for (int a = 0; a < 9; a++) big |= !below(q[a], lim - 1);
+    if (big) {
+        const double s = f[0] + f[1] + f[2] + ti[0] + ti[1] + ti[2] + tj[0] + tj[1] + tj[2];
+        flag_inst(v, I, s == s ? kStatusPairForceRange : kStatusNaN);
+    }
+    for (int a = 0; a < 3; a++) {
+        atomicAdd((unsigned long long*)&v.F[a * N + pi], (unsigned long long)q[a]);
+        atomicAdd((unsigned long long*)&v.F[a * N + pj], (unsigned long long)(-q[a]));
+    }
+    if (cls == 0)
+        for (int a = 0; a < 3; a++) {
+            atomicAdd((unsigned long long*)&v.T[a * N + pi], (unsigned long long)q[3 + a]);
+            atomicAdd((unsigned long long*)&v.T[a * N + pj], (unsigned long long)q[6 + a]);
+        }
+    if (EN) {
+        // energy and virial at 2^-38 (|U| < 2^25): exact sums per cell, one
+        // rounding to 2^-32 at its end
+        eu += __double2ll_rn(U * 274877906944.0);
+        ew += __double2ll_rn(fma(D[2], f[2], fma(D[1], f[1], D[0] * f[0])) * (-64.0 / kTwo40));
+    }
+}
+
 // Eight CTAs per SM (the shared-memory limit): 0.833 against 0.863 ms at seven.
 // MP (band-3 or glycophorin in the batch): the staged particles carry three
 // partner classes (lipid 0, cytoskeleton 1, bilayer protein 2) and each
 // particle culls them at its own cutoff for that class, so that a lipid's
 // list is not widened to the cutoff of its widest protein pair.
-template <bool MP>
-__global__ void __launch_bounds__(kPairThreads, 8)
+// DIRECT (FP64 forces): the pairs found are evaluated at once (pair_terms_d);
+// F and T are zero before the launch.  EN adds U_pair and the virial of the
+// cell's instance to energy [B][8].
+template <bool MP, bool DIRECT = false, bool Z4 = true, bool S0 = false, bool EN = false>
+__global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
     k_pair_search(View v, int* __restrict__ nlist, int* __restrict__ ncnt, int cap, int2* __restrict__ ovf,
-                  int* __restrict__ novf, int ovf_cap, int4* __restrict__ rowoff) {
+                  int* __restrict__ novf, int ovf_cap, int4* __restrict__ rowoff, long long* __restrict__ energy) {
     // sY: staged mirrors (int4 by the bulk copy), then in the tangent frame
     //     (FP32), w = 0 for a bilayer particle and 1 for a cytoskeleton protein
     // sQ: the list entry of each staged particle
@@ -816,6 +915,9 @@ __global__ void __launch_bounds__(kPairThreads, 8)
     __shared__ unsigned short spos[kPairThreads / 32][32];
     __shared__ SNbr nb[kMaxNbr];
     __shared__ int s_cnt[kPairThreads];
+    __shared__ int2 wq[DIRECT ? kPairThreads / 32 : 1][DIRECT ? kQueue64 : 1];       // queued pairs: slots
+    __shared__ unsigned char wc[DIRECT ? kPairThreads / 32 : 1][DIRECT ? kQueue64 : 1];   // class and species
+    __shared__ long long s_e[2];
     __shared__ unsigned long long bar;
     __shared__ int s_nstage, s_next, s_next_off, s_self, s_self_lo, s_self_hi, s_total;
 
@@ -827,7 +929,17 @@ __global__ void __launch_bounds__(kPairThreads, 8)
     const AdjDesc* __restrict__ row = v.adjd + (size_t)k * kAdjRow;
     const int a1 = min(v.adjn[k], kAdjRow);
     const size_t N = v.N;
-    const float sk = 2.0f * I.skinf + kFilterBand;
+    // (a list outlives the mirrors it was made from by up to a skin's move)
+    const float sk = (DIRECT ? 0.0f : 2.0f * I.skinf) + kFilterBand;
+    long long eu = 0, ew = 0;
+    int nq = 0;                       // the warp's queued pairs
+    auto drain = [&]() {              // evaluates the last 32 of them
+        __syncwarp();
+        nq -= 32;
+        const int2 pr = wq[warp][nq + lane];
+        eval_pair_d<Z4, S0, EN>(v, I, pr.x, pr.y, wc[warp][nq + lane], eu, ew);
+        __syncwarp();
+    };
     const float rsb = I.rsf + sk, rs2f = rsb * rsb;
     const float cw = sqrtf(I.rc2f_wca) + sk, cp = sqrtf(I.rc2f_pp) + sk;
     unsigned phase = 0;
@@ -858,7 +970,7 @@ __global__ void __launch_bounds__(kPairThreads, 8)
                     // each row's exact offset, written where the row is first
                     // staged (lane 0 of a pass that continues a split row
                     // was written in the pass before)
-                    if (it0 == cs && !(lane == 0 && na_off > 0))
+                    if (!DIRECT && it0 == cs && !(lane == 0 && na_off > 0))
                         rowoff[(size_t)k * kAdjRow + nn] = make_int4(d.ox, d.oy, d.oz, 0);
                     if (lane == 0) { st += na_off; c -= na_off; }
                 }
@@ -921,11 +1033,17 @@ __global__ void __launch_bounds__(kPairThreads, 8)
         const Frame F = tangent_frame(cn.x, cn.y, cn.z);
         const int r = igrp * gs + lane;
         const bool ivalid = wactive && lane < gs && r < nti;
-        int ti = 0;
+        int ti = 0, pi = 0;
+        unsigned idi = 0;
+        int4 qi = make_int4(0, 0, 0, 0);
         float yix = 1.0e18f, yiy = 1.0e18f, yiz = 1.0e18f;
         if (ivalid) {
-            const int4 qi = v.mqr[it0 + r];
+            qi = v.mqr[it0 + r];
             ti = qi.w & 0xff;
+            if (DIRECT) {
+                pi = __float_as_int(v.mor[it0 + r].w);
+                idi = (unsigned)I.id_base + v.id[pi];
+            }
             F.apply(qi.x * kMirrorUnit, qi.y * kMirrorUnit, qi.z * kMirrorUnit, yix, yiy, yiz);
         }
         // squared search radius for a bilayer and for a cytoskeleton partner
@@ -1053,6 +1171,28 @@ __global__ void __launch_bounds__(kPairThreads, 8)
                     }
                     if (cnt - c0 < 32) hits &= (1u << (cnt - c0)) - 1u;
                     if ((unsigned)(sp - c0) < 32u) hits &= ~(1u << (sp - c0));
+                    if constexpr (DIRECT) {
+                        const PairC C(I);
+                        while (__any_sync(0xffffffffu, hits)) {
+                            bool in = false;
+                            int pj = 0, code = 0;
+                            if (hits) {
+                                const int u = __ffs(hits) - 1;
+                                hits &= hits - 1u;
+                                const int e = sQ[cand[warp][c0 + u] >> 4];
+                                const AdjDesc& d = row[(unsigned)e >> kRowShift];
+                                in = own_pair_d(v, I, C, qi, pi, idi, e & ((1 << kRowShift) - 1), d.ox, d.oy, d.oz, pj, code);
+                            }
+                            const unsigned m2 = __ballot_sync(0xffffffffu, in);
+                            if (in) {
+                                const int at = nq + __popc(m2 & ((1u << lane) - 1u));
+                                wq[warp][at] = make_int2(pi, pj);
+                                wc[warp][at] = (unsigned char)code;
+                            }
+                            nq += __popc(m2);
+                            if (nq >= 32) drain();
+                        }
+                    }
                     while (hits) {
                         const int u = __ffs(hits) - 1;
                         hits &= hits - 1u;
@@ -1072,8 +1212,39 @@ __global__ void __launch_bounds__(kPairThreads, 8)
             na_off = next_off;
         }
         __syncthreads();
-        if (tid < nti) ncnt[it0 + tid] = s_cnt[tid];
+        if (!DIRECT && tid < nti) ncnt[it0 + tid] = s_cnt[tid];
         __syncthreads();
+    }
+    if constexpr (DIRECT) {
+        // the warps' remainders (fewer than 32 pairs each) together: the
+        // warps move theirs behind the first one's (room for 4 x 31 in the
+        // four queues), which saves two of four nearly empty rounds per cell
+        __shared__ int s_left[kPairThreads / 32];
+        int2 pr = make_int2(0, 0);
+        unsigned char code = 0;
+        __syncwarp();
+        if (lane < nq) { pr = wq[warp][lane]; code = wc[warp][lane]; }
+        if (lane == 0) s_left[warp] = nq;
+        __syncthreads();
+        int base = 0, total = 0;
+        for (int w = 0; w < kPairThreads / 32; w++) { base += w < warp ? s_left[w] : 0; total += s_left[w]; }
+        if (lane < nq) { (&wq[0][0])[base + lane] = pr; (&wc[0][0])[base + lane] = code; }
+        __syncthreads();
+        if (tid < total) {
+            pr = (&wq[0][0])[tid];
+            eval_pair_d<Z4, S0, EN>(v, I, pr.x, pr.y, (&wc[0][0])[tid], eu, ew);
+        }
+        if (EN) {
+            if (tid < 2) s_e[tid] = 0;
+            __syncthreads();
+            atomicAdd((unsigned long long*)&s_e[0], (unsigned long long)eu);
+            atomicAdd((unsigned long long*)&s_e[1], (unsigned long long)ew);
+            __syncthreads();
+            if (tid == 0) {
+                atomicAdd((unsigned long long*)&energy[b * 8 + 0], (unsigned long long)((s_e[0] + 32) >> 6));
+                atomicAdd((unsigned long long*)&energy[b * 8 + 4], (unsigned long long)((s_e[1] + 32) >> 6));
+            }
+        }
     }
 }
 
@@ -1103,30 +1274,15 @@ __device__ inline bool listed_pair(const View& v, const Inst& I, int zc, int pi,
     if (in && cls != 0 && is_excluded(v, I, v.id[pi], v.id[pj], pj)) in = false;
     if (!in) return false;
     if (ll && I.has_mp)
-        lipid_dispatch<float, S0, LipK>(LipK(I, m), dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, fx, fy, fz, tx,
+        lipid_dispatch<S0, LipK>(LipK(I, m), dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, fx, fy, fz, tx,
                                         ty, tz, zc, (float*)nullptr);
     else if (ll)
-        lipid_dispatch<float, S0>(I, dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, fx, fy, fz, tx, ty, tz, zc,
+        lipid_dispatch<S0>(I, dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, fx, fy, fz, tx, ty, tz, zc,
                                   (float*)nullptr);
     else
-        wca_terms<float>(I, cls == 2, dx, dy, dz, r2, fx, fy, fz);
+        wca_terms(I, cls == 2, dx, dy, dz, r2, fx, fy, fz);
     return true;
 }
-
-// The FP32 constants of the pair terms, held in registers by the evaluation.
-struct PairC {
-    float eps, rmin, mu, s0, aw, eps2z_aw, eps_wca, sig_wca, sig_pp;
-    int zeta;
-    float ll_lo, ll_hi, w_lo, w_hi, p_lo, p_hi;   // squared cutoffs -+ the FP64 decision band
-    __device__ explicit PairC(const Inst& I)
-        : eps(I.eps), rmin(I.rmin), mu(I.mu), s0(I.s0), aw(I.aw), eps2z_aw(I.eps2z_aw), eps_wca(I.eps_wca),
-          sig_wca(I.sig_wca), sig_pp(I.sig_pp), zeta(I.zeta) {
-        const float rcl = sqrtf(I.rc2f_ll), rcw = sqrtf(I.rc2f_wca), rcp = sqrtf(I.rc2f_pp);
-        ll_lo = (rcl - kCutBand) * (rcl - kCutBand); ll_hi = (rcl + kCutBand) * (rcl + kCutBand);
-        w_lo = (rcw - kCutBand) * (rcw - kCutBand); w_hi = (rcw + kCutBand) * (rcw + kCutBand);
-        p_lo = (rcp - kCutBand) * (rcp - kCutBand); p_hi = (rcp + kCutBand) * (rcp + kCutBand);
-    }
-};
 
 // One particle's list (the thread of rank q): the listed particles' mirrors
 // read from global memory (L1/L2), the constants of the pair terms in
@@ -1479,16 +1635,10 @@ template <typename Kern> static void prefer_shared(Kern k) {
 static void prefer_shared_all() {
     static std::once_flag once;
     std::call_once(once, [] {
-        prefer_shared(k_pairs<float, false, true, 0, true>);
-        prefer_shared(k_pairs<float, true, false, 4, true>);
-        prefer_shared(k_pairs<float, true, false, 4, false>);
-        prefer_shared(k_pairs<float, true, false, 0, true>);
-        prefer_shared(k_pairs<float, false, false, 4, true>);
-        prefer_shared(k_pairs<float, false, false, 4, false>);
-        prefer_shared(k_pairs<float, false, false, 0, true>);
-        prefer_shared(k_pairs<double, false, true, 0, true>);
-        prefer_shared(k_pairs<double, true, false, 0, true>);
-        prefer_shared(k_pairs<double, false, false, 0, true>);
+        prefer_shared(k_pairs<false, true, 0, true>);
+        prefer_shared(k_pairs<true, false, 4, true>);
+        prefer_shared(k_pairs<true, false, 4, false>);
+        prefer_shared(k_pairs<true, false, 0, true>);
     });
 }
 
@@ -1511,6 +1661,23 @@ void Ensemble::clear_overflow() {
     ovf_clean_ = false;
 }
 
+// The neighbour lists, once per cell reorder.
+void Ensemble::launch_search() {
+    if (list_valid) return;
+    tic("pair_search");
+    clear_overflow();
+    if (any_mp())
+        k_pair_search<true><<<Ktot, kPairThreads, 0, stream>>>(view(), d_nlist, d_ncnt, list_cap, d_novf, d_novf_n, ovf_cap,
+                                                               d_rowoff, nullptr);
+    else
+        k_pair_search<false><<<Ktot, kPairThreads, 0, stream>>>(view(), d_nlist, d_ncnt, list_cap, d_novf, d_novf_n,
+                                                                ovf_cap, d_rowoff, nullptr);
+    launches++;
+    CK(cudaGetLastError());
+    toc();
+    list_valid = true;
+}
+
 void Ensemble::launch_pairs(bool energies, bool dump) {
     View v = view();
     if (energies) CK(cudaMemsetAsync(d_energy, 0, sizeof(long long) * 8 * B, stream));
@@ -1521,18 +1688,7 @@ void Ensemble::launch_pairs(bool energies, bool dump) {
     if (!force_f64() && !energies && !dump) {
         // split path: neighbour lists (once per cell reorder), evaluation,
         // listed pairs beyond the lists' capacity
-        if (!list_valid) {
-            tic("pair_search");
-            clear_overflow();
-            if (any_mp())
-                k_pair_search<true><<<g, t, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_novf, d_novf_n, ovf_cap, d_rowoff);
-            else
-                k_pair_search<false><<<g, t, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_novf, d_novf_n, ovf_cap, d_rowoff);
-            launches++;
-            CK(cudaGetLastError());
-            toc();
-            list_valid = true;
-        }
+        launch_search();
         tic("pairs");
         const int ng = (int)((N + 127) / 128);
         // the batch's launch shape: the choice of its largest instance
@@ -1578,23 +1734,30 @@ void Ensemble::launch_pairs(bool energies, bool dump) {
         toc();
         launch_volume(false);
         return;
-    } else {
-    tic("pairs");
-    if (!force_f64()) {
-        if (dump) k_pairs<float, false, true, 0, true><<<g, t, 0, stream>>>(v, d_energy, d_dump, d_dump_count, dump_cap);
-        else if (energies && z4 && s0z) k_pairs<float, true, false, 4, false><<<g, t, 0, stream>>>(v, d_energy, nullptr, nullptr, 0);
-        else if (energies && z4) k_pairs<float, true, false, 4, true><<<g, t, 0, stream>>>(v, d_energy, nullptr, nullptr, 0);
-        else if (energies) k_pairs<float, true, false, 0, true><<<g, t, 0, stream>>>(v, d_energy, nullptr, nullptr, 0);
-        else if (z4 && s0z) k_pairs<float, false, false, 4, false><<<g, t, 0, stream>>>(v, d_energy, nullptr, nullptr, 0);
-        else if (z4) k_pairs<float, false, false, 4, true><<<g, t, 0, stream>>>(v, d_energy, nullptr, nullptr, 0);
-        else k_pairs<float, false, false, 0, true><<<g, t, 0, stream>>>(v, d_energy, nullptr, nullptr, 0);
-    } else {
-        if (dump) k_pairs<double, false, true, 0, true><<<g, t, 0, stream>>>(v, d_energy, d_dump, d_dump_count, dump_cap);
-        else if (energies) k_pairs<double, true, false, 0, true><<<g, t, 0, stream>>>(v, d_energy, nullptr, nullptr, 0);
-        else k_pairs<double, false, false, 0, true><<<g, t, 0, stream>>>(v, d_energy, nullptr, nullptr, 0);
     }
-    launches++;
-    toc();
+    if (dump || !force_f64()) {
+        // (the pair set is the same at every precision)
+        tic("pairs");
+        if (dump) k_pairs<false, true, 0, true><<<g, t, 0, stream>>>(v, d_energy, d_dump, d_dump_count, dump_cap);
+        else if (z4 && s0z) k_pairs<true, false, 4, false><<<g, t, 0, stream>>>(v, d_energy, nullptr, nullptr, 0);
+        else if (z4) k_pairs<true, false, 4, true><<<g, t, 0, stream>>>(v, d_energy, nullptr, nullptr, 0);
+        else k_pairs<true, false, 0, true><<<g, t, 0, stream>>>(v, d_energy, nullptr, nullptr, 0);
+        launches++;
+        CK(cudaGetLastError());
+        toc();
+    }
+    if (force_f64()) {
+        tic("pairs");
+        CK(cudaMemsetAsync(d_F, 0, sizeof(long long) * 3 * (size_t)N, stream));
+        CK(cudaMemsetAsync(d_T, 0, sizeof(long long) * 3 * (size_t)N, stream));
+#define ORBC_PAIRS_D(MP, Z4, S, EN)                                                                                   \
+    k_pair_search<MP, true, Z4, S, EN><<<g, t, 0, stream>>>(v, nullptr, nullptr, 0, nullptr, nullptr, 0, nullptr, d_energy)
+        if (!any_mp() && z4 && s0z) { if (energies) ORBC_PAIRS_D(false, true, false, true); else ORBC_PAIRS_D(false, true, false, false); }
+        else { if (energies) ORBC_PAIRS_D(true, false, true, true); else ORBC_PAIRS_D(true, false, true, false); }
+#undef ORBC_PAIRS_D
+        launches++;
+        CK(cudaGetLastError());
+        toc();
     }
     tic("bonds");
     const int nb = (int)((std::max(nbond, 1) + 255) / 256);
@@ -1616,16 +1779,7 @@ void Ensemble::launch_pairs_step(bool msums) {
     bool z4 = true, s0z = true;
     for (auto& I : inst_h) { z4 = z4 && I.zeta == 4; s0z = s0z && I.s0_d == 0.0; }
     prefer_shared_all();
-    if (!list_valid) {
-        tic("pair_search");
-        clear_overflow();
-        k_pair_search<false><<<Ktot, kPairThreads, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_novf, d_novf_n, ovf_cap,
-                                                                d_rowoff);
-        launches++;
-        CK(cudaGetLastError());
-        toc();
-        list_valid = true;
-    }
+    launch_search();
     tic("pairs_step");
     // what the epilogue cannot compute from a particle's own list goes to
     // the side array first: bonds, listed pairs beyond the lists' capacity;

@@ -132,6 +132,8 @@ struct Inst {
     int has_mp, bonded_bilayer;
     float mm_eps[9], mm_aw[9], mm_e2za[9], mm_lo[9], mm_hi[9], mm_rcf[3], mm_rcp[9];
     double mm_eps_d[9], mm_rc_d[9], mm_rc2[9];
+    // FP64 tail constants of each pair: w = (pi/2)/(rc - rmin) and eps 2 zeta w
+    double mm_w_d[9], mm_e2zw_d[9];
 };
 
 // ---------------------------------------------------------------- packed device arrays
