@@ -85,7 +85,7 @@ View Ensemble::view() {
     v.type = d_type[cur_]; v.id = d_id[cur_];
     v.cell = d_cell; v.slot_of_id = d_slot_of_id;
     v.F = d_F; v.T = d_T; v.Fbig = d_Fbig;
-    v.mq = d_mq; v.mo = d_mo; v.mqr = d_mqr; v.mor = d_mor; v.cnorm = d_cnorm; v.grank = d_grank;
+    v.mq = d_mq; v.mo = d_mo; v.mqr = d_mqr; v.mor = d_mor; v.cframe = d_cframe; v.grank = d_grank;
     v.cq = d_cq; v.cell_start = d_cell_start; v.R2 = d_R2; v.Rf = d_Rf; v.adj_ptr = d_adj_ptr; v.adj = d_adj; v.adj_cap = adj_cap; v.adjd = d_adjd;
     v.adjn = d_adjcount;
     v.gstart = d_gstart; v.gcf = d_gcf;
@@ -329,7 +329,7 @@ void Ensemble::alloc_core(const std::vector<int>& p0, const std::vector<int>& k0
     d_lbound = alloc<float>(N);
     d_cmove = alloc<float>(Ktot);
     d_cf = alloc<float4>(Ktot);
-    d_cnorm = alloc<float4>(Ktot);
+    d_cframe = alloc<float4>((size_t)3 * Ktot);
     d_grank = alloc<unsigned char>(N);
     d_dmax = alloc<unsigned>(B);
     d_fbcount = alloc<int>(1);

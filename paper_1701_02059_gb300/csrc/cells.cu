@@ -1269,7 +1269,7 @@ __device__ inline void warp_bitonic_u32(unsigned (&r)[4], int lane) {
 // Per-cell quantities read back from the gathered mirrors: one warp per cell
 // computes the squared cell radius R_k^2 = max |x - c_k|^2 (FP32 with the
 // FP64 definition inside a band) and the radius in FP32, the pair
-// kernel's cell normal (mean bilayer director, unit; +z without one) and, in
+// kernels' cell frame (its normal the mean bilayer director, +z without one) and, in
 // each tile of 128 particles, every particle's rank along the tile's longer
 // tangent extent.  rmax_bits: each instance's largest R_k^2 (bit pattern).
 // Launched with 256 threads (8 warps, one cell each).
@@ -1324,8 +1324,11 @@ __global__ void __launch_bounds__(256, 6) k_cell_props(View v, unsigned long lon
     const float nn = sqrtf(fmaf(nx, nx, fmaf(ny, ny, nz * nz)));
     if (nn > 1e-3f) { nx /= nn; ny /= nn; nz /= nn; }
     else { nx = 0.f; ny = 0.f; nz = 1.f; }
-    if (lane == 0) v.cnorm[k] = make_float4(nx, ny, nz, 0.f);
     const Frame F = tangent_frame(nx, ny, nz);
+    if (lane < 3)
+        v.cframe[3 * (size_t)k + lane] =
+            lane == 0 ? make_float4(F.r[0], F.r[1], F.r[2], 0.f)
+                      : (lane == 1 ? make_float4(F.r[3], F.r[4], F.r[5], 0.f) : make_float4(F.r[6], F.r[7], F.r[8], 0.f));
     // pair-kernel groups: ranks inside each tile of 128 particles
     for (int t0 = s; t0 < e; t0 += 128) {
         const int nt = min(128, e - t0);

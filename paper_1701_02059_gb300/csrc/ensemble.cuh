@@ -330,7 +330,7 @@ public:
     float* d_cmove = nullptr;                // [Ktot] k-means: move of each centroid in the last M-step
     unsigned* d_gmove = nullptr;             // [Gtot] k-means: largest move of the centroids in a grid cell               // [N] k-means: lower bound on the second-nearest centroid
     float4* d_cf = nullptr;                  // [Ktot] FP32 centroids by cell
-    float4* d_cnorm = nullptr;               // [Ktot] cell normals (pair-kernel frames)
+    float4* d_cframe = nullptr;              // [Ktot][3] cell frames (pair kernels)
     unsigned char* d_grank = nullptr;        // [N] pair-kernel group ranks
     unsigned* d_dmax = nullptr;              // [B] largest centroid move of the last M-step (float bits)
     int* d_rot_n = nullptr;                  // lipids whose rotation the fixed-point update left to FP64

@@ -267,6 +267,29 @@ __device__ inline bool mbar_wait_bounded(unsigned long long* bar, unsigned phase
     return false;
 }
 
+// the cell's tangent frame (prepared with the cell radii)
+__device__ inline Frame load_frame(const View& v, int k) {
+    const float4 a = __ldg(v.cframe + 3 * (size_t)k), b = __ldg(v.cframe + 3 * (size_t)k + 1),
+                 c = __ldg(v.cframe + 3 * (size_t)k + 2);
+    Frame f;
+    f.r[0] = a.x; f.r[1] = a.y; f.r[2] = a.z;
+    f.r[3] = b.x; f.r[4] = b.y; f.r[5] = b.z;
+    f.r[6] = c.x; f.r[7] = c.y; f.r[8] = c.z;
+    return f;
+}
+
+// extremes over the warp in one instruction each
+__device__ inline float warp_min_f32(float x) {
+    float r;
+    asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ inline float warp_max_f32(float x) {
+    float r;
+    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // ---------------------------------------------------------------- the kernel
 struct NbrInfo {
     int base;       // first staged index
@@ -415,8 +438,7 @@ __global__ void __launch_bounds__(kPairThreads, 5) k_pairs(View v, long long* __
         //      stored in the order of their rank along the tile's longer
         //      tangent extent (prepared with the cell radii), so that the
         //      group of rank range [g gs, (g + 1) gs) is compact
-        const float4 cn = v.cnorm[k];
-        const Frame F = tangent_frame(cn.x, cn.y, cn.z);
+        const Frame F = load_frame(v, k);
 
         // ---- this lane's particle: rank r of the tile, slot pi
         const int r = igrp * gs + lane;
@@ -439,11 +461,7 @@ __global__ void __launch_bounds__(kPairThreads, 5) k_pairs(View v, long long* __
         // group bounding box in the tangent frame, widened by the search radius
         float blo[3] = {ivalid ? yix : 3.0e38f, ivalid ? yiy : 3.0e38f, ivalid ? yiz : 3.0e38f};
         float bhi[3] = {ivalid ? yix : -3.0e38f, ivalid ? yiy : -3.0e38f, ivalid ? yiz : -3.0e38f};
-        for (int a = 0; a < 3; a++)
-            for (int off = 16; off; off >>= 1) {
-                blo[a] = fminf(blo[a], __shfl_xor_sync(0xffffffffu, blo[a], off));
-                bhi[a] = fmaxf(bhi[a], __shfl_xor_sync(0xffffffffu, bhi[a], off));
-            }
+        for (int a = 0; a < 3; a++) { blo[a] = warp_min_f32(blo[a]); bhi[a] = warp_max_f32(bhi[a]); }
         Acc acc;
         acc.zero();
         double up = 0, vir = 0;     // per-particle energy and virial partials, FP64 in every mode
@@ -1029,8 +1047,7 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
         };
         if (0 < a1) issue(0, 0);
 
-        const float4 cn = v.cnorm[k];
-        const Frame F = tangent_frame(cn.x, cn.y, cn.z);
+        const Frame F = load_frame(v, k);
         const int r = igrp * gs + lane;
         const bool ivalid = wactive && lane < gs && r < nti;
         int ti = 0, pi = 0;
@@ -1071,11 +1088,7 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
         const float rcull2 = glip ? rs2f : fmaxf(cw, cp) * fmaxf(cw, cp);
         float blo[3] = {ivalid ? yix : 3.0e38f, ivalid ? yiy : 3.0e38f, ivalid ? yiz : 3.0e38f};
         float bhi[3] = {ivalid ? yix : -3.0e38f, ivalid ? yiy : -3.0e38f, ivalid ? yiz : -3.0e38f};
-        for (int a = 0; a < 3; a++)
-            for (int off = 16; off; off >>= 1) {
-                blo[a] = fminf(blo[a], __shfl_xor_sync(0xffffffffu, blo[a], off));
-                bhi[a] = fmaxf(bhi[a], __shfl_xor_sync(0xffffffffu, bhi[a], off));
-            }
+        for (int a = 0; a < 3; a++) { blo[a] = warp_min_f32(blo[a]); bhi[a] = warp_max_f32(bhi[a]); }
         const int qi_idx = it0 + r;
 
         bool first_pass = true;
@@ -1101,9 +1114,11 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
             phase ^= 1u;
             // staged particles into the cell's frame (exact) and the tangent
             // frame (FP32), with their list entries
-            for (int q = 0; q < m; q++) {
+            // (a warp per neighbouring cell: with the whole CTA on one cell
+            // after the other, half of its warps found nothing to do)
+            for (int q = warp; q < m; q += kPairThreads / 32) {
                 const SNbr inf = nb[q];
-                for (int j = inf.base + tid; j < inf.base + inf.cnt; j += kPairThreads) {
+                for (int j = inf.base + lane; j < inf.base + inf.cnt; j += 32) {
                     const int4 rj = reinterpret_cast<const int4*>(sY)[j];
                     const int x = (int)((unsigned)rj.x + (unsigned)inf.ox);
                     const int y = (int)((unsigned)rj.y + (unsigned)inf.oy);
@@ -1193,17 +1208,33 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
                             if (nq >= 32) drain();
                         }
                     }
-                    while (hits) {
-                        const int u = __ffs(hits) - 1;
-                        hits &= hits - 1u;
-                        const int e = sQ[cand[warp][c0 + u] >> 4];
-                        const int pos = atomicAdd(&s_cnt[r], 1);
-                        if (pos < cap) {
-                            nlist[(size_t)pos * N + qi_idx] = e;
+                    if constexpr (!DIRECT) {
+                        // places in the list for all hits of the chunk at once
+                        // (the warps of a group share the particle's list)
+                        const int nh = __popc(hits);
+                        int pos = nh ? atomicAdd(&s_cnt[r], nh) : 0;
+                        if (pos + nh <= cap) {
+                            int* at = nlist + (size_t)pos * N + qi_idx;
+                            while (hits) {
+                                const int u = __ffs(hits) - 1;
+                                hits &= hits - 1u;
+                                *at = sQ[cand[warp][c0 + u] >> 4];
+                                at += N;
+                            }
                         } else {
-                            const int o = atomicAdd(novf, 1);
-                            if (o < ovf_cap) ovf[o] = make_int2(qi_idx, e);
-                            else atomicOr(v.status, kStatusListOverflow);
+                            while (hits) {
+                                const int u = __ffs(hits) - 1;
+                                hits &= hits - 1u;
+                                const int e = sQ[cand[warp][c0 + u] >> 4];
+                                if (pos < cap) {
+                                    nlist[(size_t)pos * N + qi_idx] = e;
+                                } else {
+                                    const int o = atomicAdd(novf, 1);
+                                    if (o < ovf_cap) ovf[o] = make_int2(qi_idx, e);
+                                    else atomicOr(v.status, kStatusListOverflow);
+                                }
+                                pos++;
+                            }
                         }
                     }
                 }
