@@ -660,9 +660,9 @@ void Ensemble::init_cells() {
     collect_times(kernel_times);
 }
 
-void Ensemble::compute_forces(bool energies) {
+void Ensemble::compute_forces(bool energies, bool one_launch) {
     if (!cells_valid) throw StateError("cells not initialised");
-    launch_pairs(energies, false);
+    launch_pairs(energies, false, one_launch);
     if (energies) launch_kinetic();
     forces_valid = true;
 }
@@ -1399,6 +1399,10 @@ int orbc_compute_forces(orbc_system* s, double* energies_out) {
         sync_device(s);
         s->ens->compute_forces(energies_out != nullptr);
         st = s->ens->read_status(true);
+        if (energies_out && (st & kStatusListOverflow)) {
+            s->ens->compute_forces(true, true);
+            st = s->ens->read_status(true);
+        }
         if (st) s->ens->forces_valid = false;
         if (!st && energies_out) {
             std::vector<double> e;

@@ -142,7 +142,7 @@ public:
     // one EM update + reorder; sums_ready: the B-A-O-A launch before it
     // already summed each cell's lipid displacements (d_msum, d_mcnt)
     void rebuild(bool sums_ready = false);
-    void compute_forces(bool energies);
+    void compute_forces(bool energies, bool one_launch = false);
     // graphs: replay captured steps where the step's launches allow it
     void integrate(int nsteps, bool graphs);
     // the captured steps are stale (launch arguments or choices changed)
@@ -225,7 +225,9 @@ public:
     void estep_bounded(int* cell);                  // k-means rounds after the first (bounds in d_lbound)
     void morton_relabel();
     void finish_cells();
-    void launch_pairs(bool energies, bool dump);
+    // one_launch: FP32 energies by the kernel without lists (for more partners
+    // than the lists and their overflow hold)
+    void launch_pairs(bool energies, bool dump, bool one_launch = false);
     // the forces of the current positions with the next step's B-A-O-A (after
     // this step's final B) in the evaluation's epilogue; the new state lands
     // in the other buffer, which becomes current; msums: the epilogue takes

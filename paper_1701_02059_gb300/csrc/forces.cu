@@ -1286,7 +1286,8 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
 template <int Z, bool S0>
 __device__ inline bool listed_pair(const View& v, const Inst& I, int zc, int pi, int ti, int4 qi, float4 oi, int4 mj,
                                    float4 oj, int4 o, float ll_lo, float ll_hi, float w_lo, float w_hi, float p_lo,
-                                   float p_hi, float& fx, float& fy, float& fz, float& tx, float& ty, float& tz) {
+                                   float p_hi, float& fx, float& fy, float& fz, float& tx, float& ty, float& tz, float& U,
+                                   float d[3]) {
     const int pj = __float_as_int(oj.w);
     const int tj = mj.w & 0xff;
     int m;
@@ -1304,14 +1305,15 @@ __device__ inline bool listed_pair(const View& v, const Inst& I, int zc, int pi,
     if (!in) in = exact_inside(v, I, pi, pj, cls, m);
     if (in && cls != 0 && is_excluded(v, I, v.id[pi], v.id[pj], pj)) in = false;
     if (!in) return false;
+    d[0] = dx; d[1] = dy; d[2] = dz;
     if (ll && I.has_mp)
-        lipid_dispatch<S0, LipK>(LipK(I, m), dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, fx, fy, fz, tx,
-                                        ty, tz, zc, (float*)nullptr);
+        U = lipid_dispatch<S0, LipK>(LipK(I, m), dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, fx, fy, fz, tx, ty, tz,
+                                     zc, (float*)nullptr);
     else if (ll)
-        lipid_dispatch<S0>(I, dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, fx, fy, fz, tx, ty, tz, zc,
-                                  (float*)nullptr);
+        U = lipid_dispatch<S0>(I, dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, fx, fy, fz, tx, ty, tz, zc,
+                               (float*)nullptr);
     else
-        wca_terms(I, cls == 2, dx, dy, dz, r2, fx, fy, fz);
+        U = wca_terms(I, cls == 2, dx, dy, dz, r2, fx, fy, fz);
     return true;
 }
 
@@ -1322,10 +1324,17 @@ __device__ inline bool listed_pair(const View& v, const Inst& I, int zc, int pi,
 // MP: the batch holds band-3 or glycophorin, whose pairs take the constants
 // of their bilayer species pair (the lipid-only instantiation tests the
 // lipid type alone).
-template <int Z, bool S0, bool MP = false>
+// EN: also the energies and virials of the particle's sides of its pairs
+// (11 FP64-pipe instructions a pair in FP64, at 16 cycles each and SM; split
+// integer sums take about 60 FP32 ones: 1M cell, energies included, 0.80 ms
+// in the one-launch kernel, 0.32 ms here on lists of 0.18 ms), as
+// exact sums (hi 2^-32 + lo 2^-52) in es: U, then d . F, both over all listed
+// pairs (each pair counted from both sides).
+template <int Z, bool S0, bool MP = false, bool EN = false>
 __device__ __forceinline__ void eval_list(const View& v, int q, const int* __restrict__ nlist,
                                           const int* __restrict__ ncnt, int cap, const int4* __restrict__ rowoff,
-                                          SplitAcc af[3], SplitAcc at[3], int& nterm, bool& big, int& pi_out) {
+                                          SplitAcc af[3], SplitAcc at[3], int& nterm, bool& big, int& pi_out,
+                                          long long* es = nullptr) {
     const size_t N = v.N;
     const int4 qi = v.mqr[q];
     const float4 oi = v.mor[q];
@@ -1346,6 +1355,13 @@ __device__ __forceinline__ void eval_list(const View& v, int q, const int* __res
     for (int a = 0; a < 3; a++) { af[a].zero(); at[a].zero(); }
     nterm = 0;
     big = false;
+    SplitAcc3 eu, ew;
+    int ne = 0;
+    if (EN) {
+        eu.zero();
+        ew.zero();
+        for (int a = 0; a < 4; a++) es[a] = 0;
+    }
     // the next list entry is in flight while a pair is evaluated; the
     // mirrors are read through the read-only data path
     int e_next = n > 0 ? __ldcs(nlist + q) : 0;
@@ -1381,6 +1397,7 @@ __device__ __forceinline__ void eval_list(const View& v, int q, const int* __res
             is_excluded(v, I, v.id[pi], v.id[__float_as_int(oj.w)], __float_as_int(oj.w)))
             continue;
         float f[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        float U = 0.f;
         if (ll && MP) {
             // one code path for every species pair (lanes with different
             // pairs stay converged): the pair's constants picked first
@@ -1391,17 +1408,17 @@ __device__ __forceinline__ void eval_list(const View& v, int q, const int* __res
                 Cm.eps2z_aw = I.mm_e2za[m];
             }
             if (zc == 4)
-                lipid_terms_f<4, S0>(Cm, dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, f[0], f[1], f[2], f[3],
+                U = lipid_terms_f<4, S0>(Cm, dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, f[0], f[1], f[2], f[3],
                                      f[4], f[5]);
             else
-                lipid_terms_f<0, true>(Cm, dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, f[0], f[1], f[2],
+                U = lipid_terms_f<0, true>(Cm, dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, f[0], f[1], f[2],
                                        f[3], f[4], f[5]);
         } else if (ll) {
             if (zc == 4)
-                lipid_terms_f<4, S0>(C, dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, f[0], f[1], f[2], f[3],
+                U = lipid_terms_f<4, S0>(C, dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, f[0], f[1], f[2], f[3],
                                      f[4], f[5]);
             else
-                lipid_terms_f<0, true>(C, dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, f[0], f[1], f[2], f[3],
+                U = lipid_terms_f<0, true>(C, dx, dy, dz, r2, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, f[0], f[1], f[2], f[3],
                                        f[4], f[5]);
         } else {
             const float sig = cls == 2 ? C.sig_pp : C.sig_wca;
@@ -1410,6 +1427,21 @@ __device__ __forceinline__ void eval_list(const View& v, int q, const int* __res
             const float s12 = s6 * s6;
             const float fr = 4.0f * C.eps_wca * (12.0f * s12 - 6.0f * s6) / r2;
             f[0] = -fr * dx; f[1] = -fr * dy; f[2] = -fr * dz;
+            U = 4.0f * C.eps_wca * (s12 - s6) + C.eps_wca;
+        }
+        if (EN) {
+            // the products with their rounding errors (fused multiply-adds),
+            // so that the virial's sum is as exact as the energy's
+            const float w0 = dx * f[0], w1 = dy * f[1], w2 = dz * f[2];
+            const float we = fmaf(dx, f[0], -w0) + fmaf(dy, f[1], -w1) + fmaf(dz, f[2], -w2);
+            if (fabsf(U) < 1000.0f && fabsf(w0) + fabsf(w1) + fabsf(w2) < 1000.0f) {
+                eu.add(U);
+                ew.add(w0); ew.add(w1); ew.add(w2); ew.add(we);
+                ne++;
+            } else {
+                es[0] += __double2ll_rn((double)U * 4294967296.0);
+                es[2] += __double2ll_rn(((double)w0 + (double)w1 + (double)w2 + (double)we) * 4294967296.0);
+            }
         }
         const float mag = fabsf(f[0]) + fabsf(f[1]) + fabsf(f[2]) + fabsf(f[3]) + fabsf(f[4]) + fabsf(f[5]);
         if (mag < 1000.0f) {
@@ -1424,6 +1456,13 @@ __device__ __forceinline__ void eval_list(const View& v, int q, const int* __res
             big = true;
         }
     }
+    if (EN) {
+        long long h, l;
+        eu.finish(ne, h, l);
+        es[0] += h; es[1] += l;
+        ew.finish(4 * ne, h, l);
+        es[2] += h; es[3] += l;
+    }
 }
 
 // Evaluation: one thread per particle (rank order) over its list (see
@@ -1434,17 +1473,42 @@ __device__ __forceinline__ void eval_list(const View& v, int q, const int* __res
 // seven (72 registers, a few spilled) hide more of the gathers' latency than
 // five without spills, 0.785 against 0.857 ms on the 4M cell.
 // MP: the batch holds band-3 or glycophorin (eval_list).
-template <int Z, bool S0, int MINB, bool MP = false>
+template <int Z, bool S0, int MINB, bool MP = false, bool EN = false>
 __global__ void __launch_bounds__(128, MINB)
     k_pair_eval(View v, const int* __restrict__ nlist, const int* __restrict__ ncnt, int cap,
-                const int4* __restrict__ rowoff) {
+                const int4* __restrict__ rowoff, long long* __restrict__ energy) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= v.N) return;
+    if (!EN && q >= v.N) return;
     const size_t N = v.N;
     SplitAcc af[3], at[3];
     int nterm, pi;
     bool big;
-    eval_list<Z, S0, MP>(v, q, nlist, ncnt, cap, rowoff, af, at, nterm, big, pi);
+    if constexpr (EN) {
+        // the block's sums (exact), halved (each pair has two sides) and
+        // rounded to 2^-32 once; energy [B][8] is summed over the instances
+        // of a membrane, so the block's go to its first particle's
+        __shared__ long long s_e[4];
+        if (threadIdx.x < 4) s_e[threadIdx.x] = 0;
+        __syncthreads();
+        long long es[4] = {0, 0, 0, 0};
+        if (q < v.N) eval_list<Z, S0, MP, true>(v, q, nlist, ncnt, cap, rowoff, af, at, nterm, big, pi, es);
+        for (int a = 0; a < 4; a++) {
+            for (int off = 16; off; off >>= 1) es[a] += __shfl_xor_sync(0xffffffffu, es[a], off);
+            if ((threadIdx.x & 31) == 0) atomicAdd((unsigned long long*)&s_e[a], (unsigned long long)es[a]);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            auto half = [](long long hi, long long lo) {
+                return (hi >> 1) + ((((hi & 1) << 20) + lo + (1ll << 20)) >> 21);
+            };
+            long long* e = energy + 8 * find_inst(v.inst_p0, v.B, blockIdx.x * blockDim.x);
+            atomicAdd((unsigned long long*)&e[0], (unsigned long long)half(s_e[0], s_e[1]));
+            atomicAdd((unsigned long long*)&e[4], (unsigned long long)half(-s_e[2], -s_e[3]));
+        }
+        if (q >= v.N) return;
+    } else {
+        eval_list<Z, S0, MP>(v, q, nlist, ncnt, cap, rowoff, af, at, nterm, big, pi);
+    }
 #pragma unroll
     for (int a = 0; a < 3; a++) {
         long long fb = 0, tb = 0;
@@ -1520,10 +1584,10 @@ __global__ void __launch_bounds__(128, 4)
 // so the totals are the same integers).
 // sflag (nullable): add to the side array instead, and flag the particle
 // (the evaluation with the update in its epilogue collects it).
-template <int Z, bool S0>
+template <int Z, bool S0, bool EN = false>
 __device__ inline void pair_overflow(const View& v, const int2* __restrict__ ovf, const int* __restrict__ novf,
                                      int ovf_cap, const int4* __restrict__ rowoff, unsigned char* __restrict__ sflag,
-                                     int at, int threads) {
+                                     int at, int threads, long long* __restrict__ energy = nullptr) {
     const int n = min(*novf, ovf_cap);
     const size_t N = v.N;
     for (int x = at; x < n; x += threads) {
@@ -1540,11 +1604,11 @@ __device__ inline void pair_overflow(const View& v, const int2* __restrict__ ovf
         const float rcl = sqrtf(I.rc2f_ll), rcw = sqrtf(I.rc2f_wca), rcp = sqrtf(I.rc2f_pp);
         const int qj = e & ((1 << kRowShift) - 1);
         const int4 o = rowoff[(size_t)k * kAdjRow + ((unsigned)e >> kRowShift)];
-        float f[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        float f[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, U, d[3];
         if (!listed_pair<Z, S0>(v, I, zc, pi, ti, qi, oi, v.mqr[qj], v.mor[qj], o, (rcl - kCutBand) * (rcl - kCutBand),
                                 (rcl + kCutBand) * (rcl + kCutBand), (rcw - kCutBand) * (rcw - kCutBand),
                                 (rcw + kCutBand) * (rcw + kCutBand), (rcp - kCutBand) * (rcp - kCutBand),
-                                (rcp + kCutBand) * (rcp + kCutBand), f[0], f[1], f[2], f[3], f[4], f[5]))
+                                (rcp + kCutBand) * (rcp + kCutBand), f[0], f[1], f[2], f[3], f[4], f[5], U, d))
             continue;
         const float mag = fabsf(f[0]) + fabsf(f[1]) + fabsf(f[2]) + fabsf(f[3]) + fabsf(f[4]) + fabsf(f[5]);
         if (!(mag < kMaxTerm)) flag_inst(v, I, (mag == mag) ? kStatusPairForceRange : kStatusNaN);
@@ -1555,6 +1619,11 @@ __device__ inline void pair_overflow(const View& v, const int2* __restrict__ ovf
             atomicAdd((unsigned long long*)&Tt[a * N + pi], (unsigned long long)__float2ll_rn(f[3 + a] * 4294967296.0f));
         }
         if (sflag) sflag[pi] = 1;
+        if (EN) {
+            const double w = (double)d[0] * (double)f[0] + (double)d[1] * (double)f[1] + (double)d[2] * (double)f[2];
+            atomicAdd((unsigned long long*)&energy[b * 8 + 0], (unsigned long long)__double2ll_rn((double)U * 2147483648.0));
+            atomicAdd((unsigned long long*)&energy[b * 8 + 4], (unsigned long long)__double2ll_rn(w * -2147483648.0));
+        }
     }
 }
 
@@ -1647,14 +1716,14 @@ __global__ void k_bonds(View v, long long* __restrict__ energy, unsigned char* _
 // The bonds and the listed pairs beyond the lists' capacity (blocks from
 // ovf_block on) in one launch: both add to F by integer atomics after the
 // evaluation wrote it.
-template <int Z, bool S0>
+template <int Z, bool S0, bool EN = false>
 __global__ void k_bonds_overflow(View v, int ovf_block, const int2* __restrict__ ovf, const int* __restrict__ novf,
-                                 int ovf_cap, const int4* __restrict__ rowoff) {
+                                 int ovf_cap, const int4* __restrict__ rowoff, long long* __restrict__ energy) {
     if ((int)blockIdx.x < ovf_block)
-        bond_one<float, false>(v, blockIdx.x * blockDim.x + threadIdx.x, nullptr, nullptr);
+        bond_one<float, EN>(v, blockIdx.x * blockDim.x + threadIdx.x, energy, nullptr);
     else
-        pair_overflow<Z, S0>(v, ovf, novf, ovf_cap, rowoff, nullptr, (blockIdx.x - ovf_block) * blockDim.x + threadIdx.x,
-                             (gridDim.x - ovf_block) * blockDim.x);
+        pair_overflow<Z, S0, EN>(v, ovf, novf, ovf_cap, rowoff, nullptr, (blockIdx.x - ovf_block) * blockDim.x + threadIdx.x,
+                                 (gridDim.x - ovf_block) * blockDim.x, energy);
 }
 
 // The pair kernel runs five CTAs per SM only with the whole unified L1 /
@@ -1709,14 +1778,14 @@ void Ensemble::launch_search() {
     list_valid = true;
 }
 
-void Ensemble::launch_pairs(bool energies, bool dump) {
+void Ensemble::launch_pairs(bool energies, bool dump, bool one_launch) {
     View v = view();
     if (energies) CK(cudaMemsetAsync(d_energy, 0, sizeof(long long) * 8 * B, stream));
     bool z4 = true, s0z = true;
     for (auto& I : inst_h) { z4 = z4 && I.zeta == 4; s0z = s0z && I.s0_d == 0.0; }
     const dim3 g(Ktot), t(kPairThreads);
     prefer_shared_all();
-    if (!force_f64() && !energies && !dump) {
+    if (!force_f64() && !one_launch && !dump) {
         // split path: neighbour lists (once per cell reorder), evaluation,
         // listed pairs beyond the lists' capacity
         launch_search();
@@ -1726,27 +1795,24 @@ void Ensemble::launch_pairs(bool energies, bool dump) {
         int ctas = prm_h[0].eval_ctas, nmax = -1;
         for (int b = 0; b < B; b++)
             if (inst_h[b].n > nmax) { nmax = inst_h[b].n; ctas = prm_h[b].eval_ctas; }
-#define ORBC_EVAL(Z, S)                                                                                    \
-    do {                                                                                                   \
-        if (ctas == 5) k_pair_eval<Z, S, 5><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff); \
-        else k_pair_eval<Z, S, 7><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff);          \
+        // (with energies: five CTAs per SM, for their registers)
+#define ORBC_EVAL(Z, S, MP)                                                                                                 \
+    do {                                                                                                                    \
+        if (energies) k_pair_eval<Z, S, 5, MP, true><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, d_energy); \
+        else if (ctas == 5) k_pair_eval<Z, S, 5, MP><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, nullptr);  \
+        else k_pair_eval<Z, S, 7, MP><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, nullptr);             \
     } while (0)
         if (any_mp()) {
             // band-3 or glycophorin present (or a bonded bilayer particle):
             // the evaluation with the bilayer species pairs' constants
-            if (z4 && s0z) {
-                if (ctas == 5) k_pair_eval<4, false, 5, true><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff);
-                else k_pair_eval<4, false, 7, true><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff);
-            } else {
-                if (ctas == 5) k_pair_eval<0, true, 5, true><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff);
-                else k_pair_eval<0, true, 7, true><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff);
-            }
+            if (z4 && s0z) ORBC_EVAL(4, false, true);
+            else ORBC_EVAL(0, true, true);
         } else if (z4 && s0z) {
-            ORBC_EVAL(4, false);
+            ORBC_EVAL(4, false, false);
         } else if (z4) {
-            ORBC_EVAL(4, true);
+            ORBC_EVAL(4, true, false);
         } else {
-            ORBC_EVAL(0, true);
+            ORBC_EVAL(0, true, false);
         }
 #undef ORBC_EVAL
         launches++;
@@ -1754,7 +1820,11 @@ void Ensemble::launch_pairs(bool energies, bool dump) {
         toc();
         tic("bonds");
         const int nbb = (nbond + 255) / 256, nov = 76;
-#define ORBC_BONDS(Z, S) k_bonds_overflow<Z, S><<<nbb + nov, 256, 0, stream>>>(v, nbb, d_novf, d_novf_n, ovf_cap, d_rowoff)
+#define ORBC_BONDS(Z, S)                                                                                              \
+    do {                                                                                                              \
+        if (energies) k_bonds_overflow<Z, S, true><<<nbb + nov, 256, 0, stream>>>(v, nbb, d_novf, d_novf_n, ovf_cap, d_rowoff, d_energy); \
+        else k_bonds_overflow<Z, S><<<nbb + nov, 256, 0, stream>>>(v, nbb, d_novf, d_novf_n, ovf_cap, d_rowoff, nullptr); \
+    } while (0)
         if (any_mp()) ORBC_BONDS(0, true);
         else if (z4 && s0z) ORBC_BONDS(4, false);
         else if (z4) ORBC_BONDS(4, true);
@@ -1763,7 +1833,7 @@ void Ensemble::launch_pairs(bool energies, bool dump) {
         launches++;
         CK(cudaGetLastError());
         toc();
-        launch_volume(false);
+        launch_volume(energies);
         return;
     }
     if (dump || !force_f64()) {

@@ -123,13 +123,21 @@ __global__ void k_kinetic(View v, long long* __restrict__ energy) {
     }
     // warp-aggregate per instance
     const unsigned grp = __match_any_sync(0xffffffffu, b);
-    long long st = 0, sr = 0;
-    unsigned m = grp;
-    while (m) {
-        int src = __ffs(m) - 1;
-        m &= m - 1;
-        st += __shfl_sync(grp, kt, src);
-        sr += __shfl_sync(grp, kr, src);
+    long long st = kt, sr = kr;
+    if (grp == 0xffffffffu) {
+        for (int off = 16; off; off >>= 1) {
+            st += __shfl_xor_sync(0xffffffffu, st, off);
+            sr += __shfl_xor_sync(0xffffffffu, sr, off);
+        }
+    } else {
+        st = sr = 0;
+        unsigned m = grp;
+        while (m) {
+            int src = __ffs(m) - 1;
+            m &= m - 1;
+            st += __shfl_sync(grp, kt, src);
+            sr += __shfl_sync(grp, kr, src);
+        }
     }
     if (b >= 0 && (int)(threadIdx.x & 31) == __ffs(grp) - 1) {
         atomicAdd((unsigned long long*)&energy[b * 8 + 2], (unsigned long long)st);

@@ -309,6 +309,28 @@ struct SplitAcc {
     }
 };
 
+// The same with a third level at 2^-52: for |f| < 1000 the sum of the terms
+// themselves is exact down to terms of 2^-28 (the pair energies).
+struct SplitAcc3 {
+    int h, l, m;
+    __device__ inline void zero() { h = 0; l = 0; m = 0; }
+    __device__ inline void add(float f) {
+        const float t = fmaf(f, 4096.0f, kMagic);
+        const float r = fmaf(f, 4096.0f, -(t - kMagic));
+        const float u = fmaf(r, 1048576.0f, kMagic);
+        const float q = fmaf(r, 1048576.0f, -(u - kMagic));
+        const float w = fmaf(q, 1048576.0f, kMagic);
+        h += __float_as_int(t);
+        l += __float_as_int(u);
+        m += __float_as_int(w);
+    }
+    // the sum as hi 2^-32 + lo 2^-52
+    __device__ inline void finish(int count, long long& hi, long long& lo) const {
+        hi = ((long long)(h - count * kMagicBits) << 20) + (long long)(l - count * kMagicBits);
+        lo = (long long)(m - count * kMagicBits);
+    }
+};
+
 // Round a float to the 2^-40 grid as int64 (exact FP32 splitting, |v| < 2^11).
 __device__ inline long long float_to_grid(float v) {
     // v * 2^40 = h * 2^20 + l  with h = round(v * 2^20), |v * 2^20| < 2^22 required -> |v| < 4
