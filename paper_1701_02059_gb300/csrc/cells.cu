@@ -1622,7 +1622,7 @@ void Ensemble::mstep_iter(const int* cell_of, int iter, unsigned* dmax) {
 }
 
 void Ensemble::mirrors() {
-    k_mirrors<<<nblk(N, 256), 256, 0, stream>>>(view());
+    k_mirrors<<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(view());
     launches++;
     CK(cudaGetLastError());
 }
@@ -1647,7 +1647,7 @@ __global__ void k_displacement(View v, const long long* __restrict__ xref, unsig
 
 bool Ensemble::displacement_exceeds_skin() {
     CK(cudaMemsetAsync(d_flag, 0, sizeof(int), stream));
-    k_displacement<<<nblk(N, 256), 256, 0, stream>>>(view(), d_xref, (unsigned*)d_flag);
+    k_displacement<<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(view(), d_xref, (unsigned*)d_flag);
     launches++;
     CK(cudaGetLastError());
     unsigned f = 0;
@@ -1701,7 +1701,7 @@ void Ensemble::finish_cells() {
     if (prev_adj_valid_) {
         k_cand_rows<<<nblk((long long)Ktot * kAdjRow, 256), 256, 0, stream>>>(v, d_adjcount, d_adjpad, d_new_of_old, d_cf,
                                                                           d_candrows, d_gidx, d_gcount);
-        k_estep_rows<<<nblk(N, 128), 128, 0, stream>>>(v, d_cell, d_adjcount, d_candrows, d_rho, d_new_of_old, d_dmax,
+        k_estep_rows<<<nblk(N, spread_block(N, 128)), spread_block(N, 128), 0, stream>>>(v, d_cell, d_adjcount, d_candrows, d_rho, d_new_of_old, d_dmax,
                                                       d_cell_new, d_cell_tmp, d_fbcount, d_cnt);
         k_estep_list<<<152 * 4, 128, 0, stream>>>(v, d_cell_tmp, d_fbcount, d_cell_new, d_cnt);
         launches += 3;
@@ -1722,12 +1722,12 @@ void Ensemble::finish_cells() {
     swap_state();
     View nv = view();
     View ov = view_alt();
-    k_gather_particles<<<nblk(N, 256), 256, 0, stream>>>(nv, ov, d_perm, d_cell_new, d_xref);
-    k_cell_props<<<nblk((long long)Ktot * 32, 256), 256, 0, stream>>>(nv, d_rmax);
+    k_gather_particles<<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(nv, ov, d_perm, d_cell_new, d_xref);
+    k_cell_props<<<nblk((long long)Ktot * 32, spread_block((long long)Ktot * 32, 256)), spread_block((long long)Ktot * 32, 256), 0, stream>>>(nv, d_rmax);
     launches += 2;
     CK(cudaGetLastError());
     // neighbouring cells
-    k_adj_warp<<<nblk((long long)Ktot * 32, 256), 256, 0, stream>>>(nv, d_rmax, d_adjcount, d_rho, d_adjpad);
+    k_adj_warp<<<nblk((long long)Ktot * 32, spread_block((long long)Ktot * 32, 256)), spread_block((long long)Ktot * 32, 256), 0, stream>>>(nv, d_rmax, d_adjcount, d_rho, d_adjpad);
     launches++;
     CK(cudaGetLastError());
     prev_adj_valid_ = true;

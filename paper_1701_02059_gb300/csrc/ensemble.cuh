@@ -97,6 +97,13 @@ struct BondSpec {
 // One instance's carried state in device buffers of its own: what a packed
 // batch needs to continue the instance bit for bit after it is re-packed
 // (state, forces, centroids, cell ownership in the cell-sorted order).
+// Threads per block of a kernel that works thread by thread or warp by warp
+// (no block-wide step): 64 while the launch has fewer threads than the chip
+// holds, so that they spread over every SM evenly (62k particles in blocks of
+// 256 leave 90 of 152 SMs with two blocks and the others with one), else the
+// kernel's own size.
+inline int spread_block(long long threads, int full) { return threads <= 152ll * 2048 ? 64 : full; }
+
 struct Snapshot {
     Inst inst;                                // descriptor (p0, k0, g0 of the batch it came from)
     Params prm;

@@ -1330,11 +1330,13 @@ __device__ inline bool listed_pair(const View& v, const Inst& I, int zc, int pi,
 // in the one-launch kernel, 0.32 ms here on lists of 0.18 ms), as
 // exact sums (hi 2^-32 + lo 2^-52) in es: U, then d . F, both over all listed
 // pairs (each pair counted from both sides).
+// The list's entries t0, t0 + dt, ... (dt > 1: several threads share a
+// particle).
 template <int Z, bool S0, bool MP = false, bool EN = false>
 __device__ __forceinline__ void eval_list(const View& v, int q, const int* __restrict__ nlist,
                                           const int* __restrict__ ncnt, int cap, const int4* __restrict__ rowoff,
                                           SplitAcc af[3], SplitAcc at[3], int& nterm, bool& big, int& pi_out,
-                                          long long* es = nullptr) {
+                                          long long* es = nullptr, int t0 = 0, int dt = 1) {
     const size_t N = v.N;
     const int4 qi = v.mqr[q];
     const float4 oi = v.mor[q];
@@ -1364,10 +1366,10 @@ __device__ __forceinline__ void eval_list(const View& v, int q, const int* __res
     }
     // the next list entry is in flight while a pair is evaluated; the
     // mirrors are read through the read-only data path
-    int e_next = n > 0 ? __ldcs(nlist + q) : 0;
-    for (int t = 0; t < n; t++) {
+    int e_next = t0 < n ? __ldcs(nlist + (size_t)t0 * N + q) : 0;
+    for (int t = t0; t < n; t += dt) {
         const int e = e_next;
-        if (t + 1 < n) e_next = __ldcs(nlist + (size_t)(t + 1) * N + q);
+        if (t + dt < n) e_next = __ldcs(nlist + (size_t)(t + dt) * N + q);
         const int qj = e & ((1 << kRowShift) - 1);
         const int4 o = __ldg(ro + ((unsigned)e >> kRowShift));
         const int4 mj = __ldg(v.mqr + qj);
@@ -1513,6 +1515,58 @@ __global__ void __launch_bounds__(128, MINB)
     for (int a = 0; a < 3; a++) {
         long long fb = 0, tb = 0;
         if (big) {
+            fb = __ldcg(&v.Fbig[(size_t)a * N + pi]);
+            tb = __ldcg(&v.Fbig[(size_t)(3 + a) * N + pi]);
+            v.Fbig[(size_t)a * N + pi] = 0;
+            v.Fbig[(size_t)(3 + a) * N + pi] = 0;
+        }
+        v.F[a * N + pi] = af[a].finish(nterm) + fb;
+        v.T[a * N + pi] = at[a].finish(nterm) + tb;
+    }
+}
+
+// The same with 2^sh threads per particle (neighbouring lanes), for batches
+// that one thread per particle spreads too thinly: a thread's chain of
+// gathers and pair terms is what such a launch lasts (2,304 particles 20.5 us
+// with one thread, 14.3 with four; 20k 26.2 and 18.0; 62k 32.7 and 26.6 with
+// two; 145k are better off with one, 44.7 against 45.9).  The partial sums
+// are integers, so the result is the same.
+template <int Z, bool S0, bool MP>
+__global__ void __launch_bounds__(128, 7)
+    k_pair_eval_split(View v, const int* __restrict__ nlist, const int* __restrict__ ncnt, int cap,
+                      const int4* __restrict__ rowoff, int sh) {
+    const long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int q = (int)(x >> sh), part = (int)(x & ((1 << sh) - 1));
+    const unsigned live = __ballot_sync(0xffffffffu, q < v.N);
+    if (q >= v.N) return;
+    const size_t N = v.N;
+    SplitAcc af[3], at[3];
+    int nterm, pi;
+    bool big;
+    eval_list<Z, S0, MP>(v, q, nlist, ncnt, cap, rowoff, af, at, nterm, big, pi, nullptr, part, 1 << sh);
+    __syncwarp(live);
+    for (int off = 1 << (sh - 1); off; off >>= 1) {
+        for (int a = 0; a < 3; a++) {
+            af[a].h += __shfl_xor_sync(live, af[a].h, off);
+            af[a].l += __shfl_xor_sync(live, af[a].l, off);
+            at[a].h += __shfl_xor_sync(live, at[a].h, off);
+            at[a].l += __shfl_xor_sync(live, at[a].l, off);
+        }
+        nterm += __shfl_xor_sync(live, nterm, off);
+    }
+    // (the large terms of the other lanes are in the side array before it is read)
+    const unsigned anybig = __ballot_sync(live, big);
+    if (anybig) {
+        __threadfence();
+        __syncwarp(live);
+    }
+    if (part != 0) return;
+    const int lane = threadIdx.x & 31;
+    const bool mine = (anybig >> lane) & ((1u << (1 << sh)) - 1u);
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        long long fb = 0, tb = 0;
+        if (mine) {
             fb = __ldcg(&v.Fbig[(size_t)a * N + pi]);
             tb = __ldcg(&v.Fbig[(size_t)(3 + a) * N + pi]);
             v.Fbig[(size_t)a * N + pi] = 0;
@@ -1795,10 +1849,17 @@ void Ensemble::launch_pairs(bool energies, bool dump, bool one_launch) {
         int ctas = prm_h[0].eval_ctas, nmax = -1;
         for (int b = 0; b < B; b++)
             if (inst_h[b].n > nmax) { nmax = inst_h[b].n; ctas = prm_h[b].eval_ctas; }
+        // threads per particle: as many as fit the chip at once (seven CTAs
+        // of 128 on each of 152 SMs), up to four (eight gain nothing more on
+        // 2,304 particles and lose 2.6 us on 20,000)
+        int sh = 0;
+        while (sh < 2 && ((long long)N << (sh + 1)) <= 152ll * 7 * 128) sh++;
+        const int nsp = (int)((((long long)N << sh) + 127) / 128);
         // (with energies: five CTAs per SM, for their registers)
 #define ORBC_EVAL(Z, S, MP)                                                                                                 \
     do {                                                                                                                    \
         if (energies) k_pair_eval<Z, S, 5, MP, true><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, d_energy); \
+        else if (sh > 0) k_pair_eval_split<Z, S, MP><<<nsp, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, sh);     \
         else if (ctas == 5) k_pair_eval<Z, S, 5, MP><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, nullptr);  \
         else k_pair_eval<Z, S, 7, MP><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, nullptr);             \
     } while (0)

@@ -218,12 +218,12 @@ void Ensemble::launch_integrate_first(bool fused, bool msums) {
     long long* ms = msums ? d_msum : nullptr;
     int* mc = msums ? d_mcnt : nullptr;
     if (step_f32()) {
-        if (fused) k_baoa<float, true><<<nblk(N, 256), 256, 0, stream>>>(view(), d_step, ms, mc);
-        else k_baoa<float, false><<<nblk(N, 256), 256, 0, stream>>>(view(), d_step, ms, mc);
+        if (fused) k_baoa<float, true><<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(view(), d_step, ms, mc);
+        else k_baoa<float, false><<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(view(), d_step, ms, mc);
     } else {
         // (the left-over list shares the E-step's, which the rebuild uses later)
-        if (fused) k_baoa_d<true><<<nblk(N, 256), 256, 0, stream>>>(view(), d_step, ms, mc, d_cell_tmp, d_rot_n);
-        else k_baoa_d<false><<<nblk(N, 256), 256, 0, stream>>>(view(), d_step, ms, mc, d_cell_tmp, d_rot_n);
+        if (fused) k_baoa_d<true><<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(view(), d_step, ms, mc, d_cell_tmp, d_rot_n);
+        else k_baoa_d<false><<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(view(), d_step, ms, mc, d_cell_tmp, d_rot_n);
     }
     launches++;
     CK(cudaGetLastError());
@@ -244,15 +244,15 @@ void Ensemble::launch_integrate_first(bool fused, bool msums) {
 }
 
 void Ensemble::launch_kick(bool energies) {
-    if (step_f32()) k_kick<float><<<nblk(N, 256), 256, 0, stream>>>(view(), d_step);
-    else k_kick_d<<<nblk(N, 256), 256, 0, stream>>>(view(), d_step);
+    if (step_f32()) k_kick<float><<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(view(), d_step);
+    else k_kick_d<<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(view(), d_step);
     launches++;
     CK(cudaGetLastError());
     (void)energies;
 }
 
 void Ensemble::launch_quench(double dt, double max_move, double max_turn) {
-    k_quench<<<nblk(N, 256), 256, 0, stream>>>(view(), dt, max_move, max_turn);
+    k_quench<<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(view(), dt, max_move, max_turn);
     launches++;
     CK(cudaGetLastError());
 }
