@@ -256,20 +256,11 @@ __device__ inline unsigned long long spread3(unsigned long long x) {
 
 // Key: 21 bits per axis, q = min(2^21 - 1, floor((c - lo) * 2^21 / (hi - lo)))
 // in FP64 exactly as the definition (c - lo is exact on the grid).  Also
-// copies the centroids for the permutation that follows, and does what the
-// step's earlier launches left to a later one (K >= B): the step counters
-// (advance), the empty list of left-over rotations, the largest radii and
-// the overflow count of the pair search to come.
+// copies the centroids for the permutation that follows.
 __global__ void k_morton_keys(View v, const long long* __restrict__ bb, unsigned long long* __restrict__ key,
-                              long long* __restrict__ cq_copy, long long* __restrict__ steps, int advance,
-                              int* __restrict__ rot_n, unsigned long long* __restrict__ rmax, int* __restrict__ novf) {
+                              long long* __restrict__ cq_copy) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= v.Ktot) return;
-    if (k < v.B) {
-        if (advance) steps[k] += 1;
-        rmax[k] = 0ull;
-        if (k == 0) { *rot_n = 0; *novf = 0; }
-    }
     int b = find_inst(v.inst_k0, v.B, k);
     unsigned long long kk = 0;
     for (int a = 0; a < 3; a++) {
@@ -361,14 +352,17 @@ __device__ inline int grid_coord(long long xq, const Inst& I, int a, float& rel)
 
 // Centroid k's grid cell: counted (gcount), noted (gidx) and its FP32 position
 // relative to the grid origin (cf).
-__device__ inline void grid_count_one(const Inst& I, int k, long long x, long long y, long long z,
-                                      int* __restrict__ gcount, int* __restrict__ gidx, float4* __restrict__ cf) {
+__device__ inline int grid_count_one(const Inst& I, int k, long long x, long long y, long long z,
+                                     int* __restrict__ gcount, int* __restrict__ gidx, float4* __restrict__ cf,
+                                     float4* f = nullptr) {
     float r[3];
     const int gx = grid_coord(x, I, 0, r[0]), gy = grid_coord(y, I, 1, r[1]), gz = grid_coord(z, I, 2, r[2]);
     const long long g = I.g0 + ((long long)gz * I.gdim[1] + gy) * I.gdim[0] + gx;
     gidx[k] = (int)g;
     cf[k] = make_float4(r[0], r[1], r[2], 0.f);
+    if (f) *f = make_float4(r[0], r[1], r[2], 0.f);
     atomicAdd(&gcount[g], 1);
+    return (int)g;
 }
 
 __global__ void k_grid_count(View v, int* __restrict__ gcount, int* __restrict__ gidx, float4* __restrict__ cf) {
@@ -456,6 +450,206 @@ __global__ void k_rank_scatter(View v, const SortRec* __restrict__ tiles, int nt
         v.cq[(size_t)a * v.Ktot + nk] = c[a];
     }
     grid_count_one(I, nk, c[0], c[1], c[2], gcount, gidx, cf);
+}
+
+// ============================================================== small batches
+// M-step, Morton relabel and centroid grid of one instance of up to kSmallK
+// cells in one block: five launches (M-step, keys, tile sort, ranks, grid
+// scan) of one to four blocks each otherwise, 32-45 us of the 98-136 us of a
+// step on 2,304 to 62k particles.  The outputs are those launches' (the
+// grid's order inside a cell aside, which nothing depends on).  The blocks
+// after the first take the left-over rotations (see k_mstep_apply).
+constexpr int kSmallK = 1024;
+constexpr int kSmallG = 1 << 16;
+
+__device__ inline long long warp_min_ll(long long x) {
+    for (int off = 16; off; off >>= 1) x = min(x, __shfl_xor_sync(0xffffffffu, x, off));
+    return x;
+}
+
+__global__ void __launch_bounds__(kSmallK) k_relabel_small(
+    View v, int mstep, long long* __restrict__ S, int* __restrict__ cnt, unsigned* __restrict__ dmax,
+    long long* __restrict__ bb, int* __restrict__ new_of_old, int* gcount, int* __restrict__ gidx, float4* __restrict__ cf,
+    int* gstart, const long long* __restrict__ steps, int fused, const int* __restrict__ rot_list,
+    const int* __restrict__ rot_n) {
+    if (blockIdx.x > 0) {
+        rot_rest(v, v, steps, fused, rot_list, rot_n, (blockIdx.x - 1) * blockDim.x + threadIdx.x,
+                 (gridDim.x - 1) * blockDim.x);
+        return;
+    }
+    __shared__ long long sc[3][kSmallK];                  // centroids by old index
+    __shared__ unsigned long long skey[kSmallK];
+    __shared__ unsigned short sidx[kSmallK];
+    __shared__ long long red[32][6];                      // per warp: min x, y, z, -max x, y, z
+    __shared__ float redm[32];
+    __shared__ long long s_lo[3], s_hi[3];
+    __shared__ unsigned long long s_m[3];                 // s = 2^21 / (hi - lo) = s_m 2^(es - 63)
+    __shared__ int s_sh[3], s_r[3];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int K = v.Ktot;
+    const size_t Ks = K;
+    const Inst& I = v.inst[0];
+    // M-step (k_mstep_apply's update)
+    long long c[3] = {0, 0, 0};
+    float mv2 = 0.f;
+    if (t < K) {
+        const int n = mstep ? cnt[t] : 0;
+        for (int a = 0; a < 3; a++) {
+            c[a] = v.cq[a * Ks + t];
+            if (mstep) {
+                long long step = 0;
+                if (n > 0) step = floor_div_ll(2 * S[a * Ks + t] + n, 2 * (long long)n);
+                const float sf = ll_to_float(step) * (float)kGridInv;
+                mv2 = fmaf(sf, sf, mv2);
+                c[a] += step;
+                if (I.periodic[a]) c[a] = floor_mod_ll(c[a], I.boxq[a]);
+                S[a * Ks + t] = 0;
+            }
+            sc[a][t] = c[a];
+        }
+        if (mstep) cnt[t] = 0;
+    }
+    // bounding box and largest move
+    for (int a = 0; a < 3; a++) {
+        const long long mn = warp_min_ll(t < K ? c[a] : 0x7fffffffffffffffll);
+        const long long mx = warp_min_ll(t < K ? -c[a] : 0x7fffffffffffffffll);
+        if (lane == 0) { red[w][a] = mn; red[w][3 + a] = mx; }
+    }
+    {
+        const float mv = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(sqrtf(mv2) * 1.0001f + 1e-6f)));
+        if (lane == 0) redm[w] = mv;
+    }
+    __syncthreads();
+    if (w == 0) {
+        for (int a = 0; a < 6; a++) {
+            const long long m = warp_min_ll(red[lane][a]);
+            if (lane == 0) { if (a < 3) s_lo[a] = m; else s_hi[a - 3] = -m; }
+        }
+        const unsigned mv = __reduce_max_sync(0xffffffffu, __float_as_uint(redm[lane]));
+        if (lane == 0 && mstep) dmax[0] = mv;
+        __syncwarp();
+        if (lane < 3) {
+            // the keys' scale as the definition computes it, split for the
+            // integer evaluation below
+            const long long D = s_hi[lane] - s_lo[lane];
+            const double s = D > 0 ? __ddiv_rn(2097152.0, __dsub_rn(grid_to_double(s_hi[lane]), grid_to_double(s_lo[lane]))) : 0.0;
+            const long long bits = __double_as_longlong(s);
+            const int es = (int)(bits >> 52) - 1023;
+            s_m[lane] = D > 0 ? ((unsigned long long)(bits & 0xfffffffffffffll) | (1ull << 52)) << 11 : 0ull;
+            s_sh[lane] = D > 0 ? __clzll(D) - 1 : 0;
+            s_r[lane] = D > 0 ? 7 + s_sh[lane] - es : 8;
+        }
+        if (lane < 6) bb[lane] = lane < 3 ? 0x7fffffffffffffffll : (-0x7fffffffffffffffll - 1);
+    }
+    __syncthreads();
+    // Morton keys: q = floor(fl((c - lo) s)).  (c - lo) s to 2^-32 in integers
+    // (FP64 here would wait for the FP64 pipe of one SM); only a fraction
+    // within 2^-32 of one can round to the next integer, and takes FP64.
+    unsigned long long key = ~0ull;
+    int idx = 0x7fff;
+    if (t < K) {
+        key = 0;
+        idx = t;
+        for (int a = 0; a < 3; a++) {
+            const unsigned long long d = (unsigned long long)(c[a] - s_lo[a]);
+            const unsigned long long f = __umul64hi(d << s_sh[a], s_m[a]) >> s_r[a];
+            unsigned long long q = f >> 32;
+            if ((unsigned)f == 0xffffffffu) {
+                const double lo = grid_to_double(s_lo[a]);
+                const double s = __ddiv_rn(2097152.0, __dsub_rn(grid_to_double(s_hi[a]), lo));
+                q = (unsigned long long)floor(__dmul_rn(__dsub_rn(grid_to_double(c[a]), lo), s));
+            }
+            key |= spread3(min(q, 2097151ull)) << a;
+        }
+    }
+    // bitonic sort of (key, index) over the next power of two (whole warps)
+    int P = 32;
+    while (P < K) P <<= 1;
+    for (int size = 2; size <= P; size <<= 1) {
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            unsigned long long ok = key;
+            int oi = idx;
+            if (stride >= 32) {
+                if (t < P) { skey[t] = key; sidx[t] = (unsigned short)idx; }
+                __syncthreads();
+                if (t < P) { ok = skey[t ^ stride]; oi = sidx[t ^ stride]; }
+                __syncthreads();
+            } else if (t < P) {
+                ok = __shfl_xor_sync(0xffffffffu, key, stride);
+                oi = __shfl_xor_sync(0xffffffffu, idx, stride);
+            }
+            const bool lower = (t & stride) == 0, up = (t & size) == 0;
+            const bool less = ok < key || (ok == key && oi < idx);
+            if (t < P && (lower == up) == less && (ok != key || oi != idx)) { key = ok; idx = oi; }
+        }
+    }
+    // the record of rank t: old cell idx becomes cell t
+    int gc = 0;
+    float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (t < K) {
+        new_of_old[idx] = t;
+        for (int a = 0; a < 3; a++) {
+            c[a] = sc[a][idx];
+            v.cq[a * Ks + t] = c[a];
+        }
+        gc = grid_count_one(I, t, c[0], c[1], c[2], gcount, gidx, cf, &f);
+    }
+    __threadfence();
+    __syncthreads();
+    // grid starts: exclusive scan of the counts (written by atomics above:
+    // read past L1), a contiguous chunk per thread, the first eight counts
+    // kept for the second pass
+    const int G = (int)v.Gtot + 1, per = ((G + kSmallK - 1) / kSmallK + 3) & ~3, g0 = min(t * per, G), g1 = min(g0 + per, G);
+    int4 k0 = make_int4(0, 0, 0, 0), k1 = k0;
+    if (g0 + 8 <= g1) {
+        k0 = __ldcg(reinterpret_cast<const int4*>(gcount + g0));
+        k1 = __ldcg(reinterpret_cast<const int4*>(gcount + g0 + 4));
+    } else {
+        int q[8];
+#pragma unroll
+        for (int u = 0; u < 8; u++) q[u] = g0 + u < g1 ? __ldcg(gcount + g0 + u) : 0;
+        k0 = make_int4(q[0], q[1], q[2], q[3]);
+        k1 = make_int4(q[4], q[5], q[6], q[7]);
+    }
+    int sum = k0.x + k0.y + k0.z + k0.w + k1.x + k1.y + k1.z + k1.w;
+    for (int g = g0 + 8; g < g1; g++) sum += __ldcg(gcount + g);
+    int x = sum;
+    for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, off);
+        if (lane >= off) x += y;
+    }
+    int* wtot = reinterpret_cast<int*>(&red[0][0]);
+    if (lane == 31) wtot[w] = x;
+    __syncthreads();
+    if (w == 0) {
+        int s = wtot[lane];
+        for (int off = 1; off < 32; off <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, s, off);
+            if (lane >= off) s += y;
+        }
+        wtot[lane] = s;
+    }
+    __syncthreads();
+    int run = x - sum + (w > 0 ? wtot[w - 1] : 0);
+    {
+        const int q[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+#pragma unroll
+        for (int u = 0; u < 8; u++) {
+            if (g0 + u < g1) gstart[g0 + u] = run;
+            run += q[u];
+        }
+    }
+    for (int g = g0 + 8; g < g1; g++) {
+        gstart[g] = run;
+        run += __ldcg(gcount + g);
+    }
+    __threadfence();
+    __syncthreads();
+    if (t < K) {
+        const int pos = __ldcg(gstart + gc) + atomicSub(&gcount[gc], 1) - 1;
+        f.w = __int_as_float(t);
+        v.gcf[pos] = f;
+    }
 }
 
 // ============================================================== E-step
@@ -890,12 +1084,12 @@ __global__ void __launch_bounds__(256) k_estep_bound(View v, const int* __restri
 // The previous rows with their cells renumbered and the renumbered cells'
 // FP32 centroids (w = new index), so the E-step reads one record per
 // candidate instead of three dependent loads; the first K threads also put
-// the centroids in grid order.
+// the centroids in grid order (gcount not null).
 __global__ void k_cand_rows(View v, const int* __restrict__ cnt_old, const int* __restrict__ pad_old,
                             const int* __restrict__ new_of_old, const float4* __restrict__ cf,
                             float4* __restrict__ rows, const int* __restrict__ gidx, int* __restrict__ gcount) {
     const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // one thread per row slot
-    if (q < v.Ktot) grid_fill_one(v, (int)q, gidx, gcount, cf);
+    if (gcount && q < v.Ktot) grid_fill_one(v, (int)q, gidx, gcount, cf);
     if (q >= (long long)v.Ktot * kAdjRow || (int)(q % kAdjRow) >= cnt_old[q / kAdjRow]) return;
     const int j = new_of_old[pad_old[q]];
     float4 c = cf[j];
@@ -999,13 +1193,18 @@ __global__ void k_hist(int N, const int* __restrict__ cell, int* __restrict__ cn
 
 // Slot of each particle inside its cell's range (in any order across warps;
 // the per-cell sort that follows restores the storage order).  The counts
-// are taken down to zero, ready for the next histogram.  dmax, fb_count
-// (nullable): the E-step's inputs, cleared for the next rebuild (N >= B).
+// are taken down to zero, ready for the next histogram.  In a rebuild
+// (B > 0 <= N) it also does what the launches before it left to a later one:
+// see ScratchReset.
 __global__ void k_scatter(int N, const int* __restrict__ cell, const int* __restrict__ start, int* __restrict__ cnt,
-                          int* __restrict__ tmp, int B, unsigned* __restrict__ dmax, int* __restrict__ fb_count) {
+                          int* __restrict__ tmp, int B, ScratchReset z) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < B) dmax[i] = 0u;
-    if (i == 0 && fb_count) *fb_count = 0;
+    if (i < B) {
+        z.dmax[i] = 0u;
+        z.rmax[i] = 0ull;
+        if (z.advance) z.steps[i] += 1;
+        if (i == 0) { *z.fb_count = 0; *z.rot_n = 0; *z.novf = 0; }
+    }
     const int c = (i < N) ? cell[i] : -1;
     const unsigned peers = __match_any_sync(0xffffffffu, c);
     const int lane = threadIdx.x & 31;
@@ -1680,10 +1879,7 @@ void Ensemble::morton_relabel() {
         launches++;
     }
     bbox_ready_ = false;
-    k_morton_keys<<<nblk(Ktot, 256), 256, 0, stream>>>(v, d_bbox, d_keys, d_cq_tmp, d_step, after_baoa_ == 1, d_rot_n,
-                                                       d_rmax, d_novf_n);
-    after_baoa_ = -1;
-    ovf_clean_ = true;
+    k_morton_keys<<<nblk(Ktot, 256), 256, 0, stream>>>(v, d_bbox, d_keys, d_cq_tmp);
     launches++;
     int ntiles = nblk(Ktot, kTile);
     k_tile_sort<<<ntiles, kTile, 0, stream>>>(v, d_keys, (SortRec*)d_sortrec);
@@ -1694,27 +1890,45 @@ void Ensemble::morton_relabel() {
     CK(cudaGetLastError());
 }
 
-void Ensemble::finish_cells() {
+bool Ensemble::small_cells() const { return B == 1 && Ktot <= kSmallK && Gtot < kSmallG; }
+
+void Ensemble::finish_cells(bool sums_ready) {
     View v = view();
-    morton_relabel();
-    scan_exclusive(d_gcount, d_gstart, Gtot + 1);
+    const bool small = small_cells();
+    if (small) {
+        const int rot = after_baoa_ >= 0 ? 4 : 0;
+        k_relabel_small<<<1 + rot, kSmallK, 0, stream>>>(v, sums_ready, d_msum, d_mcnt, d_dmax, d_bbox, d_new_of_old, d_gcount,
+                                                         d_gidx, d_cf, d_gstart, d_step, after_baoa_, d_cell_tmp, d_rot_n);
+        launches++;
+        CK(cudaGetLastError());
+        bbox_ready_ = false;
+    } else {
+        morton_relabel();
+        scan_exclusive(d_gcount, d_gstart, Gtot + 1);
+    }
     if (prev_adj_valid_) {
         k_cand_rows<<<nblk((long long)Ktot * kAdjRow, 256), 256, 0, stream>>>(v, d_adjcount, d_adjpad, d_new_of_old, d_cf,
-                                                                          d_candrows, d_gidx, d_gcount);
-        k_estep_rows<<<nblk(N, spread_block(N, 128)), spread_block(N, 128), 0, stream>>>(v, d_cell, d_adjcount, d_candrows, d_rho, d_new_of_old, d_dmax,
-                                                      d_cell_new, d_cell_tmp, d_fbcount, d_cnt);
+                                                                          d_candrows, d_gidx, small ? nullptr : d_gcount);
+        k_estep_rows<<<nblk(N, spread_block(N, 128)), spread_block(N, 128), 0, stream>>>(
+            v, d_cell, d_adjcount, d_candrows, d_rho, d_new_of_old, d_dmax, d_cell_new, d_cell_tmp, d_fbcount, d_cnt);
         k_estep_list<<<152 * 4, 128, 0, stream>>>(v, d_cell_tmp, d_fbcount, d_cell_new, d_cnt);
         launches += 3;
         CK(cudaGetLastError());
     } else {
-        k_grid_fill<<<nblk(Ktot, 256), 256, 0, stream>>>(v, d_gidx, d_gcount, d_cf);
+        if (!small) {
+            k_grid_fill<<<nblk(Ktot, 256), 256, 0, stream>>>(v, d_gidx, d_gcount, d_cf);
+            launches++;
+        }
         estep(d_cell_new, nullptr);
         k_hist<<<nblk(N, 256), 256, 0, stream>>>(N, d_cell_new, d_cnt);
-        launches += 2;
+        launches++;
     }
     // stable counting sort
     scan_exclusive(d_cnt, d_cell_start, Ktot + 1);
-    k_scatter<<<nblk(N, 256), 256, 0, stream>>>(N, d_cell_new, d_cell_start, d_cnt, d_perm, B, d_dmax, d_fbcount);
+    const ScratchReset z{d_dmax, d_rmax, d_step, after_baoa_ == 1, d_fbcount, d_rot_n, d_novf_n};
+    after_baoa_ = -1;
+    ovf_clean_ = true;
+    k_scatter<<<nblk(N, 256), 256, 0, stream>>>(N, d_cell_new, d_cell_start, d_cnt, d_perm, B, z);
     k_segsort_cells<<<nblk(Ktot, 8), 256, 0, stream>>>(Ktot, d_cell_start, d_perm, d_cell_tmp);
     launches += 2;
     CK(cudaGetLastError());
@@ -1751,6 +1965,11 @@ void Ensemble::adjacency_csr() {
 void Ensemble::rebuild(bool sums_ready) {
     // M-step on the cell-sorted particles, fused with the centroid bounding
     // box (and the B-A-O-A's left-over rotations)
+    if (sums_ready && small_cells()) {
+        // (part of the small batches' relabel)
+        finish_cells(true);
+        return;
+    }
     if (sums_ready) {
         const int nb = nblk(Ktot, 256);
         k_mstep_apply<<<nb + (after_baoa_ >= 0 ? 152 : 0), 256, 0, stream>>>(
@@ -1761,7 +1980,7 @@ void Ensemble::rebuild(bool sums_ready) {
     launches++;
     CK(cudaGetLastError());
     bbox_ready_ = true;
-    finish_cells();
+    finish_cells(false);
 }
 
 }  // namespace orbc

@@ -15,7 +15,7 @@ namespace orbc {
 // kernels defined in cells.cu
 __global__ void k_hist(int N, const int* __restrict__ cell, int* __restrict__ cnt);
 __global__ void k_scatter(int N, const int* __restrict__ cell, const int* __restrict__ start, int* __restrict__ cnt,
-                          int* __restrict__ tmp, int B, unsigned* __restrict__ dmax, int* __restrict__ fb_count);
+                          int* __restrict__ tmp, int B, ScratchReset z);
 __global__ void k_segsort_warp(int Ktot, const int* __restrict__ start, int* __restrict__ tmp);
 __global__ void k_segsort(int Ktot, const int* __restrict__ start, int* __restrict__ tmp, unsigned* status);
 __global__ void k_segrank(int N, const int* __restrict__ cell, const int* __restrict__ start, const int* __restrict__ tmp,
@@ -61,7 +61,7 @@ void cell_sort_run(const int* d_cell, int n, int K, int* d_perm, int* d_start, c
     CK(cudaMemsetAsync(counts, 0, sizeof(int) * (K + 1), st));
     k_hist<<<nblk(n, 256), 256, 0, st>>>(n, d_cell, counts);
     k_scan_single<<<1, 1024, 0, st>>>(counts, d_start, K + 1);
-    k_scatter<<<nblk(n, 256), 256, 0, st>>>(n, d_cell, d_start, counts, d_perm, 0, nullptr, nullptr);
+    k_scatter<<<nblk(n, 256), 256, 0, st>>>(n, d_cell, d_start, counts, d_perm, 0, ScratchReset{});
     k_segsort_warp<<<nblk((long long)K * 32, 256), 256, 0, st>>>(K, d_start, d_perm);
     k_segsort<<<std::min(K, 1024), 256, 0, st>>>(K, d_start, d_perm, flag);
     k_segrank<<<nblk(n, 256), 256, 0, st>>>(n, d_cell, d_start, d_perm, tmp);

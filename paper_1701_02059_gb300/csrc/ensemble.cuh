@@ -104,6 +104,18 @@ struct BondSpec {
 // kernel's own size.
 inline int spread_block(long long threads, int full) { return threads <= 152ll * 2048 ? 64 : full; }
 
+// Scratch of a rebuild that a later launch leaves ready for the next step:
+// the E-step's largest centroid move and grid-search count, the largest
+// radii, the left-over rotations, the search's overflow count; and the step
+// counters, once every reader of the old value is done.
+struct ScratchReset {
+    unsigned* dmax;
+    unsigned long long* rmax;
+    long long* steps;
+    int advance;
+    int *fb_count, *rot_n, *novf;
+};
+
 struct Snapshot {
     Inst inst;                                // descriptor (p0, k0, g0 of the batch it came from)
     Params prm;
@@ -231,7 +243,9 @@ public:
     void estep(int* cell_out, float* lbound);       // grid search; lbound: second-nearest bounds
     void estep_bounded(int* cell);                  // k-means rounds after the first (bounds in d_lbound)
     void morton_relabel();
-    void finish_cells();
+    bool small_cells() const;   // one block relabels the cells (k_relabel_small)
+    // sums_ready: the relabel of a small batch also applies the M-step's sums
+    void finish_cells(bool sums_ready = false);
     // one_launch: FP32 energies by the kernel without lists (for more partners
     // than the lists and their overflow hold)
     void launch_pairs(bool energies, bool dump, bool one_launch = false);
