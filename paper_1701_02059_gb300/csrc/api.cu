@@ -86,7 +86,7 @@ View Ensemble::view() {
     v.cell = d_cell; v.slot_of_id = d_slot_of_id;
     v.F = d_F; v.T = d_T; v.Fbig = d_Fbig;
     v.mq = d_mq; v.mo = d_mo; v.mqr = d_mqr; v.mor = d_mor; v.cframe = d_cframe; v.grank = d_grank;
-    v.cq = d_cq; v.cell_start = d_cell_start; v.R2 = d_R2; v.Rf = d_Rf; v.adj_ptr = d_adj_ptr; v.adj = d_adj; v.adj_cap = adj_cap; v.adjd = d_adjd;
+    v.cq = d_cq; v.cell_start = d_cell_start; v.rcand = d_rcand; v.R2 = d_R2; v.Rf = d_Rf; v.adj_ptr = d_adj_ptr; v.adj = d_adj; v.adj_cap = adj_cap; v.adjd = d_adjd;
     v.adjn = d_adjcount;
     v.gstart = d_gstart; v.gcf = d_gcf;
     v.bptr = d_bptr; v.bpartner = d_bpartner;
@@ -304,6 +304,7 @@ void Ensemble::alloc_core(const std::vector<int>& p0, const std::vector<int>& k0
     d_cq_tmp = alloc<long long>((size_t)3 * Ktot);
     d_cell_start = alloc<int>(Ktot + 1);
     d_R2 = alloc<double>(Ktot);
+    d_rcand = alloc<int>(Ktot);
     d_Rf = alloc<float>(Ktot);
     d_adj_ptr = alloc<int>(Ktot + 1);
     d_adjcount = alloc<int>(Ktot + 1);
@@ -324,7 +325,7 @@ void Ensemble::alloc_core(const std::vector<int>& p0, const std::vector<int>& k0
     d_cell_new = alloc<int>(N);
     d_perm = alloc<int>(N);
     d_cell_tmp = alloc<int>(N);
-    d_rmax = alloc<unsigned long long>(B);
+    d_rmax = alloc<unsigned>(B);
     d_rho = alloc<float>(Ktot);
     d_lbound = alloc<float>(N);
     d_cmove = alloc<float>(Ktot);
@@ -857,6 +858,7 @@ void Ensemble::get_forces(int b, double* f, double* t) {
 void Ensemble::get_cells(int b, int* cell_of_id, unsigned* slot_ids, double* centroids, int* cell_start,
                          double* radius, int* adj_ptr, int* adj) {
     adjacency_csr();
+    cell_radii();
     const Inst& I = inst_h[b];
     const int n = I.n, K = I.K;
     std::vector<unsigned> ids(n);
@@ -900,6 +902,7 @@ void Ensemble::get_cells(int b, int* cell_of_id, unsigned* slot_ids, double* cen
 void Ensemble::get_cells_all(int* cell_of_id, unsigned* slot_ids, double* centroids, int* cell_start, double* radius,
                              int* adj_ptr, int* adj) {
     adjacency_csr();
+    cell_radii();
     std::vector<unsigned> ids(N);
     std::vector<int> cl(N);
     CK(cudaMemcpyAsync(ids.data(), d_id[cur_], sizeof(unsigned) * N, cudaMemcpyDeviceToHost, stream));

@@ -1201,7 +1201,7 @@ __global__ void k_scatter(int N, const int* __restrict__ cell, const int* __rest
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < B) {
         z.dmax[i] = 0u;
-        z.rmax[i] = 0ull;
+        z.rmax[i] = 0u;
         if (z.advance) z.steps[i] += 1;
         if (i == 0) { *z.fb_count = 0; *z.rot_n = 0; *z.novf = 0; }
     }
@@ -1379,6 +1379,10 @@ __device__ inline int mirror_coord(long long xq, long long cq, const Inst& I, in
 // Cell radius R_k = max_i |x_i - c_k| over the cell (all types), equal to
 // the FP64 definition: FP32 from the exact mirror (error < 1e-6 sigma) finds
 // the candidates within this band of the maximum, FP64 decides among them.
+// A single candidate (nearly always) is only noted: an FP64 instruction holds
+// the FP64 pipe for a whole warp's turn, and the few radii that a neighbour
+// test inside its band or a getter wants in FP64 are computed there
+// (cell_r2).
 constexpr float kBandR = 1e-5f;
 
 // Gather of the cell-sorted state, one thread per new slot p: the particle
@@ -1465,14 +1469,27 @@ __device__ inline void warp_bitonic_u32(unsigned (&r)[4], int lane) {
     }
 }
 
+// The squared radius of cell k by the FP64 definition, from the positions x
+// that the cells were built from.
+__device__ inline double cell_r2(const View& v, const long long* __restrict__ x, const Inst& I, int k) {
+    const int p = v.rcand[k];
+    if (p < 0) return v.R2[k];
+    const size_t N = v.N, K = v.Ktot;
+    return dist2_grid_d(x[p], x[N + p], x[2 * N + p], v.cq[k], v.cq[K + k], v.cq[2 * K + k], I);
+}
+
+__global__ void k_cell_r2(View v, const long long* __restrict__ x) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < v.Ktot) v.R2[k] = cell_r2(v, x, v.inst[find_inst(v.inst_k0, v.B, k)], k);
+}
+
 // Per-cell quantities read back from the gathered mirrors: one warp per cell
-// computes the squared cell radius R_k^2 = max |x - c_k|^2 (FP32 with the
-// FP64 definition inside a band) and the radius in FP32, the pair
-// kernels' cell frame (its normal the mean bilayer director, +z without one) and, in
-// each tile of 128 particles, every particle's rank along the tile's longer
-// tangent extent.  rmax_bits: each instance's largest R_k^2 (bit pattern).
-// Launched with 256 threads (8 warps, one cell each).
-__global__ void __launch_bounds__(256, 6) k_cell_props(View v, unsigned long long* __restrict__ rmax_bits /* [B] */) {
+// finds the cell radius (in FP32, and the particle that sets it), the pair
+// kernels' cell frame (its normal the mean bilayer director, +z without one)
+// and, in each tile of 128 particles, every particle's rank along the tile's
+// longer tangent extent.  rmax_bits: each instance's largest radius (FP32
+// bits).
+__global__ void __launch_bounds__(256, 6) k_cell_props(View v, unsigned* __restrict__ rmax_bits /* [B] */) {
     const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (k >= v.Ktot) return;
@@ -1495,29 +1512,38 @@ __global__ void __launch_bounds__(256, 6) k_cell_props(View v, unsigned long lon
         ny += __shfl_xor_sync(0xffffffffu, ny, off);
         nz += __shfl_xor_sync(0xffffffffu, nz, off);
     }
-    // radius: FP64 definition for the particles within the band of the FP32 max
-    double best = 0.0;
+    // the particles within the band of the FP32 maximum: one, or the FP64
+    // definition among them
+    int cand = -1, nc = 0;
     for (int p = s + lane; p < e; p += 32) {
         const int4 m = v.mq[p];
         const float dx = m.x * kMirrorUnit, dy = m.y * kMirrorUnit, dz = m.z * kMirrorUnit;
         const float d = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-        if (d >= mx - kBandR) {
-            const double d2 = dist2_grid_d(v.xq[p], v.xq[N + p], v.xq[2 * N + p], ck[0], ck[1], ck[2], I);
-            best = fmax(best, d2);
-        }
+        if (d >= mx - kBandR) { cand = p; nc++; }
     }
-    // the max over the lanes on the bit patterns (a non-negative double's
-    // bits order like its value): integer operations, not the FP64 pipe
-    unsigned long long bb = (unsigned long long)__double_as_longlong(best);
-    for (int off = 16; off; off >>= 1) bb = max(bb, (unsigned long long)__shfl_xor_sync(0xffffffffu, bb, off));
-    best = __longlong_as_double((long long)bb);
-    // the squared radius (an FP64 square root per cell would cost a whole
-    // warp's turn on the FP64 pipe each: the neighbour rule takes the few it
-    // needs), the radius in FP32, and each instance's largest square
+    nc = (int)__reduce_add_sync(0xffffffffu, (unsigned)nc);
+    cand = __reduce_max_sync(0xffffffffu, cand);
+    if (nc > 1) {
+        // (the maximum over the lanes on the bit patterns: a non-negative
+        // double's bits order like its value)
+        unsigned long long bb = 0;
+        for (int p = s + lane; p < e; p += 32) {
+            const int4 m = v.mq[p];
+            const float dx = m.x * kMirrorUnit, dy = m.y * kMirrorUnit, dz = m.z * kMirrorUnit;
+            if (sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz))) >= mx - kBandR)
+                bb = max(bb, (unsigned long long)__double_as_longlong(
+                                 dist2_grid_d(v.xq[p], v.xq[N + p], v.xq[2 * N + p], ck[0], ck[1], ck[2], I)));
+        }
+        for (int off = 16; off; off >>= 1) bb = max(bb, (unsigned long long)__shfl_xor_sync(0xffffffffu, bb, off));
+        if (lane == 0) v.R2[k] = __longlong_as_double((long long)bb);
+        cand = -1;
+    } else if (nc == 0 && lane == 0) {
+        v.R2[k] = 0.0;      // an empty cell
+    }
     if (lane == 0) {
-        v.R2[k] = best;
-        v.Rf[k] = sqrtf((float)best);
-        atomicMax(&rmax_bits[b], bb);
+        v.rcand[k] = cand;
+        v.Rf[k] = mx;
+        atomicMax(&rmax_bits[b], __float_as_uint(mx));
     }
     // pair-kernel frame
     const float nn = sqrtf(fmaf(nx, nx, fmaf(ny, ny, nz * nz)));
@@ -1610,34 +1636,132 @@ __global__ void k_mirrors(View v) {
 // the threshold, and by an FP32 test with margin elsewhere.
 constexpr float kBandA = 2e-3f;
 
-// exact neighbouring-cell test of (k, j), FP32 with a margin outside the
-// band and the definition's FP64 operations inside it
-__device__ inline bool adj_test(const View& v, const Inst& I, int k, int j, float Rkf, float df, long long cx,
-                                long long cy, long long cz, float tailf) {
-    // FP32 prefilter: FP32 radii differ from the definition's FP64 sum by far
-    // less than the band
-    const float tf = (Rkf + v.Rf[j]) + tailf;
-    if (df < tf - kBandA) return true;
-    if (df > tf + kBandA) return false;
-    const double d = __dsqrt_rn(dist2_grid_d(cx, cy, cz, v.cq[j], v.cq[(size_t)v.Ktot + j], v.cq[(size_t)2 * v.Ktot + j], I));
+// The definition's FP64 test of (k, j), for the candidates that FP32 leaves
+// undecided; d: the distance of the centroids.
+__device__ inline bool adj_exact(const View& v, const Inst& I, int k, int j, double& d) {
+    const size_t K = v.Ktot;
+    d = __dsqrt_rn(dist2_grid_d(v.cq[k], v.cq[K + k], v.cq[2 * K + k], v.cq[j], v.cq[K + j], v.cq[2 * K + j], I));
     // same operation order as the definition: ((Rk + Rj) + rs) + (skin + skin)
-    double tt = __dadd_rn(__dadd_rn(__dadd_rn(__dsqrt_rn(v.R2[k]), __dsqrt_rn(v.R2[j])), I.rs), __dadd_rn(I.skin, I.skin));
+    double tt = __dadd_rn(__dadd_rn(__dadd_rn(__dsqrt_rn(cell_r2(v, v.xq, I, k)), __dsqrt_rn(cell_r2(v, v.xq, I, j))), I.rs),
+                          __dadd_rn(I.skin, I.skin));
     tt = __dmul_rn(tt, 1.0 + 1e-12);
     return d < tt;
 }
 
-// Neighbouring cells, one warp per cell: the lanes share the grid cells of
-// the cube around the cell's own grid cell that the reach
-// R_k + R_max + r_s + 2 skin can touch, test every centroid there with the
-// exact rule, collect the row in shared memory and sort it.  A membrane
-// whose proteins have a cell set of their own searches that set's grid too,
-// so that its rows hold the neighbouring cells of both sets.  Rows longer than
-// kAdjRow are flagged (kStatusAdjOverflow) and truncated. Each entry gets
-// the pair kernel's staging descriptor (particle range, exact centroid
-// offset at 2^-26 sigma) in the same fixed-stride row.
-__global__ void __launch_bounds__(256, 6) k_adj_warp(View v, const unsigned long long* __restrict__ rmax_bits, int* __restrict__ count,
+constexpr int kAdjRaw = 2 * kAdjRow;        // room for neighbours and undecided candidates
+constexpr int kAdjOpen = 1 << 30;           // mark of an undecided one (K < 2^30)
+
+// The warp's share of the centroids of one set, searched through the set's
+// grid G (own: the set of cell k, whose nearest non-neighbour bounds the
+// E-step's certificate; the other set's cells join the row only): the lanes
+// share the rows of grid cells of the cube that the reach R_k + R_max + r_s +
+// 2 skin can touch.  Neighbours go to row, candidates within kBandA of the
+// threshold with the mark kAdjOpen (EXACT: decided at once).
+template <bool EXACT>
+__device__ inline void adj_scan(const View& v, const Inst& I, const Inst& G, int k, float Rkf, float tailf, float reach,
+                                bool own, long long cx, long long cy, long long cz, int* row, int* rown, float& rho) {
+    const int lane = threadIdx.x & 31;
+    float p[3];
+    int g[3];
+    g[0] = grid_coord(cx, G, 0, p[0]);
+    g[1] = grid_coord(cy, G, 1, p[1]);
+    g[2] = grid_coord(cz, G, 2, p[2]);
+    // cube radius: the first shell beyond which nothing is within reach
+    int R = 0;
+    for (;; R++) {
+        bool ex;
+        const float lb = shell_bound(p, g, R, G, ex);
+        if (ex || lb > reach) break;
+    }
+    int lo[3], ext[3];
+    bool full[3];
+    for (int a = 0; a < 3; a++) {
+        int l, h;
+        full[a] = false;
+        if (G.periodic[a]) {
+            if (2 * R + 1 >= G.gdim[a]) { l = 0; h = G.gdim[a] - 1; full[a] = true; }
+            else { l = g[a] - R; h = g[a] + R; }
+        } else {
+            l = max(0, g[a] - R);
+            h = min(G.gdim[a] - 1, g[a] + R);
+        }
+        lo[a] = l;
+        ext[a] = h - l + 1;
+    }
+    const float reach2 = reach * reach;
+    // one lane per (y, z) row of the cube: the row's grid cells are
+    // contiguous along x, and so are their centroids in grid order (one
+    // or two segments when a periodic x range wraps)
+    auto axis_gap = [&](int a, int u) {
+        if (full[a]) return 0.f;
+        const float cl = (!G.periodic[a] && u == 0) ? -3.0e38f : u * G.gh[a];
+        const float ch = (!G.periodic[a] && u == G.gdim[a] - 1) ? 3.0e38f : (u + 1) * G.gh[a];
+        return fmaxf(fmaxf(cl - p[a], p[a] - ch), 0.f);
+    };
+    const int rows = ext[1] * ext[2];
+    for (int t = lane; t < rows; t += 32) {
+        const int y = lo[1] + t % ext[1], z = lo[2] + t / ext[1];
+        const float gy = axis_gap(1, y), gz = axis_gap(2, z);
+        if (fmaf(gy, gy, gz * gz) > reach2) continue;      // the whole row is beyond the reach
+        const int w1 = G.periodic[1] ? wrap_idx(y, G.gdim[1]) : y;
+        const int w2 = G.periodic[2] ? wrap_idx(z, G.gdim[2]) : z;
+        const long long rowbase = G.g0 + ((long long)w2 * G.gdim[1] + w1) * G.gdim[0];
+        int xa[2], xb[2], nseg = 1;
+        xa[0] = lo[0];
+        xb[0] = lo[0] + ext[0] - 1;
+        if (G.periodic[0] && !full[0]) {
+            const int a0 = wrap_idx(xa[0], G.gdim[0]), b0 = wrap_idx(xb[0], G.gdim[0]);
+            if (a0 <= b0) { xa[0] = a0; xb[0] = b0; }
+            else { xa[0] = a0; xb[0] = G.gdim[0] - 1; xa[1] = 0; xb[1] = b0; nseg = 2; }
+        }
+        for (int sg = 0; sg < nseg; sg++) {
+            const int q1 = v.gstart[rowbase + xb[sg] + 1];
+            for (int q = v.gstart[rowbase + xa[sg]]; q < q1; q++) {
+                const float4 c = v.gcf[q];
+                const int j = __float_as_int(c.w);
+                const float dx = axis_dist(p[0], c.x, G, 0), dy = axis_dist(p[1], c.y, G, 1), dz = axis_dist(p[2], c.z, G, 2);
+                const float df = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+                // FP32 prefilter: FP32 radii differ from the definition's
+                // FP64 sum by far less than the band
+                const float tf = (Rkf + v.Rf[j]) + tailf;
+                bool in = df <= tf + kBandA, open = in && df >= tf - kBandA;
+                if (EXACT && open) {
+                    double d;
+                    in = adj_exact(v, I, k, j, d);
+                    open = false;
+                }
+                if (in) {
+                    const int at = atomicAdd(rown, 1);
+                    if (at < kAdjRaw) row[at] = open ? j | kAdjOpen : j;
+                } else if (own) {
+                    rho = fminf(rho, df);
+                }
+            }
+        }
+    }
+}
+
+// The same with every candidate decided in the scan (out of line: only when
+// neighbours and undecided candidates together overflow the row's room).
+static __device__ __noinline__ float adj_scan_exact(const View& v, const Inst& I, const Inst& G, int k, float reach, bool own,
+                                                    int* row, int* rown, float rho) {
+    const size_t K = v.Ktot;
+    adj_scan<true>(v, I, G, k, v.Rf[k], I.rsf + 2.0f * I.skinf, reach, own, v.cq[k], v.cq[K + k], v.cq[2 * K + k], row, rown,
+                   rho);
+    return rho;
+}
+
+// Neighbouring cells, one warp per cell: candidates by adj_scan, the few
+// undecided ones by the FP64 rule afterwards (FP64 code inside the scan cost
+// it registers and spills), then the row sorted.  A membrane whose proteins
+// have a cell set of their own searches that set's grid too, so that its rows
+// hold the neighbouring cells of both sets.  Rows longer than kAdjRow are
+// flagged (kStatusAdjOverflow) and truncated. Each entry gets the pair
+// kernel's staging descriptor (particle range, exact centroid offset at 2^-26
+// sigma) in the same fixed-stride row.
+__global__ void __launch_bounds__(256, 6) k_adj_warp(View v, const unsigned* __restrict__ rmax_bits, int* __restrict__ count,
                            float* __restrict__ rho_out, int* __restrict__ pad /* [Ktot][kAdjRow] */) {
-    __shared__ int row[8][kAdjRow];
+    __shared__ int row[8][kAdjRaw];
     __shared__ int rown[8];
     const int wb = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1646,101 +1770,52 @@ __global__ void __launch_bounds__(256, 6) k_adj_warp(View v, const unsigned long
     const Inst& I = v.inst[b];
     const float Rkf = v.Rf[k];
     const long long cx = v.cq[k], cy = v.cq[(size_t)v.Ktot + k], cz = v.cq[(size_t)2 * v.Ktot + k];
-    // the cell's scalars in FP32 (every lane of the warp computes them, and
-    // an FP64 operation costs a full warp's turn on the FP64 pipe): they only
-    // set the FP32 prefilter and the search reach, whose band kBandA is far
-    // wider than their rounding
+    // the cell's scalars in FP32: they only set the FP32 prefilter and the
+    // search reach, whose band kBandA is far wider than their rounding
     const float tailf = I.rsf + 2.0f * I.skinf;
     if (lane == 0) rown[wb] = 0;
     __syncwarp();
-    auto reach_of = [&](float Rmaxf) { return ((Rkf + Rmaxf) + tailf) + kBandA; };
-    // the largest radius of the set from its largest square (FP32: it only
-    // sets the reach)
-    auto rmax_of = [&](int s) { return sqrtf((float)__longlong_as_double((long long)rmax_bits[s])); };
-    const float reach_own = reach_of(rmax_of(b));
-    float rho = reach_own - kBandA;
-    // the centroids of one set through its own grid G: every centroid within
-    // the reach R_k + R_max(G) + r_s + 2 skin is tested with the exact rule;
-    // own: the set of cell k, whose nearest non-neighbour bounds the
-    // E-step's certificate (the other set's cells join the row only)
-    auto scan = [&](const Inst& G, float Rmaxf, bool own) {
-        const float reach = reach_of(Rmaxf);
-        float p[3];
-        int g[3];
-        g[0] = grid_coord(cx, G, 0, p[0]);
-        g[1] = grid_coord(cy, G, 1, p[1]);
-        g[2] = grid_coord(cz, G, 2, p[2]);
-        // cube radius: the first shell beyond which nothing is within reach
-        int R = 0;
-        for (;; R++) {
-            bool ex;
-            const float lb = shell_bound(p, g, R, G, ex);
-            if (ex || lb > reach) break;
-        }
-        int lo[3], ext[3];
-        bool full[3];
-        for (int a = 0; a < 3; a++) {
-            int l, h;
-            full[a] = false;
-            if (G.periodic[a]) {
-                if (2 * R + 1 >= G.gdim[a]) { l = 0; h = G.gdim[a] - 1; full[a] = true; }
-                else { l = g[a] - R; h = g[a] + R; }
-            } else {
-                l = max(0, g[a] - R);
-                h = min(G.gdim[a] - 1, g[a] + R);
-            }
-            lo[a] = l;
-            ext[a] = h - l + 1;
-        }
-        const float reach2 = reach * reach;
-        // one lane per (y, z) row of the cube: the row's grid cells are
-        // contiguous along x, and so are their centroids in grid order (one
-        // or two segments when a periodic x range wraps)
-        auto axis_gap = [&](int a, int u) {
-            if (full[a]) return 0.f;
-            const float cl = (!G.periodic[a] && u == 0) ? -3.0e38f : u * G.gh[a];
-            const float ch = (!G.periodic[a] && u == G.gdim[a] - 1) ? 3.0e38f : (u + 1) * G.gh[a];
-            return fmaxf(fmaxf(cl - p[a], p[a] - ch), 0.f);
-        };
-        const int rows = ext[1] * ext[2];
-        for (int t = lane; t < rows; t += 32) {
-            const int y = lo[1] + t % ext[1], z = lo[2] + t / ext[1];
-            const float gy = axis_gap(1, y), gz = axis_gap(2, z);
-            if (fmaf(gy, gy, gz * gz) > reach2) continue;      // the whole row is beyond the reach
-            const int w1 = G.periodic[1] ? wrap_idx(y, G.gdim[1]) : y;
-            const int w2 = G.periodic[2] ? wrap_idx(z, G.gdim[2]) : z;
-            const long long rowbase = G.g0 + ((long long)w2 * G.gdim[1] + w1) * G.gdim[0];
-            int xa[2], xb[2], nseg = 1;
-            xa[0] = lo[0];
-            xb[0] = lo[0] + ext[0] - 1;
-            if (G.periodic[0] && !full[0]) {
-                const int a0 = wrap_idx(xa[0], G.gdim[0]), b0 = wrap_idx(xb[0], G.gdim[0]);
-                if (a0 <= b0) { xa[0] = a0; xb[0] = b0; }
-                else { xa[0] = a0; xb[0] = G.gdim[0] - 1; xa[1] = 0; xb[1] = b0; nseg = 2; }
-            }
-            for (int sg = 0; sg < nseg; sg++) {
-                const int q1 = v.gstart[rowbase + xb[sg] + 1];
-                for (int q = v.gstart[rowbase + xa[sg]]; q < q1; q++) {
-                    const float4 c = v.gcf[q];
-                    const int j = __float_as_int(c.w);
-                    const float dx = axis_dist(p[0], c.x, G, 0), dy = axis_dist(p[1], c.y, G, 1),
-                                dz = axis_dist(p[2], c.z, G, 2);
-                    const float df = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-                    if (adj_test(v, I, k, j, Rkf, df, cx, cy, cz, tailf)) {
-                        const int at = atomicAdd(&rown[wb], 1);
-                        if (at < kAdjRow) row[wb][at] = j;
-                    } else if (own) {
-                        rho = fminf(rho, df);
-                    }
+    auto reach_of = [&](int s) { return ((Rkf + __uint_as_float(rmax_bits[s])) + tailf) + kBandA; };
+    const float rho0 = reach_of(b) - kBandA;
+    float rho = rho0;
+    for (int s = b, own = 1; s >= 0; s = own ? I.partner : -1, own = 0)
+        adj_scan<false>(v, I, v.inst[s], k, Rkf, tailf, reach_of(s), own != 0, cx, cy, cz, row[wb], &rown[wb], rho);
+    __syncwarp();
+    if (rown[wb] > kAdjRaw) {
+        __syncwarp();
+        if (lane == 0) rown[wb] = 0;
+        __syncwarp();
+        rho = adj_scan_exact(v, I, I, k, reach_of(b), true, row[wb], &rown[wb], rho0);
+        if (I.partner >= 0) adj_scan_exact(v, I, v.inst[I.partner], k, reach_of(I.partner), false, row[wb], &rown[wb], 0.f);
+        __syncwarp();
+    }
+    int n = min(rown[wb], kAdjRaw);
+    {
+        // the undecided ones, and the row without those that fail
+        bool any = false;
+        for (int u = lane; u < n; u += 32) any |= (row[wb][u] & kAdjOpen) != 0;
+        if (__any_sync(0xffffffffu, any)) {
+            int m = 0;
+            for (int u0 = 0; u0 < n; u0 += 32) {
+                int j = u0 + lane < n ? row[wb][u0 + lane] : -1;
+                bool keep = j >= 0;
+                if (keep && (j & kAdjOpen)) {
+                    double d;
+                    j &= ~kAdjOpen;
+                    keep = adj_exact(v, I, k, j, d);
+                    // (a cell of the own set)
+                    if (!keep && j >= I.k0 && j < I.k0 + I.K) rho = fminf(rho, (float)d);
                 }
+                const unsigned bal = __ballot_sync(0xffffffffu, keep);
+                if (keep) row[wb][m + __popc(bal & ((1u << lane) - 1u))] = j;
+                m += __popc(bal);
+                __syncwarp();
             }
+            n = m;
         }
-    };
-    scan(I, rmax_of(b), true);
-    if (I.partner >= 0) scan(v.inst[I.partner], rmax_of(I.partner), false);
+    }
     for (int off = 16; off; off >>= 1) rho = fminf(rho, __shfl_xor_sync(0xffffffffu, rho, off));
     __syncwarp();
-    int n = rown[wb];
     if (n > kAdjRow) {
         if (lane == 0) flag_inst(v, I, kStatusAdjOverflow);
         n = kAdjRow;
@@ -1950,6 +2025,14 @@ void Ensemble::finish_cells(bool sums_ready) {
     forces_valid = false;
     list_valid = false;
     n_rebuilds++;
+}
+
+void Ensemble::cell_radii() {
+    if (!cells_valid) return;
+    // (with a skin the particles may have moved since the cells were built)
+    k_cell_r2<<<nblk(Ktot, 256), 256, 0, stream>>>(view(), d_xref ? d_xref : d_state[cur_][0]);
+    launches++;
+    CK(cudaGetLastError());
 }
 
 void Ensemble::adjacency_csr() {

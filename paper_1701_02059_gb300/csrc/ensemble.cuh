@@ -110,7 +110,7 @@ inline int spread_block(long long threads, int full) { return threads <= 152ll *
 // counters, once every reader of the old value is done.
 struct ScratchReset {
     unsigned* dmax;
-    unsigned long long* rmax;
+    unsigned* rmax;
     long long* steps;
     int advance;
     int *fb_count, *rot_n, *novf;
@@ -193,6 +193,8 @@ public:
     long long adjacency_len_all();
     // the neighbour rows as CSR (adj_ptr, adj), built on demand for the getters
     void adjacency_csr();
+    // squared FP64 radii of every cell into d_R2 (for the getters)
+    void cell_radii();
     long long dump_pairs(int b, long long cap, unsigned* pairs);
     unsigned read_status(bool clear);
     std::vector<unsigned> read_instance_status(bool clear);
@@ -321,6 +323,7 @@ public:
     float4* d_mor = nullptr;
     long long *d_cq = nullptr, *d_cq_tmp = nullptr;
     int* d_cell_start = nullptr;
+    int* d_rcand = nullptr;
     double* d_R2 = nullptr;
     float* d_Rf = nullptr;
     int *d_adj_ptr = nullptr, *d_adj = nullptr, *d_adjcount = nullptr;
@@ -347,7 +350,7 @@ public:
     void* d_sortrec = nullptr;
     int* d_new_of_old = nullptr;
     int *d_cell_new = nullptr, *d_perm = nullptr, *d_cell_tmp = nullptr;
-    unsigned long long* d_rmax = nullptr;
+    unsigned* d_rmax = nullptr;              // [B] largest cell radius (FP32 bits)
     float* d_rho = nullptr;                  // [Ktot] distance to the nearest non-neighbour centroid
     float* d_lbound = nullptr;
     float* d_cmove = nullptr;                // [Ktot] k-means: move of each centroid in the last M-step

@@ -177,7 +177,10 @@ struct View {
     // cells
     long long* cq;                  // [3][Ktot] centroids on the 2^-40 grid
     int* cell_start;                // [Ktot+1]
-    double* R2;                     // [Ktot] squared cell radius
+    // [Ktot] the particle that sets the cell's radius (its slot), when FP32
+    // tells it from the others; else -1 and the squared FP64 radius in R2
+    int* rcand;
+    double* R2;
     float* Rf;                      // [Ktot] cell radius in FP32 (the neighbour rule's prefilter)
     int* adj_ptr;                   // [Ktot+1]
     int* adj;                       // [adj_cap]
