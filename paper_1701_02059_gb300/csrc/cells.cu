@@ -158,11 +158,16 @@ __global__ void k_mstep_sorted(View v, long long* __restrict__ bb, unsigned* __r
     }
 }
 
+__device__ inline long long warp_min_ll(long long x) {
+    for (int off = 16; off; off >>= 1) x = min(x, __shfl_xor_sync(0xffffffffu, x, off));
+    return x;
+}
+
 // M-step from the sums the B-A-O-A launch accumulated (same terms as
 // k_mstep_sorted, so the same centroids): one thread per cell updates c_k,
 // clears the sums for the next step and folds the centroid into the
-// instance's bounding box and its largest move (warp-reduced before the
-// atomics).  The blocks from rot_block on take the B-A-O-A's left-over
+// instance's bounding box and its largest move (reduced over the block before
+// the atomics).  The blocks from rot_block on take the B-A-O-A's left-over
 // rotations instead (rot_rest; one launch fewer than on their own).
 __global__ void __launch_bounds__(256) k_mstep_apply(View v, long long* __restrict__ S, int* __restrict__ cnt,
                                                      long long* __restrict__ bb, unsigned* __restrict__ dmax,
@@ -173,40 +178,61 @@ __global__ void __launch_bounds__(256) k_mstep_apply(View v, long long* __restri
                  (gridDim.x - rot_block) * blockDim.x);
         return;
     }
+    __shared__ long long red[8][6];
+    __shared__ unsigned redm[8];
+    __shared__ int s_b;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= v.Ktot) return;
+    const bool act = k < v.Ktot;
     const size_t K = v.Ktot;
-    const int b = find_inst(v.inst_k0, v.B, k);
-    const Inst& I = v.inst[b];
-    const int n = cnt[k];
-    long long c[3];
+    const int b = act ? find_inst(v.inst_k0, v.B, k) : -1;
+    long long c[3] = {0, 0, 0};
     float mv2 = 0.f;
-    for (int a = 0; a < 3; a++) {
-        c[a] = v.cq[a * K + k];
-        long long step = 0;
-        if (n > 0) step = floor_div_ll(2 * S[a * K + k] + n, 2 * (long long)n);
-        const float sf = ll_to_float(step) * (float)kGridInv;
-        mv2 = fmaf(sf, sf, mv2);
-        c[a] += step;
-        if (I.periodic[a]) c[a] = floor_mod_ll(c[a], I.boxq[a]);
-        v.cq[a * K + k] = c[a];
-        S[a * K + k] = 0;
+    if (act) {
+        const Inst& I = v.inst[b];
+        const int n = cnt[k];
+        for (int a = 0; a < 3; a++) {
+            c[a] = v.cq[a * K + k];
+            long long step = 0;
+            if (n > 0) step = floor_div_ll(2 * S[a * K + k] + n, 2 * (long long)n);
+            const float sf = ll_to_float(step) * (float)kGridInv;
+            mv2 = fmaf(sf, sf, mv2);
+            c[a] += step;
+            if (I.periodic[a]) c[a] = floor_mod_ll(c[a], I.boxq[a]);
+            v.cq[a * K + k] = c[a];
+            S[a * K + k] = 0;
+        }
+        cnt[k] = 0;
     }
-    cnt[k] = 0;
-    const unsigned grp = __match_any_sync(__activemask(), b);
-    const unsigned mv = __reduce_max_sync(grp, __float_as_uint(sqrtf(mv2) * 1.0001f + 1e-6f));
-    long long mn[3] = {c[0], c[1], c[2]}, mx[3] = {c[0], c[1], c[2]};
-    if (grp == 0xffffffffu) {
-        for (int off = 16; off; off >>= 1)
-            for (int a = 0; a < 3; a++) {
-                mn[a] = min(mn[a], __shfl_xor_sync(0xffffffffu, mn[a], off));
-                mx[a] = max(mx[a], __shfl_xor_sync(0xffffffffu, mx[a], off));
-            }
+    const unsigned mv = __float_as_uint(sqrtf(mv2) * 1.0001f + 1e-6f);
+    if (threadIdx.x == 0) s_b = b;
+    __syncthreads();
+    if (!__syncthreads_and(b == s_b || !act)) {
+        // a block with cells of several instances
+        if (act) {
+            atomicMax(&dmax[b], mv);
+            for (int a = 0; a < 3; a++) { atomicMin(&bb[b * 6 + a], c[a]); atomicMax(&bb[b * 6 + 3 + a], c[a]); }
+        }
+        return;
     }
-    const bool leader = (int)(threadIdx.x & 31) == __ffs(grp) - 1;
-    if (leader && dmax) atomicMax(&dmax[b], mv);
-    if (grp != 0xffffffffu || leader)
-        for (int a = 0; a < 3; a++) { atomicMin(&bb[b * 6 + a], mn[a]); atomicMax(&bb[b * 6 + 3 + a], mx[a]); }
+    // one set of atomics per block
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int a = 0; a < 6; a++) {
+        const long long m = warp_min_ll(act ? (a < 3 ? c[a] : -c[a - 3]) : 0x7fffffffffffffffll);
+        if (lane == 0) red[w][a] = m;
+    }
+    const unsigned mw = __reduce_max_sync(0xffffffffu, act ? mv : 0u);
+    if (lane == 0) redm[w] = mw;
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        long long m = red[0][threadIdx.x];
+        for (int q = 1; q < 8; q++) m = min(m, red[q][threadIdx.x]);
+        if (threadIdx.x < 3) atomicMin(&bb[s_b * 6 + threadIdx.x], m);
+        else atomicMax(&bb[s_b * 6 + threadIdx.x], -m);
+    } else if (threadIdx.x == 32) {
+        unsigned m = redm[0];
+        for (int q = 1; q < 8; q++) m = max(m, redm[q]);
+        atomicMax(&dmax[s_b], m);
+    }
 }
 
 // ============================================================== Morton relabel
@@ -397,14 +423,20 @@ constexpr int kBoundTiles = 1024;   // tiles whose bounds a block keeps in share
 __global__ void k_rank_scatter(View v, const SortRec* __restrict__ tiles, int ntiles, const long long* __restrict__ cq_old,
                                int* __restrict__ new_of_old, int* __restrict__ gcount, int* __restrict__ gidx,
                                float4* __restrict__ cf, long long* __restrict__ bb) {
-    // first and last record of every tile (most tiles lie wholly below or
-    // above a record, which these settle without a search)
-    __shared__ SortRec tb[2][kBoundTiles];
+    // first and last key of every tile and its instance (-1: several): most
+    // tiles lie wholly below or above a record, which these settle without a
+    // search
+    __shared__ unsigned long long tmin[kBoundTiles], tmax[kBoundTiles];
+    __shared__ int tinst[kBoundTiles];
     const bool cached = ntiles <= kBoundTiles;
     if (cached)
         for (int t = threadIdx.x; t < ntiles; t += blockDim.x) {
-            tb[0][t] = tiles[(size_t)t * kTile];
-            tb[1][t] = tiles[(size_t)t * kTile + kTile - 1];
+            // (the last tile ends in padding records)
+            const int last = min(kTile, v.Ktot - t * kTile) - 1;
+            const SortRec a = tiles[(size_t)t * kTile], b = tiles[(size_t)t * kTile + last];
+            tmin[t] = a.key;
+            tmax[t] = b.key;
+            tinst[t] = a.inst == b.inst ? a.inst : -1;
         }
     __syncthreads();
     int pos = blockIdx.x * blockDim.x + threadIdx.x;   // position in the tiled array
@@ -423,18 +455,23 @@ __global__ void k_rank_scatter(View v, const SortRec* __restrict__ tiles, int nt
     int rank = 0;
     int t0 = I.k0 / kTile, t1 = (I.k0 + I.K - 1) / kTile;
     for (int t = t0; t <= t1; t++) {
+        if (cached && tinst[t] == me.inst) {
+            // (equal keys go by index: searched)
+            if (me.key > tmax[t]) { rank += min(kTile, v.Ktot - t * kTile); continue; }
+            if (me.key < tmin[t]) continue;
+        }
         const SortRec* T = tiles + (size_t)t * kTile;
-        const SortRec tmin = cached ? tb[0][t] : T[0], tmax = cached ? tb[1][t] : T[kTile - 1];
+        const SortRec tfirst = T[0], tlast = T[kTile - 1];
         int lo, lo2;
-        if (rec_less(tmax, me)) lo = kTile;
-        else if (!rec_less(tmin, me)) lo = 0;
+        if (rec_less(tlast, me)) lo = kTile;
+        else if (!rec_less(tfirst, me)) lo = 0;
         else {
             int a = 0, c = kTile;
             while (a < c) { int mid = (a + c) >> 1; if (rec_less(T[mid], me)) a = mid + 1; else c = mid; }
             lo = a;
         }
-        if (rec_less(tmax, first)) lo2 = kTile;
-        else if (!rec_less(tmin, first)) lo2 = 0;
+        if (rec_less(tlast, first)) lo2 = kTile;
+        else if (!rec_less(tfirst, first)) lo2 = 0;
         else {
             int a = 0, c = kTile;
             while (a < c) { int mid = (a + c) >> 1; if (rec_less(T[mid], first)) a = mid + 1; else c = mid; }
@@ -461,11 +498,6 @@ __global__ void k_rank_scatter(View v, const SortRec* __restrict__ tiles, int nt
 // after the first take the left-over rotations (see k_mstep_apply).
 constexpr int kSmallK = 1024;
 constexpr int kSmallG = 1 << 16;
-
-__device__ inline long long warp_min_ll(long long x) {
-    for (int off = 16; off; off >>= 1) x = min(x, __shfl_xor_sync(0xffffffffu, x, off));
-    return x;
-}
 
 __global__ void __launch_bounds__(kSmallK) k_relabel_small(
     View v, int mstep, long long* __restrict__ S, int* __restrict__ cnt, unsigned* __restrict__ dmax,
@@ -1085,16 +1117,21 @@ __global__ void __launch_bounds__(256) k_estep_bound(View v, const int* __restri
 // FP32 centroids (w = new index), so the E-step reads one record per
 // candidate instead of three dependent loads; the first K threads also put
 // the centroids in grid order (gcount not null).
+constexpr int kRowLanes = 8;    // (a membrane's rows hold about 8 cells)
 __global__ void k_cand_rows(View v, const int* __restrict__ cnt_old, const int* __restrict__ pad_old,
                             const int* __restrict__ new_of_old, const float4* __restrict__ cf,
                             float4* __restrict__ rows, const int* __restrict__ gidx, int* __restrict__ gcount) {
-    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // one thread per row slot
-    if (gcount && q < v.Ktot) grid_fill_one(v, (int)q, gidx, gcount, cf);
-    if (q >= (long long)v.Ktot * kAdjRow || (int)(q % kAdjRow) >= cnt_old[q / kAdjRow]) return;
-    const int j = new_of_old[pad_old[q]];
-    float4 c = cf[j];
-    c.w = __int_as_float(j);
-    rows[q] = c;
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;   // kRowLanes threads per row
+    if (gcount && q < v.Ktot) grid_fill_one(v, q, gidx, gcount, cf);
+    const int k = q / kRowLanes;
+    if (k >= v.Ktot) return;
+    const int n = min(cnt_old[k], kAdjRow);
+    for (int r = q % kRowLanes; r < n; r += kRowLanes) {
+        const int j = new_of_old[pad_old[(size_t)k * kAdjRow + r]];
+        float4 c = cf[j];
+        c.w = __int_as_float(j);
+        rows[(size_t)k * kAdjRow + r] = c;
+    }
 }
 
 // Rebuild E-step from the previous cell list (the paper's guess from the
@@ -1244,31 +1281,32 @@ __global__ void k_segsort(int Ktot, const int* __restrict__ start, int* __restri
     }
 }
 
-// Cells of up to 128 particles: one warp, bitonic network over 4 values per
+// Cells of up to 32 NE particles: one warp, bitonic network over NE values per
 // lane (element e = lane + 32 q), shuffles for strides < 32.
-__device__ inline void segsort_warp(int s, int n, int* __restrict__ tmp) {
+template <int NE>
+__device__ inline void segsort_net(int s, int n, int* __restrict__ tmp) {
     const int lane = threadIdx.x & 31;
-    int val[4];
+    int val[NE];
 #pragma unroll
-    for (int q = 0; q < 4; q++) val[q] = (lane + 32 * q < n) ? tmp[s + lane + 32 * q] : 0x7fffffff;
+    for (int q = 0; q < NE; q++) val[q] = (lane + 32 * q < n) ? tmp[s + lane + 32 * q] : 0x7fffffff;
 #pragma unroll
-    for (int size = 2; size <= 128; size <<= 1) {
+    for (int size = 2; size <= 32 * NE; size <<= 1) {
 #pragma unroll
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
             if (stride >= 32) {
                 const int qs = stride >> 5;
 #pragma unroll
-                for (int q = 0; q < 4; q++) {
+                for (int q = 0; q < NE; q++) {
                     if (q & qs) continue;
                     const int e = lane + 32 * q;
                     const bool up = (e & size) == 0;
-                    const int a = val[q], c = val[q | qs];
+                    const int a = val[q], c = val[q + qs];
                     val[q] = up ? min(a, c) : max(a, c);
-                    val[q | qs] = up ? max(a, c) : min(a, c);
+                    val[q + qs] = up ? max(a, c) : min(a, c);
                 }
             } else {
 #pragma unroll
-                for (int q = 0; q < 4; q++) {
+                for (int q = 0; q < NE; q++) {
                     const int e = lane + 32 * q;
                     const int other = __shfl_xor_sync(0xffffffffu, val[q], stride);
                     const bool up = (e & size) == 0;
@@ -1279,8 +1317,12 @@ __device__ inline void segsort_warp(int s, int n, int* __restrict__ tmp) {
         }
     }
 #pragma unroll
-    for (int q = 0; q < 4; q++)
+    for (int q = 0; q < NE; q++)
         if (lane + 32 * q < n) tmp[s + lane + 32 * q] = val[q];
+}
+__device__ inline void segsort_warp(int s, int n, int* __restrict__ tmp) {   // n <= 128
+    if (n <= 64) segsort_net<2>(s, n, tmp);
+    else segsort_net<4>(s, n, tmp);
 }
 
 __global__ void k_segsort_warp(int Ktot, const int* __restrict__ start, int* __restrict__ tmp) {
@@ -1489,7 +1531,7 @@ __global__ void k_cell_r2(View v, const long long* __restrict__ x) {
 // and, in each tile of 128 particles, every particle's rank along the tile's
 // longer tangent extent.  rmax_bits: each instance's largest radius (FP32
 // bits).
-__global__ void __launch_bounds__(256, 6) k_cell_props(View v, unsigned* __restrict__ rmax_bits /* [B] */) {
+__global__ void __launch_bounds__(256, 6) k_cell_props(View v, unsigned* rmax_bits /* [B] */) {
     const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (k >= v.Ktot) return;
@@ -1543,7 +1585,9 @@ __global__ void __launch_bounds__(256, 6) k_cell_props(View v, unsigned* __restr
     if (lane == 0) {
         v.rcand[k] = cand;
         v.Rf[k] = mx;
-        atomicMax(&rmax_bits[b], __float_as_uint(mx));
+        // (a possibly stale value read through L1 saves nearly all atomics on
+        // the one address)
+        if (__float_as_uint(mx) > __ldca(rmax_bits + b)) atomicMax(&rmax_bits[b], __float_as_uint(mx));
     }
     // pair-kernel frame
     const float nn = sqrtf(fmaf(nx, nx, fmaf(ny, ny, nz * nz)));
@@ -1982,7 +2026,7 @@ void Ensemble::finish_cells(bool sums_ready) {
         scan_exclusive(d_gcount, d_gstart, Gtot + 1);
     }
     if (prev_adj_valid_) {
-        k_cand_rows<<<nblk((long long)Ktot * kAdjRow, 256), 256, 0, stream>>>(v, d_adjcount, d_adjpad, d_new_of_old, d_cf,
+        k_cand_rows<<<nblk((long long)Ktot * kRowLanes, 256), 256, 0, stream>>>(v, d_adjcount, d_adjpad, d_new_of_old, d_cf,
                                                                           d_candrows, d_gidx, small ? nullptr : d_gcount);
         k_estep_rows<<<nblk(N, spread_block(N, 128)), spread_block(N, 128), 0, stream>>>(
             v, d_cell, d_adjcount, d_candrows, d_rho, d_new_of_old, d_dmax, d_cell_new, d_cell_tmp, d_fbcount, d_cnt);

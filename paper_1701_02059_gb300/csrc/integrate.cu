@@ -103,8 +103,32 @@ __global__ void k_kick(View v, long long* __restrict__ steps) {
     if (p == I.p0) steps[b] += 1;
 }
 
-// Kinetic energies K_trans = sum m v^2 / 2, K_rot = sum_lipids I w^2 / 2,
-// per particle in FP64, summed exactly as 2^-32 fixed point.
+// m u^2 / 2 of a vector on the 2^-40 grid, at 2^-32: the square summed exactly
+// (u = h 2^23 + l) to 2^-48 and multiplied by m/2 = c 2^-k in integers (c in
+// [2^61, 2^62)); FP64 for |component| of 2^6 and above and for other masses.
+// (Two energies in FP64 hold the FP64 pipe for 24 instructions a particle.)
+__device__ inline long long kinetic_fix(const long long u[3], double mass, Half c, int k) {
+    const long long lim = 1ll << 46;
+    if (k >= 49 && k <= 80 && below(u[0], lim - 1) && below(u[1], lim - 1) && below(u[2], lim - 1)) {
+        long long hh = 0, hl = 0, ll = 0;
+        for (int a = 0; a < 3; a++) {
+            const int l = (int)((unsigned)(unsigned long long)u[a] & 0x7fffffu), h = (int)(u[a] >> 23);
+            hh += (long long)h * h;
+            hl += (long long)h * l;
+            ll += (long long)l * l;
+        }
+        // u^2 2^-32: hh 2^46 + hl 2^24 + ll, below 2^62
+        const long long s = (hh << 14) + (hl >> 8) + (ll >> 32);
+        const long long x = mulh(halves(s), c);
+        return (x + (1ll << (k - 49))) >> (k - 48);
+    }
+    double s = 0.0;
+    for (int a = 0; a < 3; a++) { const double x = grid_to_double(u[a]); s += x * x; }
+    return __double2ll_rn(0.5 * mass * s * 4294967296.0);
+}
+
+// Kinetic energies K_trans = sum m v^2 / 2, K_rot = sum_lipids I w^2 / 2, per
+// particle to 2^-32 and summed exactly.
 __global__ void k_kinetic(View v, long long* __restrict__ energy) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     long long kt = 0, kr = 0;
@@ -113,31 +137,41 @@ __global__ void k_kinetic(View v, long long* __restrict__ energy) {
         b = find_inst(v.inst_p0, v.B, p);
         const Inst& I = v.inst[b];
         const size_t N = v.N;
-        double s = 0.0, r = 0.0;
-        for (int a = 0; a < 3; a++) { double x = grid_to_double(v.vq[a * N + p]); s += x * x; }
-        kt = __double2ll_rn(0.5 * I.mass * s * 4294967296.0);
+        const long long u[3] = {v.vq[p], v.vq[N + p], v.vq[2 * N + p]};
+        kt = kinetic_fix(u, I.mass, Half{I.km_h, I.km_l}, I.km_k);
         if (bilayer(v.type[p])) {
-            for (int a = 0; a < 3; a++) { double x = grid_to_double(v.wq[a * N + p]); r += x * x; }
-            kr = __double2ll_rn(0.5 * I.inertia * r * 4294967296.0);
+            const long long w[3] = {v.wq[p], v.wq[N + p], v.wq[2 * N + p]};
+            kr = kinetic_fix(w, I.inertia, Half{I.ki_h, I.ki_l}, I.ki_k);
         }
     }
-    // warp-aggregate per instance
-    const unsigned grp = __match_any_sync(0xffffffffu, b);
-    long long st = kt, sr = kr;
-    if (grp == 0xffffffffu) {
+    // a block of one instance: one atomic per block (one per warp, all on the
+    // same address, took most of the kernel's time: 47 against 17 us on the
+    // 1M cell); otherwise per instance and warp
+    __shared__ long long s_k[2];
+    __shared__ int s_b;
+    if (threadIdx.x == 0) { s_k[0] = 0; s_k[1] = 0; s_b = b; }
+    __syncthreads();
+    if (__syncthreads_and(b == s_b || b < 0)) {
         for (int off = 16; off; off >>= 1) {
-            st += __shfl_xor_sync(0xffffffffu, st, off);
-            sr += __shfl_xor_sync(0xffffffffu, sr, off);
+            kt += __shfl_xor_sync(0xffffffffu, kt, off);
+            kr += __shfl_xor_sync(0xffffffffu, kr, off);
         }
-    } else {
-        st = sr = 0;
-        unsigned m = grp;
-        while (m) {
-            int src = __ffs(m) - 1;
-            m &= m - 1;
-            st += __shfl_sync(grp, kt, src);
-            sr += __shfl_sync(grp, kr, src);
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd((unsigned long long*)&s_k[0], (unsigned long long)kt);
+            atomicAdd((unsigned long long*)&s_k[1], (unsigned long long)kr);
         }
+        __syncthreads();
+        if (threadIdx.x < 2) atomicAdd((unsigned long long*)&energy[s_b * 8 + 2 + threadIdx.x], (unsigned long long)s_k[threadIdx.x]);
+        return;
+    }
+    const unsigned grp = __match_any_sync(0xffffffffu, b);
+    long long st = 0, sr = 0;
+    unsigned m = grp;
+    while (m) {
+        int src = __ffs(m) - 1;
+        m &= m - 1;
+        st += __shfl_sync(grp, kt, src);
+        sr += __shfl_sync(grp, kr, src);
     }
     if (b >= 0 && (int)(threadIdx.x & 31) == __ffs(grp) - 1) {
         atomicAdd((unsigned long long*)&energy[b * 8 + 2], (unsigned long long)st);

@@ -101,6 +101,7 @@ struct Inst {
     // not possible, see mul_round), and v << ou_vt, noise << ou_nt (ou_lim)
     int hm8_t, hdt_t, ou_vt, ou_nt;
     long long hm8_lim, hdt_lim, ou_lim;
+    int km_h, km_l, km_k, ki_h, ki_l, ki_k;   // m/2 and I/2 for the kinetic energies (norm61)
     RotK rot;           // the rotational update's constants in fixed point
     // st and sr 2^40 times the noise's scale sqrt(12) 2^-33 (multiplying the
     // noise's exact integer part)

@@ -49,20 +49,22 @@ ORBC_HD inline Half halves(long long x) {
     return r;
 }
 
+// x = m 2^-k, m in [2^61, 2^62) in halves (k = 62 and m = 0 unless x > 0)
+inline int norm61(double x, int& h, int& l) {
+    h = l = 0;
+    if (!(x > 0)) return 62;
+    int e = 0;
+    const double f = std::frexp(x, &e);
+    const Half m = halves((long long)std::ldexp(f, 62));
+    h = m.h;
+    l = m.l;
+    return 62 - e;
+}
+
 // The constants of one instance: dt/4, dt/2/I, exp(-gamma_r dt) - 1 and the
 // noise amplitude per integer noise unit (grid units).
 inline RotK rot_constants(double quarter_dt, double h_i, double cr_m1, double srn) {
     RotK R;
-    auto norm61 = [](double x, int& h, int& l) {
-        h = l = 0;
-        if (!(x > 0)) return 62;
-        int e = 0;
-        const double f = std::frexp(x, &e);
-        const Half m = halves((long long)std::ldexp(f, 62));
-        h = m.h;
-        l = m.l;
-        return 62 - e;
-    };
     auto shifts = [](int s, int& left, int& right) {
         left = std::max(s, 0);
         right = std::min(std::max(-s, 0), 63);
