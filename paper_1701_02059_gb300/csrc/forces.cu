@@ -703,12 +703,8 @@ struct PairC {
     float ll_lo, ll_hi, w_lo, w_hi, p_lo, p_hi;   // squared cutoffs -+ the FP64 decision band
     __device__ explicit PairC(const Inst& I)
         : eps(I.eps), rmin(I.rmin), mu(I.mu), s0(I.s0), aw(I.aw), eps2z_aw(I.eps2z_aw), eps_wca(I.eps_wca),
-          sig_wca(I.sig_wca), sig_pp(I.sig_pp), zeta(I.zeta) {
-        const float rcl = sqrtf(I.rc2f_ll), rcw = sqrtf(I.rc2f_wca), rcp = sqrtf(I.rc2f_pp);
-        ll_lo = (rcl - kCutBand) * (rcl - kCutBand); ll_hi = (rcl + kCutBand) * (rcl + kCutBand);
-        w_lo = (rcw - kCutBand) * (rcw - kCutBand); w_hi = (rcw + kCutBand) * (rcw + kCutBand);
-        p_lo = (rcp - kCutBand) * (rcp - kCutBand); p_hi = (rcp + kCutBand) * (rcp + kCutBand);
-    }
+          sig_wca(I.sig_wca), sig_pp(I.sig_pp), zeta(I.zeta), ll_lo(I.ll_lo), ll_hi(I.ll_hi), w_lo(I.w_lo), w_hi(I.w_hi),
+          p_lo(I.p_lo), p_hi(I.p_hi) {}
 };
 
 // ================================================================ FP64 pair forces
@@ -917,10 +913,11 @@ __device__ inline void eval_pair_d(const View& v, const Inst& I, int pi, int pj,
 // DIRECT (FP64 forces): the pairs found are evaluated at once (pair_terms_d);
 // F and T are zero before the launch.  EN adds U_pair and the virial of the
 // cell's instance to energy [B][8].
-template <bool MP, bool DIRECT = false, bool Z4 = true, bool S0 = false, bool EN = false>
-__global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
+template <bool MP, bool DIRECT = false, bool Z4 = true, bool S0 = false, bool EN = false, bool ONE = false>
+__global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 9)
     k_pair_search(View v, int* __restrict__ nlist, int* __restrict__ ncnt, int cap, int2* __restrict__ ovf,
-                  int* __restrict__ novf, int ovf_cap, int4* __restrict__ rowoff, long long* __restrict__ energy) {
+                  int* __restrict__ novf, int ovf_cap, int4* __restrict__ rowoff, long long* __restrict__ energy,
+                  const __grid_constant__ Inst one) {
     // sY: staged mirrors (int4 by the bulk copy), then in the tangent frame
     //     (FP32), w = 0 for a bilayer particle and 1 for a cytoskeleton protein
     // sQ: the list entry of each staged particle
@@ -940,8 +937,8 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
     __shared__ int s_nstage, s_next, s_next_off, s_self, s_self_lo, s_self_hi, s_total;
 
     const int k = blockIdx.x;
-    const int b = find_inst(v.inst_k0, v.B, k);
-    const Inst& I = v.inst[b];
+    const int b = ONE ? 0 : find_inst(v.inst_k0, v.B, k);
+    const Inst& I = ONE ? one : v.inst[b];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int cs = v.cell_start[k], ce = v.cell_start[k + 1];
     const AdjDesc* __restrict__ row = v.adjd + (size_t)k * kAdjRow;
@@ -1336,7 +1333,7 @@ template <int Z, bool S0, bool MP = false, bool EN = false>
 __device__ __forceinline__ void eval_list(const View& v, int q, const int* __restrict__ nlist,
                                           const int* __restrict__ ncnt, int cap, const int4* __restrict__ rowoff,
                                           SplitAcc af[3], SplitAcc at[3], int& nterm, bool& big, int& pi_out,
-                                          long long* es = nullptr, int t0 = 0, int dt = 1) {
+                                          const Inst* one, long long* es = nullptr, int t0 = 0, int dt = 1) {
     const size_t N = v.N;
     const int4 qi = v.mqr[q];
     const float4 oi = v.mor[q];
@@ -1344,8 +1341,7 @@ __device__ __forceinline__ void eval_list(const View& v, int q, const int* __res
     pi_out = pi;
     const int ti = qi.w & 0xff;
     const int k = v.cell[pi];
-    const int b = find_inst(v.inst_p0, v.B, pi);
-    const Inst& I = v.inst[b];
+    const Inst& I = one ? *one : v.inst[find_inst(v.inst_p0, v.B, pi)];
     const PairC C(I);
     const int zc = (Z > 0) ? Z : C.zeta;
     const int4* __restrict__ ro = rowoff + (size_t)k * kAdjRow;
@@ -1451,7 +1447,8 @@ __device__ __forceinline__ void eval_list(const View& v, int q, const int* __res
             nterm++;
         } else {
             // terms of 1000 or more go to the int64 side array (exact, rare)
-            if (!(mag < kMaxTerm)) flag_inst(v, I, (mag == mag) ? kStatusPairForceRange : kStatusNaN);
+            if (!(mag < kMaxTerm))
+                flag_inst(v, v.inst[find_inst(v.inst_p0, v.B, pi)], (mag == mag) ? kStatusPairForceRange : kStatusNaN);
             for (int a = 0; a < 6; a++)
                 atomicAdd((unsigned long long*)&v.Fbig[(size_t)a * N + pi],
                           (unsigned long long)__float2ll_rn(f[a] * 4294967296.0f));
@@ -1475,10 +1472,10 @@ __device__ __forceinline__ void eval_list(const View& v, int q, const int* __res
 // seven (72 registers, a few spilled) hide more of the gathers' latency than
 // five without spills, 0.785 against 0.857 ms on the 4M cell.
 // MP: the batch holds band-3 or glycophorin (eval_list).
-template <int Z, bool S0, int MINB, bool MP = false, bool EN = false>
+template <int Z, bool S0, int MINB, bool MP = false, bool EN = false, bool ONE = false>
 __global__ void __launch_bounds__(128, MINB)
     k_pair_eval(View v, const int* __restrict__ nlist, const int* __restrict__ ncnt, int cap,
-                const int4* __restrict__ rowoff, long long* __restrict__ energy) {
+                const int4* __restrict__ rowoff, long long* __restrict__ energy, const __grid_constant__ Inst one) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (!EN && q >= v.N) return;
     const size_t N = v.N;
@@ -1493,7 +1490,7 @@ __global__ void __launch_bounds__(128, MINB)
         if (threadIdx.x < 4) s_e[threadIdx.x] = 0;
         __syncthreads();
         long long es[4] = {0, 0, 0, 0};
-        if (q < v.N) eval_list<Z, S0, MP, true>(v, q, nlist, ncnt, cap, rowoff, af, at, nterm, big, pi, es);
+        if (q < v.N) eval_list<Z, S0, MP, true>(v, q, nlist, ncnt, cap, rowoff, af, at, nterm, big, pi, ONE ? &one : nullptr, es);
         for (int a = 0; a < 4; a++) {
             for (int off = 16; off; off >>= 1) es[a] += __shfl_xor_sync(0xffffffffu, es[a], off);
             if ((threadIdx.x & 31) == 0) atomicAdd((unsigned long long*)&s_e[a], (unsigned long long)es[a]);
@@ -1509,7 +1506,7 @@ __global__ void __launch_bounds__(128, MINB)
         }
         if (q >= v.N) return;
     } else {
-        eval_list<Z, S0, MP>(v, q, nlist, ncnt, cap, rowoff, af, at, nterm, big, pi);
+        eval_list<Z, S0, MP>(v, q, nlist, ncnt, cap, rowoff, af, at, nterm, big, pi, ONE ? &one : nullptr);
     }
 #pragma unroll
     for (int a = 0; a < 3; a++) {
@@ -1531,10 +1528,10 @@ __global__ void __launch_bounds__(128, MINB)
 // with one thread, 14.3 with four; 20k 26.2 and 18.0; 62k 32.7 and 26.6 with
 // two; 145k are better off with one, 44.7 against 45.9).  The partial sums
 // are integers, so the result is the same.
-template <int Z, bool S0, bool MP>
+template <int Z, bool S0, bool MP, bool ONE>
 __global__ void __launch_bounds__(128, 7)
     k_pair_eval_split(View v, const int* __restrict__ nlist, const int* __restrict__ ncnt, int cap,
-                      const int4* __restrict__ rowoff, int sh) {
+                      const int4* __restrict__ rowoff, int sh, const __grid_constant__ Inst one) {
     const long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int q = (int)(x >> sh), part = (int)(x & ((1 << sh) - 1));
     const unsigned live = __ballot_sync(0xffffffffu, q < v.N);
@@ -1543,7 +1540,8 @@ __global__ void __launch_bounds__(128, 7)
     SplitAcc af[3], at[3];
     int nterm, pi;
     bool big;
-    eval_list<Z, S0, MP>(v, q, nlist, ncnt, cap, rowoff, af, at, nterm, big, pi, nullptr, part, 1 << sh);
+    eval_list<Z, S0, MP>(v, q, nlist, ncnt, cap, rowoff, af, at, nterm, big, pi, ONE ? &one : nullptr, nullptr, part,
+                         1 << sh);
     __syncwarp(live);
     for (int off = 1 << (sh - 1); off; off >>= 1) {
         for (int a = 0; a < 3; a++) {
@@ -1599,7 +1597,7 @@ __global__ void __launch_bounds__(128, 4)
     SplitAcc af[3], at[3];
     int nterm, pi;
     bool big;
-    eval_list<Z, S0>(v, q, nlist, ncnt, cap, rowoff, af, at, nterm, big, pi);
+    eval_list<Z, S0>(v, q, nlist, ncnt, cap, rowoff, af, at, nterm, big, pi, nullptr);
     const bool side = big || sflag[pi];
     long long F[3], Tq[3];
 #pragma unroll
@@ -1629,7 +1627,7 @@ __global__ void __launch_bounds__(128, 4)
     }
     for (int a = 0; a < 3; a++) { v.F[a * N + pi] = F[a]; v.T[a * N + pi] = Tq[a]; }
     __syncwarp(live);
-    if (D) baoa_d_body<true>(v, o, pi, F, Tq, steps, msum, mcnt, live, true, rot_list, rot_n);
+    if (D) baoa_d_body<true>(v, o, pi, F, Tq, steps, msum, mcnt, live, true, rot_list, rot_n, nullptr);
     else baoa_body<float, true>(v, o, pi, F, Tq, steps, msum, mcnt, live, true);
 }
 
@@ -1820,12 +1818,12 @@ void Ensemble::launch_search() {
     if (list_valid) return;
     tic("pair_search");
     clear_overflow();
-    if (any_mp())
-        k_pair_search<true><<<Ktot, kPairThreads, 0, stream>>>(view(), d_nlist, d_ncnt, list_cap, d_novf, d_novf_n, ovf_cap,
-                                                               d_rowoff, nullptr);
-    else
-        k_pair_search<false><<<Ktot, kPairThreads, 0, stream>>>(view(), d_nlist, d_ncnt, list_cap, d_novf, d_novf_n,
-                                                                ovf_cap, d_rowoff, nullptr);
+#define ORBC_SEARCH(MP, ONE)                                                                                              \
+    k_pair_search<MP, false, true, false, false, ONE><<<Ktot, kPairThreads, 0, stream>>>(                                 \
+        view(), d_nlist, d_ncnt, list_cap, d_novf, d_novf_n, ovf_cap, d_rowoff, nullptr, inst_h[0])
+    if (any_mp()) { if (B == 1) ORBC_SEARCH(true, true); else ORBC_SEARCH(true, false); }
+    else { if (B == 1) ORBC_SEARCH(false, true); else ORBC_SEARCH(false, false); }
+#undef ORBC_SEARCH
     launches++;
     CK(cudaGetLastError());
     toc();
@@ -1856,12 +1854,22 @@ void Ensemble::launch_pairs(bool energies, bool dump, bool one_launch) {
         while (sh < 2 && ((long long)N << (sh + 1)) <= 152ll * 7 * 128) sh++;
         const int nsp = (int)((((long long)N << sh) + 127) / 128);
         // (with energies: five CTAs per SM, for their registers)
+        // one instance: its constants as a kernel argument (ONE)
+#define ORBC_EVAL_N(Z, S, MP, ONE)                                                                                          \
+    do {                                                                                                                    \
+        if (energies)                                                                                                       \
+            k_pair_eval<Z, S, 5, MP, true, ONE><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, d_energy, inst_h[0]); \
+        else if (sh > 0)                                                                                                    \
+            k_pair_eval_split<Z, S, MP, ONE><<<nsp, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, sh, inst_h[0]); \
+        else if (ctas == 5)                                                                                                 \
+            k_pair_eval<Z, S, 5, MP, false, ONE><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, nullptr, inst_h[0]); \
+        else                                                                                                                \
+            k_pair_eval<Z, S, ONE ? 8 : 7, MP, false, ONE><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, nullptr, inst_h[0]); \
+    } while (0)
 #define ORBC_EVAL(Z, S, MP)                                                                                                 \
     do {                                                                                                                    \
-        if (energies) k_pair_eval<Z, S, 5, MP, true><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, d_energy); \
-        else if (sh > 0) k_pair_eval_split<Z, S, MP><<<nsp, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, sh);     \
-        else if (ctas == 5) k_pair_eval<Z, S, 5, MP><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, nullptr);  \
-        else k_pair_eval<Z, S, 7, MP><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, nullptr);             \
+        if (B == 1) ORBC_EVAL_N(Z, S, MP, true);                                                                            \
+        else ORBC_EVAL_N(Z, S, MP, false);                                                                                  \
     } while (0)
         if (any_mp()) {
             // band-3 or glycophorin present (or a bonded bilayer particle):
@@ -1876,6 +1884,7 @@ void Ensemble::launch_pairs(bool energies, bool dump, bool one_launch) {
             ORBC_EVAL(0, true, false);
         }
 #undef ORBC_EVAL
+#undef ORBC_EVAL_N
         launches++;
         CK(cudaGetLastError());
         toc();
@@ -1913,7 +1922,7 @@ void Ensemble::launch_pairs(bool energies, bool dump, bool one_launch) {
         CK(cudaMemsetAsync(d_F, 0, sizeof(long long) * 3 * (size_t)N, stream));
         CK(cudaMemsetAsync(d_T, 0, sizeof(long long) * 3 * (size_t)N, stream));
 #define ORBC_PAIRS_D(MP, Z4, S, EN)                                                                                   \
-    k_pair_search<MP, true, Z4, S, EN><<<g, t, 0, stream>>>(v, nullptr, nullptr, 0, nullptr, nullptr, 0, nullptr, d_energy)
+    k_pair_search<MP, true, Z4, S, EN><<<g, t, 0, stream>>>(v, nullptr, nullptr, 0, nullptr, nullptr, 0, nullptr, d_energy, inst_h[0])
         if (!any_mp() && z4 && s0z) { if (energies) ORBC_PAIRS_D(false, true, false, true); else ORBC_PAIRS_D(false, true, false, false); }
         else { if (energies) ORBC_PAIRS_D(true, false, true, true); else ORBC_PAIRS_D(true, false, true, false); }
 #undef ORBC_PAIRS_D

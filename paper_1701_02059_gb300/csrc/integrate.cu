@@ -35,16 +35,17 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 4) k_baoa(View v, co
 // fixed-point rotation it is bound by integer issue: 0.47 ms with
 // k_rot_rest.  Four CTAs per SM (64 registers, some spilled) against 0.48 ms
 // at three.
-template <bool FUSED>
+template <bool FUSED, bool ONE>
 __global__ void __launch_bounds__(256, 4) k_baoa_d(View v, const long long* __restrict__ steps,
                                                    long long* __restrict__ msum, int* __restrict__ mcnt,
-                                                   int* __restrict__ rot_list, int* __restrict__ rot_n) {
+                                                   int* __restrict__ rot_list, int* __restrict__ rot_n,
+                                                   const __grid_constant__ Inst one) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= v.N) return;
     const size_t N = v.N;
     long long F[3], Tq[3];
     for (int a = 0; a < 3; a++) { F[a] = v.F[a * N + p]; Tq[a] = v.T[a * N + p]; }
-    baoa_d_body<FUSED>(v, v, p, F, Tq, steps, msum, mcnt, __activemask(), false, rot_list, rot_n);
+    baoa_d_body<FUSED>(v, v, p, F, Tq, steps, msum, mcnt, __activemask(), false, rot_list, rot_n, ONE ? &one : nullptr);
 }
 
 // The left-over rotations in a launch of their own (when no rebuild follows).
@@ -256,8 +257,12 @@ void Ensemble::launch_integrate_first(bool fused, bool msums) {
         else k_baoa<float, false><<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(view(), d_step, ms, mc);
     } else {
         // (the left-over list shares the E-step's, which the rebuild uses later)
-        if (fused) k_baoa_d<true><<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(view(), d_step, ms, mc, d_cell_tmp, d_rot_n);
-        else k_baoa_d<false><<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(view(), d_step, ms, mc, d_cell_tmp, d_rot_n);
+#define ORBC_BAOA(F, ONE)                                                                                        \
+    k_baoa_d<F, ONE><<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(view(), d_step, ms, mc, \
+                                                                                         d_cell_tmp, d_rot_n, inst_h[0])
+        if (fused) { if (B == 1) ORBC_BAOA(true, true); else ORBC_BAOA(true, false); }
+        else { if (B == 1) ORBC_BAOA(false, true); else ORBC_BAOA(false, false); }
+#undef ORBC_BAOA
     }
     launches++;
     CK(cudaGetLastError());

@@ -386,9 +386,9 @@ template <bool FUSED>
 __device__ inline void baoa_d_body(const View& v, const View& o, int p, const long long F[3], const long long Tq[3],
                                    const long long* __restrict__ steps, long long* __restrict__ msum,
                                    int* __restrict__ mcnt, unsigned mask, bool copy_static,
-                                   int* __restrict__ rot_list, int* __restrict__ rot_n) {
-    const int b = find_inst(v.inst_p0, v.B, p);
-    const Inst& I = v.inst[b];
+                                   int* __restrict__ rot_list, int* __restrict__ rot_n, const Inst* one) {
+    const int b = one ? 0 : find_inst(v.inst_p0, v.B, p);
+    const Inst& I = one ? *one : v.inst[b];
     const size_t N = v.N;
     const unsigned char type = v.type[p];
     const bool lipid = bilayer(type);

@@ -205,10 +205,7 @@ void Ensemble::set_volume(int b, double kv, double v0, double area, const double
     CK(cudaStreamSynchronize(stream));
     bool any = false;
     for (const Inst& J : inst_h) any = any || J.vol_on;
-    if (any != vol_any) {
-        // the captured step holds the volume launches or not
-        drop_graphs();
-    }
+    drop_graphs();   // the captured steps hold the descriptor and the volume launches, or not
     vol_any = any;
     forces_valid = false;
 }
