@@ -186,6 +186,8 @@ static Inst make_inst(const Params& P) {
     I.eps2z_aw = (float)(P.eps * 2.0 * P.zeta * (1.5707963267948966 / (P.rc_lipid - two_sixth * P.sigma)));
     {
         const float rcl = std::sqrt(I.rc2f_ll), rw = std::sqrt(I.rc2f_wca), rp = std::sqrt(I.rc2f_pp);
+        I.rcf_wca = rw;
+        I.rcf_pp = rp;
         I.ll_lo = (rcl - kCutBand) * (rcl - kCutBand); I.ll_hi = (rcl + kCutBand) * (rcl + kCutBand);
         I.w_lo = (rw - kCutBand) * (rw - kCutBand); I.w_hi = (rw + kCutBand) * (rw + kCutBand);
         I.p_lo = (rp - kCutBand) * (rp - kCutBand); I.p_hi = (rp + kCutBand) * (rp + kCutBand);

@@ -687,7 +687,8 @@ __global__ void __launch_bounds__(kPairThreads, 5) k_pairs(View v, long long* __
 // whose exact offset c_l - c_k the search writes to rowoff.  Lists hold
 // kListCap entries per particle (t-major: entry t of particle q at t N + q);
 // further entries go to an overflow list evaluated with integer atomics.
-constexpr int kSearchStage = 768;
+constexpr int kSearchStage = 640;
+constexpr int kFragRow = 12;        // floats between fragment rows (48 B: no bank conflicts)
 constexpr int kListCap = 32;
 constexpr int kRowShift = 26;
 
@@ -905,7 +906,37 @@ __device__ inline void eval_pair_d(const View& v, const Inst& I, int pi, int pj,
     }
 }
 
-// Eight CTAs per SM (the shared-memory limit): 0.833 against 0.863 ms at seven.
+// ---- distance tests on the tensor cores (TF32, FP32 accumulation)
+// A warp tests its 32 particles against 32 candidates as the product of a
+// 32 x 8 and an 8 x 32 matrix,
+//   d^2 - cut = -2 x_i.x_j + |x_j|^2 + (|x_i|^2 - cut_i) - (cut of the class)_i,
+// whose sign is the hit: eight m16n8k8 products and one funnel shift per
+// result instead of about ten FP32 instructions per test (159M -> 126M
+// instructions on the 1M cell; 0.66 -> 0.61 ms on the 4M cell, its species-pair
+// form 195 -> 169 us at 1M).  Coordinates are
+// rounded to TF32 first (and the squares taken of the rounded ones, split in
+// two TF32 terms), so the result is the distance of points moved by at most
+// 2^-11 of their distance from the cell's centre: the cutoffs grow by
+// filter_band, and a list holds up to a few pairs more, which the exact
+// decision drops.
+__device__ inline float tf32_rna(float x) {
+    unsigned r;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+    return __uint_as_float(r);
+}
+__device__ inline float tf32_down(float x) {      // towards minus infinity
+    const float r = __uint_as_float(__float_as_uint(x) & 0xffffe000u);
+    return r <= x ? r : __uint_as_float(__float_as_uint(r) + 0x2000u);
+}
+__device__ inline void mma_tf32(float d[4], const float a[4], float b0, float b1) {
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%10, %10, %10, %10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(__float_as_uint(a[0])), "r"(__float_as_uint(a[1])), "r"(__float_as_uint(a[2])), "r"(__float_as_uint(a[3])),
+          "r"(__float_as_uint(b0)), "r"(__float_as_uint(b1)), "f"(0.f));
+}
+
+// Eight CTAs per SM: 0.608 ms on the 4M cell against 0.613 at seven or nine.
 // MP (band-3 or glycophorin in the batch): the staged particles carry three
 // partner classes (lipid 0, cytoskeleton 1, bilayer protein 2) and each
 // particle culls them at its own cutoff for that class, so that a lipid's
@@ -914,7 +945,7 @@ __device__ inline void eval_pair_d(const View& v, const Inst& I, int pi, int pj,
 // F and T are zero before the launch.  EN adds U_pair and the virial of the
 // cell's instance to energy [B][8].
 template <bool MP, bool DIRECT = false, bool Z4 = true, bool S0 = false, bool EN = false, bool ONE = false>
-__global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 9)
+__global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
     k_pair_search(View v, int* __restrict__ nlist, int* __restrict__ ncnt, int cap, int2* __restrict__ ovf,
                   int* __restrict__ novf, int ovf_cap, int4* __restrict__ rowoff, long long* __restrict__ energy,
                   const __grid_constant__ Inst one) {
@@ -925,11 +956,9 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 9)
     __shared__ alignas(16) float4 sY[kSearchStage];
     __shared__ int sQ[kSearchStage];
     __shared__ alignas(16) unsigned short cand[kPairThreads / 32][kSearchStage];
-    // each lane's own particle's position in its warp's candidate list (the
-    // self pair is removed once per 32 candidates instead of per test)
-    __shared__ unsigned short spos[kPairThreads / 32][32];
     __shared__ SNbr nb[kMaxNbr];
     __shared__ int s_cnt[kPairThreads];
+    __shared__ alignas(16) float frag[kPairThreads / 32][32 * kFragRow];   // per warp: fragment rows
     __shared__ int2 wq[DIRECT ? kPairThreads / 32 : 1][DIRECT ? kQueue64 : 1];       // queued pairs: slots
     __shared__ unsigned char wc[DIRECT ? kPairThreads / 32 : 1][DIRECT ? kQueue64 : 1];   // class and species
     __shared__ long long s_e[2];
@@ -956,7 +985,13 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 9)
         __syncwarp();
     };
     const float rsb = I.rsf + sk, rs2f = rsb * rsb;
-    const float cw = sqrtf(I.rc2f_wca) + sk, cp = sqrtf(I.rc2f_pp) + sk;
+    const float cw = I.rcf_wca + sk, cp = I.rcf_pp + sk;
+    // candidate c of 32 goes to the fragment column whose hit is bit c; the
+    // byte transpose within four lanes that brings a row's hits to one lane
+    const int fcol = (((lane >> 1) & 3) * 8 + 2 * (lane >> 3) + (lane & 1)) * kFragRow;
+    const unsigned q4 = lane & 3;
+    const unsigned selA = q4 | ((4 + q4) << 4), selC = 0x5410u,
+                   selD = (0 ^ q4) | ((1 ^ q4) << 4) | ((2 ^ q4) << 8) | ((3 ^ q4) << 12);
     unsigned phase = 0;
     if (tid == 0) mbar_init(&bar, 1);
     __syncthreads();
@@ -964,11 +999,12 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 9)
     for (int it0 = cs; it0 < ce; it0 += kPairThreads) {
         const int nti = min(kPairThreads, ce - it0);
         const int groups = (nti + 31) >> 5;
-        const int nsplit = (groups == 1) ? 4 : (groups == 2 ? 2 : 1);
-        const int igrp = warp % groups;
-        const int jsplit = warp / groups;
+        const int lsplit = (groups == 1) ? 2 : (groups == 2 ? 1 : 0), nsplit = 1 << lsplit;
+        // (groups is 1 to 4: no divisions)
+        const int jsplit = groups == 1 ? warp : (groups == 2 ? warp >> 1 : (groups == 3 ? (warp == 3) : 0));
+        const int igrp = warp - jsplit * groups;
         const bool wactive = jsplit < nsplit;
-        const int gs = (nti + groups - 1) / groups;
+        const int gs = groups == 1 ? nti : (groups == 2 ? (nti + 1) >> 1 : (groups == 3 ? (nti + 2) / 3 : (nti + 3) >> 2));
         s_cnt[tid] = 0;
 
         auto issue = [&](const int na, const int na_off) {
@@ -1062,21 +1098,46 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 9)
         }
         // squared search radius for a bilayer and for a cytoskeleton partner
         // (for a bilayer particle the widest cutoff of its species; with MP
-        // the lipid partners' and the bilayer proteins' apart)
+        // the lipid partners' and the bilayer proteins' apart), widened by
+        // what the rounded coordinates may move: 2^-11 (|x_i| + |x_j|) with
+        // |x_i| <= R_k (plus what it moved since), |x_j| <= |x_i| + r_s, and
+        // the rounding of the products' sum
         const bool bi = bilayer(ti);
         const int si = species(ti);
-        const float cl = (MP ? I.mm_rcp[3 * si] : I.mm_rcf[si]) + sk;
-        const float cutL = bi ? cl * cl : cw * cw;
-        const float cutP = bi ? cw * cw : cp * cp;
-        const float cutD = cutP - cutL;
-        // MP: the cutoff of a partner of class c in {0, 1, 2} as
-        // cutL + c (qa + c qb), through cutP at c = 1 and cutM at c = 2
-        float qa = cutD, qb = 0.f;
+        const float reach = 2.0f * (v.Rf[k] + 2.0f * I.skinf) + rsb;
+        const float fb = sk + 5.0e-4f * reach, fb2 = 1.0e-5f * reach * reach + 1.0e-4f;
+        const float cl = (MP ? I.mm_rcp[3 * si] : I.mm_rcf[si]) + fb;
+        const float cwb = I.rcf_wca + fb, cpb = I.rcf_pp + fb;
+        const float cutL = (bi ? cl * cl : cwb * cwb) + fb2;
+        const float cutP = (bi ? cwb * cwb : cpb * cpb) + fb2;
+        float cutM = cutP;
         if (MP) {
-            const float cm = fmaxf(I.mm_rcp[3 * si + 1], I.mm_rcp[3 * si + 2]) + sk;
-            const float cutM = bi ? cm * cm : cw * cw;
-            qb = 0.5f * (cutM - cutL) - cutD;
-            qa = cutD - qb;
+            const float cm = fmaxf(I.mm_rcp[3 * si + 1], I.mm_rcp[3 * si + 2]) + fb;
+            cutM = (bi ? cm * cm : cwb * cwb) + fb2;
+        }
+        // A fragments: lane l's particle is row (l >> 2) + 8 (l & 3), which is
+        // the row whose hits the lane ends up with
+        float af[2][4];
+        float* const fr = frag[warp];
+        {
+            const float x = tf32_rna(yix), y = tf32_rna(yiy), z = tf32_rna(yiz);
+            float c = fmaf(x, x, fmaf(y, y, z * z)) - cutL;
+            float ax = -2.0f * x, ay = -2.0f * y, az = -2.0f * z;
+            if (!ivalid) { c = 1.0e30f; ax = ay = az = 0.f; }
+            const float ch = tf32_rna(c);
+            float* w = fr + ((lane >> 2) + 8 * (lane & 3)) * kFragRow;
+            *reinterpret_cast<float4*>(w) = make_float4(ax, ay, az, 1.0f);
+            *reinterpret_cast<float4*>(w + 4) = make_float4(MP ? tf32_down(cutL - cutP) : 1.0f, ch, ivalid ? c - ch : 0.f,
+                                                            tf32_down(cutL - (MP ? cutM : cutP)));
+            __syncwarp();
+            const float* p = fr + (lane >> 2) * kFragRow + (lane & 3);
+            for (int h = 0; h < 2; h++) {
+                af[h][0] = p[16 * h * kFragRow];
+                af[h][1] = p[(16 * h + 8) * kFragRow];
+                af[h][2] = p[16 * h * kFragRow + 4];
+                af[h][3] = p[(16 * h + 8) * kFragRow + 4];
+            }
+            __syncwarp();
         }
         // the group box's cull radius: the search cutoff, or for a group
         // without bilayer particles (a protein cell) the larger of its two
@@ -1131,11 +1192,13 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 9)
             __syncthreads();
 
             if (wactive) {
-                int cnt = 0;
-                spos[warp][lane] = 0xffffu;
-                __syncwarp();
-                // staged index of lane 0's own particle (own cell, this pass)
+                int cnt = 0, p0 = 0;
+                // the warp's first own particle in this pass: the group's
+                // particles are staged one after the other and lie in its
+                // box, so they follow each other in the candidate list too
                 const int self0 = sself + (it0 + igrp * gs - cs);
+                int jf = max(self0, sslo);
+                jf += (jsplit - jf) & (nsplit - 1);
                 for (int c0 = 0; c0 < total; c0 += nsplit * 32) {
                     const int j = c0 + lane * nsplit + jsplit;
                     bool in = false;
@@ -1147,41 +1210,59 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 9)
                         in = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) < rcull2;
                     }
                     const unsigned bal = __ballot_sync(0xffffffffu, in);
-                    if (in) {
-                        const int at = cnt + __popc(bal & ((1u << lane) - 1u));
-                        cand[warp][at] = (unsigned short)(j << 4);   // byte offset of sY[j]
-                        // the own particle of lane t of this group
-                        const int t = j - self0;
-                        if (sslo >= 0 && j >= sslo && j < sshi && t >= 0 && t < gs) spos[warp][t] = (unsigned short)at;
-                    }
+                    if ((unsigned)(jf - c0) < (unsigned)(nsplit * 32))
+                        p0 = cnt + __popc(bal & ((1u << ((jf - jsplit - c0) >> lsplit)) - 1u));
+                    if (in) cand[warp][cnt + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)(j << 4);   // byte offset of sY[j]
                     cnt += __popc(bal);
                 }
-                // pad to a multiple of 32 with a valid staged index
-                if (cnt + lane < ((cnt + 31) & ~31)) cand[warp][cnt + lane] = 0;
                 __syncwarp();
-                const int sp = selfj >= 0 ? (int)spos[warp][lane] : -1;   // 0xffff: not in this warp's list
-                // every lane tests the same 32 candidates (broadcast reads)
-                // into a bit mask, then writes its hits; the padding of the
-                // candidate list past cnt is never read as a hit
-                static_assert(kSearchStage % 32 == 0, "candidate lists are read 32 at a time");
+                // the own particle's place in this warp's list (-1: the other warps')
+                const int sp = selfj >= 0 && ((selfj - jsplit) & (nsplit - 1)) == 0 ? p0 + ((selfj - jf) >> lsplit) : -1;
+                // 32 candidates at a time (past the list: far away, no hit)
                 static_assert(kSearchStage * 16 <= 65536, "candidate byte offsets fit 16 bits");
                 for (int c0 = 0; c0 < cnt; c0 += 32) {
-                    unsigned hits = 0u;
-#pragma unroll
-                    for (int h = 0; h < 4; h++) {
-                        const uint4 c8 = *reinterpret_cast<const uint4*>(&cand[warp][c0 + 8 * h]);
-                        const unsigned cw8[4] = {c8.x, c8.y, c8.z, c8.w};
-#pragma unroll
-                        for (int u = 0; u < 8; u++) {
-                            const unsigned off = (cw8[u >> 1] >> (16 * (u & 1))) & 0xffffu;
-                            const float4 y = *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(sY) + off);
-                            const float ex = y.x - yix, ey = y.y - yiy, ez = y.z - yiz;
-                            const float d2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
-                            const float cut = MP ? fmaf(y.w, fmaf(y.w, qb, qa), cutL) : fmaf(y.w, cutD, cutL);
-                            if (d2 < cut) hits |= 1u << (8 * h + u);
+                    {
+                        float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+                        float n = 1.0e30f;
+                        if (c0 + lane < cnt) {
+                            y = *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(sY) + cand[warp][c0 + lane]);
+                            y.x = tf32_rna(y.x); y.y = tf32_rna(y.y); y.z = tf32_rna(y.z);
+                            n = fmaf(y.x, y.x, fmaf(y.y, y.y, y.z * y.z));
                         }
+                        // (MP has no room for the square's second term: rounded down)
+                        const float nh = MP ? __uint_as_float(__float_as_uint(n) & 0xffffe000u) : tf32_rna(n);
+                        float* w = fr + fcol;
+                        *reinterpret_cast<float4*>(w) = make_float4(y.x, y.y, y.z, nh);
+                        *reinterpret_cast<float4*>(w + 4) =
+                            make_float4(MP ? (y.w == 1.0f ? 1.0f : 0.f) : n - nh, 1.0f, 1.0f, MP ? (y.w == 2.0f ? 1.0f : 0.f) : y.w);
                     }
-                    if (cnt - c0 < 32) hits &= (1u << (cnt - c0)) - 1u;
+                    __syncwarp();
+                    unsigned m0 = 0, m1 = 0, m2 = 0, m3 = 0;       // rows g, g + 8, g + 16, g + 24
+                    const float* p = fr + (lane >> 2) * kFragRow + (lane & 3);
+#pragma unroll
+                    for (int nt = 3; nt >= 0; nt--) {
+                        const float b0 = p[8 * nt * kFragRow], b1 = p[8 * nt * kFragRow + 4];
+                        float d[4];
+                        mma_tf32(d, af[0], b0, b1);
+                        m0 = __funnelshift_l(__float_as_uint(d[1]), m0, 1);
+                        m0 = __funnelshift_l(__float_as_uint(d[0]), m0, 1);
+                        m1 = __funnelshift_l(__float_as_uint(d[3]), m1, 1);
+                        m1 = __funnelshift_l(__float_as_uint(d[2]), m1, 1);
+                        mma_tf32(d, af[1], b0, b1);
+                        m2 = __funnelshift_l(__float_as_uint(d[1]), m2, 1);
+                        m2 = __funnelshift_l(__float_as_uint(d[0]), m2, 1);
+                        m3 = __funnelshift_l(__float_as_uint(d[3]), m3, 1);
+                        m3 = __funnelshift_l(__float_as_uint(d[2]), m3, 1);
+                    }
+                    __syncwarp();
+                    // bytes (row, lane of four) -> (lane, row): byte u of the
+                    // result is this lane's row in lane u of the four
+                    const unsigned mm = m0 | (m1 << 8) | (m2 << 16) | (m3 << 24);
+                    const unsigned w1 = __shfl_xor_sync(0xffffffffu, mm, 1), w2 = __shfl_xor_sync(0xffffffffu, mm, 2),
+                                   w3 = __shfl_xor_sync(0xffffffffu, mm, 3);
+                    // own, lane ^ 1, lane ^ 2, lane ^ 3 in this order, then by lane
+                    unsigned hits = __byte_perm(__byte_perm(mm, w1, selA), __byte_perm(w2, w3, selA), selC);
+                    hits = __byte_perm(hits, 0u, selD);
                     if ((unsigned)(sp - c0) < 32u) hits &= ~(1u << (sp - c0));
                     if constexpr (DIRECT) {
                         const PairC C(I);

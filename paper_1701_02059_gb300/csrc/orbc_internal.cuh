@@ -74,6 +74,7 @@ struct Inst {
     double rs, skin;            // search cutoff and skin
     float rc2f_ll, rc2f_wca, rc2f_pp, rsf, skinf;
     float aw, eps2z_aw;         // (pi/2)/(rc - rmin) and eps 2 zeta aw
+    float rcf_wca, rcf_pp;      // the WCA cutoffs
     float ll_lo, ll_hi, w_lo, w_hi, p_lo, p_hi;   // squared cutoffs -+ the FP64 decision band
     // integrator (host-computed constants)
     float h_m, h_i;             // dt/2/m, dt/2/I
