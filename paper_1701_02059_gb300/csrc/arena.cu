@@ -60,13 +60,6 @@ __global__ void k_offset(int* __restrict__ a, long long n, int delta) {
     if (i < n) a[i] += delta;
 }
 
-__global__ void k_slot_of_id(View v) {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= v.N) return;
-    const int b = find_inst(v.inst_p0, v.B, p);
-    v.slot_of_id[v.inst[b].p0 + (int)v.id[p]] = p;
-}
-
 static inline int nblk(long long n, int t) { return (int)((n + t - 1) / t); }
 
 // defined with the plain system's getters: int64 fixed point of a slot range
@@ -130,7 +123,9 @@ void Ensemble::setup_from(const std::vector<const Snapshot*>& list) {
         p0[b + 1] = N;
         k0[b + 1] = Ktot;
     }
-    alloc_core(p0, k0, false);
+    int nb = 0;
+    for (const Snapshot* x : list) nb += (int)x->r0.size();
+    alloc_core(p0, k0, false, nb);
     Gtot = 0;
     for (int b = 0; b < B; b++) {
         inst_h[b].g0 = Gtot;
@@ -159,9 +154,7 @@ void Ensemble::setup_from(const std::vector<const Snapshot*>& list) {
         k_offset<<<nblk(K + 1, 256), 256, 0, stream>>>(d_cell_start + k0[b], K + 1, p0[b]);
         launches += 2;
     }
-    k_slot_of_id<<<nblk(N, 256), 256, 0, stream>>>(view());
-    launches++;
-    CK(cudaGetLastError());
+    slots_of_ids();
     std::vector<BondSpec> bl(B);
     for (int b = 0; b < B; b++) bl[b] = BondSpec{&list[b]->bonds, &list[b]->r0, &list[b]->kb};
     upload_bonds(bl, p0);

@@ -275,13 +275,25 @@ public:
 
 private:
     void free_all();
-    void alloc_core(const std::vector<int>& p0, const std::vector<int>& k0, bool any_skin);
+    void alloc_core(const std::vector<int>& p0, const std::vector<int>& k0, bool any_skin, int nb);
+    void open_block(bool any_skin);
+    void lay_core(bool any_skin);
+    struct BondScratch {
+        int *cnt, *fill;
+        unsigned* flag;
+    };
+    BondScratch lay_bonds();
+    void slots_of_ids();
     void upload_bonds(const std::vector<BondSpec>& bl, const std::vector<int>& p0);
     // fused: the previous step's final B is still due; baoa_done: this step's
     // B-A-O-A already ran in the previous step's force launch; eval_step: the
     // force launch also runs the next step's B-A-O-A
     void step_body(bool fused, bool baoa_done = false, bool eval_step = false);
     size_t bytes_ = 0;
+    char* block_ = nullptr;        // the next free byte of the arrays' block
+    size_t block_left_ = 0;
+    bool laying_ = false;          // the block's size is being added up (lay_bytes_)
+    size_t lay_bytes_ = 0;
     // one step as a CUDA graph, by kind (first step of a call, a later one,
     // quench step) and state-buffer parity
     struct StepGraph {
