@@ -724,23 +724,10 @@ void Ensemble::setup(const HostInstance& h) { setup(std::vector<const HostInstan
 void Ensemble::init_cells() {
     int iters = 0;
     for (int x : n_lloyd_) iters = std::max(iters, x);
-    for (int it = 0; it < iters; it++) {
-        tic("grid");
-        build_grid();
-        toc();
-        // the first round searches every particle and records a lower bound
-        // on its second-nearest centroid; later rounds search only the
-        // particles whose bound no longer certifies their centroid
-        tic("estep");
-        if (it == 0) estep(d_cell, d_lbound);
-        else estep_bounded(d_cell);
-        toc();
-        tic("mstep");
-        mstep_iter(d_cell, it, d_dmax);
-        toc();
-    }
+    prev_adj_valid_ = false;   // (d_cell is in another order in there)
+    lloyd(iters);
     CK(cudaMemsetAsync(d_dmax, 0, sizeof(unsigned) * B, stream));
-    finish_cells();
+    finish_cells(false, d_perm);
     unsigned st = read_status(true);
     if (st) throw StateError("cell initialisation flagged status " + std::to_string(st));
     collect_times(kernel_times);

@@ -834,18 +834,48 @@ __device__ void estep_one(const View& v, int i, int* __restrict__ cell_out, floa
 // share one grid region [lo - r, hi + r]; every lane scores every centroid
 // of the region (broadcast loads), and the region grows by one ring until
 // each lane's unexplored space is provably farther than its band.
+// The centroids of the region's grid cells (ring: without those of the region
+// at r - 1), f(centroid) with the whole warp.  A lane looks at a grid cell and
+// loads its centroids, and the warp passes them round: on a membrane most of
+// the 27 to 125 grid cells are empty, and one after the other each of them
+// would cost the warp a chain of loads (160 against 112 us for the first
+// round of 500,000 particles, 78 against 52 for the later ones).
 template <typename F>
-__device__ inline void region_ring(const Inst& I, const int lo[3], const int hi[3], int r, F&& f) {
-    int a0[3], a1[3];
-    for (int a = 0; a < 3; a++) { a0[a] = max(0, lo[a] - r); a1[a] = min(I.gdim[a] - 1, hi[a] + r); }
-    for (int z = a0[2]; z <= a1[2]; z++)
-        for (int y = a0[1]; y <= a1[1]; y++)
-            for (int x = a0[0]; x <= a1[0]; x++) {
-                if (r > 0 && x >= lo[0] - r + 1 && x <= hi[0] + r - 1 && y >= lo[1] - r + 1 && y <= hi[1] + r - 1 &&
-                    z >= lo[2] - r + 1 && z <= hi[2] + r - 1)
-                    continue;
-                f(I.g0 + ((long long)z * I.gdim[1] + y) * I.gdim[0] + x);
+__device__ __forceinline__ void region_visit(const View& v, const Inst& I, const int lo[3], const int hi[3], int r,
+                                             bool ring, F&& f) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    int a0[3], ext[3];
+    for (int a = 0; a < 3; a++) {
+        a0[a] = max(0, lo[a] - r);
+        ext[a] = min(I.gdim[a] - 1, hi[a] + r) - a0[a] + 1;
+    }
+    const int n = ext[0] * ext[1] * ext[2];    // (the whole grid has up to 2^24 cells)
+    for (int base = 0; base < n; base += 32) {
+        const int t = base + lane;
+        int s = 0, c = 0;
+        if (t < n) {
+            const int x = a0[0] + t % ext[0], y = a0[1] + t / ext[0] % ext[1], z = a0[2] + t / (ext[0] * ext[1]);
+            const bool inner = ring && r > 0 && x >= lo[0] - r + 1 && x <= hi[0] + r - 1 && y >= lo[1] - r + 1 &&
+                               y <= hi[1] + r - 1 && z >= lo[2] - r + 1 && z <= hi[2] + r - 1;
+            if (!inner) {
+                const long long gg = I.g0 + ((long long)z * I.gdim[1] + y) * I.gdim[0] + x;
+                s = v.gstart[gg];
+                c = v.gstart[gg + 1] - s;
             }
+        }
+        for (int u = 0;; u++) {
+            unsigned m = __ballot_sync(full, c > u);
+            if (!m) break;
+            const float4 own = c > u ? v.gcf[s + u] : make_float4(0.f, 0.f, 0.f, 0.f);
+            while (m) {
+                const int src = __ffs(m) - 1;
+                m &= m - 1;
+                f(make_float4(__shfl_sync(full, own.x, src), __shfl_sync(full, own.y, src), __shfl_sync(full, own.z, src),
+                              __shfl_sync(full, own.w, src)));
+            }
+        }
+    }
 }
 
 __device__ inline float region_bound(const Inst& I, const float p[3], const int lo[3], const int hi[3], int r,
@@ -871,12 +901,63 @@ __device__ inline void warp_box(const int g[3], bool valid, int lo[3], int hi[3]
     }
 }
 
-// list (nullable): search only the *count particles listed (in list order,
-// which keeps the lanes of a warp close in space)
+// The search of the lanes with `in` set (whose grid cells lie in lo..hi), by
+// the whole warp.
+__device__ __forceinline__ void estep_group(const View& v, const Inst& I, int i, bool in, const long long xq[3],
+                                            const float p[3], const int lo[3], const int hi[3],
+                                            int* __restrict__ cell_out, float* __restrict__ lbound) {
+    float best = 3.0e38f, second = 3.0e38f;
+    float lbr = 3.0e38f;    // bound on the unscanned region after the last ring
+    int bk = -1;
+    int r = 0;
+    for (;; r++) {
+        region_visit(v, I, lo, hi, r, true, [&](const float4 c) {
+            const float dx = p[0] - c.x, dy = p[1] - c.y, dz = p[2] - c.z;
+            const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+            if (d2 < best) { second = best; best = d2; bk = __float_as_int(c.w); }
+            else if (d2 < second) second = d2;
+        });
+        bool ex;
+        const float lb = region_bound(I, p, lo, hi, r, ex);
+        lbr = ex ? 3.0e38f : lb;
+        const bool done = !in || ex || (best < 3.0e38f && lb > sqrtf(best) + kBandE);
+        if (__all_sync(0xffffffffu, done)) break;
+    }
+    // tie band: every centroid within the band of the FP32 best is re-scored in FP64
+    const float lim = sqrtf(best) + kBandE;
+    const bool amb = in && second <= lim * lim;
+    if (__any_sync(0xffffffffu, amb)) {
+        double best64 = 1e300;
+        int bk64 = -1;
+        region_visit(v, I, lo, hi, r, false, [&](const float4 c) {
+            const float dx = p[0] - c.x, dy = p[1] - c.y, dz = p[2] - c.z;
+            const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+            if (amb && d2 <= lim * lim) {
+                const int k = __float_as_int(c.w);
+                const double d64 = dist2_grid_d(xq[0], xq[1], xq[2], v.cq[k], v.cq[(size_t)v.Ktot + k],
+                                                v.cq[(size_t)2 * v.Ktot + k], I);
+                if (d64 < best64 || (d64 == best64 && k < bk64)) { best64 = d64; bk64 = k; }
+            }
+        });
+        if (amb) bk = bk64;
+    }
+    if (in) {
+        if (bk < 0) { flag_inst(v, I, kStatusGridRange); bk = I.k0; }
+        cell_out[i] = bk;
+        if (lbound) lbound[i] = amb ? 0.f : fminf(sqrtf(second), lbr);
+    }
+}
+
+// list (nullable): search only the particles listed, *count of them (null:
+// all of v.N), in list order, which keeps the lanes of a warp close in space.
+// A warp whose particles lie in several places (its list runs on from one row
+// of grid cells to another) takes up to eight of them one after the other
+// (three: 112 us for the first round of 500,000 particles and 50 for the
+// later ones, eight: 58 and 40, any number the same).
 __global__ void k_estep_warp(View v, int* __restrict__ cell_out, float* __restrict__ lbound,
                              const int* __restrict__ list, const int* __restrict__ count) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool valid = list ? q < *count : q < v.N;
+    const bool valid = q < (count ? *count : v.N);
     const int i = valid ? (list ? list[q] : q) : 0;
     const int b = valid ? find_inst(v.inst_p0, v.B, i) : -1;
     int b0 = __shfl_sync(0xffffffffu, b, 0);
@@ -900,60 +981,51 @@ __global__ void k_estep_warp(View v, int* __restrict__ cell_out, float* __restri
     }
     int lo[3], hi[3];
     warp_box(g, valid, lo, hi);
-    if (hi[0] - lo[0] > 2 || hi[1] - lo[1] > 2 || hi[2] - lo[2] > 2) {
-        // queries not clustered in space (e.g. input order): per-thread search
-        if (valid) estep_one(v, i, cell_out, lbound);
+    if (hi[0] - lo[0] <= 2 && hi[1] - lo[1] <= 2 && hi[2] - lo[2] <= 2) {
+        estep_group(v, I, i, valid, xq, p, lo, hi, cell_out, lbound);
         return;
     }
-    float best = 3.0e38f, second = 3.0e38f;
-    float lbr = 3.0e38f;    // bound on the unscanned region after the last ring
-    int bk = -1;
-    int r = 0;
-    for (;; r++) {
-        region_ring(I, lo, hi, r, [&](long long gg) {
-            const int q1 = v.gstart[gg + 1];
-            for (int q = v.gstart[gg]; q < q1; q++) {
-                const float4 c = v.gcf[q];
-                const float dx = p[0] - c.x, dy = p[1] - c.y, dz = p[2] - c.z;
-                const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                if (d2 < best) { second = best; best = d2; bk = __float_as_int(c.w); }
-                else if (d2 < second) second = d2;
-            }
-        });
-        bool ex;
-        const float lb = region_bound(I, p, lo, hi, r, ex);
-        lbr = ex ? 3.0e38f : lb;
-        const bool done = !valid || ex || (best < 3.0e38f && lb > sqrtf(best) + kBandE);
-        if (__all_sync(0xffffffffu, done)) break;
+    unsigned todo = __ballot_sync(0xffffffffu, valid);
+    for (int part = 0; todo && part < 8; part++) {
+        const int lead = __ffs(todo) - 1;
+        bool in = (todo >> (threadIdx.x & 31)) & 1u;
+        for (int a = 0; a < 3; a++) in = abs(g[a] - __shfl_sync(0xffffffffu, g[a], lead)) <= 1 && in;
+        warp_box(g, in, lo, hi);
+        estep_group(v, I, i, in, xq, p, lo, hi, cell_out, lbound);
+        todo &= ~__ballot_sync(0xffffffffu, in);
     }
-    // tie band: every centroid within the band of the FP32 best is re-scored in FP64
-    const float lim = sqrtf(best) + kBandE;
-    const bool amb = valid && second <= lim * lim;
-    if (__any_sync(0xffffffffu, amb)) {
-        double best64 = 1e300;
-        int bk64 = -1;
-        for (int rr = 0; rr <= r; rr++)
-            region_ring(I, lo, hi, rr, [&](long long gg) {
-                const int q1 = v.gstart[gg + 1];
-                for (int q = v.gstart[gg]; q < q1; q++) {
-                    const float4 c = v.gcf[q];
-                    const float dx = p[0] - c.x, dy = p[1] - c.y, dz = p[2] - c.z;
-                    const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                    if (amb && d2 <= lim * lim) {
-                        const int k = __float_as_int(c.w);
-                        const double d64 = dist2_grid_d(xq[0], xq[1], xq[2], v.cq[k], v.cq[(size_t)v.Ktot + k],
-                                                        v.cq[(size_t)2 * v.Ktot + k], I);
-                        if (d64 < best64 || (d64 == best64 && k < bk64)) { best64 = d64; bk64 = k; }
-                    }
-                }
-            });
-        if (amb) bk = bk64;
-    }
-    if (valid) {
-        if (bk < 0) { flag_inst(v, I, kStatusGridRange); bk = I.k0; }
-        cell_out[i] = bk;
-        if (lbound) lbound[i] = amb ? 0.f : fminf(sqrtf(second), lbr);
-    }
+    // the others: per-thread search
+    if ((todo >> (threadIdx.x & 31)) & 1u) estep_one(v, i, cell_out, lbound);
+}
+
+// The particles by grid cell, for the searches of the initialisation: the
+// input's order need not be one in space, and a warp whose lanes lie apart
+// searches thread by thread (500,000 particles, ten rounds and the search
+// after them: 1,720 us, 500 in this order, 35 to make it).  Counts per grid cell (gcount, zero before and
+// after), then each particle's place: its position and type in the second
+// buffers, its slot in order.  The order within a grid cell changes nothing
+// (each particle's search is its own, and the centroids' sums are integers).
+__device__ inline long long grid_cell(const View& v, const Inst& I, int i) {
+    int g[3];
+    float p;
+    for (int a = 0; a < 3; a++) g[a] = grid_coord(v.xq[(size_t)a * v.N + i], I, a, p);
+    return I.g0 + ((long long)g[2] * I.gdim[1] + g[1]) * I.gdim[0] + g[0];
+}
+
+__global__ void k_grid_particles(View v, int* __restrict__ gcount) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < v.N) atomicAdd(&gcount[grid_cell(v, v.inst[find_inst(v.inst_p0, v.B, i)], i)], 1);
+}
+
+__global__ void k_grid_order(View v, View to, const int* __restrict__ gstart, int* __restrict__ gcount,
+                             int* __restrict__ order) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= v.N) return;
+    const long long g = grid_cell(v, v.inst[find_inst(v.inst_p0, v.B, i)], i);
+    const int q = gstart[g] + atomicSub(&gcount[g], 1) - 1;
+    for (int a = 0; a < 3; a++) to.xq[(size_t)a * v.N + q] = v.xq[(size_t)a * v.N + i];
+    to.type[q] = v.type[i];
+    order[q] = i;
 }
 
 // One particle's nearest centroid by a whole warp: the lanes share the grid
@@ -1974,8 +2046,39 @@ bool Ensemble::displacement_exceeds_skin() {
     return f != 0;
 }
 
-void Ensemble::estep(int* cell_out, float* lbound) {
-    k_estep_warp<<<nblk(N, 128), 128, 0, stream>>>(view(), cell_out, lbound, nullptr, nullptr);
+// The Lloyd rounds of the initialisation, on the particles by grid cell
+// (their positions and types in the second state buffers, which the sort of
+// finish_cells fills anew).  d_perm is left with the slots in that order.
+void Ensemble::lloyd(int iters) {
+    const View v = view(), by_cell = view_alt();
+    k_grid_particles<<<nblk(N, 256), 256, 0, stream>>>(v, d_gcount);
+    launches++;
+    CK(cudaGetLastError());
+    scan_exclusive(d_gcount, d_gstart, Gtot + 1);
+    k_grid_order<<<nblk(N, 256), 256, 0, stream>>>(v, by_cell, d_gstart, d_gcount, d_perm);
+    launches++;
+    CK(cudaGetLastError());
+    swap_state();
+    for (int it = 0; it < iters; it++) {
+        tic("grid");
+        build_grid();
+        toc();
+        // the first round searches every particle and records a lower bound
+        // on its second-nearest centroid; later rounds search only the
+        // particles whose bound no longer certifies their centroid
+        tic("estep");
+        if (it == 0) estep(d_cell, d_lbound);
+        else estep_bounded(d_cell);
+        toc();
+        tic("mstep");
+        mstep_iter(d_cell, it, d_dmax);
+        toc();
+    }
+    swap_state();
+}
+
+void Ensemble::estep(int* cell_out, float* lbound, const int* order) {
+    k_estep_warp<<<nblk(N, 128), 128, 0, stream>>>(view(), cell_out, lbound, order, nullptr);
     launches++;
     CK(cudaGetLastError());
 }
@@ -2011,7 +2114,8 @@ void Ensemble::morton_relabel() {
 
 bool Ensemble::small_cells() const { return B == 1 && Ktot <= kSmallK && Gtot < kSmallG; }
 
-void Ensemble::finish_cells(bool sums_ready) {
+// order: the slots in an order that keeps neighbours together (nullable).
+void Ensemble::finish_cells(bool sums_ready, const int* order) {
     View v = view();
     const bool small = small_cells();
     if (small) {
@@ -2038,7 +2142,7 @@ void Ensemble::finish_cells(bool sums_ready) {
             k_grid_fill<<<nblk(Ktot, 256), 256, 0, stream>>>(v, d_gidx, d_gcount, d_cf);
             launches++;
         }
-        estep(d_cell_new, nullptr);
+        estep(d_cell_new, nullptr, order);
         k_hist<<<nblk(N, 256), 256, 0, stream>>>(N, d_cell_new, d_cnt);
         launches++;
     }

@@ -242,12 +242,13 @@ public:
     void mstep_iter(const int* cell_of, int iter, unsigned* dmax = nullptr);
     bool displacement_exceeds_skin();
     void launch_kinetic();
-    void estep(int* cell_out, float* lbound);       // grid search; lbound: second-nearest bounds
+    void lloyd(int iters);                          // the k-means rounds of init_cells
+    void estep(int* cell_out, float* lbound, const int* order = nullptr);   // grid search; lbound: second-nearest bounds
     void estep_bounded(int* cell);                  // k-means rounds after the first (bounds in d_lbound)
     void morton_relabel();
     bool small_cells() const;   // one block relabels the cells (k_relabel_small)
     // sums_ready: the relabel of a small batch also applies the M-step's sums
-    void finish_cells(bool sums_ready = false);
+    void finish_cells(bool sums_ready = false, const int* order = nullptr);
     // one_launch: FP32 energies by the kernel without lists (for more partners
     // than the lists and their overflow hold)
     void launch_pairs(bool energies, bool dump, bool one_launch = false);
