@@ -1356,11 +1356,10 @@ __global__ void k_segsort(int Ktot, const int* __restrict__ start, int* __restri
 // Cells of up to 32 NE particles: one warp, bitonic network over NE values per
 // lane (element e = lane + 32 q), shuffles for strides < 32.
 template <int NE>
-__device__ inline void segsort_net(int s, int n, int* __restrict__ tmp) {
+__device__ __forceinline__ void segsort_net(const int* __restrict__ tmp, int n, int (&val)[NE]) {
     const int lane = threadIdx.x & 31;
-    int val[NE];
 #pragma unroll
-    for (int q = 0; q < NE; q++) val[q] = (lane + 32 * q < n) ? tmp[s + lane + 32 * q] : 0x7fffffff;
+    for (int q = 0; q < NE; q++) val[q] = (lane + 32 * q < n) ? tmp[lane + 32 * q] : 0x7fffffff;
 #pragma unroll
     for (int size = 2; size <= 32 * NE; size <<= 1) {
 #pragma unroll
@@ -1388,13 +1387,19 @@ __device__ inline void segsort_net(int s, int n, int* __restrict__ tmp) {
             }
         }
     }
+}
+template <int NE>
+__device__ inline void segsort_store(int s, int n, int* __restrict__ tmp) {
+    const int lane = threadIdx.x & 31;
+    int val[NE];
+    segsort_net<NE>(tmp + s, n, val);
 #pragma unroll
     for (int q = 0; q < NE; q++)
         if (lane + 32 * q < n) tmp[s + lane + 32 * q] = val[q];
 }
 __device__ inline void segsort_warp(int s, int n, int* __restrict__ tmp) {   // n <= 128
-    if (n <= 64) segsort_net<2>(s, n, tmp);
-    else segsort_net<4>(s, n, tmp);
+    if (n <= 64) segsort_store<2>(s, n, tmp);
+    else segsort_store<4>(s, n, tmp);
 }
 
 __global__ void k_segsort_warp(int Ktot, const int* __restrict__ start, int* __restrict__ tmp) {
@@ -1404,19 +1409,11 @@ __global__ void k_segsort_warp(int Ktot, const int* __restrict__ start, int* __r
     if (n > 1 && n <= 128) segsort_warp(s, n, tmp);
 }
 
-// The rebuild's form, one launch for every size: 256 threads, eight cells; a
-// warp sorts its cell when it holds up to 128 particles, then the block takes
-// the larger ones (rare) one after the other, bitonic in shared memory up to
-// kSegMax, beyond it each slot's rank among its cell's (distinct) slots, out
-// being scratch.
-__global__ void __launch_bounds__(256) k_segsort_cells(int Ktot, const int* __restrict__ start, int* __restrict__ tmp,
-                                                       int* __restrict__ out) {
-    __shared__ int sh[kSegMax];
-    const int k0 = blockIdx.x * 8, k = k0 + (threadIdx.x >> 5);
-    const int s = k < Ktot ? start[k] : 0, n = k < Ktot ? start[k + 1] - s : 0;
-    if (n > 1 && n <= 128) segsort_warp(s, n, tmp);
-    if (!__syncthreads_or(n > 128)) return;
-    for (int c = k0; c < min(k0 + 8, Ktot); c++) {
+// The cells k0..k1 - 1 of more than 128 particles, by the block one after the
+// other: bitonic in shared memory up to kSegMax, beyond it each slot's rank
+// among its cell's (distinct) slots, out being scratch.
+__device__ void segsort_large(int k0, int k1, const int* __restrict__ start, int* tmp, int* out, int* sh) {
+    for (int c = k0; c < k1; c++) {
         const int s0 = start[c], m0 = start[c + 1] - s0;
         if (m0 <= 128) continue;
         if (m0 <= kSegMax) {
@@ -1449,6 +1446,18 @@ __global__ void __launch_bounds__(256) k_segsort_cells(int Ktot, const int* __re
         }
         __syncthreads();
     }
+}
+
+// The rebuild's form for large cells, one launch for every size: 256 threads,
+// eight cells; a warp sorts its cell when it holds up to 128 particles, then
+// the block takes the larger ones.
+__global__ void __launch_bounds__(256) k_segsort_cells(int Ktot, const int* __restrict__ start, int* __restrict__ tmp,
+                                                       int* __restrict__ out) {
+    __shared__ int sh[kSegMax];
+    const int k0 = blockIdx.x * 8, k = k0 + (threadIdx.x >> 5);
+    const int s = k < Ktot ? start[k] : 0, n = k < Ktot ? start[k + 1] - s : 0;
+    if (n > 1 && n <= 128) segsort_warp(s, n, tmp);
+    if (__syncthreads_or(n > 128)) segsort_large(k0, min(k0 + 8, Ktot), start, tmp, out, sh);
 }
 
 // Cells larger than kSegMax: each slot's rank among its cell's (distinct)
@@ -1499,55 +1508,68 @@ __device__ inline int mirror_coord(long long xq, long long cq, const Inst& I, in
 // (cell_r2).
 constexpr float kBandR = 1e-5f;
 
-// Gather of the cell-sorted state, one thread per new slot p: the particle
-// of old slot perm[p] moves with its state, type and id, learns its new cell
-// (the E-step's result for the old slot) and gets its exact mirror relative
-// to that cell's centroid.  Every load and the mirror come before the first
+// Gather of the cell-sorted state: the particle of old slot so moves to slot p
+// of cell k with its state, type and id and gets its exact mirror relative to
+// that cell's centroid.  Every load and the mirror come before the first
 // store: as far as the compiler knows the stores may alias the sources, and
 // interleaved they would serialise the loads' latencies.
+struct Moved {
+    long long x[3], vq[3], nq[3], wq[3];
+    unsigned id;
+    int q0;          // p0 + id
+    int4 m;
+    float4 no;
+};
+
+__device__ __forceinline__ void move_load(const View& v, const View& o, const Inst& I, int k, int so, int p, Moved& g) {
+    const size_t N = v.N;
+    g.id = o.id[so];        // (first: the bond list's look-up waits for it)
+    for (int a = 0; a < 3; a++) {
+        g.x[a] = o.xq[a * N + so];
+        g.vq[a] = o.vq[a * N + so];
+        g.nq[a] = o.nq[a * N + so];
+        g.wq[a] = o.wq[a * N + so];
+    }
+    const unsigned char t = o.type[so];
+    g.m.x = mirror_coord(g.x[0], v.cq[k], I, 0, v);
+    g.m.y = mirror_coord(g.x[1], v.cq[(size_t)v.Ktot + k], I, 1, v);
+    g.m.z = mirror_coord(g.x[2], v.cq[(size_t)2 * v.Ktot + k], I, 2, v);
+    g.q0 = I.p0 + (int)g.id;
+    g.m.w = t | (v.bptr[g.q0] < v.bptr[g.q0 + 1] ? kMirrorBonded : 0);
+    g.no.x = ll_to_float(g.nq[0]) * (float)kGridInv;
+    g.no.y = ll_to_float(g.nq[1]) * (float)kGridInv;
+    g.no.z = ll_to_float(g.nq[2]) * (float)kGridInv;
+    g.no.w = __int_as_float(p);
+}
+
+__device__ __forceinline__ void move_store(const View& v, int k, int p, const Moved& g, long long* __restrict__ xref) {
+    const size_t N = v.N;
+    for (int a = 0; a < 3; a++) {
+        v.xq[a * N + p] = g.x[a];
+        v.vq[a * N + p] = g.vq[a];
+        v.nq[a * N + p] = g.nq[a];
+        v.wq[a * N + p] = g.wq[a];
+        if (xref) xref[a * N + p] = g.x[a];
+    }
+    v.type[p] = (unsigned char)(g.m.w & 0xff);
+    v.id[p] = g.id;
+    v.cell[p] = k;
+    v.slot_of_id[g.q0] = p;
+}
+
+// One thread per new slot (large cells; k_build_cells otherwise): the old slot
+// is perm[p], the cell the E-step's result for it.
 __global__ void __launch_bounds__(256) k_gather_particles(View v, View o, const int* __restrict__ perm,
                                                           const int* __restrict__ cell_new,
                                                           long long* __restrict__ xref) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= v.N) return;
-    const size_t N = v.N;
-    const int so = perm[p];
-    const int k = cell_new[so];
-    long long x[3], vq[3], nq[3], wq[3];
-    for (int a = 0; a < 3; a++) {
-        x[a] = o.xq[a * N + so];
-        vq[a] = o.vq[a * N + so];
-        nq[a] = o.nq[a * N + so];
-        wq[a] = o.wq[a * N + so];
-    }
-    const unsigned char t = o.type[so];
-    const unsigned id = o.id[so];
-    const int b = find_inst(v.inst_p0, v.B, p);
-    const Inst& I = v.inst[b];
-    int4 m;
-    m.x = mirror_coord(x[0], v.cq[k], I, 0, v);
-    m.y = mirror_coord(x[1], v.cq[(size_t)v.Ktot + k], I, 1, v);
-    m.z = mirror_coord(x[2], v.cq[(size_t)2 * v.Ktot + k], I, 2, v);
-    const int q0 = I.p0 + (int)id;
-    m.w = t | (v.bptr[q0] < v.bptr[q0 + 1] ? kMirrorBonded : 0);
-    float4 no;
-    no.x = ll_to_float(nq[0]) * (float)kGridInv;
-    no.y = ll_to_float(nq[1]) * (float)kGridInv;
-    no.z = ll_to_float(nq[2]) * (float)kGridInv;
-    no.w = __int_as_float(p);
-    for (int a = 0; a < 3; a++) {
-        v.xq[a * N + p] = x[a];
-        v.vq[a * N + p] = vq[a];
-        v.nq[a * N + p] = nq[a];
-        v.wq[a * N + p] = wq[a];
-        if (xref) xref[a * N + p] = x[a];
-    }
-    v.type[p] = t;
-    v.id[p] = id;
-    v.cell[p] = k;
-    v.slot_of_id[q0] = p;
-    v.mq[p] = m;
-    v.mo[p] = no;
+    const int so = perm[p], k = cell_new[so];
+    Moved g;
+    move_load(v, o, v.inst[find_inst(v.inst_p0, v.B, p)], k, so, p, g);
+    move_store(v, k, p, g, xref);
+    v.mq[p] = g.m;
+    v.mo[p] = g.no;
 }
 
 // Bitonic sort of 32 * NE records over a warp, slot lane + 32 u held in
@@ -1597,57 +1619,44 @@ __global__ void k_cell_r2(View v, const long long* __restrict__ x) {
     if (k < v.Ktot) v.R2[k] = cell_r2(v, x, v.inst[find_inst(v.inst_k0, v.B, k)], k);
 }
 
-// Per-cell quantities read back from the gathered mirrors: one warp per cell
-// finds the cell radius (in FP32, and the particle that sets it), the pair
-// kernels' cell frame (its normal the mean bilayer director, +z without one)
-// and, in each tile of 128 particles, every particle's rank along the tile's
-// longer tangent extent.  rmax_bits: each instance's largest radius (FP32
-// bits).
-__global__ void __launch_bounds__(256, 6) k_cell_props(View v, unsigned* rmax_bits /* [B] */) {
-    const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (k >= v.Ktot) return;
-    const int b = find_inst(v.inst_k0, v.B, k);
-    const Inst& I = v.inst[b];
-    const int s = v.cell_start[k], e = v.cell_start[k + 1];
-    const size_t N = v.N;
-    const long long ck[3] = {v.cq[k], v.cq[(size_t)v.Ktot + k], v.cq[(size_t)2 * v.Ktot + k]};
+// What the pair kernels and the neighbour search want of a cell, by one warp:
+// the cell radius (in FP32, and the particle that sets it), the pair kernels'
+// cell frame (its normal the mean bilayer director, +z without one) and, in
+// each tile of 128 particles, every particle's rank along the tile's longer
+// tangent extent.  rmax_bits: each instance's largest radius (FP32 bits).
+struct CellSums {        // a lane's share, then the cell's
     float mx = 0.f, nx = 0.f, ny = 0.f, nz = 0.f;
-    for (int p = s + lane; p < e; p += 32) {
-        const int4 m = v.mq[p];
-        const float4 no = v.mo[p];
+    __device__ __forceinline__ static float dist(const int4& m) {
         const float dx = m.x * kMirrorUnit, dy = m.y * kMirrorUnit, dz = m.z * kMirrorUnit;
-        mx = fmaxf(mx, sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz))));
-        if (bilayer(m.w & 0xff)) { nx += no.x; ny += no.y; nz += no.z; }
+        return sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
     }
-    for (int off = 16; off; off >>= 1) {
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-        nx += __shfl_xor_sync(0xffffffffu, nx, off);
-        ny += __shfl_xor_sync(0xffffffffu, ny, off);
-        nz += __shfl_xor_sync(0xffffffffu, nz, off);
+    __device__ __forceinline__ void add(const int4& m, float x, float y, float z) {
+        mx = fmaxf(mx, dist(m));
+        if (bilayer(m.w & 0xff)) { nx += x; ny += y; nz += z; }
     }
-    // the particles within the band of the FP32 maximum: one, or the FP64
-    // definition among them
-    int cand = -1, nc = 0;
-    for (int p = s + lane; p < e; p += 32) {
-        const int4 m = v.mq[p];
-        const float dx = m.x * kMirrorUnit, dy = m.y * kMirrorUnit, dz = m.z * kMirrorUnit;
-        const float d = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-        if (d >= mx - kBandR) { cand = p; nc++; }
+    __device__ __forceinline__ void reduce() {
+        for (int off = 16; off; off >>= 1) {
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+            nx += __shfl_xor_sync(0xffffffffu, nx, off);
+            ny += __shfl_xor_sync(0xffffffffu, ny, off);
+            nz += __shfl_xor_sync(0xffffffffu, nz, off);
+        }
     }
+};
+
+// The radius: of the particles within the band of the FP32 maximum (cand, the
+// last of the nc in this lane) the only one is noted, or exact(), a lane's
+// largest FP64 distance squared among its own, decides.
+template <typename F>
+__device__ __forceinline__ void cell_radius(const View& v, int k, int b, float mx, int cand, int nc, unsigned* rmax_bits,
+                                            F&& exact) {
+    const int lane = threadIdx.x & 31;
     nc = (int)__reduce_add_sync(0xffffffffu, (unsigned)nc);
     cand = __reduce_max_sync(0xffffffffu, cand);
     if (nc > 1) {
         // (the maximum over the lanes on the bit patterns: a non-negative
         // double's bits order like its value)
-        unsigned long long bb = 0;
-        for (int p = s + lane; p < e; p += 32) {
-            const int4 m = v.mq[p];
-            const float dx = m.x * kMirrorUnit, dy = m.y * kMirrorUnit, dz = m.z * kMirrorUnit;
-            if (sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz))) >= mx - kBandR)
-                bb = max(bb, (unsigned long long)__double_as_longlong(
-                                 dist2_grid_d(v.xq[p], v.xq[N + p], v.xq[2 * N + p], ck[0], ck[1], ck[2], I)));
-        }
+        unsigned long long bb = exact();
         for (int off = 16; off; off >>= 1) bb = max(bb, (unsigned long long)__shfl_xor_sync(0xffffffffu, bb, off));
         if (lane == 0) v.R2[k] = __longlong_as_double((long long)bb);
         cand = -1;
@@ -1661,7 +1670,16 @@ __global__ void __launch_bounds__(256, 6) k_cell_props(View v, unsigned* rmax_bi
         // the one address)
         if (__float_as_uint(mx) > __ldca(rmax_bits + b)) atomicMax(&rmax_bits[b], __float_as_uint(mx));
     }
-    // pair-kernel frame
+}
+
+__device__ __forceinline__ unsigned long long exact_r2_bits(const View& v, const Inst& I, int k, int p) {
+    const size_t N = v.N, K = v.Ktot;
+    return (unsigned long long)__double_as_longlong(
+        dist2_grid_d(v.xq[p], v.xq[N + p], v.xq[2 * N + p], v.cq[k], v.cq[K + k], v.cq[2 * K + k], I));
+}
+
+__device__ __forceinline__ Frame cell_frame(const View& v, int k, float nx, float ny, float nz) {
+    const int lane = threadIdx.x & 31;
     const float nn = sqrtf(fmaf(nx, nx, fmaf(ny, ny, nz * nz)));
     if (nn > 1e-3f) { nx /= nn; ny /= nn; nz /= nn; }
     else { nx = 0.f; ny = 0.f; nz = 1.f; }
@@ -1670,43 +1688,80 @@ __global__ void __launch_bounds__(256, 6) k_cell_props(View v, unsigned* rmax_bi
         v.cframe[3 * (size_t)k + lane] =
             lane == 0 ? make_float4(F.r[0], F.r[1], F.r[2], 0.f)
                       : (lane == 1 ? make_float4(F.r[3], F.r[4], F.r[5], 0.f) : make_float4(F.r[6], F.r[7], F.r[8], 0.f));
-    // pair-kernel groups: ranks inside each tile of 128 particles
+    return F;
+}
+
+// A tile of nt <= 32 NE particles (particle lane + 32 u at tangent coordinates
+// ya[u], yb[u]) in the order of its longer tangent extent: rank lane + 32 u
+// goes to the particle (r[u] & 127), none where r[u] is ~0.  32-bit records:
+// the key quantised to 24 bits over the tile's extent (monotone), the tile
+// index in the low 7 bits (equal keys go by index), sorted over the warp.
+template <int NE>
+__device__ __forceinline__ void tile_ranks(const float (&ya)[4], const float (&yb)[4], int nt, unsigned (&r)[4]) {
+    const int lane = threadIdx.x & 31;
+    float lo_a = 3.0e38f, hi_a = -3.0e38f, lo_b = 3.0e38f, hi_b = -3.0e38f;
+#pragma unroll
+    for (int u = 0; u < NE; u++)
+        if (lane + 32 * u < nt) {
+            lo_a = fminf(lo_a, ya[u]); hi_a = fmaxf(hi_a, ya[u]);
+            lo_b = fminf(lo_b, yb[u]); hi_b = fmaxf(hi_b, yb[u]);
+        }
+    for (int off = 16; off; off >>= 1) {
+        lo_a = fminf(lo_a, __shfl_xor_sync(0xffffffffu, lo_a, off));
+        hi_a = fmaxf(hi_a, __shfl_xor_sync(0xffffffffu, hi_a, off));
+        lo_b = fminf(lo_b, __shfl_xor_sync(0xffffffffu, lo_b, off));
+        hi_b = fmaxf(hi_b, __shfl_xor_sync(0xffffffffu, hi_b, off));
+    }
+    const bool use_a = (hi_a - lo_a) >= (hi_b - lo_b);
+    const float klo = use_a ? lo_a : lo_b, kext = use_a ? hi_a - lo_a : hi_b - lo_b;
+    const float ksc = kext > 0.f ? 16777215.0f / kext : 0.f;
+#pragma unroll
+    for (int u = 0; u < NE; u++) {
+        const int t = lane + 32 * u;
+        const float y = use_a ? ya[u] : yb[u];
+        r[u] = (t < nt) ? (min(16777215u, (unsigned)((y - klo) * ksc)) << 7) | (unsigned)t : 0xffffffffu;
+    }
+    warp_bitonic_u32<NE>(r, lane);
+}
+
+// Cell k from the gathered mirrors mq, mo (written by the same lanes, or by an
+// earlier launch).
+__device__ void cell_props(const View& v, int k, unsigned* rmax_bits) {
+    const int lane = threadIdx.x & 31;
+    const int b = find_inst(v.inst_k0, v.B, k);
+    const Inst& I = v.inst[b];
+    const int s = v.cell_start[k], e = v.cell_start[k + 1];
+    CellSums c;
+    for (int p = s + lane; p < e; p += 32) {
+        const float4 no = v.mo[p];
+        c.add(v.mq[p], no.x, no.y, no.z);
+    }
+    c.reduce();
+    int cand = -1, nc = 0;
+    for (int p = s + lane; p < e; p += 32)
+        if (CellSums::dist(v.mq[p]) >= c.mx - kBandR) { cand = p; nc++; }
+    cell_radius(v, k, b, c.mx, cand, nc, rmax_bits, [&] {
+        unsigned long long bb = 0;
+        for (int p = s + lane; p < e; p += 32)
+            if (CellSums::dist(v.mq[p]) >= c.mx - kBandR) bb = max(bb, exact_r2_bits(v, I, k, p));
+        return bb;
+    });
+    const Frame F = cell_frame(v, k, c.nx, c.ny, c.nz);
     for (int t0 = s; t0 < e; t0 += 128) {
         const int nt = min(128, e - t0);
         float ya[4], yb[4];
-        float lo_a = 3.0e38f, hi_a = -3.0e38f, lo_b = 3.0e38f, hi_b = -3.0e38f;
         for (int u = 0; u < 4; u++) {
             const int t = lane + 32 * u;
             ya[u] = 0.f; yb[u] = 0.f;
             if (t < nt) {
                 const int4 m = v.mq[t0 + t];
-                float c;
-                F.apply(m.x * kMirrorUnit, m.y * kMirrorUnit, m.z * kMirrorUnit, ya[u], yb[u], c);
-                lo_a = fminf(lo_a, ya[u]); hi_a = fmaxf(hi_a, ya[u]);
-                lo_b = fminf(lo_b, yb[u]); hi_b = fmaxf(hi_b, yb[u]);
+                float h;
+                F.apply(m.x * kMirrorUnit, m.y * kMirrorUnit, m.z * kMirrorUnit, ya[u], yb[u], h);
             }
         }
-        for (int off = 16; off; off >>= 1) {
-            lo_a = fminf(lo_a, __shfl_xor_sync(0xffffffffu, lo_a, off));
-            hi_a = fmaxf(hi_a, __shfl_xor_sync(0xffffffffu, hi_a, off));
-            lo_b = fminf(lo_b, __shfl_xor_sync(0xffffffffu, lo_b, off));
-            hi_b = fmaxf(hi_b, __shfl_xor_sync(0xffffffffu, hi_b, off));
-        }
-        const bool use_a = (hi_a - lo_a) >= (hi_b - lo_b);
-        // 32-bit records: the key quantised to 24 bits over the tile's
-        // extent (monotone), the tile index in the low 7 bits (equal keys
-        // go by index); the rank of a particle is the slot its record ends
-        // in after a warp bitonic sort
-        const float klo = use_a ? lo_a : lo_b, kext = use_a ? hi_a - lo_a : hi_b - lo_b;
-        const float ksc = kext > 0.f ? 16777215.0f / kext : 0.f;
-        unsigned r[4];
-        for (int u = 0; u < 4; u++) {
-            const int t = lane + 32 * u;
-            const float y = use_a ? ya[u] : yb[u];
-            r[u] = (t < nt) ? (min(16777215u, (unsigned)((y - klo) * ksc)) << 7) | (unsigned)t : 0xffffffffu;
-        }
-        if (nt <= 64) warp_bitonic_u32<2>(r, lane);
-        else warp_bitonic_u32<4>(r, lane);
+        unsigned r[4] = {~0u, ~0u, ~0u, ~0u};
+        if (nt <= 64) tile_ranks<2>(ya, yb, nt, r);
+        else tile_ranks<4>(ya, yb, nt, r);
         for (int u = 0; u < 4; u++) {
             if (r[u] == 0xffffffffu) continue;
             const int t = (int)(r[u] & 127u), q = lane + 32 * u;
@@ -1718,6 +1773,124 @@ __global__ void __launch_bounds__(256, 6) k_cell_props(View v, unsigned* rmax_bi
     }
 }
 
+__global__ void __launch_bounds__(256, 6) k_cell_props(View v, unsigned* rmax_bits /* [B] */) {
+    const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (k < v.Ktot) cell_props(v, k, rmax_bits);
+}
+
+// A cell of more than 128 particles (its old slots sorted): the mirrors go
+// through mq, mo.
+__device__ __noinline__ void build_large(const View& v, const View& o, int k, int s, int n, const int* perm,
+                                         long long* __restrict__ xref, unsigned* rmax_bits) {
+    const Inst& I = v.inst[find_inst(v.inst_k0, v.B, k)];
+    for (int p = s + (threadIdx.x & 31); p < s + n; p += 32) {
+        Moved g;
+        move_load(v, o, I, k, perm[p], p, g);
+        move_store(v, k, p, g, xref);
+        v.mq[p] = g.m;
+        v.mo[p] = g.no;
+    }
+    __syncwarp();
+    cell_props(v, k, rmax_bits);
+}
+
+// What a warp of k_build_cells keeps of its cell.
+struct CellTile {
+    int4 m[128];
+    float nx[128], ny[128], nz[128];
+    int so[128];
+};
+
+template <int NE>
+__device__ __forceinline__ void tile_sort(const int* __restrict__ perm, int n, int* so) {
+    const int lane = threadIdx.x & 31;
+    int val[NE];
+    segsort_net<NE>(perm, n, val);
+#pragma unroll
+    for (int u = 0; u < NE; u++) so[lane + 32 * u] = val[u];
+}
+
+template <int NE>
+__device__ __forceinline__ void tile_write(const View& v, const CellTile& T, const Frame& F, int s, int n) {
+    const int lane = threadIdx.x & 31;
+    float ya[4], yb[4];
+#pragma unroll
+    for (int u = 0; u < NE; u++) {
+        const int t = lane + 32 * u;
+        ya[u] = yb[u] = 0.f;
+        if (t < n) {
+            float h;
+            F.apply(T.m[t].x * kMirrorUnit, T.m[t].y * kMirrorUnit, T.m[t].z * kMirrorUnit, ya[u], yb[u], h);
+        }
+    }
+    unsigned r[4];
+    tile_ranks<NE>(ya, yb, n, r);
+#pragma unroll
+    for (int u = 0; u < NE; u++) {
+        if (r[u] == 0xffffffffu) continue;
+        const int t = (int)(r[u] & 127u), q = lane + 32 * u;
+        v.grank[s + t] = (unsigned char)q;
+        v.mqr[s + q] = T.m[t];
+        v.mor[s + q] = make_float4(T.nx[t], T.ny[t], T.nz[t], __int_as_float(s + t));
+    }
+}
+
+// The cell sort's last part, the gather and the cells' properties in one
+// launch, a warp per cell, the mirrors in shared memory throughout.  Bound by
+// the latency of the gather's loads (in 1,000,000 particles 42% of the DRAM
+// bandwidth, warps waiting for loads half of the time): as launches of their
+// own the three took 8, 51 and 27 us there, together 62, as the sorts and the
+// sums of one warp run under the loads of others and the mirrors are not
+// written and read back.  Registers decide: the mirrors in registers (80, 24
+// warps an SM) 80 us, here 64 registers and 32 warps; 48 registers spill (75).
+// Rebuild of the 4M cell 637 -> 555 us, of the 62k vesicle 94 -> 87.
+constexpr int kBuildWarps = 4;
+__global__ void __launch_bounds__(32 * kBuildWarps, 8)
+    k_build_cells(View v, View o, int* __restrict__ perm, int* __restrict__ out, long long* __restrict__ xref,
+                  unsigned* rmax_bits) {
+    __shared__ CellTile tile[kBuildWarps];
+    static_assert(sizeof(tile) >= kSegMax * sizeof(int), "the large cells' sort uses the tiles' memory");
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int k0 = blockIdx.x * kBuildWarps, k = k0 + w;
+    const int s = k < v.Ktot ? v.cell_start[k] : 0, n = k < v.Ktot ? v.cell_start[k + 1] - s : 0;
+    if (__syncthreads_or(n > 128))
+        segsort_large(k0, min(k0 + kBuildWarps, v.Ktot), v.cell_start, perm, out, reinterpret_cast<int*>(tile));
+    if (k >= v.Ktot) return;
+    if (n > 128) {
+        build_large(v, o, k, s, n, perm, xref, rmax_bits);
+        return;
+    }
+    CellTile& T = tile[w];
+    if (n <= 64) tile_sort<2>(perm + s, n, T.so);
+    else tile_sort<4>(perm + s, n, T.so);
+    __syncwarp();
+    const int b = find_inst(v.inst_k0, v.B, k);
+    const Inst& I = v.inst[b];
+    CellSums c;
+#pragma unroll 1
+    for (int t = lane; t < n; t += 32) {
+        Moved g;
+        move_load(v, o, I, k, T.so[t], s + t, g);
+        move_store(v, k, s + t, g, xref);
+        T.m[t] = g.m;
+        T.nx[t] = g.no.x; T.ny[t] = g.no.y; T.nz[t] = g.no.z;
+        c.add(g.m, g.no.x, g.no.y, g.no.z);
+    }
+    __syncwarp();
+    c.reduce();
+    int cand = -1, nc = 0;
+    for (int t = lane; t < n; t += 32)
+        if (CellSums::dist(T.m[t]) >= c.mx - kBandR) { cand = s + t; nc++; }
+    cell_radius(v, k, b, c.mx, cand, nc, rmax_bits, [&] {
+        unsigned long long bb = 0;
+        for (int t = lane; t < n; t += 32)
+            if (CellSums::dist(T.m[t]) >= c.mx - kBandR) bb = max(bb, exact_r2_bits(v, I, k, s + t));
+        return bb;
+    });
+    const Frame F = cell_frame(v, k, c.nx, c.ny, c.nz);
+    if (n <= 64) tile_write<2>(v, T, F, s, n);
+    else tile_write<4>(v, T, F, s, n);
+}
 
 // Mirrors of the current order (after integration without a rebuild),
 // written where the pair kernel reads them: slot p of its cell's tile of 128
@@ -2114,6 +2287,13 @@ void Ensemble::morton_relabel() {
 
 bool Ensemble::small_cells() const { return B == 1 && Ktot <= kSmallK && Gtot < kSmallG; }
 
+// Whether k_build_cells does the rebuild's last part, or the sort, the gather
+// (a thread per particle) and the cells' properties a launch each: up to a
+// mean of 300 particles a cell the one launch was the faster one (rebuild of
+// 620k particles: 61 a cell 172 against 186 us, 150: 204 and 222, 300: 246 and
+// 256); few cells of thousands would leave each to one warp.
+bool Ensemble::build_fused() const { return N <= 256ll * Ktot; }
+
 // order: the slots in an order that keeps neighbours together (nullable).
 void Ensemble::finish_cells(bool sums_ready, const int* order) {
     View v = view();
@@ -2152,16 +2332,22 @@ void Ensemble::finish_cells(bool sums_ready, const int* order) {
     after_baoa_ = -1;
     ovf_clean_ = true;
     k_scatter<<<nblk(N, 256), 256, 0, stream>>>(N, d_cell_new, d_cell_start, d_cnt, d_perm, B, z);
-    k_segsort_cells<<<nblk(Ktot, 8), 256, 0, stream>>>(Ktot, d_cell_start, d_perm, d_cell_tmp);
-    launches += 2;
+    launches++;
     CK(cudaGetLastError());
     // gather into the second buffer set, then swap
     swap_state();
     View nv = view();
     View ov = view_alt();
-    k_gather_particles<<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(nv, ov, d_perm, d_cell_new, d_xref);
-    k_cell_props<<<nblk((long long)Ktot * 32, spread_block((long long)Ktot * 32, 256)), spread_block((long long)Ktot * 32, 256), 0, stream>>>(nv, d_rmax);
-    launches += 2;
+    if (build_fused()) {
+        k_build_cells<<<nblk(Ktot, kBuildWarps), 32 * kBuildWarps, 0, stream>>>(nv, ov, d_perm, d_cell_tmp, d_xref, d_rmax);
+        launches++;
+    } else {
+        const long long warps = (long long)Ktot * 32;
+        k_segsort_cells<<<nblk(Ktot, 8), 256, 0, stream>>>(Ktot, d_cell_start, d_perm, d_cell_tmp);
+        k_gather_particles<<<nblk(N, spread_block(N, 256)), spread_block(N, 256), 0, stream>>>(nv, ov, d_perm, d_cell_new, d_xref);
+        k_cell_props<<<nblk(warps, spread_block(warps, 256)), spread_block(warps, 256), 0, stream>>>(nv, d_rmax);
+        launches += 3;
+    }
     CK(cudaGetLastError());
     // neighbouring cells
     k_adj_warp<<<nblk((long long)Ktot * 32, spread_block((long long)Ktot * 32, 256)), spread_block((long long)Ktot * 32, 256), 0, stream>>>(nv, d_rmax, d_adjcount, d_rho, d_adjpad);

@@ -248,6 +248,7 @@ public:
     void morton_relabel();
     bool small_cells() const;   // one block relabels the cells (k_relabel_small)
     // sums_ready: the relabel of a small batch also applies the M-step's sums
+    bool build_fused() const;
     void finish_cells(bool sums_ready = false, const int* order = nullptr);
     // one_launch: FP32 energies by the kernel without lists (for more partners
     // than the lists and their overflow hold)
