@@ -39,22 +39,6 @@ MAX_SM_MHZ = 2070.0
 # candidate test), counted from the pair expression
 FLOP_PER_PAIR = 100.0
 FLOP_PER_CANDIDATE = 9.0
-# FP64 arithmetic of the integrator's B-A-O-A per step (both half kicks, both
-# drifts with their Cayley maps and the renormalisation, the
-# Ornstein-Uhlenbeck update with its noise scaling), counted from the
-# kernel's expressions with FMA = 2 and a division as 1: per lipid (the
-# angular kick 15, first drift's Cayley map 32 and second drift's 36 with the
-# Cayley factor's three-term series and the renormalisation's exact integer
-# norm, the angular Ornstein-Uhlenbeck update 21); a point particle has none.
-# The translational kick, the drifts and the velocity's Ornstein-Uhlenbeck
-# update are exact 128-bit integer products (and a sum of two) of the int64
-# state with the FP64 constants (integer pipes, one rounding) and are not
-# FP64 flops; the int64 <-> FP64 conversions (about 40 per lipid) use the
-# FP64 pipe but are not counted.
-FLOP64_PER_LIPID_STEP = 104.0
-FLOP64_PER_BEAD_STEP = 0.0
-# FP64 peak: the recipe's nominal GB300 figure (no measured FP64 peak exists)
-FP64_TFLOPS = 1.25
 # algorithmic HBM bytes of one step per particle (cells rebuilt every step):
 # B-A-O-A 240, M-step 24, E-step 32, histogram/scatter/per-cell order 16,
 # gather 238 (state in and out, mirrors, slot), pair kernel 80 (mirrors in,
@@ -288,8 +272,6 @@ def run_ours(args, rank, world):
     # work counts of the step: half-list pairs and quad-loop candidate tests
     # (counted from the cell list), lipids and point particles
     npairs, ncand = algorithmic_work(g, mem)
-    n_lip = int((mem.type == 0).sum())
-    n_bead = mem.n - n_lip
     peak32 = SM_COUNT * FP32_LANES * 2 * MAX_SM_MHZ * 1e6 / 1e12
     pk_meas, src = peaks()
     hbm = float(pk_meas.get("hbm_gbs", 6800.0)) * 1e9
@@ -297,7 +279,6 @@ def run_ours(args, rank, world):
     per = lambda name: times.get(name, {"ms": 0.0, "launches": 1})["ms"] / max(times.get(name, {}).get("launches", 1), 1)
     flops_pair = npairs * FLOP_PER_PAIR
     flops_search = ncand * FLOP_PER_CANDIDATE
-    flops64 = n_lip * FLOP64_PER_LIPID_STEP + n_bead * FLOP64_PER_BEAD_STEP
     # candidates for the dominant single kernel: the list search, the pair
     # evaluation and the B-A-O-A update, each against its own bound
     cands = {
@@ -306,13 +287,12 @@ def run_ours(args, rank, world):
         "k_pair_eval": {"ms": per("pairs"), "bound": "alu", "unit": "TFLOP/s", "work": flops_pair, "peak": peak32,
                         "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 x 2070 MHz"},
     }
-    if f64_step:
-        cands["k_baoa_d"] = {"ms": per("integrate_baoa"), "bound": "alu", "unit": "TFLOP/s", "work": flops64,
-                             "peak": FP64_TFLOPS, "peak_source": "nominal GB300 FP64 (no measured FP64 peak)",
-                             "dtype": "f64"}
-    else:
-        cands["k_baoa"] = {"ms": per("integrate_baoa"), "bound": "hbm", "unit": "GB/s",
-                           "work": 240.0 * mem.n, "peak": hbm / 1e9, "peak_source": f"{src} copy bandwidth"}
+    # the B-A-O-A update reads and writes the state and reads the forces; its
+    # increments (rounded like FP64 arithmetic when f64_step) are 64-bit
+    # integer products
+    cands["k_baoa_d" if f64_step else "k_baoa"] = {
+        "ms": per("integrate_baoa"), "bound": "hbm", "unit": "GB/s", "work": 240.0 * mem.n, "peak": hbm / 1e9,
+        "peak_source": f"{src} copy bandwidth"}
     dom = max(cands, key=lambda k: cands[k]["ms"])
     d = cands[dom]
     achieved = d["work"] / (d["ms"] * 1e-3) / (1e12 if d["unit"] == "TFLOP/s" else 1e9)
@@ -330,9 +310,8 @@ def run_ours(args, rank, world):
                  "eval_frac": round(flops_pair / (per("pairs") * 1e-3) / 1e12 / peak32, 4)}
     breakdown = {k: round(v["ms"] / max(v["launches"], 1), 4) for k, v in times.items()}
     # step roofline: each phase at the larger of its HBM time and its
-    # arithmetic time (FP32 pair work; FP64 integrator work when the step
-    # computes its increments in FP64)
-    t_int = max(240.0 * mem.n / hbm, flops64 / (FP64_TFLOPS * 1e12) if f64_step else 0.0)
+    # arithmetic time (FP32 pair work)
+    t_int = 240.0 * mem.n / hbm
     t_rest = (STEP_BYTES_PER_PARTICLE - 240.0 - PAIR_BYTES_PER_PARTICLE) * mem.n / hbm
     t_pair = max(PAIR_BYTES_PER_PARTICLE * mem.n / hbm, (flops_pair + flops_search) / (peak32 * 1e12))
     t_roof = t_int + t_rest + t_pair
@@ -340,8 +319,7 @@ def run_ours(args, rank, world):
                  "frac": round(t_roof * 1e3 / (ms / args.steps), 4), "hbm_gbs": hbm / 1e9, "hbm_source": src,
                  "bytes_per_particle": STEP_BYTES_PER_PARTICLE,
                  "phases_ms": {"integrator": round(t_int * 1e3, 4), "rebuild": round(t_rest * 1e3, 4),
-                               "pairs": round(t_pair * 1e3, 4)},
-                 "fp64_tflops": FP64_TFLOPS if f64_step else None}
+                               "pairs": round(t_pair * 1e3, 4)}}
 
     g.close()
 
@@ -617,7 +595,7 @@ def run_reference(args, rank, world):
 
 
 # revisions of the kernels whose ncu summaries are committed under profiles/
-KERNEL_REV = {"k_pair_search": "search-v7", "k_pair_eval": "eval-v4", "k_baoa_d": "baoa-d-v7"}
+KERNEL_REV = {"k_pair_search": "search-v8", "k_pair_eval": "eval-v5", "k_baoa_d": "baoa-d-v8"}
 
 
 def ensemble_jobs(n_instances: int, steps: int):

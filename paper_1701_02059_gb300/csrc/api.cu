@@ -761,8 +761,8 @@ void Ensemble::drop_graphs() {
 // as a CUDA graph from its third use on (a step that is captured at once
 // would charge a short run for a graph it hardly uses).  Replaying saves about
 // 38 us a step at every size (2,304 particles 145 -> 107 us, 62k 180 -> 142,
-// 4M 2,715 -> 2,677): the host launches one graph instead of 18 kernels, and
-// the gaps between the kernels shrink.
+// 4M 2,715 -> 2,677): the host launches one graph instead of a step's
+// kernels, and the gaps between them shrink.
 template <typename F>
 void Ensemble::step_or_replay(int kind, bool graphs, F&& body) {
     const int p = cur_;

@@ -4,7 +4,8 @@
 // the wider search cutoff for protein pairs and the bond list for linked
 // proteins.
 //
-// GPU design (one CTA of 4 warps per cell):
+// GPU design (one CTA of 4 warps per cell; what the search of the step's path
+// and the FP64 forces do in its place stands at k_pair_search):
 //   1. the mirrors of every neighbouring cell (contiguous after the sort) are
 //      staged in shared memory by 1-D bulk async copies (TMA) completing on
 //      an mbarrier, then moved into the cell's own frame: an exact int32
@@ -14,11 +15,12 @@
 //      their longer tangent extent; each group's warps cull the staged
 //      particles against the group's bounding box (r_s + band) into a
 //      candidate list, then every lane tests the same candidate at once
-//      (broadcast reads) against its own particle, appending hits to a
-//      per-lane queue in shared memory;
+//      (broadcast reads; in the search the tests of 16 particles and 8
+//      candidates are one matrix product) against its own particle,
+//      appending hits to a per-lane queue in shared memory;
 //   3. queued pairs are evaluated with the exact integer displacement
 //      (2^-26 sigma), the type-pair cutoff decided in FP64 inside a 1e-6 sigma
-//      band, and the FP32 (or FP64) potential; force and torque on i are
+//      band, and the FP32 potential; force and torque on i are
 //      accumulated exactly in split integers, so the sum does not depend on
 //      the order or on how candidates are split across warps;
 //   4. every pair is computed from both sides (no atomics to other cells, as
@@ -184,7 +186,6 @@ struct Acc {
         add3(v, p, f, nf, 0, fx, fy, fz);
         add3(v, p, t, nt, 3, tx, ty, tz);
     }
-    __device__ void add_bond(const View& v, int p, float fx, float fy, float fz) { add3(v, p, f, nf, 0, fx, fy, fz); }
 };
 // exact FP64 inclusion decision for a pair inside the cutoff band; m: the
 // bilayer species pair (cls 0)
@@ -1404,9 +1405,9 @@ __device__ inline bool listed_pair(const View& v, const Inst& I, int zc, int pi,
 // lipid type alone).
 // EN: also the energies and virials of the particle's sides of its pairs
 // (11 FP64-pipe instructions a pair in FP64, at 16 cycles each and SM; split
-// integer sums take about 60 FP32 ones: 1M cell, energies included, 0.80 ms
-// in the one-launch kernel, 0.32 ms here on lists of 0.18 ms), as
-// exact sums (hi 2^-32 + lo 2^-52) in es: U, then d . F, both over all listed
+// integer sums take about 60 FP32 ones: forces and energies of the 1M cell in
+// one call 1.17 ms with the one-launch kernel, 0.45 with the lists), as exact
+// sums (hi 2^-32 + lo 2^-52) in es: U, then d . F, both over all listed
 // pairs (each pair counted from both sides).
 // The list's entries t0, t0 + dt, ... (dt > 1: several threads share a
 // particle).

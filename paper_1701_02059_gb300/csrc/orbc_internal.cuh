@@ -392,10 +392,6 @@ __device__ inline float noise_f(unsigned w) {
     float s = (float)(int)(w ^ 0x80000000u);            // w - 2^31
     return 3.46410161513775f * fmaf(s, 2.3283064365386963e-10f, 1.16415321826934814e-10f);
 }
-__device__ inline double noise_d(unsigned w) {
-    double u = (__uint2double_rn(w) + 0.5) * 2.3283064365386963e-10;
-    return 3.4641016151377544 * (u - 0.5);
-}
 
 __device__ inline int find_inst(const int* off, int B, int x) {   // off[B+1], returns b with off[b] <= x < off[b+1]
     int lo = 0, hi = B - 1;

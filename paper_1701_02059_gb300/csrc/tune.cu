@@ -73,7 +73,7 @@ static void cache_store(const char* path, const std::string& key, int K, int cta
 }
 
 // Milliseconds per step of h with K centroids and the evaluation at ctas
-// CTAs per SM: initialisation and two warm-up steps untimed, then `steps`
+// CTAs per SM: initialisation and seven warm-up steps untimed, then `steps`
 // steps timed with events on the stream.
 static double time_tile(const HostInstance& h, int K, int ctas, int steps, cudaStream_t st) {
     HostInstance c = h;
