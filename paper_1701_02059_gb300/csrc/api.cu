@@ -54,6 +54,14 @@ void Ensemble::free_all() {
     bytes_ = 0;
     block_ = nullptr;
     block_left_ = 0;
+    if (skin_event_) {
+        cudaEventSynchronize(skin_event_);    // (the test writes skin_host_)
+        cudaEventDestroy(skin_event_);
+    }
+    skin_event_ = nullptr;
+    if (skin_host_) cudaFreeHost(skin_host_);
+    skin_host_ = nullptr;
+    skin_tests_ = 0;
     if (d_scan_) cudaFreeAsync(d_scan_, stream);
     d_scan_ = nullptr;
     scan_words_ = 0;
@@ -405,6 +413,11 @@ void Ensemble::alloc_core(const std::vector<int>& p0, const std::vector<int>& k0
     CK(cudaMemcpyAsync(d_p0, p0.data(), sizeof(int) * (B + 1), cudaMemcpyHostToDevice, stream));
     CK(cudaMemcpyAsync(d_k0, k0.data(), sizeof(int) * (B + 1), cudaMemcpyHostToDevice, stream));
     CK(cudaMemcpyAsync(d_step, step_h.data(), sizeof(long long) * B, cudaMemcpyHostToDevice, stream));
+    if (any_skin) {
+        CK(cudaHostAlloc(&skin_host_, sizeof(int), cudaHostAllocMapped));
+        *skin_host_ = 0;
+        CK(cudaEventCreateWithFlags(&skin_event_, cudaEventDisableTiming));
+    }
     cur_ = 0;
     prev_adj_valid_ = false;
     csr_valid_ = false;
@@ -864,18 +877,23 @@ void Ensemble::step_body(bool fused, bool baoa_done, bool eval_step) {
     // per-cell displacements of the centroid members
     const int re = prm_h[0].rebuild_every;
     const bool every = re <= 1 && !d_xref;
+    bool due = (re <= 1) || ((step_h[0] + 1) % re == 0);
+    const bool test = !due && d_xref;
+    // (timed, each phase stands alone)
+    const bool ahead = test && !timing;
     if (!baoa_done) {
         tic("integrate_baoa");
-        launch_integrate_first(fused, every);
+        launch_integrate_first(fused, every, ahead);
         toc();
     }
-    bool due = (re <= 1) || ((step_h[0] + 1) % re == 0);
-    if (!due && d_xref) due = displacement_exceeds_skin();
+    if (test && (timing || baoa_done)) launch_skin_test();
+    if (ahead) mirrors(true);
+    if (test) due = skin_exceeded();
     if (due) {
         tic("rebuild");
         rebuild(every);
         toc();
-    } else {
+    } else if (!ahead) {
         tic("mirrors");
         mirrors();
         toc();

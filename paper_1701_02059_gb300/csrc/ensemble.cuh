@@ -240,7 +240,8 @@ public:
     void mstep(const int* cell_of) { mstep_iter(cell_of, -1); }
     // iter < 0: every instance updates; dmax (nullable): largest centroid move per instance
     void mstep_iter(const int* cell_of, int iter, unsigned* dmax = nullptr);
-    bool displacement_exceeds_skin();
+    void launch_skin_test();                        // has a particle moved beyond the skin?
+    bool skin_exceeded();                           // waits for the answer
     void launch_kinetic();
     void lloyd(int iters);                          // the k-means rounds of init_cells
     void estep(int* cell_out, float* lbound, const int* order = nullptr);   // grid search; lbound: second-nearest bounds
@@ -264,11 +265,11 @@ public:
     void alloc_lists();
     void launch_search();
     void clear_overflow();
-    void launch_integrate_first(bool fused, bool msums = false);
+    void launch_integrate_first(bool fused, bool msums = false, bool skin_test = false);
     void launch_kick(bool energies);
     void launch_quench(double dt, double max_move, double max_turn);
     double quench_end();                     // zero velocities; the largest |F|
-    void mirrors();
+    void mirrors(bool unless_exceeded = false);
 
     // timing helpers
     struct Timer;
@@ -358,7 +359,10 @@ public:
     long long* d_msum = nullptr;   // [3][Ktot] M-step sums from the B-A-O-A launch (zero between uses)
     int* d_mcnt = nullptr;         // [Ktot] lipids per cell, same
     int* d_cnt = nullptr;          // [Ktot + 1] particles per cell (zero between uses)
-    int* d_flag = nullptr;         // skin trigger
+    int* d_flag = nullptr;         // skin trigger: the last test that said yes
+    int* skin_host_ = nullptr;     // its copy in mapped host memory (systems with a skin)
+    cudaEvent_t skin_event_ = nullptr;
+    int skin_tests_ = 0;
     long long* d_bbox = nullptr;
     unsigned long long* d_keys = nullptr;
     void* d_sortrec = nullptr;

@@ -249,7 +249,7 @@ __global__ void k_fmax(View v, unsigned long long* __restrict__ out) {
 
 static inline int nblk(long long n, int t) { return (int)((n + t - 1) / t); }
 
-void Ensemble::launch_integrate_first(bool fused, bool msums) {
+void Ensemble::launch_integrate_first(bool fused, bool msums, bool skin_test) {
     long long* ms = msums ? d_msum : nullptr;
     int* mc = msums ? d_mcnt : nullptr;
     if (step_f32()) {
@@ -271,6 +271,7 @@ void Ensemble::launch_integrate_first(bool fused, bool msums) {
         after_baoa_ = fused ? 1 : 0;
         return;
     }
+    if (skin_test) launch_skin_test();
     if (!step_f32()) {
         k_rot_rest<<<152, 128, 0, stream>>>(view(), view(), d_step, fused, d_cell_tmp, d_rot_n);
         launches++;
