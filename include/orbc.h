@@ -127,9 +127,8 @@ typedef struct {
     orbc_precision precision;
     int n_protein_centroids;                       /* > 0: a separate cell set for the     */
                                                    /* proteins (detached cytoskeleton)     */
-    int eval_ctas;                                 /* pair evaluation CTAs per SM: 5 or 7  */
-                                                   /* (8 for one instance), 0 = 7; launch  */
-                                                   /* shape only: results are equal        */
+    int eval_ctas;                                 /* pair evaluation CTAs per SM: 5 or 7, */
+                                                   /* 0 = 7 (launch shape; results equal)  */
     double eps_mem[3][3];                          /* bilayer species pairs: well depth,   */
     double rc_mem[3][3];                           /* cutoff; symmetric, >= 0, 0 = eps or  */
                                                    /* rc_lipid; [0][0] must be 0           */

@@ -1546,19 +1546,51 @@ __device__ __forceinline__ void eval_list(const View& v, int q, const int* __res
     }
 }
 
-// Evaluation: one thread per particle (rank order) over its list (see
-// eval_list).  (Measured on the 4M cell: evaluating from mirrors staged in
-// shared memory per cell, with each list split over two or four threads,
-// took 1.31 ms against 1.06 ms for this kernel.)
-// Compiled for 5 and 7 CTAs per SM (the autotuner's second dimension):
-// seven (72 registers, a few spilled) hide more of the gathers' latency than
-// five without spills, 0.785 against 0.857 ms on the 4M cell.
+// The block's particles by the length of their lists, the longest first:
+// thread t takes the particle of the returned rank.  A warp lasts as long as
+// its longest list, and a cell's beads have a few partners where its lipids
+// have twenty.
+__device__ __forceinline__ int by_length(const int* __restrict__ ncnt, int cap, int N) {
+    __shared__ int bin_n[64];           // by list length + 1, 0: no particle; counts, then starts
+    __shared__ unsigned char order[kPairThreads];
+    static_assert(kListCap + 2 <= 64 && kPairThreads <= 256, "a bin per length, a byte per thread");
+    const int t = threadIdx.x, q = blockIdx.x * kPairThreads + t;
+    if (t < 64) bin_n[t] = 0;
+    __syncthreads();
+    const int bin = q < N ? min(ncnt[q], cap) + 1 : 0;
+    const int r = atomicAdd(&bin_n[bin], 1);
+    __syncthreads();
+    if (t < 32) {
+        const int c0 = bin_n[63 - 2 * t], c1 = bin_n[62 - 2 * t];
+        int x = c0 + c1;
+        for (int off = 1; off < 32; off <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, off);
+            if (t >= off) x += y;
+        }
+        bin_n[63 - 2 * t] = x - c0 - c1;
+        bin_n[62 - 2 * t] = x - c1;
+    }
+    __syncthreads();
+    order[bin_n[bin] + r] = (unsigned char)t;
+    __syncthreads();
+    return blockIdx.x * kPairThreads + order[t];
+}
+
+// Evaluation: one thread per particle over its list (see eval_list), the
+// block's particles by the length of their lists (4M cell 0.62 ms against
+// 0.65 in rank order, with a skin of 0.3 at 1M 0.236 against 0.254; blocks of
+// 256 are slower, 0.68).  (Evaluating from mirrors staged in shared memory per
+// cell, with each list split over two or four threads, took 1.31 ms against
+// 1.06 ms of an earlier form of this kernel.)
+// Compiled for 5 and 7 CTAs per SM (the autotuner's second dimension), 72
+// registers at seven; at six 0.70 ms on the 4M cell, at eight (64 registers,
+// more spills) 0.66.
 // MP: the batch holds band-3 or glycophorin (eval_list).
 template <int Z, bool S0, int MINB, bool MP = false, bool EN = false, bool ONE = false>
-__global__ void __launch_bounds__(128, MINB)
+__global__ void __launch_bounds__(kPairThreads, MINB)
     k_pair_eval(View v, const int* __restrict__ nlist, const int* __restrict__ ncnt, int cap,
                 const int4* __restrict__ rowoff, long long* __restrict__ energy, const __grid_constant__ Inst one) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    const int q = by_length(ncnt, cap, v.N);
     if (!EN && q >= v.N) return;
     const size_t N = v.N;
     SplitAcc af[3], at[3];
@@ -1924,7 +1956,7 @@ void Ensemble::launch_pairs(bool energies, bool dump, bool one_launch) {
         // listed pairs beyond the lists' capacity
         launch_search();
         tic("pairs");
-        const int ng = (int)((N + 127) / 128);
+        const int ng = (int)((N + kPairThreads - 1) / kPairThreads);
         // the batch's launch shape: the choice of its largest instance
         int ctas = prm_h[0].eval_ctas, nmax = -1;
         for (int b = 0; b < B; b++)
@@ -1940,13 +1972,13 @@ void Ensemble::launch_pairs(bool energies, bool dump, bool one_launch) {
 #define ORBC_EVAL_N(Z, S, MP, ONE)                                                                                          \
     do {                                                                                                                    \
         if (energies)                                                                                                       \
-            k_pair_eval<Z, S, 5, MP, true, ONE><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, d_energy, inst_h[0]); \
+            k_pair_eval<Z, S, 5, MP, true, ONE><<<ng, kPairThreads, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, d_energy, inst_h[0]); \
         else if (sh > 0)                                                                                                    \
             k_pair_eval_split<Z, S, MP, ONE><<<nsp, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, sh, inst_h[0]); \
         else if (ctas == 5)                                                                                                 \
-            k_pair_eval<Z, S, 5, MP, false, ONE><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, nullptr, inst_h[0]); \
+            k_pair_eval<Z, S, 5, MP, false, ONE><<<ng, kPairThreads, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, nullptr, inst_h[0]); \
         else                                                                                                                \
-            k_pair_eval<Z, S, ONE ? 8 : 7, MP, false, ONE><<<ng, 128, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, nullptr, inst_h[0]); \
+            k_pair_eval<Z, S, 7, MP, false, ONE><<<ng, kPairThreads, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, nullptr, inst_h[0]); \
     } while (0)
 #define ORBC_EVAL(Z, S, MP)                                                                                                 \
     do {                                                                                                                    \
