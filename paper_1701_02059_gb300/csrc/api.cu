@@ -355,7 +355,6 @@ void Ensemble::lay_core(bool any_skin) {
     d_F = alloc<long long>((size_t)3 * N);
     d_T = alloc<long long>((size_t)3 * N);
     d_Fbig = alloc<long long>((size_t)6 * N);
-    d_mq = alloc<int4>(N);
     d_mo = alloc<float4>(N);
     d_mqr = alloc<int4>(N);
     d_mor = alloc<float4>(N);

@@ -1910,10 +1910,16 @@ static void prefer_shared_all() {
 
 void Ensemble::alloc_lists() {
     list_cap = kListCap;
-    ovf_cap = std::max(N / 4, 4096);
+    // the overflow list and the unranked mirrors of large cells share their
+    // memory: the mirrors are read by the launch that writes them or the next
+    // one of the rebuild, the overflow list is written by the search after it.
+    // So the list holds the pairs that the tests' margin adds (up to about one
+    // a particle) beside the N / 4 it is meant for
+    ovf_cap = (int)std::min<long long>(std::max(N / 4, 4096) + 2ll * N, 0x7fffffff);
     d_nlist = alloc<int>((size_t)list_cap * N);
     d_ncnt = alloc<int>(N);
     d_novf = alloc<int2>(ovf_cap);
+    d_mq = (int4*)d_novf;
     d_novf_n = alloc<int>(1);
     d_rowoff = alloc<int4>(adj_cap);
     d_sflag = alloc<unsigned char>(N);

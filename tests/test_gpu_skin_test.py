@@ -33,3 +33,20 @@ def test_skin_equals_every_step(n, skin, every):
         got = run(n, rebuild_every=every, skin=skin, **mode)
         for k in ("pos", "vel", "ori", "angvel"):
             assert np.array_equal(got[k], want[k]), (mode, k)
+
+
+def test_wide_skin_beyond_the_lists():
+    """A skin that sends about one listed pair in ten beyond the lists' 32
+    entries: the overflow list holds them, also those that the search lists
+    within its margin only."""
+    mem = M.biconcave(n_lipids=446_378, n_junctions=4_125, n_centroids=8_192, seed=2, name="rbc-500k")
+    out = []
+    for kw in ({}, {"rebuild_every": 20, "skin": 0.35}):
+        with G.System(G.make_params(kT=mem.kT, n_centroids=mem.n_centroids, box=mem.box, periodic=mem.periodic, seed=4,
+                                    **kw)) as g:
+            g.load_membrane(mem)
+            g.init_cells()
+            g.integrate(3)
+            out.append(g.state())
+    for k in ("pos", "vel", "ori", "angvel"):
+        assert np.array_equal(out[0][k], out[1][k]), k
