@@ -2062,7 +2062,9 @@ void Ensemble::launch_pairs(bool energies, bool dump, bool one_launch) {
     launches++;
     CK(cudaGetLastError());
     toc();
-    if (!dump) launch_volume(energies);
+    // (also after a dump: it writes F and T anew, and the next step starts
+    // from them)
+    launch_volume(energies);
 }
 
 void Ensemble::launch_pairs_step(bool msums) {
