@@ -1,5 +1,6 @@
 // Host orchestration of the hot path and the C ABI declared in orbc.h.
 #include "abi_common.cuh"
+#include "capture.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -769,59 +770,58 @@ void Ensemble::drop_graphs() {
         }
 }
 
+Ensemble::HostStep Ensemble::host_step() const {
+    return {cur_, after_baoa_, bbox_ready_, ovf_clean_, csr_valid_, prev_adj_valid_, cells_valid, forces_valid,
+            list_valid, launches, n_rebuilds};
+}
+
+void Ensemble::set_host_step(const HostStep& h) {
+    cur_ = h.cur;
+    after_baoa_ = h.after_baoa;
+    bbox_ready_ = h.bbox_ready;
+    ovf_clean_ = h.ovf_clean;
+    csr_valid_ = h.csr_valid;
+    prev_adj_valid_ = h.prev_adj_valid;
+    cells_valid = h.cells_valid;
+    forces_valid = h.forces_valid;
+    list_valid = h.list_valid;
+    launches = h.launches;
+    n_rebuilds = h.n_rebuilds;
+}
+
 // One step (body: its launches, swapping the state buffers once), replayed
 // as a CUDA graph from its third use on (a step that is captured at once
 // would charge a short run for a graph it hardly uses).  Replaying saves about
 // 38 us a step at every size (2,304 particles 145 -> 107 us, 62k 180 -> 142,
 // 4M 2,715 -> 2,677): the host launches one graph instead of a step's
-// kernels, and the gaps between them shrink.
+// kernels, and the gaps between them shrink.  A replay leaves the host's
+// notes as the body would.
 template <typename F>
 void Ensemble::step_or_replay(int kind, bool graphs, F&& body) {
-    const int p = cur_;
-    StepGraph& G = graph_[kind][p];
+    StepGraph& G = graph_[kind][cur_];
     if (!graphs || graphs_off_ || (!G.exec && G.uses++ < 2)) {
         body();
         return;
     }
+    const HostStep h0 = host_step();
     if (!G.exec) {
-        const long long l0 = launches, r0 = n_rebuilds;
-        if (cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-            cudaGetLastError();
+        G.exec = capture_graph(stream, body, [&] {
+            G.after = host_step();
+            G.after.launches -= h0.launches;
+            G.after.n_rebuilds -= h0.n_rebuilds;
+            set_host_step(h0);
+        });
+        if (!G.exec) {
             graphs_off_ = true;       // e.g. the legacy default stream
-            body();
-            return;
-        }
-        cudaGraph_t g = nullptr;
-        try {
-            body();
-        } catch (...) {
-            cudaStreamEndCapture(stream, &g);
-            if (g) cudaGraphDestroy(g);
-            cudaGetLastError();
-            cur_ = p;
-            throw;
-        }
-        CK(cudaStreamEndCapture(stream, &g));
-        const cudaError_t e = cudaGraphInstantiate(&G.exec, g, 0);
-        cudaGraphDestroy(g);
-        // capturing ran no kernel: restore the host-side state it advanced
-        G.launches = launches - l0;
-        launches = l0;
-        n_rebuilds = r0;
-        cur_ = p;
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            G.exec = nullptr;
-            graphs_off_ = true;
             body();
             return;
         }
     }
     CK(cudaGraphLaunch(G.exec, stream));
-    cur_ = p ^ 1;   // the step's gather swapped the state buffers
-    launches += G.launches;
-    n_rebuilds++;
-    csr_valid_ = false;
+    HostStep h = G.after;
+    h.launches += h0.launches;
+    h.n_rebuilds += h0.n_rebuilds;
+    set_host_step(h);
 }
 
 void Ensemble::integrate(int nsteps, bool graphs) {

@@ -299,9 +299,18 @@ private:
     size_t lay_bytes_ = 0;
     // one step as a CUDA graph, by kind (first step of a call, a later one,
     // quench step) and state-buffer parity
+    // what a step leaves on the host: the current state buffer, notes on what
+    // its launches left ready, counts
+    struct HostStep {
+        int cur, after_baoa;
+        bool bbox_ready, ovf_clean, csr_valid, prev_adj_valid, cells_valid, forces_valid, list_valid;
+        long long launches, n_rebuilds;
+    };
+    HostStep host_step() const;
+    void set_host_step(const HostStep& h);
     struct StepGraph {
         cudaGraphExec_t exec = nullptr;
-        long long launches = 0;
+        HostStep after = {};       // after the step, its launches and rebuilds counted from it
         int uses = 0;
     };
     StepGraph graph_[3][2];
