@@ -805,14 +805,21 @@ void Ensemble::step_or_replay(int kind, bool graphs, F&& body) {
     }
     const HostStep h0 = host_step();
     if (!G.exec) {
-        G.exec = capture_graph(stream, body, [&] {
-            G.after = host_step();
-            G.after.launches -= h0.launches;
-            G.after.n_rebuilds -= h0.n_rebuilds;
-            set_host_step(h0);
-        });
+        const cudaStream_t own = stream;
+        G.exec = capture_graph(
+            [&](cudaStream_t s) {
+                stream = s;
+                body();
+            },
+            [&] {
+                stream = own;
+                G.after = host_step();
+                G.after.launches -= h0.launches;
+                G.after.n_rebuilds -= h0.n_rebuilds;
+                set_host_step(h0);
+            });
         if (!G.exec) {
-            graphs_off_ = true;       // e.g. the legacy default stream
+            graphs_off_ = true;
             body();
             return;
         }

@@ -314,7 +314,7 @@ private:
         int uses = 0;
     };
     StepGraph graph_[3][2];
-    bool graphs_off_ = false;      // the stream cannot be captured
+    bool graphs_off_ = false;      // a capture failed
     double quench_key_[3] = {0, 0, 0};
     template <typename F> void step_or_replay(int kind, bool graphs, F&& body);
     template <typename T> T* alloc(size_t count);

@@ -1,8 +1,10 @@
 // capture_graph (capture.cuh) against a fake of the CUDA calls it makes:
-// argv[1] is the call that fails ("none", "begin", "end", "end_null",
-// "instantiate"; "throw": the body).  Prints whether a graph came back, what
+// argv[1] is the call that fails ("none", "stream", "begin", "end",
+// "end_null", "instantiate"; "throw": the body).  Prints whether a graph came back, what
 // the host's note holds afterwards (1 while the body has advanced it), the
-// body's runs, the captures left open, the graphs left and a pending error.
+// body's runs, the captures left open, the graphs and streams left, a pending
+// error, and whether each capture was of a non-blocking stream made for it,
+// which the body got.
 #include "capture.cuh"
 
 #include <cstdio>
@@ -10,11 +12,25 @@
 #include <stdexcept>
 
 static const char* fail = "none";
-static int open_captures = 0, graphs = 0, error = 0;
+static int open_captures = 0, graphs = 0, streams = 0, error = 0, own = 1;
+static cudaStream_t const made = (cudaStream_t)&streams;
 static int hit(const char* what, cudaError_t e) { return std::strcmp(fail, what) ? 0 : (error = e); }
 
 extern "C" {
-cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) {
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned flags) {
+    if (hit("stream", cudaErrorMemoryAllocation)) return (cudaError_t)error;
+    own &= flags == cudaStreamNonBlocking;
+    streams++;
+    *s = made;
+    return cudaSuccess;
+}
+cudaError_t cudaStreamDestroy(cudaStream_t s) {
+    own &= s == made;
+    streams--;
+    return cudaSuccess;
+}
+cudaError_t cudaStreamBeginCapture(cudaStream_t s, cudaStreamCaptureMode) {
+    own &= s == made;
     if (hit("begin", cudaErrorStreamCaptureUnsupported)) return (cudaError_t)error;
     open_captures++;
     return cudaSuccess;
@@ -43,8 +59,8 @@ int main(int argc, char** argv) {
     cudaGraphExec_t exec = nullptr;
     try {
         exec = orbc::capture_graph(
-            (cudaStream_t)&note,
-            [&] {
+            [&](cudaStream_t s) {
+                own &= s == made;
                 runs++;
                 note = 1;
                 if (!std::strcmp(fail, "throw")) throw std::runtime_error("body");
@@ -53,6 +69,6 @@ int main(int argc, char** argv) {
     } catch (const std::runtime_error&) {
         thrown = 1;
     }
-    std::printf("graph %d note %d runs %d thrown %d open %d graphs %d error %d\n", exec != nullptr, note, runs, thrown,
-                open_captures, graphs, error);
+    std::printf("graph %d note %d runs %d thrown %d open %d graphs %d streams %d error %d own %d\n", exec != nullptr, note, runs, thrown,
+                open_captures, graphs, streams, error, own);
 }

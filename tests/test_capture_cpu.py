@@ -1,7 +1,8 @@
 """A step's capture (csrc/capture.cuh) when one of the CUDA calls fails, on the
 host with a fake of them: no failure leaves the host's notes advanced, a
-capture open, a graph behind or an error pending, and the caller learns that
-there is no graph."""
+capture open, a graph or a stream behind or an error pending, and the caller
+learns that there is no graph.  The captured stream is the capture's own: a
+caller's stream may carry other handles' work."""
 import os
 import subprocess
 
@@ -24,10 +25,11 @@ def check(tmp_path_factory):
     return run
 
 
-@pytest.mark.parametrize("fail", ["none", "begin", "end", "end_null", "instantiate", "throw"])
+@pytest.mark.parametrize("fail", ["none", "stream", "begin", "end", "end_null", "instantiate", "throw"])
 def test_host_state(check, fail):
     r = check(fail)
     assert r["graph"] == (fail == "none")
     assert r["thrown"] == (fail == "throw")
-    assert r["runs"] == (fail != "begin")
-    assert (r["note"], r["open"], r["graphs"], r["error"]) == (0, 0, 0, 0)
+    assert r["runs"] == (fail not in ("stream", "begin"))
+    assert (r["note"], r["open"], r["graphs"], r["streams"], r["error"]) == (0, 0, 0, 0, 0)
+    assert r["own"] == 1
