@@ -27,7 +27,7 @@ def steps(mem, seed, stream):
 
 
 def test_two_threads():
-    mems = [M.vesicle(3000, 5, f=2, chain_beads=5, n_centroids=50), M.patch(2, seed=7)]
+    mems = [M.vesicle(n, 5, f=2, chain_beads=5, n_centroids=n // 60) for n in (3000, 1300)]
     want = [steps(m, k, None) for k, m in enumerate(mems)]
     stream = torch.cuda.Stream()
     got, err = [None, None], []
