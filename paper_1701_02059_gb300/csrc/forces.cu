@@ -1174,10 +1174,14 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
             // staged particles into the cell's frame (exact) and the tangent
             // frame (FP32), with their list entries
             // (a warp per neighbouring cell: with the whole CTA on one cell
-            // after the other, half of its warps found nothing to do)
-            for (int q = warp; q < m; q += kPairThreads / 32) {
+            // after the other, half of its warps found nothing to do; the
+            // whole CTA for the few cells of a pass that large ones fill,
+            // where warps would go without one: the search of eight cells of
+            // 1,359 particles 885 us against 1,024)
+            const bool wide = m < kPairThreads / 32;
+            for (int q = wide ? 0 : warp; q < m; q += wide ? 1 : kPairThreads / 32) {
                 const SNbr inf = nb[q];
-                for (int j = inf.base + lane; j < inf.base + inf.cnt; j += 32) {
+                for (int j = inf.base + (wide ? tid : lane); j < inf.base + inf.cnt; j += wide ? kPairThreads : 32) {
                     const int4 rj = reinterpret_cast<const int4*>(sY)[j];
                     const int x = (int)((unsigned)rj.x + (unsigned)inf.ox);
                     const int y = (int)((unsigned)rj.y + (unsigned)inf.oy);
