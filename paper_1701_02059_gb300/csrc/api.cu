@@ -178,6 +178,8 @@ unsigned Ensemble::read_status(bool clear) {
     CK(cudaStreamSynchronize(stream));
     // a flagged launch may have left the neighbour lists partial
     if (s) list_valid = false;
+    if (s & kStatusListOverflow) lists_full = true;
+    else if (list_valid) lists_full = false;
     if (clear && s) CK(cudaMemsetAsync(d_status, 0, sizeof(unsigned), stream));
     return s;
 }
@@ -421,6 +423,7 @@ void Ensemble::alloc_core(const std::vector<int>& p0, const std::vector<int>& k0
     cur_ = 0;
     prev_adj_valid_ = false;
     csr_valid_ = false;
+    lists_full = false;
     vol_any = false;
     for (const Inst& I : inst_h) vol_any = vol_any || I.vol_on;
     reset_scratch();
@@ -1510,9 +1513,13 @@ int orbc_compute_forces(orbc_system* s, double* energies_out) {
     unsigned st = 0;
     int rc = guarded(s, [&] {
         sync_device(s);
-        s->ens->compute_forces(energies_out != nullptr);
+        // energies of more pairs than the lists hold come from the kernel
+        // without lists, at once when the last search is known to have met
+        // that (a search and an evaluation in vain double the call)
+        const bool one_launch = energies_out && s->ens->lists_full;
+        s->ens->compute_forces(energies_out != nullptr, one_launch);
         st = s->ens->read_status(true);
-        if (energies_out && (st & kStatusListOverflow)) {
+        if (energies_out && !one_launch && (st & kStatusListOverflow)) {
             s->ens->compute_forces(true, true);
             st = s->ens->read_status(true);
         }

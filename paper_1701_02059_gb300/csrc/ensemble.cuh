@@ -400,6 +400,7 @@ public:
     int4* d_rowoff = nullptr;                // [adj_cap] exact offset c_l - c_k of each row entry
     int list_cap = 0, ovf_cap = 0;
     bool list_valid = false;
+    bool lists_full = false;                 // the last search found more pairs than the lists hold
     long long* d_xref = nullptr;
     long long* d_energy = nullptr;           // [B][8] fixed-point sums
     long long* d_vol = nullptr;              // [B][2] sum of (x - c).n (floors at 2^-24, remainders at 2^-48)
