@@ -131,8 +131,6 @@ void Ensemble::setup_from(const std::vector<const Snapshot*>& list) {
         inst_h[b].g0 = Gtot;
         Gtot += (long long)inst_h[b].gdim[0] * inst_h[b].gdim[1] * inst_h[b].gdim[2];
     }
-    d_gstart = alloc<int>(Gtot + 1);
-    d_gcount = alloc<int>(Gtot + 1);
     CK(cudaMemcpyAsync(d_inst, inst_h.data(), sizeof(Inst) * B, cudaMemcpyHostToDevice, stream));
     for (int b = 0; b < B; b++) {
         const Snapshot& s = *list[b];
@@ -158,6 +156,9 @@ void Ensemble::setup_from(const std::vector<const Snapshot*>& list) {
     std::vector<BondSpec> bl(B);
     for (int b = 0; b < B; b++) bl[b] = BondSpec{&list[b]->bonds, &list[b]->r0, &list[b]->kb};
     upload_bonds(bl, p0);
+    // (after the bonds, whose room in the arrays' block they would take)
+    d_gstart = alloc<int>(Gtot + 1);
+    d_gcount = alloc<int>(Gtot + 1);
     // warm the scan scratch (outputs into arrays the next rebuild rewrites)
     scan_exclusive(d_gcount, d_gstart, Gtot + 1);
     scan_exclusive(d_cnt, d_adj_ptr, Ktot + 1);
