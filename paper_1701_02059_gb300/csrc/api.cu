@@ -756,13 +756,14 @@ void Ensemble::compute_forces(bool energies, bool one_launch) {
     forces_valid = true;
 }
 
-void Ensemble::energies(std::vector<double>& out) {
+void Ensemble::energies(double out[5]) {
     std::vector<long long> e((size_t)8 * B);
     CK(cudaMemcpyAsync(e.data(), d_energy, sizeof(long long) * 8 * B, cudaMemcpyDeviceToHost, stream));
     CK(cudaStreamSynchronize(stream));
-    out.assign((size_t)5 * B, 0.0);
-    for (int b = 0; b < B; b++)
-        for (int q = 0; q < 5; q++) out[(size_t)5 * b + q] = (double)e[(size_t)8 * b + q] * kForceUnit;
+    for (int q = 0; q < 5; q++) {
+        out[q] = 0.0;
+        for (int b = 0; b < B; b++) out[q] += (double)e[(size_t)8 * b + q] * kForceUnit;
+    }
 }
 
 void Ensemble::drop_graphs() {
@@ -1524,15 +1525,7 @@ int orbc_compute_forces(orbc_system* s, double* energies_out) {
             st = s->ens->read_status(true);
         }
         if (st) s->ens->forces_valid = false;
-        if (!st && energies_out) {
-            std::vector<double> e;
-            s->ens->energies(e);
-            // the membrane's totals over the instances of its batch
-            for (int q = 0; q < 5; q++) {
-                energies_out[q] = 0.0;
-                for (int b = 0; b < s->ens->B; b++) energies_out[q] += e[(size_t)5 * b + q];
-            }
-        }
+        if (!st && energies_out) s->ens->energies(energies_out);
     });
     if (rc == ORBC_OK && st) return fail(s, status_code(st), "device status " + std::to_string(st));
     return rc;

@@ -168,7 +168,10 @@ public:
     void drop_graphs();
     // velocity quench; returns the largest |F| at the end
     double quench(int nsteps, double dt, double max_move, double max_turn, bool graphs);
-    void energies(std::vector<double>& out); // [B][5] after compute_forces(true)
+    // after compute_forces(true): the energies and virial of the membrane whose
+    // cell sets the batch holds (only the sum over the instances is one: the
+    // evaluation adds a block's pairs to the instance of its first particle)
+    void energies(double out[5]);
     // volume constraint of instance b (kv = 0: off); forces become stale
     void set_volume(int b, double kv, double v0, double area, const double xc[3]);
     // enclosed volume of instance b for the given area per lipid and centre
@@ -402,7 +405,7 @@ public:
     bool list_valid = false;
     bool lists_full = false;                 // the last search found more pairs than the lists hold
     long long* d_xref = nullptr;
-    long long* d_energy = nullptr;           // [B][8] fixed-point sums
+    long long* d_energy = nullptr;           // [B][8] fixed-point sums (see energies())
     long long* d_vol = nullptr;              // [B][2] sum of (x - c).n (floors at 2^-24, remainders at 2^-48)
     bool vol_any = false;                    // some instance has the volume constraint on
     long long* d_step = nullptr;             // [B]
