@@ -955,47 +955,6 @@ void Ensemble::get_forces(int b, double* f, double* t) {
     CK(cudaFreeAsync(tmp, stream));
 }
 
-void Ensemble::get_cells(int b, int* cell_of_id, unsigned* slot_ids, double* centroids, int* cell_start,
-                         double* radius, int* adj_ptr, int* adj) {
-    adjacency_csr();
-    cell_radii();
-    const Inst& I = inst_h[b];
-    const int n = I.n, K = I.K;
-    std::vector<unsigned> ids(n);
-    std::vector<int> cl(n);
-    CK(cudaMemcpyAsync(ids.data(), d_id[cur_] + I.p0, sizeof(unsigned) * n, cudaMemcpyDeviceToHost, stream));
-    CK(cudaMemcpyAsync(cl.data(), d_cell + I.p0, sizeof(int) * n, cudaMemcpyDeviceToHost, stream));
-    std::vector<int> cs(K + 1), ap(K + 1);
-    CK(cudaMemcpyAsync(cs.data(), d_cell_start + I.k0, sizeof(int) * (K + 1), cudaMemcpyDeviceToHost, stream));
-    CK(cudaMemcpyAsync(ap.data(), d_adj_ptr + I.k0, sizeof(int) * (K + 1), cudaMemcpyDeviceToHost, stream));
-    std::vector<double> R(K);
-    CK(cudaMemcpyAsync(R.data(), d_R2 + I.k0, sizeof(double) * K, cudaMemcpyDeviceToHost, stream));
-    std::vector<long long> c((size_t)3 * K);
-    for (int a = 0; a < 3; a++)
-        CK(cudaMemcpyAsync(c.data() + (size_t)a * K, d_cq + (size_t)a * Ktot + I.k0, sizeof(long long) * K,
-                           cudaMemcpyDeviceToHost, stream));
-    CK(cudaStreamSynchronize(stream));
-    for (int i = 0; i < n; i++) {
-        if (cell_of_id) cell_of_id[ids[i]] = cl[i] - I.k0;
-        if (slot_ids) slot_ids[i] = ids[i];
-    }
-    if (centroids)
-        for (int k = 0; k < K; k++)
-            for (int a = 0; a < 3; a++) centroids[(size_t)3 * k + a] = (double)c[(size_t)a * K + k] * kGridInv;
-    if (cell_start) for (int k = 0; k <= K; k++) cell_start[k] = cs[k] - I.p0;
-    // (the device keeps the squares; the host's square root is correctly rounded too)
-    if (radius) std::transform(R.begin(), R.end(), radius, [](double r2) { return std::sqrt(r2); });
-    if (adj_ptr) for (int k = 0; k <= K; k++) adj_ptr[k] = ap[k] - ap[0];
-    if (adj) {
-        long long L = ap[K] - ap[0];
-        std::vector<int> a((size_t)std::max(L, 1ll));
-        if (L > 0)
-            CK(cudaMemcpyAsync(a.data(), d_adj + ap[0], sizeof(int) * L, cudaMemcpyDeviceToHost, stream));
-        CK(cudaStreamSynchronize(stream));
-        for (long long q = 0; q < L; q++) adj[q] = a[q] - I.k0;
-    }
-}
-
 // The cells of every instance of the batch as one list (global cell
 // numbers, ids offset by each instance's id_base): a membrane with separate
 // protein cells, or a single instance.
@@ -1040,16 +999,6 @@ long long Ensemble::adjacency_len_all() {
     int ap[2];
     CK(cudaMemcpyAsync(&ap[0], d_adj_ptr, sizeof(int), cudaMemcpyDeviceToHost, stream));
     CK(cudaMemcpyAsync(&ap[1], d_adj_ptr + Ktot, sizeof(int), cudaMemcpyDeviceToHost, stream));
-    CK(cudaStreamSynchronize(stream));
-    return ap[1] - ap[0];
-}
-
-long long Ensemble::adjacency_len(int b) {
-    adjacency_csr();
-    const Inst& I = inst_h[b];
-    int ap[2];
-    CK(cudaMemcpyAsync(&ap[0], d_adj_ptr + I.k0, sizeof(int), cudaMemcpyDeviceToHost, stream));
-    CK(cudaMemcpyAsync(&ap[1], d_adj_ptr + I.k0 + I.K, sizeof(int), cudaMemcpyDeviceToHost, stream));
     CK(cudaStreamSynchronize(stream));
     return ap[1] - ap[0];
 }

@@ -60,15 +60,15 @@ __global__ void k_mstep_accum(View v, const int* __restrict__ cell_of, long long
 }
 
 // c_k <- c_k + floor((2 S_k + n_k) / (2 n_k)); periodic axes wrap into [0, L).
-// dmax (nullable): the largest move of an instance's centroids, as FP32 bits
-// rounded up (warp-reduced before the atomics).
+// cmove: the move of each centroid; dmax: the largest one of an instance's, as
+// FP32 bits rounded up (warp-reduced before the atomics).
 __global__ void k_mstep_finish(View v, long long* __restrict__ S, int* __restrict__ cnt, int iter,
                                unsigned* __restrict__ dmax, float* __restrict__ cmove) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= v.Ktot) return;
     int b = find_inst(v.inst_k0, v.B, k);
     const Inst& I = v.inst[b];
-    int n = (iter < 0 || iter < I.n_lloyd) ? cnt[k] : 0;   // instances past their k-means rounds keep c
+    int n = iter < I.n_lloyd ? cnt[k] : 0;   // instances past their k-means rounds keep c
     float mv2 = 0.f;
     for (int a = 0; a < 3; a++) {
         long long c = v.cq[(size_t)a * v.Ktot + k];
@@ -82,12 +82,11 @@ __global__ void k_mstep_finish(View v, long long* __restrict__ S, int* __restric
         S[(size_t)a * v.Ktot + k] = 0;
     }
     cnt[k] = 0;
-    if (cmove) cmove[k] = sqrtf(mv2) * 1.0001f + 1e-6f;
-    if (dmax) {
-        const unsigned grp = __match_any_sync(__activemask(), b);
-        const unsigned mv = __reduce_max_sync(grp, __float_as_uint(sqrtf(mv2) * 1.0001f + 1e-6f));
-        if ((int)(threadIdx.x & 31) == __ffs(grp) - 1) atomicMax(&dmax[b], mv);
-    }
+    const float move = sqrtf(mv2) * 1.0001f + 1e-6f;
+    cmove[k] = move;
+    const unsigned grp = __match_any_sync(__activemask(), b);
+    const unsigned mv = __reduce_max_sync(grp, __float_as_uint(move));
+    if ((int)(threadIdx.x & 31) == __ffs(grp) - 1) atomicMax(&dmax[b], mv);
 }
 
 // Rebuild M-step on cell-sorted particles: one warp per cell sums its members'
@@ -2186,13 +2185,13 @@ void Ensemble::build_grid() {
     CK(cudaGetLastError());
 }
 
-void Ensemble::mstep_iter(const int* cell_of, int iter, unsigned* dmax) {
+void Ensemble::mstep_iter(const int* cell_of, int iter) {
     View v = view();
     k_mstep_accum<<<nblk(N, 256), 256, 0, stream>>>(v, cell_of, d_S, d_cnt);
     launches++;
     CK(cudaGetLastError());
-    if (dmax) CK(cudaMemsetAsync(dmax, 0, sizeof(unsigned) * B, stream));
-    k_mstep_finish<<<nblk(Ktot, 256), 256, 0, stream>>>(v, d_S, d_cnt, iter, dmax, dmax ? d_cmove : nullptr);
+    CK(cudaMemsetAsync(d_dmax, 0, sizeof(unsigned) * B, stream));
+    k_mstep_finish<<<nblk(Ktot, 256), 256, 0, stream>>>(v, d_S, d_cnt, iter, d_dmax, d_cmove);
     launches++;
     CK(cudaGetLastError());
 }
@@ -2272,7 +2271,7 @@ void Ensemble::lloyd(int iters) {
         else estep_bounded(d_cell);
         toc();
         tic("mstep");
-        mstep_iter(d_cell, it, d_dmax);
+        mstep_iter(d_cell, it);
         toc();
     }
     swap_state();

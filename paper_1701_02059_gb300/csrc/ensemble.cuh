@@ -187,9 +187,6 @@ public:
     // per-slot int64 array q of instance b to FP64 [n][3] in id order (device)
     void to_id_order(int b, const long long* q, double unit, double* out);
     void get_forces_device(int b, double* f, double* t);
-    void get_cells(int b, int* cell_of_id, unsigned* slot_ids, double* centroids, int* cell_start, double* radius,
-                   int* adj_ptr, int* adj);
-    long long adjacency_len(int b);
     // every instance of the batch as one list (global cell numbers, ids offset by id_base)
     void get_cells_all(int* cell_of_id, unsigned* slot_ids, double* centroids, int* cell_start, double* radius,
                        int* adj_ptr, int* adj);
@@ -240,9 +237,7 @@ public:
     // phases
     void reset_scratch();       // the scratch that each step's launches leave ready for the next
     void build_grid();
-    void mstep(const int* cell_of) { mstep_iter(cell_of, -1); }
-    // iter < 0: every instance updates; dmax (nullable): largest centroid move per instance
-    void mstep_iter(const int* cell_of, int iter, unsigned* dmax = nullptr);
+    void mstep_iter(const int* cell_of, int iter);  // k-means round iter
     void launch_skin_test();                        // has a particle moved beyond the skin?
     bool skin_exceeded();                           // waits for the answer
     void launch_kinetic();

@@ -19,7 +19,7 @@ namespace orbc {
 // without a second pass over memory.  The previous step is then not yet
 // counted in steps[], so this step's index is steps[b] + 1.
 template <typename T, bool FUSED>
-__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 4) k_baoa(View v, const long long* __restrict__ steps,
+__global__ void __launch_bounds__(256, 4) k_baoa(View v, const long long* __restrict__ steps,
                                                  long long* __restrict__ msum, int* __restrict__ mcnt) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= v.N) return;
