@@ -2141,10 +2141,14 @@ __global__ void __launch_bounds__(256, 6) k_adj_warp(View v, const unsigned* __r
         AdjDesc d;
         d.start = v.cell_start[j];
         d.cnt = v.cell_start[j + 1] - d.start;
-        d.ox = (int)(unsigned)(unsigned long long)((dx + (1ll << (kMirrorShift - 1))) >> kMirrorShift);
-        d.oy = (int)(unsigned)(unsigned long long)((dy + (1ll << (kMirrorShift - 1))) >> kMirrorShift);
-        d.oz = (int)(unsigned)(unsigned long long)((dz + (1ll << (kMirrorShift - 1))) >> kMirrorShift);
-        d.cell = j;
+        const long long off[3] = {(dx + (1ll << (kMirrorShift - 1))) >> kMirrorShift,
+                                  (dy + (1ll << (kMirrorShift - 1))) >> kMirrorShift,
+                                  (dz + (1ll << (kMirrorShift - 1))) >> kMirrorShift};
+        d.ox = (int)(unsigned)(unsigned long long)off[0];
+        d.oy = (int)(unsigned)(unsigned long long)off[1];
+        d.oz = (int)(unsigned)(unsigned long long)off[2];
+        d.cell_turns = (unsigned)j;
+        for (int a = 0; a < 3; a++) d.cell_turns |= turn_code(off[a]) << (kCellBits + 2 * a);
         v.adjd[(size_t)k * kAdjRow + rk[u]] = d;
     }
     if (lane == 0) {

@@ -9,8 +9,9 @@
 //   1. the mirrors of every neighbouring cell (contiguous after the sort) are
 //      staged in shared memory by 1-D bulk async copies (TMA) completing on
 //      an mbarrier, then moved into the cell's own frame: an exact int32
-//      offset (wrap-around arithmetic) and an FP32 copy rotated into the
-//      cell's tangent frame (normal = mean lipid director) for filtering;
+//      offset (wrap-around arithmetic) and, for filtering, an FP32 copy
+//      (without the wrap) rotated into the cell's tangent frame (normal =
+//      mean lipid director);
 //   2. the cell's particles are split into compact groups of <= 32 along
 //      their longer tangent extent; each group's warps cull the staged
 //      particles against the group's bounding box (r_s + band) into a
@@ -297,6 +298,7 @@ struct NbrInfo {
     int cnt;
     int start;      // global slot of the first particle
     int ox, oy, oz; // exact offset c_l - c_k at 2^-26 sigma (wrap-around int32)
+    float fx, fy, fz;   // the same without the wrap, in sigma (FP32)
 };
 
 template <bool S0, typename IC = Inst>
@@ -368,7 +370,7 @@ __global__ void __launch_bounds__(kPairThreads, 5) k_pairs(View v, long long* __
                     AdjDesc d;
                     if (has) {
                         d = row[nn];
-                        l = d.cell;
+                        l = d.cell();
                         st = d.start;
                         c = d.cnt;
                         if (lane == 0) { st += na_off; c -= na_off; }
@@ -389,6 +391,7 @@ __global__ void __launch_bounds__(kPairThreads, 5) k_pairs(View v, long long* __
                         NbrInfo inf;
                         inf.base = excl; inf.cnt = take; inf.start = st;
                         inf.ox = d.ox; inf.oy = d.oy; inf.oz = d.oz;
+                        whole_offset(d, inf.fx, inf.fy, inf.fz);
                         nb[lane] = inf;
                     }
                     const unsigned selfm = __ballot_sync(0xffffffffu, staged && l == k);
@@ -498,12 +501,13 @@ __global__ void __launch_bounds__(kPairThreads, 5) k_pairs(View v, long long* __
                 const NbrInfo inf = nb[q];
                 for (int j = inf.base + tid; j < inf.base + inf.cnt; j += kPairThreads) {
                     int4 rj = sy[j];
+                    float4 y;
+                    F.apply(fmaf((float)rj.x, kMirrorUnit, inf.fx), fmaf((float)rj.y, kMirrorUnit, inf.fy),
+                            fmaf((float)rj.z, kMirrorUnit, inf.fz), y.x, y.y, y.z);
                     rj.x = (int)((unsigned)rj.x + (unsigned)inf.ox);
                     rj.y = (int)((unsigned)rj.y + (unsigned)inf.oy);
                     rj.z = (int)((unsigned)rj.z + (unsigned)inf.oz);
                     sy[j] = rj;
-                    float4 y;
-                    F.apply(rj.x * kMirrorUnit, rj.y * kMirrorUnit, rj.z * kMirrorUnit, y.x, y.y, y.z);
                     y.w = 0.f;
                     sY[j] = y;
                 }
@@ -695,7 +699,7 @@ constexpr int kRowShift = 26;
 
 struct SNbr {
     int base, cnt, start, row;
-    int ox, oy, oz;
+    float ox, oy, oz;       // c_l - c_k without the wrap, in sigma
 };
 
 // The FP32 constants of the pair terms, held in registers by the evaluation.
@@ -1016,7 +1020,7 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
                 AdjDesc d;
                 if (has) {
                     d = row[nn];
-                    l = d.cell;
+                    l = d.cell();
                     st = d.start;
                     c = d.cnt;
                     // each row's exact offset, written where the row is first
@@ -1041,7 +1045,7 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
                 if (staged) {
                     SNbr inf;
                     inf.base = excl; inf.cnt = take; inf.start = st; inf.row = nn;
-                    inf.ox = d.ox; inf.oy = d.oy; inf.oz = d.oz;
+                    whole_offset(d, inf.ox, inf.oy, inf.oz);
                     nb[lane] = inf;
                 }
                 const unsigned selfm = __ballot_sync(0xffffffffu, staged && l == k);
@@ -1171,8 +1175,8 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
                 return;
             }
             phase ^= 1u;
-            // staged particles into the cell's frame (exact) and the tangent
-            // frame (FP32), with their list entries
+            // staged particles into the cell's tangent frame (FP32), with
+            // their list entries
             // (a warp per neighbouring cell: with the whole CTA on one cell
             // after the other, half of its warps found nothing to do; the
             // whole CTA for the few cells of a pass that large ones fill,
@@ -1183,11 +1187,9 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
                 const SNbr inf = nb[q];
                 for (int j = inf.base + (wide ? tid : lane); j < inf.base + inf.cnt; j += wide ? kPairThreads : 32) {
                     const int4 rj = reinterpret_cast<const int4*>(sY)[j];
-                    const int x = (int)((unsigned)rj.x + (unsigned)inf.ox);
-                    const int y = (int)((unsigned)rj.y + (unsigned)inf.oy);
-                    const int z = (int)((unsigned)rj.z + (unsigned)inf.oz);
                     float4 w;
-                    F.apply(x * kMirrorUnit, y * kMirrorUnit, z * kMirrorUnit, w.x, w.y, w.z);
+                    F.apply(fmaf((float)rj.x, kMirrorUnit, inf.ox), fmaf((float)rj.y, kMirrorUnit, inf.oy),
+                            fmaf((float)rj.z, kMirrorUnit, inf.oz), w.x, w.y, w.z);
                     const int tj = rj.w & 0xff;
                     w.w = MP ? (tj == kLipid ? 0.0f : (bilayer(tj) ? 2.0f : 1.0f)) : (bilayer(tj) ? 0.0f : 1.0f);
                     sY[j] = w;

@@ -140,17 +140,43 @@ struct Inst {
 };
 
 // ---------------------------------------------------------------- packed device arrays
-// What the pair kernel needs to stage neighbouring cell l of cell k: its
-// particle range and the exact offset c_l - c_k (minimum image) at the mirror
-// resolution 2^-26 sigma, as wrap-around int32.
 // Longest row of neighbouring cells; rows are stored at this fixed stride.
 constexpr int kAdjRow = 64;
 
+// What the pair kernel needs to stage neighbouring cell l of cell k: its
+// particle range and the exact offset c_l - c_k (minimum image) at the mirror
+// resolution 2^-26 sigma, as wrap-around int32: exact for the displacement of
+// two close particles.  The staged coordinates that the distance filters work
+// on must not wrap (cells may reach 32 sigma, and two particles 64 sigma apart
+// would look close): each axis' turns of 64 sigma stand in two bits (turn_code)
+// above the cell's number (K < 2^26: the rows of 2^26 cells alone would take
+// more than the device holds).
+constexpr int kCellBits = 26;
 struct AdjDesc {
     int start, cnt;
     int ox, oy, oz;
-    int cell;
+    unsigned cell_turns;
+    __device__ int cell() const { return (int)(cell_turns & ((1u << kCellBits) - 1u)); }
 };
+// off: an axis' whole offset at 2^-26 sigma.  0, 1 (+64), 2 (-64) or 3: so far
+// (96 sigma) that no particle of the one cell is close to one of the other.
+__device__ inline unsigned turn_code(long long off) {
+    const long long t = (off - (long long)(int)(unsigned)(unsigned long long)off) >> 32;
+    return t == 0 ? 0u : (t == 1 ? 1u : (t == -1 ? 2u : 3u));
+}
+// The offset without the wrap, in sigma (FP32).  (Ordinary cells have no turns.)
+__device__ inline void whole_offset(const AdjDesc& d, float& x, float& y, float& z) {
+    x = (float)d.ox * kMirrorUnit;
+    y = (float)d.oy * kMirrorUnit;
+    z = (float)d.oz * kMirrorUnit;
+    const unsigned t = d.cell_turns >> kCellBits;
+    if (t) {
+        auto turn = [](unsigned c) { return c == 0u ? 0.f : (c == 1u ? 64.f : (c == 2u ? -64.f : 1.0e6f)); };
+        x += turn(t & 3u);
+        y += turn((t >> 2) & 3u);
+        z += turn(t >> 4);
+    }
+}
 
 struct View {
     int B;                      // instances
