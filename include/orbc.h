@@ -176,7 +176,8 @@ ORBC_API int orbc_create(const orbc_params* params, void* cuda_stream, orbc_syst
  * a permutation of 0..n-1.  The arrays are validated and copied on the host;
  * the device set-up (allocation, upload, bond lists) runs at the first call
  * that needs the device, which then reports its errors (ORBC_E_NOMEM,
- * ORBC_E_CUDA, and the bond limit of orbc_set_bonds as ORBC_E_ARG).
+ * ORBC_E_CUDA, and as ORBC_E_ARG the bond limit of orbc_set_bonds and, with
+ * FP32 forces, more than 67,108,864 particles).
  * Invalidates cells and forces.
  * Errors: ORBC_E_ARG (null pointer, n < 1, non-finite value, |x| >= 4096
  * sigma, unknown type, ids not a permutation), ORBC_E_NOMEM. */

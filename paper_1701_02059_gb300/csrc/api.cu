@@ -546,6 +546,11 @@ void Ensemble::setup(const std::vector<const HostInstance*>& list) {
     B = (int)list.size();
     if (B < 1) throw ArgError("no instance");
     precision = list[0]->prm.precision;
+    // (the instances are one membrane's cell sets)
+    long long total = 0;
+    for (const HostInstance* hp : list) total += hp->n;
+    if (!force_f64() && total > 1ll << kListBits)
+        throw ArgError("more than 67,108,864 particles of a membrane (neighbour lists; FP64 forces take more)");
     N = 0; Ktot = 0;
     inst_h.assign(B, Inst());
     prm_h.clear();

@@ -687,15 +687,23 @@ __global__ void __launch_bounds__(kPairThreads, 5) k_pairs(View v, long long* __
 // the evaluation has no barriers and full lanes.  Forces are the same exact
 // integer sums as in the one-launch kernel, whatever order the list holds.
 //
-// List entry: (row << 26) | q, where q indexes the rank-ordered mirrors and
-// row is the neighbouring cell's place in the row of the particle's cell,
-// whose exact offset c_l - c_k the search writes to rowoff.  Lists hold
+// List entry: (row << 26) | q, where q indexes the rank-ordered mirrors from the
+// membrane's first slot on (a batch may hold more than 2^26 particles, a
+// membrane with lists not: Ensemble::setup) and row is the neighbouring cell's
+// place in the row of the particle's cell, whose exact offset c_l - c_k the
+// search writes to rowoff.  Lists hold
 // kListCap entries per particle (t-major: entry t of particle q at t N + q);
 // further entries go to an overflow list evaluated with integer atomics.
 constexpr int kSearchStage = 640;
 constexpr int kFragRow = 12;        // floats between fragment rows (48 B: no bank conflicts)
 constexpr int kListCap = 32;
-constexpr int kRowShift = 26;
+constexpr int kRowShift = kListBits;
+
+// The slot that the list entries of instance I count from: the first one of
+// its membrane (of both its cell sets).
+__device__ inline int list_base(const View& v, const Inst& I) {
+    return I.partner < 0 ? I.p0 : min(I.p0, v.inst[I.partner].p0);
+}
 
 struct SNbr {
     int base, cnt, start, row;
@@ -956,10 +964,12 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
                   const __grid_constant__ Inst one) {
     // sY: staged mirrors (int4 by the bulk copy), then in the tangent frame
     //     (FP32), w = 0 for a bilayer particle and 1 for a cytoskeleton protein
-    // sQ: the list entry of each staged particle
+    // sQ: the list entry of each staged particle (DIRECT: its slot in the
+    //     rank-ordered mirrors, its row in sR)
     // cand: per warp, the byte offsets (16 j) in sY of the culled candidates
     __shared__ alignas(16) float4 sY[kSearchStage];
     __shared__ int sQ[kSearchStage];
+    __shared__ unsigned char sR[DIRECT ? kSearchStage : 1];
     __shared__ alignas(16) unsigned short cand[kPairThreads / 32][kSearchStage];
     __shared__ SNbr nb[kMaxNbr];
     __shared__ int s_cnt[kPairThreads];
@@ -990,6 +1000,7 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
         __syncwarp();
     };
     const float rsb = I.rsf + sk, rs2f = rsb * rsb;
+    const int qbase = DIRECT || ONE ? 0 : list_base(v, I);
     const float cw = I.rcf_wca + sk, cp = I.rcf_pp + sk;
     // candidate c of 32 goes to the fragment column whose hit is bit c; the
     // byte transpose within four lanes that brings a row's hits to one lane
@@ -1193,7 +1204,9 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
                     const int tj = rj.w & 0xff;
                     w.w = MP ? (tj == kLipid ? 0.0f : (bilayer(tj) ? 2.0f : 1.0f)) : (bilayer(tj) ? 0.0f : 1.0f);
                     sY[j] = w;
-                    sQ[j] = (inf.row << kRowShift) | (inf.start + (j - inf.base));
+                    const int at = inf.start + (j - inf.base);
+                    if (DIRECT) sR[j] = (unsigned char)inf.row;
+                    sQ[j] = DIRECT ? at : (inf.row << kRowShift) | (at - qbase);
                 }
             }
             __syncthreads();
@@ -1279,9 +1292,9 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
                             if (hits) {
                                 const int u = __ffs(hits) - 1;
                                 hits &= hits - 1u;
-                                const int e = sQ[cand[warp][c0 + u] >> 4];
-                                const AdjDesc& d = row[(unsigned)e >> kRowShift];
-                                in = own_pair_d(v, I, C, qi, pi, idi, e & ((1 << kRowShift) - 1), d.ox, d.oy, d.oz, pj, code);
+                                const int j = cand[warp][c0 + u] >> 4;
+                                const AdjDesc& d = row[sR[j]];
+                                in = own_pair_d(v, I, C, qi, pi, idi, sQ[j], d.ox, d.oy, d.oz, pj, code);
                             }
                             const unsigned m2 = __ballot_sync(0xffffffffu, in);
                             if (in) {
@@ -1433,6 +1446,7 @@ __device__ __forceinline__ void eval_list(const View& v, int q, const int* __res
     const PairC C(I);
     const int zc = (Z > 0) ? Z : C.zeta;
     const int4* __restrict__ ro = rowoff + (size_t)k * kAdjRow;
+    const int qbase = one ? 0 : list_base(v, I);
     const int n = min(ncnt[q], cap);
     // a particle without bonds has no excluded pair: its list skips the test
     // (the lipid-only instantiation runs only when no bilayer particle has a
@@ -1454,7 +1468,7 @@ __device__ __forceinline__ void eval_list(const View& v, int q, const int* __res
     for (int t = t0; t < n; t += dt) {
         const int e = e_next;
         if (t + dt < n) e_next = __ldcs(nlist + (size_t)(t + dt) * N + q);
-        const int qj = e & ((1 << kRowShift) - 1);
+        const int qj = qbase + (e & ((1 << kRowShift) - 1));
         const int4 o = __ldg(ro + ((unsigned)e >> kRowShift));
         const int4 mj = __ldg(v.mqr + qj);
         const float4 oj = __ldg(v.mor + qj);
@@ -1774,7 +1788,7 @@ __device__ inline void pair_overflow(const View& v, const int2* __restrict__ ovf
         const Inst& I = v.inst[b];
         const int zc = (Z > 0) ? Z : I.zeta;
         const float rcl = sqrtf(I.rc2f_ll), rcw = sqrtf(I.rc2f_wca), rcp = sqrtf(I.rc2f_pp);
-        const int qj = e & ((1 << kRowShift) - 1);
+        const int qj = list_base(v, I) + (e & ((1 << kRowShift) - 1));
         const int4 o = rowoff[(size_t)k * kAdjRow + ((unsigned)e >> kRowShift)];
         float f[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, U, d[3];
         if (!listed_pair<Z, S0>(v, I, zc, pi, ti, qi, oi, v.mqr[qj], v.mor[qj], o, (rcl - kCutBand) * (rcl - kCutBand),

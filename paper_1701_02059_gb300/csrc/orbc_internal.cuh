@@ -152,6 +152,7 @@ constexpr int kAdjRow = 64;
 // above the cell's number (K < 2^26: the rows of 2^26 cells alone would take
 // more than the device holds).
 constexpr int kCellBits = 26;
+constexpr int kListBits = 26;     // bits of a particle in the neighbour lists' entries
 struct AdjDesc {
     int start, cnt;
     int ox, oy, oz;
