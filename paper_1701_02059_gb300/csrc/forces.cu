@@ -687,9 +687,9 @@ __global__ void __launch_bounds__(kPairThreads, 5) k_pairs(View v, long long* __
 // the evaluation has no barriers and full lanes.  Forces are the same exact
 // integer sums as in the one-launch kernel, whatever order the list holds.
 //
-// List entry: (row << 26) | q, where q indexes the rank-ordered mirrors from the
-// membrane's first slot on (a batch may hold more than 2^26 particles, a
-// membrane with lists not: Ensemble::setup) and row is the neighbouring cell's
+// List entry: (row << 26) | q, where q indexes the rank-ordered mirrors (in a
+// batch of more than 2^26 particles from the membrane's first slot on: FAR; a
+// membrane has no more, see Ensemble::setup) and row is the neighbouring cell's
 // place in the row of the particle's cell, whose exact offset c_l - c_k the
 // search writes to rowoff.  Lists hold
 // kListCap entries per particle (t-major: entry t of particle q at t N + q);
@@ -699,8 +699,11 @@ constexpr int kFragRow = 12;        // floats between fragment rows (48 B: no ba
 constexpr int kListCap = 32;
 constexpr int kRowShift = kListBits;
 
-// The slot that the list entries of instance I count from: the first one of
-// its membrane (of both its cell sets).
+// The slot that the list entries of instance I count from in a FAR batch: the
+// first one of its membrane (of both its cell sets).  A form of its own: in
+// every batch, one more register and addition a pair make the steps of 400,000
+// particles in twelve membranes 1 per cent slower.
+inline __host__ __device__ bool far_batch(int N) { return N > 1 << kListBits; }
 __device__ inline int list_base(const View& v, const Inst& I) {
     return I.partner < 0 ? I.p0 : min(I.p0, v.inst[I.partner].p0);
 }
@@ -957,7 +960,7 @@ __device__ inline void mma_tf32(float d[4], const float a[4], float b0, float b1
 // DIRECT (FP64 forces): the pairs found are evaluated at once (pair_terms_d);
 // F and T are zero before the launch.  EN adds U_pair and the virial of the
 // cell's instance to energy [B][8].
-template <bool MP, bool DIRECT = false, bool Z4 = true, bool S0 = false, bool EN = false, bool ONE = false>
+template <bool MP, bool DIRECT = false, bool Z4 = true, bool S0 = false, bool EN = false, bool ONE = false, bool FAR = false>
 __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
     k_pair_search(View v, int* __restrict__ nlist, int* __restrict__ ncnt, int cap, int2* __restrict__ ovf,
                   int* __restrict__ novf, int ovf_cap, int4* __restrict__ rowoff, long long* __restrict__ energy,
@@ -1000,7 +1003,7 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
         __syncwarp();
     };
     const float rsb = I.rsf + sk, rs2f = rsb * rsb;
-    const int qbase = DIRECT || ONE ? 0 : list_base(v, I);
+    const int qbase = FAR ? list_base(v, I) : 0;
     const float cw = I.rcf_wca + sk, cp = I.rcf_pp + sk;
     // candidate c of 32 goes to the fragment column whose hit is bit c; the
     // byte transpose within four lanes that brings a row's hits to one lane
@@ -1430,7 +1433,7 @@ __device__ inline bool listed_pair(const View& v, const Inst& I, int zc, int pi,
 // pairs (each pair counted from both sides).
 // The list's entries t0, t0 + dt, ... (dt > 1: several threads share a
 // particle).
-template <int Z, bool S0, bool MP = false, bool EN = false>
+template <int Z, bool S0, bool MP = false, bool EN = false, bool FAR = false>
 __device__ __forceinline__ void eval_list(const View& v, int q, const int* __restrict__ nlist,
                                           const int* __restrict__ ncnt, int cap, const int4* __restrict__ rowoff,
                                           SplitAcc af[3], SplitAcc at[3], int& nterm, bool& big, int& pi_out,
@@ -1446,7 +1449,7 @@ __device__ __forceinline__ void eval_list(const View& v, int q, const int* __res
     const PairC C(I);
     const int zc = (Z > 0) ? Z : C.zeta;
     const int4* __restrict__ ro = rowoff + (size_t)k * kAdjRow;
-    const int qbase = one ? 0 : list_base(v, I);
+    const int qbase = FAR ? list_base(v, I) : 0;
     const int n = min(ncnt[q], cap);
     // a particle without bonds has no excluded pair: its list skips the test
     // (the lipid-only instantiation runs only when no bilayer particle has a
@@ -1606,7 +1609,7 @@ __device__ __forceinline__ int by_length(const int* __restrict__ ncnt, int cap, 
 // registers at seven; at six 0.70 ms on the 4M cell, at eight (64 registers,
 // more spills) 0.66.
 // MP: the batch holds band-3 or glycophorin (eval_list).
-template <int Z, bool S0, int MINB, bool MP = false, bool EN = false, bool ONE = false>
+template <int Z, bool S0, int MINB, bool MP = false, bool EN = false, bool ONE = false, bool FAR = false>
 __global__ void __launch_bounds__(kPairThreads, MINB)
     k_pair_eval(View v, const int* __restrict__ nlist, const int* __restrict__ ncnt, int cap,
                 const int4* __restrict__ rowoff, long long* __restrict__ energy, const __grid_constant__ Inst one) {
@@ -1640,7 +1643,7 @@ __global__ void __launch_bounds__(kPairThreads, MINB)
         }
         if (q >= v.N) return;
     } else {
-        eval_list<Z, S0, MP>(v, q, nlist, ncnt, cap, rowoff, af, at, nterm, big, pi, ONE ? &one : nullptr);
+        eval_list<Z, S0, MP, false, FAR>(v, q, nlist, ncnt, cap, rowoff, af, at, nterm, big, pi, ONE ? &one : nullptr);
     }
 #pragma unroll
     for (int a = 0; a < 3; a++) {
@@ -1788,7 +1791,7 @@ __device__ inline void pair_overflow(const View& v, const int2* __restrict__ ovf
         const Inst& I = v.inst[b];
         const int zc = (Z > 0) ? Z : I.zeta;
         const float rcl = sqrtf(I.rc2f_ll), rcw = sqrtf(I.rc2f_wca), rcp = sqrtf(I.rc2f_pp);
-        const int qj = list_base(v, I) + (e & ((1 << kRowShift) - 1));
+        const int qj = (far_batch(v.N) ? list_base(v, I) : 0) + (e & ((1 << kRowShift) - 1));
         const int4 o = rowoff[(size_t)k * kAdjRow + ((unsigned)e >> kRowShift)];
         float f[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, U, d[3];
         if (!listed_pair<Z, S0>(v, I, zc, pi, ti, qi, oi, v.mqr[qj], v.mor[qj], o, (rcl - kCutBand) * (rcl - kCutBand),
@@ -1958,11 +1961,18 @@ void Ensemble::launch_search() {
     if (list_valid) return;
     tic("pair_search");
     clear_overflow();
-#define ORBC_SEARCH(MP, ONE)                                                                                              \
-    k_pair_search<MP, false, true, false, false, ONE><<<Ktot, kPairThreads, 0, stream>>>(                                 \
+#define ORBC_SEARCH(MP, ONE, FAR)                                                                                         \
+    k_pair_search<MP, false, true, false, false, ONE, FAR><<<Ktot, kPairThreads, 0, stream>>>(                                 \
         view(), d_nlist, d_ncnt, list_cap, d_novf, d_novf_n, ovf_cap, d_rowoff, nullptr, inst_h[0])
-    if (any_mp()) { if (B == 1) ORBC_SEARCH(true, true); else ORBC_SEARCH(true, false); }
-    else { if (B == 1) ORBC_SEARCH(false, true); else ORBC_SEARCH(false, false); }
+    if (any_mp()) {
+        if (B == 1) ORBC_SEARCH(true, true, false);
+        else if (far_batch(N)) ORBC_SEARCH(true, false, true);
+        else ORBC_SEARCH(true, false, false);
+    } else {
+        if (B == 1) ORBC_SEARCH(false, true, false);
+        else if (far_batch(N)) ORBC_SEARCH(false, false, true);
+        else ORBC_SEARCH(false, false, false);
+    }
 #undef ORBC_SEARCH
     launches++;
     CK(cudaGetLastError());
@@ -2009,6 +2019,8 @@ void Ensemble::launch_pairs(bool energies, bool dump, bool one_launch) {
 #define ORBC_EVAL(Z, S, MP)                                                                                                 \
     do {                                                                                                                    \
         if (B == 1) ORBC_EVAL_N(Z, S, MP, true);                                                                            \
+        else if (far_batch(N)) /* (an arena's: no energies) */                                                              \
+            k_pair_eval<Z, S, 7, MP, false, false, true><<<ng, kPairThreads, 0, stream>>>(v, d_nlist, d_ncnt, list_cap, d_rowoff, nullptr, inst_h[0]); \
         else ORBC_EVAL_N(Z, S, MP, false);                                                                                  \
     } while (0)
         if (any_mp()) {
