@@ -2316,14 +2316,19 @@ void Ensemble::morton_relabel() {
     CK(cudaGetLastError());
 }
 
+// (As many cells as a block has threads: 60,000 particles in 1,000 cells 120 us
+// a step, 126 by the five launches, which cells beyond the limit take: 1,025
+// cells 124, 1,100 126.)
 bool Ensemble::small_cells() const { return B == 1 && Ktot <= kSmallK && Gtot < kSmallG; }
 
-// Whether k_build_cells does the rebuild's last part, or the sort, the gather
-// (a thread per particle) and the cells' properties a launch each: up to a
-// mean of 300 particles a cell the one launch was the faster one (rebuild of
-// 620k particles: 61 a cell 172 against 186 us, 150: 204 and 222, 300: 246 and
-// 256); few cells of thousands would leave each to one warp.
-bool Ensemble::build_fused() const { return N <= 256ll * Ktot; }
+// Whether k_build_cells does the rebuild's last part, or the sort (a block per
+// cell), the gather (a thread per particle) and the cells' properties a launch
+// each.  The line lies where cells begin to exceed the 128 particles that a
+// warp holds: steps of 60,000 particles at a mean of 61 a cell 118 us against
+// 122, 95 118 / 122, 105 137 / 130, 128 159 / 130; of 605,000 417 / 432, 425 /
+// 424, 435 / 431, 455 / 457; of 1,445,000 857 / 893, 862 / 886, 874 / 886,
+// 950 / 949.
+bool Ensemble::build_fused() const { return N <= 100ll * Ktot; }
 
 // order: the slots in an order that keeps neighbours together (nullable).
 void Ensemble::finish_cells(bool sums_ready, const int* order) {

@@ -1195,7 +1195,7 @@ __global__ void __launch_bounds__(kPairThreads, DIRECT ? 4 : 8)
             // after the other, half of its warps found nothing to do; the
             // whole CTA for the few cells of a pass that large ones fill,
             // where warps would go without one: the search of eight cells of
-            // 1,359 particles 885 us against 1,024)
+            // 1,359 particles 0.9 ms against 1.0)
             const bool wide = m < kPairThreads / 32;
             for (int q = wide ? 0 : warp; q < m; q += wide ? 1 : kPairThreads / 32) {
                 const SNbr inf = nb[q];
