@@ -918,7 +918,7 @@ void Ensemble::step_body(bool fused, bool baoa_done, bool eval_step) {
 }
 
 // ---------------------------------------------------------------- getters
-// Host copies in id order: converted on the device (k_to_id_order), then one
+// Host copies in id order: converted on the device (k_gather_ids), then one
 // copy per array.
 void Ensemble::get_state(int b, double* pos, double* vel, double* ori, double* angvel, long long* step) {
     const Inst& I = inst_h[b];

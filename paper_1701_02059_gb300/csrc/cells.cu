@@ -1301,9 +1301,9 @@ __global__ void k_hist(int N, const int* __restrict__ cell, int* __restrict__ cn
 
 // Slot of each particle inside its cell's range (in any order across warps;
 // the per-cell sort that follows restores the storage order).  The counts
-// are taken down to zero, ready for the next histogram.  In a rebuild
-// (B > 0 <= N) it also does what the launches before it left to a later one:
-// see ScratchReset.
+// are taken down to zero, ready for the next histogram.  In a rebuild (B > 0,
+// B <= N) it also does what the launches before it left to a later one: see
+// ScratchReset.
 __global__ void k_scatter(int N, const int* __restrict__ cell, const int* __restrict__ start, int* __restrict__ cnt,
                           int* __restrict__ tmp, int B, ScratchReset z) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;

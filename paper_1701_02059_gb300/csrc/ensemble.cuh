@@ -94,9 +94,6 @@ struct BondSpec {
     const std::vector<double>* kb;
 };
 
-// One instance's carried state in device buffers of its own: what a packed
-// batch needs to continue the instance bit for bit after it is re-packed
-// (state, forces, centroids, cell ownership in the cell-sorted order).
 // Threads per block of a kernel that works thread by thread or warp by warp
 // (no block-wide step): 64 while the launch has fewer threads than the chip
 // holds, so that they spread over every SM evenly (62k particles in blocks of
@@ -116,6 +113,9 @@ struct ScratchReset {
     int *fb_count, *rot_n, *novf;
 };
 
+// One instance's carried state in device buffers of its own: what a packed
+// batch needs to continue the instance bit for bit after it is re-packed
+// (state, forces, centroids, cell ownership in the cell-sorted order).
 struct Snapshot {
     Inst inst;                                // descriptor (p0, k0, g0 of the batch it came from)
     Params prm;
@@ -377,9 +377,9 @@ public:
     int *d_cell_new = nullptr, *d_perm = nullptr, *d_cell_tmp = nullptr;
     unsigned* d_rmax = nullptr;              // [B] largest cell radius (FP32 bits)
     float* d_rho = nullptr;                  // [Ktot] distance to the nearest non-neighbour centroid
-    float* d_lbound = nullptr;
+    float* d_lbound = nullptr;               // [N] k-means: lower bound on the second-nearest centroid
     float* d_cmove = nullptr;                // [Ktot] k-means: move of each centroid in the last M-step
-    unsigned* d_gmove = nullptr;             // [Gtot] k-means: largest move of the centroids in a grid cell               // [N] k-means: lower bound on the second-nearest centroid
+    unsigned* d_gmove = nullptr;             // [Gtot] k-means: largest move of the centroids in a grid cell
     float4* d_cf = nullptr;                  // [Ktot] FP32 centroids by cell
     float4* d_cframe = nullptr;              // [Ktot][3] cell frames (pair kernels)
     unsigned char* d_grank = nullptr;        // [N] pair-kernel group ranks

@@ -32,9 +32,10 @@ __global__ void __launch_bounds__(256, 4) k_baoa(View v, const long long* __rest
 // FP64-accurate increments on the integer pipes.  With the rotation in FP64
 // the kernel was bound by the FP64 pipe (85% busy): 0.81 ms on the 4M cell,
 // against 0.14 ms for its 240 B per particle at the copy bandwidth; with the
-// fixed-point rotation it is bound by integer issue: 0.47 ms with
-// k_rot_rest.  Four CTAs per SM (64 registers, some spilled) against 0.48 ms
-// at three.
+// fixed-point rotation it is bound by integer issue: 0.47 ms with the
+// left-over rotations, 0.41 since one instance's constants are a kernel
+// argument.  Four CTAs per SM (64 registers, some spilled); at three and at
+// five 0.43 ms.
 template <bool FUSED, bool ONE>
 __global__ void __launch_bounds__(256, 4) k_baoa_d(View v, const long long* __restrict__ steps,
                                                    long long* __restrict__ msum, int* __restrict__ mcnt,

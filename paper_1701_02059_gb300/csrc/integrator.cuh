@@ -361,7 +361,8 @@ static __device__ __noinline__ void rot_fp64(const long long* ni, const long lon
 // evaluation with the update in its epilogue) listed: from the state of v
 // into the state arrays of o, thread `at` of `threads`.  About 1e-3 of the
 // lipids; taken inside k_baoa_d, 4% of its warps would wait for one lane's
-// FP64 code (0.49-0.50 against 0.47 ms for both launches on the 4M cell).
+// FP64 code (0.49-0.50 against 0.47 ms for both launches on the 4M cell, each
+// with the constants read from memory).
 __device__ inline void rot_rest(const View& v, const View& o, const long long* __restrict__ steps, int fused,
                                 const int* __restrict__ rot_list, const int* __restrict__ rot_n, int at, int threads) {
     const int n = *rot_n;
