@@ -61,11 +61,13 @@ typedef enum {
  * exact 2^-32 fixed point, so sums do not depend on the order of the terms. */
 typedef enum {
     ORBC_F32_FORCE_F64_STATE = 0,  /* FP32 pair/bond forces; FP64 integrator increments (angular kicks,
-                                      Ornstein-Uhlenbeck update, Cayley map, renormalisation; the
-                                      translational kick, the drifts and the velocity's Ornstein-Uhlenbeck
-                                      update as exact integer products of the int64 state with the FP64
-                                      constants, rounded once) and FP64
-                                      per-particle energy/virial partials                               */
+                                      Ornstein-Uhlenbeck update, Cayley map, renormalisation, taken in
+                                      fixed point where that gives the FP64 arithmetic's results bit for
+                                      bit; the translational kick, the drifts and the velocity's
+                                      Ornstein-Uhlenbeck update as exact integer products of the int64
+                                      state with the FP64 constants, rounded once); energies and virials
+                                      as exact sums of the FP32 pair terms, FP64 bond terms and integer
+                                      kinetic terms                                                     */
     ORBC_F64_ALL = 1,              /* FP64 pair/bond forces and FP64 integrator increments             */
     ORBC_F32_FORCE_F32_STEP = 2    /* FP32 pair/bond forces and FP32 integrator increments (rounded onto
                                       the same int64 grid): the narrowest, fastest variant             */
@@ -200,11 +202,17 @@ ORBC_API int orbc_set_bonds(orbc_system* s, int nb, const int* ij, const double*
  * nearest-centroid assignment and centroid update; then the two-level
  * reorder (centroids along a Morton curve, particles stably by cell) and the
  * neighbouring-cell lists.  Errors: ORBC_E_ARG (more centroids than bilayer particles),
- * ORBC_E_STATE (no particles, or a cell with more than 64 neighbouring cells:
+ * ORBC_E_STATE (no particles; a cell with more than 64 neighbouring cells:
  * each cell's row is held at a fixed stride of 64, which a membrane with
  * about 60 particles per cell fills to about 8; a particle cloud in 3-D or a
- * large skin can exceed it, and fewer, larger cells bring it back),
- * ORBC_E_NOMEM, ORBC_E_CUDA. */
+ * large skin can exceed it, and fewer, larger cells bring it back; a particle
+ * more than 32 sigma from its cell's centroid, which smaller cells bring back),
+ * ORBC_E_NOMEM, ORBC_E_CUDA.
+ * On a periodic axis the cells have to be small against the box: a pair is
+ * looked for through the nearest image of its cells, so two cells that touch
+ * both directly and through the box miss pairs (no error tells; the
+ * 2,304-particle patch, 36 sigma wide, is right with 16 cells and more, wrong
+ * with 11). */
 ORBC_API int orbc_init_cells(orbc_system* s, const double* centroids);
 
 /* One update of the Voronoi cells ("Spatial Searching Algorithm": online EM
