@@ -595,7 +595,7 @@ def run_reference(args, rank, world):
 
 
 # revisions of the kernels whose ncu summaries are committed under profiles/
-KERNEL_REV = {"k_pair_search": "search-v8", "k_pair_eval": "eval-v6", "k_baoa_d": "baoa-d-v8"}
+KERNEL_REV = {"k_pair_search": "search-v9", "k_pair_eval": "eval-v6", "k_baoa_d": "baoa-d-v8"}
 
 
 def ensemble_jobs(n_instances: int, steps: int):
